@@ -487,6 +487,63 @@ __device__ __forceinline__ double warp_sum64(double v) {
   return v;
 }
 
+// A sum kept as h + l in two FP32 words (about 48 bits): the window pass adds
+// its row terms this way. FP64 issues at 1/64 of the FP32 rate on this chip (2
+// lane operations per clock and SM), and the 24 FP64 instructions that each of
+// the 16 epilogue warps took per item (conversions, products and three
+// 32-lane reductions) were about 6100 cycles of it, more than the rest of an
+// item. As pairs the same work is about 170 FP32 instructions per warp. The
+// terms are FP32 row sums, 2^-24 off by themselves. With the columns and row
+// quadrants outside an item's ranges skipped, the iteration went from 88.1 to
+// 79.2 us on the 1e6 x 128 workload (k = 100, b = 4096).
+struct Pair32 {
+  float h, l;
+};
+// a b exactly
+__device__ __forceinline__ Pair32 pair_mul(float a, float b) {
+  const float h = __fmul_rn(a, b);
+  return Pair32{h, __fmaf_rn(a, b, -h)};
+}
+__device__ __forceinline__ Pair32 pair_scale(Pair32 x, float w) {
+  const float h = __fmul_rn(x.h, w);
+  return Pair32{h, __fmaf_rn(x.l, w, __fmaf_rn(x.h, w, -h))};
+}
+__device__ __forceinline__ Pair32 pair_add(Pair32 a, Pair32 b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float t = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));   // a.h + b.h = s + e
+  return Pair32{s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+}
+__device__ __forceinline__ Pair32 warp_pair_sum(Pair32 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = pair_add(v, Pair32{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+  return v;
+}
+
+// The window pass's sum of one warp's 32 rows: pairs where kernel values are
+// at most 1 (Gaussian, Laplacian), FP64 where they have FP32's whole range.
+template <int KIND> struct WindowSum {
+  using T = Pair32;
+  static __device__ __forceinline__ T zero() { return T{0.0f, 0.0f}; }
+  static __device__ __forceinline__ T rows(float w, float fac, float f) {
+    return warp_pair_sum(pair_scale(pair_mul(fac, f), w));
+  }
+  static __device__ __forceinline__ T add(T a, T b) { return pair_add(a, b); }
+  static __device__ __forceinline__ double value(T a) { return (double)a.h + (double)a.l; }
+};
+struct WindowSum64 {
+  using T = double;
+  static __device__ __forceinline__ T zero() { return 0.0; }
+  static __device__ __forceinline__ T rows(float w, float fac, float f) {
+    return warp_sum64((double)w * (double)fac * (double)f);
+  }
+  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+  static __device__ __forceinline__ double value(T a) { return a; }
+};
+template <> struct WindowSum<K_LINEAR> : WindowSum64 {};
+template <> struct WindowSum<K_POLY> : WindowSum64 {};
+
 struct Range {
   int lo, hi;
 };
@@ -631,8 +688,8 @@ __device__ __forceinline__ void dist_epilogue(const Dev& s, Shared<TNV>& sh, uin
 
 // Window-pass epilogue: per element K(a, b) once, three weighted column sums
 // per row (A: w_q on W, Bdd: w_q on D, E: 1 on B), then per row the weight
-// w_p (kind 0) or 1 (kind 1) and an FP64 sum over the warp's 32 rows. A row
-// meeting its own copy (same data index) gets K = 1.
+// w_p (kind 0) or 1 (kind 1) and the sum over the warp's 32 rows (WindowSum).
+// A row meeting its own copy (same data index) gets K = 1.
 template <int KIND, int TNV>
 __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rg, int warp,
                                               int lane, bool all) {
@@ -643,6 +700,9 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
   const float2 C2 = make_float2(-2.0f * negc, -2.0f * negc);
   const float coef0 = (float)s.coef0;
   const int degree = s.degree;
+  using WS = WindowSum<KIND>;
+  using Sum = typename WS::T;
+  static_assert(sizeof(Sum) == sizeof(double), "a shared-memory slot holds one sum");
   // teams, halves and the all-groups mode as in dist_epilogue; partial ph
   // of an item is its slot set ((item GPT + ph) 4 + quadrant) of wpart
   const int team = g / GPT, h = g % GPT;
@@ -666,7 +726,7 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
       if (lane == 0 && !dead) atomicOr(s.status, ST_TIMEOUT);
       dead = true;
     }
-    double tA = 0.0, tB = 0.0, tE = 0.0;
+    Sum tA = WS::zero(), tB = WS::zero(), tE = WS::zero();
     int kind = 0;
     if (!dead) {
       tc_fence_after();
@@ -694,15 +754,14 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
       auto run = [&](auto nbt) {
         constexpr int NB = decltype(nbt)::value;
         constexpr int CW = 8 * NB;
-        const int nch = ncols / CW;
+        // columns from tnew on are in no range, and a quadrant may hold no row
+        // of the item (a dropped prefix or a new block is a few dozen rows)
+        const bool rows_here = dsc.rlo < q * 32 + 32 && dsc.rhi > q * 32;
+        const int live = rows_here ? min(ncols, dsc.tnew - cbeg) : 0;
+        const int nch = live > 0 ? (live + CW - 1) / CW : 0;
         float v0[4 * NB], v1[4 * NB];
         for (int ch = 0; ch < nch; ++ch) {
           chunk_load<NB>(tq + ch * CW, v0, v1);
-          if (!all && ch == nch - 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.tempty[buf]);
-          }
 #pragma unroll
           for (int j = 0; j < NB; ++j) {
             const int c = cbeg + ch * CW + 8 * j + c2;
@@ -736,6 +795,11 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
         }
       };
       run(std::integral_constant<int, 2>{});     // 16-column chunks: three sets of row sums stay in registers
+      if (!all) {                                // the accumulator is free again
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.tempty[buf]);
+      }
       float fa[4], fb[4], fe[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -743,20 +807,25 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
         fb[u] = quad_sum(aB[u].x + aB[u].y);
         fe[u] = quad_sum(aE[u].x + aE[u].y);
       }
-      // this lane's row rq = g4 + 8 us: its row term and row weight, summed over the warp in FP64
+      // this lane's row rq = g4 + 8 us: its row term and row weight, summed over
+      // the warp (a new block's item needs only the sum over B)
       const float fac = (KIND == K_GAUSS && fast) ? ex2_approx(pick4(rc, us)) : 1.0f;
-      const double wr = (double)pick4(wp, us) * (double)fac;
-      tA = warp_sum64(wr * (double)pick4(fa, us));
-      tB = warp_sum64(wr * (double)pick4(fb, us));
-      tE = warp_sum64(wr * (double)pick4(fe, us));
+      const float wr = pick4(wp, us);
+      tE = WS::rows(wr, fac, pick4(fe, us));
+      if (kind == 0) {
+        tA = WS::rows(wr, fac, pick4(fa, us));
+        tB = WS::rows(wr, fac, pick4(fb, us));
+      }
     }
     // The item's four sums (A, Bdd, E for kind 0; M for kind 1) over its 128
-    // rows: the quadrant warps' FP64 sums meet in shared memory and one warp
+    // rows: the quadrant warps' sums meet in shared memory and one warp
     // adds them in quadrant order (group by group in the all-groups mode).
     double* out = s.wpart + ((int64_t)item * GPT + ph) * 4;
     const bool first = ((warp - 2) & 3) == 0;   // the group's first warp
+    const int src = lane == 3 ? 2 : lane;       // M is the E sum of a kind-1 item
+    const bool keep = (lane < 3) == (kind == 0);
     if (!all) {
-      double (*wq)[4] = sh.x.wq[g][gi & 1u];
+      Sum (*wq)[4] = reinterpret_cast<Sum (*)[4]>(sh.x.wq[g][gi & 1u]);
       if (lane == 0) {
         wq[q][0] = tA;
         wq[q][1] = tB;
@@ -766,31 +835,26 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
       if (lane == 0 && !dead) mbar_arrive(&sh.mempty[ms]);
       asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory");   // every warp of the group, dead or not
       if (first && !dead && lane < 4) {
-        const int src = lane == 3 ? 2 : lane;   // M is the E sum of a kind-1 item
-        const bool keep = (lane < 3) == (kind == 0);
-        const double v = ((wq[0][src] + wq[1][src]) + wq[2][src]) + wq[3][src];
-        out[lane] = keep ? v : 0.0;
+        const Sum v = WS::add(WS::add(WS::add(wq[0][src], wq[1][src]), wq[2][src]), wq[3][src]);
+        out[lane] = keep ? WS::value(v) : 0.0;
       }
       ++gi;
     } else {
-      double (*wr)[4][4] = sh.x.wred[local & 1u];
+      Sum (*wr)[4][4] = reinterpret_cast<Sum (*)[4][4]>(sh.x.wred[local & 1u]);
       if (lane == 0) {
         wr[g][q][0] = tA;
         wr[g][q][1] = tB;
         wr[g][q][2] = tE;
-        wr[g][q][3] = (double)kind;
       }
       tc_fence_before();
       asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory");
       if (lead) {
         if (first && !dead && lane < 4) {
-          const int k0 = (int)wr[g][0][3];
-          const int src = lane == 3 ? 2 : lane;
-          const bool keep = (lane < 3) == (k0 == 0);
-          double v = 0.0;
+          Sum v = WS::zero();
           for (int o = 0; o < QPP; ++o)
-            v += ((wr[g + o][0][src] + wr[g + o][1][src]) + wr[g + o][2][src]) + wr[g + o][3][src];
-          out[lane] = keep ? v : 0.0;
+            v = WS::add(v, WS::add(WS::add(WS::add(wr[g + o][0][src], wr[g + o][1][src]), wr[g + o][2][src]),
+                                   wr[g + o][3][src]));
+          out[lane] = keep ? WS::value(v) : 0.0;
         }
         __syncwarp();
         if (lane == 0 && !dead) {
