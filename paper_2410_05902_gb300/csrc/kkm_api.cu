@@ -58,7 +58,15 @@ struct kkm_ctx {
   size_t q_nb4 = 0;
   cudaEvent_t qdone[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec_q[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [slot][host indices]
-  bool fin_pending = false;          // the last step's k_finalize is still to run (see flush)
+  bool fin_pending = false;          // the last step's window pass and norms are still to run (see flush)
+  // the second set of batch buffers and its descriptors: within a captured run
+  // of steps the batches alternate, so that one can be gathered while the
+  // rows of the other still move (the first set is s's own)
+  float* xb32_2 = nullptr;
+  __nv_bfloat16* xbh_2 = nullptr;
+  float* xbn_2 = nullptr;
+  int32_t* xbi_2 = nullptr;
+  alignas(64) unsigned char tmaps2[512];
   double* d_objpart = nullptr;
   double* d_obj2 = nullptr;   // kkm_fit: f_B before and after the update
   int32_t objpart_len = 0;
@@ -151,15 +159,16 @@ kkm_status check_usable(kkm_ctx* c) {
   return KKM_OK;
 }
 
-// A step (windows form, kkm_step) ends with its window pass and leaves its
-// weight update, k_finalize, to the start of the next step, where it runs
-// beside the next batch's gather. Every call that reads or replaces the
-// centers first runs it here (on the context's stream).
+// A step (windows form, kkm_step) ends with its row moves and weights and
+// leaves its window pass, and the center norms that follow from it, to the
+// next step's distance pass. Every call that reads or replaces the centers
+// first runs it here (on the context's stream).
 kkm_status flush(kkm_ctx* c) {
   if (!c->fin_pending) return KKM_OK;
-  cudaError_t e = kkm::launch_finalize(c->s, c->stream, true);
+  cudaError_t e = c->use_tc ? kkm::launch_wgram_tc(c->s, c->tmaps, c->stream, true)
+                            : kkm::launch_wgram(c->s, c->stream, true);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->s.fin_pending, 0, sizeof(int32_t), c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "pending weight update");
+  if (e != cudaSuccess) return cuda_fail(c, e, "pending center norms");
   c->fin_pending = false;
   c->launches += 1;
   return KKM_OK;
@@ -197,6 +206,25 @@ kkm_status sync_and_check(kkm_ctx* c) {
     cudaError_t _e = (expr);                                 \
     if (_e != cudaSuccess) return cuda_fail(c, _e, where);   \
   } while (0)
+
+// The run with batch buffer set `buf` in the place of its own (set 0).
+Dev batch_view(const kkm_ctx* c, int buf) {
+  Dev v = c->s;
+  if (buf) {
+    v.xb32 = c->xb32_2;
+    v.xbh = c->xbh_2;
+    v.xbn = c->xbn_2;
+    v.xbi = c->xbi_2;
+  }
+  return v;
+}
+
+// A run whose window pass has a launch of its own ahead of the distance pass:
+// the FP32 form, and 64-row distance tiles (narrower than a window item's).
+bool split_window(const kkm_ctx* c) { return !c->use_tc || c->s.tn < kkm::WPASS_TNV; }
+
+// Kernels of one step of a run's own sequence, its gather aside.
+int step_kernels(const kkm_ctx* c) { return c->tab ? 6 : split_window(c) ? 5 : 4; }
 
 kkm_status launch_distance_pass(kkm_ctx* c, int rows) {
   if (c->use_tc) KKM_CU(kkm::launch_dist_tc(c->s, c->tmaps, rows, c->stream), "distance kernel (tcgen05)");
@@ -360,6 +388,12 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   s.pair_rows = c->use_tc ? 128 : 64;
   s.pair_cols = c->use_tc ? kkm::WPASS_TNV : 64;
   s.walign = c->use_tc ? 4 : 1;
+  if (c->use_tc) {
+    const int64_t tile_bytes = kkm::tc_item_bytes(s, s.tn, false);
+    // operand copies in units of about 470 cycles, at 64 bytes per clock and SM
+    s.tile_floor = (int32_t)std::min<int64_t>(tile_bytes / (64 * 470), 4096);
+    s.win_work = (int32_t)std::max<int64_t>(22, std::min<int64_t>(kkm::tc_item_bytes(s, kkm::WPASS_TNV, true) / (64 * 470), 4096));
+  }
   const int64_t TR = s.pair_rows, TC = s.pair_cols;   // window-pass tile
   s.max_tiles = tab ? (int32_t)(k + (b + s.tn - 1) / s.tn + 1)
                     : (int32_t)((int64_t)k * ((wmax + s.tn - 1) / s.tn + 1));
@@ -374,6 +408,11 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
     return bail(KKM_EINVAL);
   }
   s.max_pairs = (int32_t)(p1 + p2);
+
+  // CTAs of a step's tcgen05 launch: one per SM, but never more than its items
+  s.nsplit = (int32_t)std::min<int64_t>(std::min(s.num_sms, 1023),
+                                        (int64_t)((b + 127) / 128) * s.max_tiles + s.max_pairs);
+  if (!c->use_tc) s.win_work = 1;
 
   const int esz = kkm::f32_rows(s.form) ? 4 : 2;
   cudaError_t e = cudaSuccess;
@@ -396,6 +435,16 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   ALLOC(s.yi, srows);
   ALLOC(s.w64, srows);
   ALLOC(s.w32, srows);
+  if (!tab) {
+    ALLOC(s.wo32, srows);
+    if (s.form == kkm::FORM_FP32) ALLOC(s.wo64, srows);
+    s.wwin = s.wo32;
+    s.wwin64 = s.wo64;
+    if (esz == 4) ALLOC(c->xb32_2, (size_t)s.bpad * s.ld);
+    else ALLOC(c->xbh_2, (size_t)s.bpad * s.ld);
+    ALLOC(c->xbn_2, s.bpad);
+    ALLOC(c->xbi_2, s.bpad);
+  }
   ALLOC(s.head, k); ALLOC(s.tail, k); ALLOC(s.c1, k); ALLOC(s.wsum, k); ALLOC(s.cnorm, k);
   ALLOC(s.cnorm32, k); ALLOC(s.cmpart, (size_t)k * 32);
   ALLOC(s.blk_iter, (size_t)k * s.nbcap); ALLOC(s.blk_cnt, (size_t)k * s.nbcap);
@@ -403,13 +452,13 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   ALLOC(s.assign, s.bpad); ALLOC(s.mind, s.bpad); ALLOC(s.inner_a, s.bpad);
   ALLOC(s.counts, k); ALLOC(s.alpha, k); ALLOC(s.coff, k + 1); ALLOC(s.perm, s.bpad); ALLOC(s.mvdst, s.bpad);
   ALLOC(s.cmc, k); ALLOC(s.ncum, k); ALLOC(c->d_obj2, 2); ALLOC(s.plan, k); ALLOC(s.comp_off, k); ALLOC(s.comp_total, 1);
-  ALLOC(s.tiles, s.max_tiles); ALLOC(s.ntiles, 1); ALLOC(s.tile_first, k); ALLOC(s.tile_cnt, k);
+  ALLOC(s.tiles, s.max_tiles); ALLOC(s.ntiles, 1); ALLOC(s.tile_first, k);
+  if (!tab) ALLOC(s.split, s.nsplit + 1); ALLOC(s.tile_cnt, k);
   ALLOC(s.part, (size_t)s.max_tiles * s.ppt * s.bpad);
   ALLOC(s.wpairs, s.max_pairs); ALLOC(s.nwpairs, 1); ALLOC(s.wpair_first, k); ALLOC(s.wpair_cnt, k);
-  // window-pass partial slots (of four sums) per item: one per group of a team
-  s.wslots = c->use_tc ? kkm::tc_parts_per_tile(kkm::WPASS_TNV) : 4;
+  s.wslots = c->use_tc ? 1 : 4;   // window-pass partial slots (of four sums) per item
   ALLOC(s.wpart, (size_t)s.max_pairs * s.wslots * 4);
-  ALLOC(s.iter, 1); ALLOC(s.fin_pending, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
+  ALLOC(s.iter, 1); ALLOC(s.gnext, 1); ALLOC(s.wdone, k); ALLOC(s.fin_pending, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
   {
     // the finalise step's rate sqrt(n/b) and 1/n, by the host's correctly rounded
     // FP64 operations (the same values the device would compute)
@@ -525,6 +574,10 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   } else {
     if (e == cudaSuccess) e = kkm::launch_init_centers(s, c->d_init_idx, c->stream);
     if (e == cudaSuccess && c->use_tc) e = kkm::tc_prepare(s, c->tmaps);
+    if (e == cudaSuccess && c->use_tc) {
+      Dev v = batch_view(c, 1);
+      e = kkm::tc_prepare(v, c->tmaps2);
+    }
     if (e == cudaSuccess) e = kkm::launch_build_tiles(s, c->stream);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -542,13 +595,22 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   return KKM_OK;
 }
 
+// Place of a step in a run of steps queued together.
+struct StepPlace {
+  int buf = 0;                       // batch buffer set
+  bool gathered = false;             // the step before gathered this batch
+  bool next = false;                 // gather the next step's batch beside this step's row moves
+  const int32_t* next_idx = nullptr; // its indices (NULL: built-in sampler)
+};
+
 // The kernel sequence of one step, queued on `st`.
-// rotated (kkm_step, windows form): the previous step's k_finalize first (a
-// no-op unless one is pending), the gather beside it, and this step's
-// k_finalize left pending. Otherwise (run groups) finalize ends the step.
+// rotated (a run's own steps, windows form): the window pass and the center
+// norms of the step before run in this step's distance pass (nothing unless
+// they are pending), and this step leaves its own pending. Otherwise (run
+// groups) the window pass and k_finalize end the step.
 static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch_idx,
                                const int32_t* forced_assign, int32_t* assign_out, float* dist_out,
-                               double* batch_obj_out, bool timed, bool rotated) {
+                               double* batch_obj_out, bool timed, bool rotated, const StepPlace& at = StepPlace{}) {
   const Dev& s = c->s;
   if (c->tab) {
     // table form (Appendix A): distances off the table, sort, lay out the batch,
@@ -572,24 +634,58 @@ static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch
     return KKM_OK;
   }
   // with batch_idx NULL the gather draws the indices itself (SplitMix64)
-  if (rotated) KKM_CU(kkm::launch_finalize(s, st, true), "pending weight update");
-  KKM_CU(kkm::launch_gather_batch(s, batch_idx, st, rotated), "batch gather");
+  const unsigned char* maps = at.buf ? c->tmaps2 : c->tmaps;
+  Dev v = batch_view(c, at.buf);
+  if (!rotated) {   // the window pass comes before the weight update
+    v.wwin = s.w32;
+    v.wwin64 = s.w64;
+  }
+  if (rotated && (timed || split_window(c))) {
+    KKM_CU(c->use_tc ? kkm::launch_wgram_tc(v, maps, st, true) : kkm::launch_wgram(v, st, true), "window Gram");
+    if (timed) KKM_CU(cudaMemsetAsync(s.fin_pending, 0, sizeof(int32_t), st), "pending flag");
+  }
+  if (!at.gathered) KKM_CU(kkm::launch_gather_batch(v, batch_idx, st), "batch gather");
   if (timed) KKM_CU(cudaEventRecord(c->ev[2 * c->ev_used], st), "timing event");
-  for (int r = 0; r < (timed ? c->timing_reps : 1); ++r) {   // the pass is idempotent
-    if (c->use_tc) KKM_CU(kkm::launch_dist_tc(s, c->tmaps, s.b, st, true), "distance kernel (tcgen05)");
-    else KKM_CU(kkm::launch_dist_simt(s, s.b, st), "distance kernel");
+  for (int r = 0; r < (timed ? c->timing_reps : 1); ++r) {   // the distance pass alone is idempotent
+    if (rotated && !timed && !split_window(c)) KKM_CU(kkm::launch_step_tc(v, maps, st), "step kernel (tcgen05)");
+    else if (c->use_tc) KKM_CU(kkm::launch_dist_tc(v, maps, s.b, st, true), "distance kernel (tcgen05)");
+    else KKM_CU(kkm::launch_dist_simt(v, s.b, st), "distance kernel");
   }
   if (timed) {
     KKM_CU(cudaEventRecord(c->ev[2 * c->ev_used + 1], st), "timing event");
     c->ev_reps[c->ev_used++] = c->timing_reps;
   }
-  KKM_CU(kkm::launch_argmin(s, s.b, forced_assign, assign_out, nullptr, dist_out, true, st), "argmin");
-  KKM_CU(kkm::launch_sort_plan(s, batch_obj_out, st, rotated), "sort/plan");
-  KKM_CU(kkm::launch_move(s, st), "row moves");
-  if (c->use_tc) KKM_CU(kkm::launch_wgram_tc(s, c->tmaps, st), "window Gram (tcgen05)");
-  else KKM_CU(kkm::launch_wgram(s, st), "window Gram");
-  if (!rotated) KKM_CU(kkm::launch_finalize(s, st), "finalize");
+  KKM_CU(kkm::launch_argmin(v, s.b, forced_assign, assign_out, nullptr, dist_out, true, st), "argmin");
+  KKM_CU(kkm::launch_sort_plan(v, batch_obj_out, st, rotated), "sort/plan");
+  if (rotated) {
+    const Dev nx = batch_view(c, at.buf ^ 1);
+    KKM_CU(kkm::launch_update(v, at.next ? &nx : nullptr, at.next_idx, st), "row moves and weights");
+    return KKM_OK;
+  }
+  KKM_CU(kkm::launch_move(v, st), "row moves");
+  if (c->use_tc) KKM_CU(kkm::launch_wgram_tc(v, maps, st), "window Gram (tcgen05)");
+  else KKM_CU(kkm::launch_wgram(v, st), "window Gram");
+  KKM_CU(kkm::launch_finalize(v, st), "finalize");
   return KKM_OK;
+}
+
+// `m` steps queued together on `st`: in the windows form the batches alternate
+// between the two buffer sets, each gathered beside the row moves of the step
+// before. idx, asg and obj give step i's pointers.
+template <class Idx, class Asg, class Obj>
+static kkm_status enqueue_steps(kkm_ctx* c, cudaStream_t st, int m, Idx idx, Asg asg, Obj obj) {
+  kkm_status r = KKM_OK;
+  for (int i = 0; i < m && r == KKM_OK; ++i) {
+    StepPlace at;
+    if (!c->tab) {
+      at.buf = i & 1;
+      at.gathered = i > 0;
+      at.next = i + 1 < m;
+      at.next_idx = at.next ? idx(i + 1) : nullptr;
+    }
+    r = enqueue_step(c, st, idx(i), nullptr, asg(i), nullptr, obj(i), false, !c->tab, at);
+  }
+  return r;
 }
 
 KKM_API kkm_status kkm_step(kkm_ctx* c, const int32_t* batch_idx, const int32_t* forced_assign,
@@ -627,9 +723,7 @@ KKM_API kkm_status kkm_step(kkm_ctx* c, const int32_t* batch_idx, const int32_t*
     if (st != KKM_OK) return st;
     ++c->eager_steps;
   }
-  // (the previous step's finalize), gather, distance, argmin, sort/plan, moves,
-  // window Gram (+ timing repeats)
-  c->launches += 7 + (timed ? c->timing_reps - 1 : 0);
+  c->launches += 1 + step_kernels(c) + (timed ? c->timing_reps - (split_window(c) || c->tab ? 1 : 0) : 0);
   c->fin_pending = !c->tab;
   ++c->iteration;
   return KKM_OK;
@@ -660,8 +754,9 @@ KKM_API kkm_status kkm_steps(kkm_ctx* c, int64_t n) {
       if (!c->cap_stream)
         KKM_CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
       KKM_CU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-      for (int i = 0; i < STEPS_PER_GRAPH && st == KKM_OK; ++i)
-        st = enqueue_step(c, c->cap_stream, nullptr, nullptr, nullptr, nullptr, nullptr, false, !c->tab);
+      st = enqueue_steps(
+          c, c->cap_stream, STEPS_PER_GRAPH, [](int) -> const int32_t* { return nullptr; },
+          [](int) -> int32_t* { return nullptr; }, [](int) -> double* { return nullptr; });
       cudaGraph_t g = nullptr;
       const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
       if (st != KKM_OK) {
@@ -678,7 +773,7 @@ KKM_API kkm_status kkm_steps(kkm_ctx* c, int64_t n) {
     }
     for (; left >= STEPS_PER_GRAPH; left -= STEPS_PER_GRAPH) {
       KKM_CU(cudaGraphLaunch(c->gexec_multi, c->stream), "graph launch");
-      c->launches += 7 * STEPS_PER_GRAPH;
+      c->launches += STEPS_PER_GRAPH * step_kernels(c) + (c->tab ? STEPS_PER_GRAPH : 1);
       c->iteration += STEPS_PER_GRAPH;
       c->fin_pending = !c->tab;
     }
@@ -740,16 +835,16 @@ double* q_obj(char* slot, size_t nb4, int i) {
 kkm_status q_enqueue(kkm_ctx* c, int q, int m, bool host_idx) {
   const size_t nb4 = c->q_nb4;
   char* d = c->d_qslot[q];
+  auto idx = [=](int i) -> const int32_t* { return host_idx ? q_idx(d, nb4, i) : nullptr; };
+  auto asg = [=](int i) { return q_asg(d, nb4, i); };
+  auto obj = [=](int i) { return q_obj(d, nb4, i); };
   if (c->graph_on && m == HOST_CHUNK) {
     cudaGraphExec_t& ge = c->gexec_q[q][host_idx ? 1 : 0];
     if (!ge) {
       if (!c->cap_stream)
         KKM_CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
       KKM_CU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-      kkm_status st = KKM_OK;
-      for (int i = 0; i < HOST_CHUNK && st == KKM_OK; ++i)
-        st = enqueue_step(c, c->cap_stream, host_idx ? q_idx(d, nb4, i) : nullptr, nullptr, q_asg(d, nb4, i),
-                          nullptr, q_obj(d, nb4, i), false, !c->tab);
+      const kkm_status st = enqueue_steps(c, c->cap_stream, HOST_CHUNK, idx, asg, obj);
       cudaGraph_t g = nullptr;
       const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
       if (st != KKM_OK) {
@@ -766,14 +861,11 @@ kkm_status q_enqueue(kkm_ctx* c, int q, int m, bool host_idx) {
     }
     KKM_CU(cudaGraphLaunch(ge, c->stream), "graph launch");
   } else {
-    for (int i = 0; i < m; ++i) {
-      const kkm_status st = enqueue_step(c, c->stream, host_idx ? q_idx(d, nb4, i) : nullptr, nullptr,
-                                         q_asg(d, nb4, i), nullptr, q_obj(d, nb4, i), false, !c->tab);
-      if (st != KKM_OK) return st;
-      ++c->eager_steps;
-    }
+    const kkm_status st = enqueue_steps(c, c->stream, m, idx, asg, obj);
+    if (st != KKM_OK) return st;
+    c->eager_steps += m;
   }
-  c->launches += 7 * m;
+  c->launches += m * step_kernels(c) + (c->tab ? m : 1);
   c->iteration += m;
   c->fin_pending = !c->tab;
   return KKM_OK;
@@ -1462,6 +1554,8 @@ cudaError_t group_build_batched(kkm_group* g, int nchains) {
     std::memcpy(hr[i].maps, c->tmaps, sizeof(hr[i].maps));
     hr[i].s = c->s;
     hr[i].s.pre_b = 0;   // the group passes read item counts after their grid-dependency wait
+    hr[i].s.wwin = c->s.w32;       // their window pass comes before the weight update
+    hr[i].s.wwin64 = c->s.w64;
   }
   cudaError_t e = cudaMalloc(&g->d_runs, sizeof(kkm::GroupRun) * (size_t)n);
   if (e != cudaSuccess) return e;

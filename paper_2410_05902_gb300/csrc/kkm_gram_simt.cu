@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(NT) k_dist_simt(Dev s, int rows) { dist_simt_b
 
 // Pair w of a run's window pass; its four sums go to wpart[w] (slot 0).
 template <int F>
-__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, float (*As)[BM + 4], float (*Bs)[BN + 4],
-                                                double (*red)[NT / 32]) {
+__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms, float (*As)[BM + 4],
+                                                float (*Bs)[BN + 4], double (*red)[NT / 32]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
   {
     const WPair pr = s.wpairs[w];
@@ -193,7 +193,7 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, float (*As)
       const int64_t p = base + rs + ty * 4 + i;
       const float xn = s.yn[p];
       const int xi = s.yi[p];
-      const double wp = s.w64[p];
+      const double wp = s.wwin64[p];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int qc = pr.ct * BN + tx * 4 + j;
@@ -204,7 +204,7 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, float (*As)
                                                    s.negc, (float)s.coef0, s.degree);
         if (pr.kind == 0) {
           if (qpos < P.tail_c) {
-            const double ww = wp * s.w64[q] * kv;
+            const double ww = wp * s.wwin64[q] * kv;
             sA += ww;
             if (qpos < P.head_new) sB += ww;
           } else {
@@ -232,22 +232,35 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, float (*As)
       s.wpart[(int64_t)w * 16 + tid] = v;
     }
     __syncthreads();
+    if (norms && warp == 0) {   // whoever finishes a center's last pair carries its norm
+      int last = 0;
+      if (lane == 0) {
+        __threadfence();
+        last = atomicAdd(&s.wdone[pr.j], 1) + 1 == s.wpair_cnt[pr.j];
+      }
+      if (__shfl_sync(0xffffffffu, last, 0)) {
+        __threadfence();
+        norm_update(s, pr.j);
+      }
+    }
   }
 }
 
 template <int F>
-__device__ __forceinline__ void wgram_simt_body(const Dev& s, int bid, int nblk) {
+__device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bid, int nblk) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
   __shared__ double red[4][NT / 32];
-  const int total = *s.nwpairs;
-  for (int w = bid; w < total; w += nblk) wgram_simt_item<F>(s, w, As, Bs, red);
+  const int total = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
+  for (int w = bid; w < total; w += nblk) wgram_simt_item<F>(s, w, norms, As, Bs, red);
 }
 
 template <int F>
-__global__ void __launch_bounds__(NT) k_wgram_simt(Dev s) { wgram_simt_body<F>(s, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(NT) k_wgram_simt(Dev s, int norms) {
+  wgram_simt_body<F>(s, norms != 0, blockIdx.x, gridDim.x);
+}
 
 // Run groups: the items of all the launch's runs laid end to end (distance
 // pass: row tiles x support tiles; window pass: pairs), block-strided, so the
@@ -285,7 +298,7 @@ __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
     }
     const Dev& s = g.runs[lo].s;
     if constexpr (MODE == 0) dist_simt_item<F>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], As, Bs);
-    else wgram_simt_item<F>(s, w - off[lo], As, Bs, red);
+    else wgram_simt_item<F>(s, w - off[lo], false, As, Bs, red);
   }
 }
 
@@ -302,14 +315,13 @@ cudaError_t launch_dist_simt(const Dev& s, int rows, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_wgram(const Dev& s, cudaStream_t st) {
+cudaError_t launch_wgram(const Dev& s, cudaStream_t st, bool norms) {
   const int blocks = s.num_sms * 4;
   switch (s.form) {
-    case FORM_FP32: return launch_pdl(k_wgram_simt<FORM_FP32>, dim3(blocks), dim3(NT), 0, st, s);
-    case FORM_BF16: return launch_pdl(k_wgram_simt<FORM_BF16>, dim3(blocks), dim3(NT), 0, st, s);
-    default: return launch_pdl(k_wgram_simt<FORM_BF16X3>, dim3(blocks), dim3(NT), 0, st, s);
+    case FORM_FP32: return launch_pdl(k_wgram_simt<FORM_FP32>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
+    case FORM_BF16: return launch_pdl(k_wgram_simt<FORM_BF16>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
+    default: return launch_pdl(k_wgram_simt<FORM_BF16X3>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_group_simt(const GroupPhase& g, int mode, int form, int blocks, cudaStream_t st) {

@@ -6,44 +6,6 @@
 namespace kkm {
 namespace {
 
-template <int KIND, int MODE, int OP, int TNV>
-cudaError_t launch_form(const Dev& s, const CUtensorMap& a, const CUtensorMap& b, int rows, cudaStream_t st) {
-  static std::atomic<uint64_t> attr{0};
-  {
-    const cudaError_t e = smem_limit_once(k_dist_tc<KIND, MODE, OP, TNV>, smem_bytes<TNV>(), attr);
-    if (e != cudaSuccess) return e;
-  }
-  // one CTA per SM, but never more CTAs than the most items this launch can
-  // have: small runs then leave SMs free for the kernels of other runs
-  const int64_t most = MODE == 0 ? (int64_t)((rows + TM - 1) / TM) * s.max_tiles : (int64_t)s.max_pairs;
-  const int grid = (int)(most < s.num_sms ? (most > 0 ? most : 1) : s.num_sms);
-  return launch_pdl(k_dist_tc<KIND, MODE, OP, TNV>, dim3(grid), dim3(NTHREADS), smem_bytes<TNV>(), st, s, rows, a,
-                    b);
-}
-
-template <int MODE, int OP, int TNV>
-cudaError_t launch_kind(const Dev& s, const CUtensorMap& a, const CUtensorMap& b, int rows, cudaStream_t st) {
-  switch (s.kind) {
-    case K_GAUSS: return launch_form<K_GAUSS, MODE, OP, TNV>(s, a, b, rows, st);
-    case K_LAPLACE: return launch_form<K_LAPLACE, MODE, OP, TNV>(s, a, b, rows, st);
-    case K_LINEAR: return launch_form<K_LINEAR, MODE, OP, TNV>(s, a, b, rows, st);
-    default: return launch_form<K_POLY, MODE, OP, TNV>(s, a, b, rows, st);
-  }
-}
-
-// maps: [0] batch rows, 128-row boxes; support rows with [1] 128-row, [2] 64-row, [3] 256-row boxes
-template <int MODE, int TNV>
-cudaError_t launch_mode(const Dev& s, const void* maps_in, int rows, cudaStream_t st) {
-  const CUtensorMap* m = static_cast<const CUtensorMap*>(maps_in);
-  const CUtensorMap& a = (MODE == 0) ? m[0] : m[1];
-  const CUtensorMap& b = (TNV == 256) ? m[3] : (TNV == 128) ? m[1] : m[2];
-  switch (s.form) {
-    case FORM_BF16X3: return launch_kind<MODE, OP_X3, TNV>(s, a, b, rows, st);
-    case FORM_TF32: return launch_kind<MODE, OP_TF32, TNV>(s, a, b, rows, st);
-    default: return launch_kind<MODE, OP_BF16, TNV>(s, a, b, rows, st);
-  }
-}
-
 // The passes' failure-detection path: thread 0 waits on an mbarrier of one
 // arrival with the passes' bounded wait. With arrive = 0 nothing arrives, so
 // the wait runs out after limit_ns; out[0] = 1 if it did.
@@ -100,6 +62,13 @@ cudaError_t tc_prepare(Dev& s, void* maps_out) {
   return cudaSuccess;
 }
 
+int64_t tc_item_bytes(const Dev& s, int cols, bool with_a) {
+  const int nsl = s.dp / (s.form == FORM_TF32 ? 32 : KS) * (s.form == FORM_BF16X3 ? 2 : 1);
+  const int64_t b = (int64_t)nsl * cols * KS * 2, a = (int64_t)nsl * A_BYTES;
+  const bool resident = a <= A_RES_MAX && (RING_BYTES - a) / b >= 2;   // layout()
+  return b + (with_a || !resident ? a : 0);
+}
+
 int tc_parts_per_tile(int tn) {
   return tn == 256 ? Geo<256>::GPT : tn == 64 ? Geo<64>::GPT : Geo<128>::GPT;
 }
@@ -110,13 +79,13 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
   // ahead writes none of what it stages (the gather, or this pass itself)
   Dev d = s;
   d.pre_b = (stage_early && s.pre_b) ? 1 : 0;
-  if (d.tn == 64) return launch_mode<0, 64>(d, maps, rows, st);
-  if (d.tn == 256) return launch_mode<0, 256>(d, maps, rows, st);
-  return launch_mode<0, 128>(d, maps, rows, st);
+  if (d.tn == 64) return launch_mode<0, 64>(d, maps, rows, false, st);
+  if (d.tn == 256) return launch_mode<0, 256>(d, maps, rows, false, st);
+  return launch_mode<0, 128>(d, maps, rows, false, st);
 }
 
-cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st) {
-  return launch_mode<1, WPASS_TNV>(s, maps, 0, st);
+cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st, bool norms) {
+  return launch_mode<1, WPASS_TNV>(s, maps, 0, norms, st);
 }
 
 }  // namespace kkm

@@ -16,17 +16,20 @@
 // Window pass (mode 1, the norm recurrence of Sec. 4 with the drops of
 // Eq. (1)): an item is (128 support rows, 128 support rows) of one center,
 // rows from the dropped prefix D (kind 0) or the new block B (kind 1), and it
-// writes four sums per TMEM lane quadrant:
+// writes four sums:
 //   kind 0: A = sum_{p in D, q in W} w_p w_q K, Bdd = sum_{p, q in D} w_p w_q K,
 //           E = sum_{p in D, q in B} w_p K          (W: the old window)
 //   kind 1: M = sum_{p, q in B} K.
+// Mode 2 runs the window items of the previous step's update and the distance
+// items of this step in one launch.
 //
 // Roles: warp 0 issues the operand tiles' TMA copies; warp 1 issues the MMAs
 // (one elected lane) and owns the TMEM allocation (up to four accumulators);
 // warps 2-17 are the epilogue, four groups of four warps, one warp per TMEM
 // lane quadrant; warp 18 stages each item's metadata (norms, weights, data
-// indices, and for the window pass the item's row and column ranges) into a
-// ring of slots with per-lane 16-byte asynchronous copies. A copy through the
+// indices, and the item's row and column ranges) into a ring of slots with
+// per-lane 16-byte asynchronous copies; warp 19 (modes 1 and 2) carries the
+// norm of every center whose last window item has finished. A copy through the
 // TMA unit costs the issuing thread a few hundred cycles, so an item takes as
 // few of them as possible: its B tile, and its A tile only when the row tile
 // changes (the batch tile stays resident while consecutive items share it).
@@ -80,7 +83,9 @@ constexpr int A_RES_MAX = 96 * 1024;            // largest batch tile kept resid
 constexpr int NEPI = 16;                         // epilogue warps (2 .. 17): four on each scheduler
 constexpr int NGRP = 4;                          // epilogue groups, one warp per TMEM lane quadrant each
 constexpr int MWARP = 2 + NEPI;                  // the metadata warp
-constexpr int NTHREADS = 32 * (MWARP + 1);      // TMA warp, MMA warp, epilogue, metadata warp
+// TMA warp, MMA warp, epilogue, metadata warp and, where there are window items, the norm warp
+template <int MODE> constexpr int nthreads() { return 32 * (MWARP + (MODE == 0 ? 1 : 2)); }
+constexpr int NSLOT = 4;                         // finished window items waiting for the norm warp
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;   // 2 s per wait
 constexpr float ROW_EXP_FLOOR = -100.0f;        // Gaussian: rc at or above it keeps 2^t finite
 #ifndef DIST_NB
@@ -94,12 +99,13 @@ template <int TNV> struct Geo {
   static constexpr int NACC = 512 / TNV < 4 ? 512 / TNV : 4;
   static constexpr int NTEAM = NACC < NGRP ? NACC : NGRP;
   static constexpr int GPT = NGRP / NTEAM;
-  static constexpr int MS = TNV == 256 ? 4 : 8;
+  static constexpr int MS = TNV == 256 ? 4 : TNV == 128 ? 6 : 8;
   static constexpr uint32_t TMEM_COLS = (uint32_t)(NACC * TNV);
 };
 constexpr uint32_t META_ARRIVALS = 33;           // 32 lanes' asynchronous arrivals + lane 0's release
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y);
+__device__ __forceinline__ void tma_load_2d(bool lead, void* dst, const CUtensorMap* map, uint64_t* bar, int x,
+                                            int y);
 
 // Operand layout of one launch (identical in every role). Byte offsets are
 // from the 1024-aligned start of the operand region; every tile starts on a
@@ -127,38 +133,37 @@ __device__ __forceinline__ Layout layout(int nks) {
   return L;
 }
 
-// Lane t < n issues slice t of a tile (hi slices, then lo slices at column
-// dp) into dst + t * tb: the whole tile leaves in one warp instruction.
-__device__ __forceinline__ void tile_issue(int lane, int n, int nks, int dp, int kse, uint8_t* dst, int tb,
+// The slices of a whole tile (hi slices, then lo slices at column dp) into dst + t * tb.
+__device__ __forceinline__ void tile_issue(bool lead, int n, int nks, int dp, int kse, uint8_t* dst, int tb,
                                            const CUtensorMap* tm, uint64_t* bar, int y) {
-  if (lane < n) {
-    const int x = lane < nks ? lane * kse : dp + (lane - nks) * kse;
-    tma_load_2d(dst + lane * tb, tm, bar, x, y);
-  }
+  for (int t = 0; t < n; ++t)
+    tma_load_2d(lead, dst + t * tb, tm, bar, t < nks ? t * kse : dp + (t - nks) * kse, y);
 }
 
 // Instruction descriptor of tcgen05.mma kind::f16 / kind::tf32: D FP32
 // (bits 4-5 = 1), A and B BF16 (type 1) or TF32 (type 2) in bits 7-9 and
 // 10-12, both K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in
 // bits 24-28.
-template <int N, int OP>
-__host__ __device__ constexpr uint32_t idesc() {
+template <int OP>
+__device__ __forceinline__ uint32_t idesc(uint32_t n) {
   constexpr uint32_t t = OP == OP_TF32 ? 2u : 1u;
-  return (1u << 4) | (t << 7) | (t << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+  return (1u << 4) | (t << 7) | (t << 10) | ((n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// Window-pass item: row and column ranges relative to the item's first row
-// and column (both 4-aligned positions of the center's region).
+// An item's ranges. Distance item: only tnew, the tile's columns. Window item:
+// row and column ranges relative to the item's first row and column (both
+// 4-aligned positions of the center's region).
 struct ItemDesc {
   int32_t kind;        // 0: rows of D against W and B; 1: rows of B against B
   int32_t rlo, rhi;    // rows [rlo, rhi) of the tile are in the row range
   int32_t dnew;        // columns below dnew are dropped rows (D)
   int32_t told;        // columns below told are the old window W (D included)
   int32_t tnew;        // columns in [told, tnew) are the new block B
-  int32_t pad0, pad1;
+  int32_t j;           // center
+  int32_t pad0;
 };
 
-// Metadata of one item, copied by the producer. col[0] = ||y||^2, col[1] = w,
+// Metadata of one item, copied by the metadata warp. col[0] = ||y||^2, col[1] = w,
 // col[2] = data index (bits) of the TNV B rows; row[0] = ||a||^2, row[1] =
 // data index, row[2] = w (window pass) of the 128 A rows.
 template <int TNV> struct MetaSlot {
@@ -172,23 +177,24 @@ template <int TNV> struct Shared {
   uint64_t empty[STAGES];
   uint64_t afull;                // resident A tile landed
   uint64_t afree;                // the MMAs on the previous resident A tile are done
-  uint32_t anew[STAGES];         // resident A: the stage's item brings a new A tile
+  uint32_t mark[STAGES];         // 1: the stage's item brings a new resident A tile
   uint64_t tfull[4];
   uint64_t tempty[4];
   uint64_t mfull[8];
   uint64_t mempty[8];
   uint64_t mma_done;
+  uint64_t nfull[NSLOT];         // window items finished, for the norm warp
+  uint64_t nempty[NSLOT];
+  int32_t nj[NSLOT];             // their centers (-1: the item was skipped)
   uint32_t tmem_base;
   uint32_t pad;
   long long gtot;                // run groups: the class's weighted item total
   int gseg[4];                   // run groups: the next segment (run, first item, end item)
   alignas(16) Dev gdev;          // run groups: the segment's run (a shared copy: no reloads after global stores)
   alignas(16) MetaSlot<TNV> ring[Geo<TNV>::MS];   // 16-byte asynchronous copies land here
-  union alignas(16) {
-    float red[2][NGRP][4][32];     // distance pass, all groups on one item: row sums (item parity, group, quadrant, row)
-    double wred[2][NGRP][4][4];    // window pass, the same: the four sums
-    double wq[NGRP][2][4][4];      // window pass, a group per item: (group, buffer, quadrant, sum)
-  } x;
+  float red[2][NGRP][4][32];     // distance items, all-groups mode: row sums (item parity, group, quadrant, row)
+  float ex[4][3][TM];            // window items: the other groups' quarter sums (quarter, sum, row)
+  double wq[NGRP][2][4][4];      // window items: quadrant sums (team, parity, quadrant, sum)
 };
 
 template <int TNV> constexpr int smem_bytes() { return 1024 + RING_BYTES + (int)sizeof(Shared<TNV>); }
@@ -222,9 +228,12 @@ __device__ __forceinline__ void mbar_inval(uint64_t* b) {
 // invalidate the barriers before initialising them (a later segment)
 constexpr int TC_ALLOC = 1, TC_FREE = 2, TC_REINIT = 4;
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes)
-               : "memory");
+__device__ __forceinline__ void mbar_expect_tx(bool lead, uint64_t* b, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(b)), "r"(bytes),
+      "r"((uint32_t)lead)
+      : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
@@ -254,10 +263,17 @@ __device__ bool mbar_wait(uint64_t* b, uint32_t parity, uint64_t limit_ns = WAIT
   }
 }
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
+// The producer and MMA warps run converged, all lanes computing the same
+// values, and one lane (`lead`) issues: the copy and MMA instructions take their
+// operands from uniform registers, which the compiler can use only for values
+// that are the same over a converged warp. Issued from a one-lane branch every
+// operand went through a register move first, about 170 cycles an MMA.
+__device__ __forceinline__ void tma_load_2d(bool lead, void* dst, const CUtensorMap* map, uint64_t* bar, int x,
+                                            int y) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"((uint32_t)lead)
       : "memory");
 }
 
@@ -273,40 +289,39 @@ __device__ __forceinline__ void tc_fence_after() {
 // CU_TENSOR_MAP_SWIZZLE_128B): start address >> 4 in bits 0-13, leading byte
 // offset 16 (unused by swizzled K-major layouts), stride byte offset 1024
 // (8 rows x 128 B) in bits 32-45, descriptor version 1 in bits 46-47,
-// swizzle mode 2 (128B) in bits 61-63.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1u << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1u << 46;
-  d |= (uint64_t)2u << 61;
-  return d;
-}
+// swizzle mode 2 (128B) in bits 61-63. The low word changes with the tile (a
+// 32-byte K step adds 2 to it), the high word never.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // One MMA on a 32-byte K step of the 128-byte swizzled rows: K = 16 BF16
 // values (kind::f16) or K = 8 TF32 values (kind::tf32).
 template <int OP>
-__device__ __forceinline__ void mma_op(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_op(bool lead, uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
                                        uint32_t accum) {
-  if constexpr (OP == OP_TF32) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-  }
+#define KKM_MMA(kind)                                                                            \
+  asm volatile(                                                                                  \
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t" \
+      "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"                                       \
+      "@q tcgen05.mma.cta_group::1." kind " [%0], da, db, %3, p;\n\t}"                           \
+      ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(idesc), "r"(accum), "r"(DESC_HI), "r"((uint32_t)lead) \
+      : "memory")
+  if constexpr (OP == OP_TF32) KKM_MMA("kind::tf32");
+  else KKM_MMA("kind::f16");
+#undef KKM_MMA
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-               ::"r"(smem_u32(bar))
-               : "memory");
+__device__ __forceinline__ void mma_commit(bool lead, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(smem_u32(bar)), "r"((uint32_t)lead)
+      : "memory");
+}
+
+// A whole warp's wait, the same answer on every lane.
+__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(b, parity));
 }
 
 // tcgen05.ld .16x256b.xNB: 16 TMEM lanes starting at the address's lane, NB
@@ -481,12 +496,6 @@ __device__ __forceinline__ float quad_sum(float v) {
   return v;
 }
 
-__device__ __forceinline__ double warp_sum64(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // A sum kept as h + l in two FP32 words (about 48 bits): the window pass adds
 // its row terms this way. FP64 issues at 1/64 of the FP32 rate on this chip (2
 // lane operations per clock and SM), and the 24 FP64 instructions that each of
@@ -499,11 +508,6 @@ __device__ __forceinline__ double warp_sum64(double v) {
 struct Pair32 {
   float h, l;
 };
-// a b exactly
-__device__ __forceinline__ Pair32 pair_mul(float a, float b) {
-  const float h = __fmul_rn(a, b);
-  return Pair32{h, __fmaf_rn(a, b, -h)};
-}
 __device__ __forceinline__ Pair32 pair_scale(Pair32 x, float w) {
   const float h = __fmul_rn(x.h, w);
   return Pair32{h, __fmaf_rn(x.l, w, __fmaf_rn(x.h, w, -h))};
@@ -521,23 +525,22 @@ __device__ __forceinline__ Pair32 warp_pair_sum(Pair32 v) {
   return v;
 }
 
-// The window pass's sum of one warp's 32 rows: pairs where kernel values are
-// at most 1 (Gaussian, Laplacian), FP64 where they have FP32's whole range.
+// The window pass's sums: pairs where kernel values are at most 1 (Gaussian,
+// Laplacian), FP64 where they have FP32's whole range. addf adds an FP32
+// quarter sum to a row's sum; rows gives the sum of w r over a warp's 32 rows.
 template <int KIND> struct WindowSum {
   using T = Pair32;
   static __device__ __forceinline__ T zero() { return T{0.0f, 0.0f}; }
-  static __device__ __forceinline__ T rows(float w, float fac, float f) {
-    return warp_pair_sum(pair_scale(pair_mul(fac, f), w));
-  }
+  static __device__ __forceinline__ T addf(T a, float b) { return pair_add(a, T{b, 0.0f}); }
+  static __device__ __forceinline__ T rows(T r, float w) { return warp_pair_sum(pair_scale(r, w)); }
   static __device__ __forceinline__ T add(T a, T b) { return pair_add(a, b); }
   static __device__ __forceinline__ double value(T a) { return (double)a.h + (double)a.l; }
 };
 struct WindowSum64 {
   using T = double;
   static __device__ __forceinline__ T zero() { return 0.0; }
-  static __device__ __forceinline__ T rows(float w, float fac, float f) {
-    return warp_sum64((double)w * (double)fac * (double)f);
-  }
+  static __device__ __forceinline__ T addf(T a, float b) { return a + (double)b; }
+  static __device__ __forceinline__ T rows(T r, float w) { return warp_sum_f64(r * (double)w); }
   static __device__ __forceinline__ T add(T a, T b) { return a + b; }
   static __device__ __forceinline__ double value(T a) { return a; }
 };
@@ -548,320 +551,388 @@ struct Range {
   int lo, hi;
 };
 
-// Distance-pass epilogue (warps 2-17). Group g = (warp - 2) / 4 takes the
-// items of local index = g (mod 4), or, when the CTA has fewer than four
-// items, a quarter of the columns of every item. A warp covers its quadrant's
-// 32 rows; it releases the accumulator once its last chunk is in registers
-// and the metadata slot once its arithmetic is done. Part 0 (the only part,
-// or group 0 after the groups' sums meet) writes part[tile][row].
+// What an epilogue warp knows about its place: its group, its row quadrant and
+// its share of an item (teams, column halves and the all-groups mode of the
+// header comment).
+template <int TNV> struct Place {
+  static constexpr int GPT = Geo<TNV>::GPT, QPP = NGRP / GPT;
+  int g, q, team, h, lane;
+  bool all;
+  __device__ Place(int warp, int lane_, bool all_)
+      : g((warp - 2) >> 2), q(warp & 3), team(g / GPT), h(g % GPT), lane(lane_), all(all_) {}
+  __device__ bool mine(uint32_t local) const { return all || (int)(local % Geo<TNV>::NTEAM) == team; }
+  // all-groups mode: the groups that free the accumulator and the slot (4 GPT arrivals on each)
+  __device__ bool frees() const { return !all || g % QPP == 0; }
+  __device__ void arrive(uint64_t* b) const {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(b);
+  }
+  __device__ void sync_all() const { asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory"); }
+  __device__ void sync_group() const { asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory"); }
+  __device__ void sync_team() const {
+    if constexpr (GPT == 2) asm volatile("bar.sync %0, 256;" ::"r"(6 + team) : "memory");
+  }
+};
+
+// One distance-pass item: group h of the team takes the columns [h TNV / GPT,
+// (h+1) TNV / GPT), written as partial h of the tile (in the all-groups mode
+// every group a quarter of the columns, and the quarters of each partial meet
+// in shared memory). Columns from the tile's width on carry weight 0: the
+// chunks past it are skipped, and the last partial may be plain 0. A warp
+// covers its quadrant's 32 rows; it releases the accumulator once its last
+// chunk is in registers and the metadata slot once its arithmetic is done.
 template <int KIND, int TNV>
-__device__ __forceinline__ void dist_epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rg, int T,
-                                              int rows, int warp, int lane, bool all) {
-  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, NTEAM = Geo<TNV>::NTEAM, GPT = Geo<TNV>::GPT;
-  const int g = (warp - 2) >> 2, q = warp & 3;
+__device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem, const Place<TNV>& pl,
+                                          uint32_t local, int tile, int row0, int rows, bool dead) {
+  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT, QPP = Place<TNV>::QPP;
+  const int g = pl.g, q = pl.q, lane = pl.lane;
+  const bool all = pl.all;
   const int g4 = lane >> 2, us = lane & 3, c2 = 2 * us;
   const int rq = g4 + 8 * us;                   // the row this lane reports
   const float negc = s.negc;
   const float2 C2 = make_float2(-2.0f * negc, -2.0f * negc);
   const float coef0 = (float)s.coef0;
   const int degree = s.degree;
-  // Team team = g / GPT takes the items of local index = team (mod NTEAM),
-  // using accumulator `team` on each, and its group h = g % GPT the columns
-  // [h TNV / GPT, (h+1) TNV / GPT), written as partial h of the tile. In the
-  // all-groups mode (a run with fewer than NTEAM items per SM) every group
-  // takes every item (a quarter of the columns) and the quarters of each
-  // partial meet in shared memory.
-  const int team = g / GPT, h = g % GPT;
   const int ncols = all ? TNV / NGRP : TNV / GPT;
-  const int cbeg = all ? g * ncols : h * ncols;
-  constexpr int QPP = NGRP / GPT;                // all-mode quarters per partial
-  const int ph = all ? g / QPP : h;             // this group's partial
-  const bool lead = !all || g % QPP == 0;        // writes the partial and frees the slot and accumulator
-  // part[] must hold GPT partials per tile, as the host sized it (Dev::ppt)
-  bool dead = s.ppt != GPT;                     // a wait ran out (or bad layout): skip the work, keep the barriers
-  if (dead && lane == 0 && warp == 2) atomicOr(s.status, ST_CAPACITY);
-  uint32_t local = 0;
-  for (int item = rg.lo; item < rg.hi; ++item, ++local) {
-    if (!all && (int)(local % NTEAM) != team) continue;
-    const uint32_t buf = local % NACC, bph = (local / NACC) & 1u;
-    const uint32_t ms = local % MS, mph = (local / MS) & 1u;
-    const MetaSlot<TNV>& m = sh.ring[ms];
-    const bool ok = dead || (mbar_wait(&sh.mfull[ms], mph) && mbar_wait(&sh.tfull[buf], bph));
-    if (__any_sync(0xffffffffu, !ok)) {
-      if (lane == 0 && !dead) atomicOr(s.status, ST_TIMEOUT);
-      dead = true;
+  const int cbeg = all ? g * ncols : pl.h * ncols;
+  const int ph = all ? g / QPP : pl.h;          // this group's partial
+  const bool lead = !all || g % QPP == 0;       // writes the partial
+  const uint32_t buf = local % NACC, ms = local % MS;
+  const MetaSlot<TNV>& m = sh.ring[ms];
+  float f = 0.0f;
+  if (!dead) {
+    float rc[4];
+    int xi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = q * 32 + g4 + 8 * u;
+      rc[u] = (KIND == K_GAUSS) ? m.row[0][r] * negc : m.row[0][r];
+      xi[u] = __float_as_int(m.row[1][r]);
     }
-    float f = 0.0f;
-    if (!dead) {
-      tc_fence_after();
-      float rc[4];
-      int xi[4];
+    float2 acc[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = q * 32 + g4 + 8 * u;
-        rc[u] = (KIND == K_GAUSS) ? m.row[0][r] * negc : m.row[0][r];
-        xi[u] = __float_as_int(m.row[1][r]);
+    for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.0f, 0.0f);
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * TNV + cbeg;
+    bool fast = false;
+    if constexpr (KIND == K_GAUSS)
+      fast = __all_sync(0xffffffffu, fminf(fminf(rc[0], rc[1]), fminf(rc[2], rc[3])) >= ROW_EXP_FLOOR);
+    // chunks of CW columns, two in flight: the next chunk's TMEM loads are
+    // issued before the current chunk's arithmetic and waited for after it
+    // (tcgen05.wait::ld waits for every load in flight, so a chunk's
+    // arithmetic is what hides the next chunk's load latency)
+    auto release = [&]() {                      // the accumulator is free again
+      if (!all) {
+        tc_fence_before();
+        pl.arrive(&sh.tempty[buf]);
       }
-      float2 acc[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.0f, 0.0f);
-      const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * TNV + cbeg;
-      bool fast = false;
-      if constexpr (KIND == K_GAUSS)
-        fast = __all_sync(0xffffffffu, fminf(fminf(rc[0], rc[1]), fminf(rc[2], rc[3])) >= ROW_EXP_FLOOR);
-      // chunks of CW columns, two in flight: the next chunk's TMEM loads are
-      // issued before the current chunk's arithmetic and waited for after it
-      // (tcgen05.wait::ld waits for every load in flight, so a chunk's
-      // arithmetic is what hides the next chunk's load latency)
-      auto release = [&]() {                    // the accumulator is free again
-        if (!all) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sh.tempty[buf]);
-        }
-      };
-      auto run = [&](auto nbt) {
-        constexpr int NB = decltype(nbt)::value, CW = 8 * NB;
-        const int nch = ncols / CW;
-        auto math = [&](const float (&w0)[4 * NB], const float (&w1)[4 * NB], int ch) {
-          const int c = cbeg + ch * CW + c2;
-          if constexpr (KIND == K_GAUSS) {
-            if (fast) gauss_chunk<NB, true>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
-            else gauss_chunk<NB, false>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
-          } else {
-            generic_chunk<KIND, NB>(w0, w1, m.col[0], m.col[1], m.col[2], c, negc, coef0, degree, rc, xi, acc);
-          }
-        };
-        float a0[4 * NB], a1[4 * NB], b0[4 * NB], b1[4 * NB];
-        chunk_issue<NB>(tq, a0, a1);
-        tmem_wait_ld();
-        for (int ch = 0; ch < nch; ch += 2) {
-          if (ch + 1 < nch) chunk_issue<NB>(tq + (ch + 1) * CW, b0, b1);
-          else release();
-          math(a0, a1, ch);
-          if (ch + 1 < nch) {
-            tmem_wait_ld();
-            if (ch + 2 < nch) chunk_issue<NB>(tq + (ch + 2) * CW, a0, a1);
-            else release();
-            math(b0, b1, ch + 1);
-            if (ch + 2 < nch) tmem_wait_ld();
-          }
-        }
-      };
-      if (ncols % (8 * DIST_NB) == 0) run(std::integral_constant<int, DIST_NB>{});
-      else if (ncols % 32 == 0) run(std::integral_constant<int, 4>{});
-      else run(std::integral_constant<int, 2>{});
-      float fr[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) fr[u] = quad_sum(acc[u].x + acc[u].y);
-      f = pick4(fr, us);
-      if (KIND == K_GAUSS && fast) f *= ex2_approx(pick4(rc, us));   // the row term 2^rc
-    }
-    const int row = (item / T) * TM + q * 32 + rq;
-    float* out = s.part + ((int64_t)(item % T) * GPT + ph) * s.bpad + row;
-    if (!all) {
-      if (!dead) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.mempty[ms]);        // this warp is done with the slot
-        if (row < rows) *out = f;
+    };
+    constexpr int NB = DIST_NB, CW = 8 * NB;
+    static_assert(TNV / NGRP % CW == 0, "whole chunks per group");
+    const int live = min(ncols, m.desc.tnew - cbeg);
+    const int nch = live > 0 ? (live + CW - 1) / CW : 0;
+    auto math = [&](const float (&w0)[4 * NB], const float (&w1)[4 * NB], int ch) {
+      const int c = cbeg + ch * CW + c2;
+      if constexpr (KIND == K_GAUSS) {
+        if (fast) gauss_chunk<NB, true>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
+        else gauss_chunk<NB, false>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
+      } else {
+        generic_chunk<KIND, NB>(w0, w1, m.col[0], m.col[1], m.col[2], c, negc, coef0, degree, rc, xi, acc);
       }
+    };
+    if (nch == 0) {
+      release();
     } else {
-      float (*red)[4][32] = sh.x.red[local & 1u];
-      red[g][q][rq] = f;
-      tc_fence_before();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory");
-      if (lead) {
-        if (!dead && row < rows) {
-          float v = red[g][q][rq];
-          for (int o = 1; o < QPP; ++o) v += red[g + o][q][rq];
-          *out = v;
+      float a0[4 * NB], a1[4 * NB], b0[4 * NB], b1[4 * NB];
+      chunk_issue<NB>(tq, a0, a1);
+      tmem_wait_ld();
+      for (int ch = 0; ch < nch; ch += 2) {
+        if (ch + 1 < nch) chunk_issue<NB>(tq + (ch + 1) * CW, b0, b1);
+        else release();
+        math(a0, a1, ch);
+        if (ch + 1 < nch) {
+          tmem_wait_ld();
+          if (ch + 2 < nch) chunk_issue<NB>(tq + (ch + 2) * CW, a0, a1);
+          else release();
+          math(b0, b1, ch + 1);
+          if (ch + 2 < nch) tmem_wait_ld();
         }
-        __syncwarp();
-        if (lane == 0 && !dead) {
-          mbar_arrive(&sh.tempty[buf]);
-          mbar_arrive(&sh.mempty[ms]);
-        }
+      }
+    }
+    float fr[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) fr[u] = quad_sum(acc[u].x + acc[u].y);
+    f = pick4(fr, us);
+    if (KIND == K_GAUSS && fast) f *= ex2_approx(pick4(rc, us));   // the row term 2^rc
+  }
+  const int row = row0 + q * 32 + rq;
+  float* out = s.part + ((int64_t)tile * GPT + ph) * s.bpad + row;
+  if (!all) {
+    if (!dead) {
+      pl.arrive(&sh.mempty[ms]);                // this warp is done with the slot
+      if (row < rows) *out = f;
+    }
+  } else {
+    float (*red)[4][32] = sh.red[local & 1u];
+    red[g][q][rq] = f;
+    tc_fence_before();
+    pl.sync_all();
+    if (lead) {
+      if (!dead && row < rows) {
+        float v = red[g][q][rq];
+        for (int o = 1; o < QPP; ++o) v += red[g + o][q][rq];
+        *out = v;
+      }
+      if (!dead) {
+        pl.arrive(&sh.tempty[buf]);
+        pl.arrive(&sh.mempty[ms]);
       }
     }
   }
 }
 
-// Window-pass epilogue: per element K(a, b) once, three weighted column sums
-// per row (A: w_q on W, Bdd: w_q on D, E: 1 on B), then per row the weight
-// w_p (kind 0) or 1 (kind 1) and the sum over the warp's 32 rows (WindowSum).
-// A row meeting its own copy (same data index) gets K = 1.
+// One window-pass item: per element K(a, b) (its full exponent) into one of
+// three column sums per row (A: w_q on W, Bdd: w_q on D, E: 1 on B), then per
+// row the weight w_p (kind 0) or 1 (kind 1) and the sum over the 128 rows
+// (WindowSum). A row meeting its own copy (same data index) gets K = 1.
+//
+// The sums of an item do not depend on how its 128 columns are dealt to the
+// groups: the columns are four quarters of 32, a row's FP32 sum of each quarter
+// is taken by one thread quad, and the quarters are added in order, as pairs.
+// A team of two groups takes two quarters each, a team of one takes all four,
+// and in the all-groups mode each group takes one; the lead group gets the
+// others' quarter sums through shared memory. `turn` counts the team's items
+// (buffer parity).
 template <int KIND, int TNV>
-__device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rg, int warp,
-                                              int lane, bool all) {
-  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, NTEAM = Geo<TNV>::NTEAM, GPT = Geo<TNV>::GPT;
-  const int g = (warp - 2) >> 2, q = warp & 3;
-  const int g4 = lane >> 2, us = lane & 3, c2 = 2 * us;
+__device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem, const Place<TNV>& pl,
+                                            uint32_t local, uint32_t turn, int item, bool norms, bool dead) {
+  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT;
+  using WS = WindowSum<KIND>;
+  using Sum = typename WS::T;
+  static_assert(sizeof(Sum) == sizeof(double), "a shared-memory slot holds one sum");
+  const int q = pl.q, lane = pl.lane;
+  const int g4 = lane >> 2, us = lane & 3, c2 = 2 * us, rq = g4 + 8 * us;
+  const bool all = pl.all;
   const float negc = s.negc;
   const float2 C2 = make_float2(-2.0f * negc, -2.0f * negc);
   const float coef0 = (float)s.coef0;
   const int degree = s.degree;
-  using WS = WindowSum<KIND>;
-  using Sum = typename WS::T;
-  static_assert(sizeof(Sum) == sizeof(double), "a shared-memory slot holds one sum");
-  // teams, halves and the all-groups mode as in dist_epilogue; partial ph
-  // of an item is its slot set ((item GPT + ph) 4 + quadrant) of wpart
-  const int team = g / GPT, h = g % GPT;
-  const int ncols = all ? TNV / NGRP : TNV / GPT;
-  const int cbeg = all ? g * ncols : h * ncols;
-  constexpr int QPP = NGRP / GPT;
-  const int ph = all ? g / QPP : h;
-  const bool lead = !all || g % QPP == 0;
-  // wpart[] must hold GPT slots of four sums per item, as the host sized it (Dev::wslots)
-  bool dead = s.wslots != GPT;
-  uint32_t gi = 0;                               // items this group has taken (shared-memory buffer parity)
-  if (dead && lane == 0 && warp == 2) atomicOr(s.status, ST_CAPACITY);
-  uint32_t local = 0;
-  for (int item = rg.lo; item < rg.hi; ++item, ++local) {
-    if (!all && (int)(local % NTEAM) != team) continue;
-    const uint32_t buf = local % NACC, bph = (local / NACC) & 1u;
-    const uint32_t ms = local % MS, mph = (local / MS) & 1u;
-    const MetaSlot<TNV>& m = sh.ring[ms];
-    const bool ok = dead || (mbar_wait(&sh.mfull[ms], mph) && mbar_wait(&sh.tfull[buf], bph));
-    if (__any_sync(0xffffffffu, !ok)) {
-      if (lane == 0 && !dead) atomicOr(s.status, ST_TIMEOUT);
-      dead = true;
+  const uint32_t buf = local % NACC, ms = local % MS;
+  const MetaSlot<TNV>& m = sh.ring[ms];
+  const int nq = all ? 1 : NGRP / GPT, qlo = all ? pl.g : pl.h * nq;   // this group's quarters
+  const bool lead = qlo == 0;
+  const int slot = all ? 0 : pl.team;
+  Sum rA = WS::zero(), rB = WS::zero(), rE = WS::zero();   // this lane's row rq: W, D and B columns
+  auto add_class = [&](int cls, float v) {       // D is part of W
+    if (cls == 2) rE = WS::addf(rE, v);
+    else rA = WS::addf(rA, v);
+    if (cls == 0) rB = WS::addf(rB, v);
+  };
+  float wrow = 0.0f;
+  int kind = 0, center = -1;
+  bool rows_here = false;
+  if (!dead) {
+    const ItemDesc dsc = m.desc;
+    kind = dsc.kind;
+    center = dsc.j;
+    rows_here = dsc.rlo < q * 32 + 32 && dsc.rhi > q * 32;   // a quadrant may hold no row of the item
+    float rc[4];
+    int xi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = q * 32 + g4 + 8 * u;
+      rc[u] = (KIND == K_GAUSS) ? __fmul_rn(m.row[0][r], negc) : m.row[0][r];
+      xi[u] = __float_as_int(m.row[1][r]);
     }
-    Sum tA = WS::zero(), tB = WS::zero(), tE = WS::zero();
-    int kind = 0;
-    if (!dead) {
-      tc_fence_after();
-      const ItemDesc dsc = m.desc;
-      kind = dsc.kind;
-      float rc[4], wp[4], self[4];
-      int xi[4];
-      bool fast = false;
+    {
+      const int r = q * 32 + rq;
+      wrow = r >= dsc.rlo && r < dsc.rhi ? (kind == 0 ? m.row[2][r] : 1.0f) : 0.0f;
+    }
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * TNV;
+    constexpr int NB = 2, CW = 8 * NB;
+    for (int t = 0; t < nq; ++t) {
+      const int cb = (qlo + t) * 32;
+      // the quarter's columns by class: 0 dropped rows D, 1 the rest of the old
+      // window W, 2 the new block B (columns from tnew on are in none); a chunk
+      // that straddles two classes goes through once for each
+#pragma unroll 1
+      for (int cls = 0; cls < 3; ++cls) {
+        const int lo = max(cb, cls == 0 ? 0 : cls == 1 ? dsc.dnew : dsc.told);
+        const bool need = rows_here && (kind == 0 || cls == 2);   // a new block's item needs only B
+        const int hi = need ? min(cb + 32, cls == 0 ? dsc.dnew : cls == 1 ? dsc.told : dsc.tnew) : 0;
+        float2 acc[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = q * 32 + g4 + 8 * u;
-        rc[u] = (KIND == K_GAUSS) ? m.row[0][r] * negc : m.row[0][r];
-        xi[u] = __float_as_int(m.row[1][r]);
-        const bool in = r >= dsc.rlo && r < dsc.rhi;
-        wp[u] = in ? (dsc.kind == 0 ? m.row[2][r] : 1.0f) : 0.0f;
-      }
-      if constexpr (KIND == K_GAUSS)
-        fast = __all_sync(0xffffffffu, fminf(fminf(rc[0], rc[1]), fminf(rc[2], rc[3])) >= ROW_EXP_FLOOR);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) self[u] = fast ? ex2_approx(-rc[u]) : 1.0f;   // 2^t of K = 1
-      float2 aA[4], aB[4], aE[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) aA[u] = aB[u] = aE[u] = make_float2(0.0f, 0.0f);
-      const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * TNV + cbeg;
-      auto run = [&](auto nbt) {
-        constexpr int NB = decltype(nbt)::value;
-        constexpr int CW = 8 * NB;
-        // columns from tnew on are in no range, and a quadrant may hold no row
-        // of the item (a dropped prefix or a new block is a few dozen rows)
-        const bool rows_here = dsc.rlo < q * 32 + 32 && dsc.rhi > q * 32;
-        const int live = rows_here ? min(ncols, dsc.tnew - cbeg) : 0;
-        const int nch = live > 0 ? (live + CW - 1) / CW : 0;
-        float v0[4 * NB], v1[4 * NB];
-        for (int ch = 0; ch < nch; ++ch) {
-          chunk_load<NB>(tq + ch * CW, v0, v1);
+        for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.0f, 0.0f);
+        for (int c0 = lo & ~(CW - 1); c0 < hi; c0 += CW) {
+          float v0[4 * NB], v1[4 * NB];
+          chunk_load<NB>(tq + c0, v0, v1);
 #pragma unroll
           for (int j = 0; j < NB; ++j) {
-            const int c = cbeg + ch * CW + 8 * j + c2;
+            const int c = c0 + 8 * j + c2;
             const float2 y2 = *reinterpret_cast<const float2*>(&m.col[0][c]);
-            const float2 w2 = *reinterpret_cast<const float2*>(&m.col[1][c]);
+            float2 w2 = *reinterpret_cast<const float2*>(&m.col[1][c]);
             const int2 i2 = *reinterpret_cast<const int2*>(&m.col[2][c]);
-            const float2 cc = (KIND == K_GAUSS) ? __fmul2_rn(y2, make_float2(negc, negc)) : y2;
-            const float2 wa = make_float2(c < dsc.told ? w2.x : 0.0f, c + 1 < dsc.told ? w2.y : 0.0f);
-            const float2 wb = make_float2(c < dsc.dnew ? w2.x : 0.0f, c + 1 < dsc.dnew ? w2.y : 0.0f);
-            const float2 we = make_float2(c >= dsc.told && c < dsc.tnew ? 1.0f : 0.0f,
-                                          c + 1 >= dsc.told && c + 1 < dsc.tnew ? 1.0f : 0.0f);
+            if (cls == 2) w2 = make_float2(1.0f, 1.0f);
+            const bool in0 = c >= lo && c < hi, in1 = c + 1 >= lo && c + 1 < hi;
+            w2 = make_float2(in0 ? w2.x : 0.0f, in1 ? w2.y : 0.0f);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const float2 gg = gram2<NB>(v0, v1, j, u);
               float2 kv;
-              if (KIND == K_GAUSS && fast) {
-                const float2 t = __ffma2_rn(gg, C2, cc);
-                kv.x = xi[u] == i2.x ? self[u] : ex2_approx(t.x);
-                kv.y = xi[u] == i2.y ? self[u] : ex2_approx(t.y);
+              if constexpr (KIND == K_GAUSS) {
+                // every rounding spelled out: a run's norms must not depend on which
+                // kernel's compilation fuses a product into a sum
+                const float2 a = __ffma2_rn(gg, C2, __ffma2_rn(y2, make_float2(negc, negc),
+                                                               make_float2(rc[u], rc[u])));
+                kv.x = ex2_approx(xi[u] == i2.x ? 0.0f : a.x);
+                kv.y = ex2_approx(xi[u] == i2.y ? 0.0f : a.y);
               } else {
-                kv = kernel_pair<KIND>(gg, rc[u], cc, xi[u], i2, negc, coef0, degree);
-                // columns outside every range contribute nothing (unbounded kernels included)
-                kv.x = (wa.x != 0.0f || wb.x != 0.0f || we.x != 0.0f) ? kv.x : 0.0f;
-                kv.y = (wa.y != 0.0f || wb.y != 0.0f || we.y != 0.0f) ? kv.y : 0.0f;
+                kv = kernel_pair<KIND>(gg, rc[u], y2, xi[u], i2, negc, coef0, degree);
               }
-              aA[u] = __ffma2_rn(wa, kv, aA[u]);
-              aB[u] = __ffma2_rn(wb, kv, aB[u]);
-              aE[u] = __ffma2_rn(we, kv, aE[u]);
+              if constexpr (KIND == K_LINEAR || KIND == K_POLY) {   // unbounded outside the class
+                kv.x = in0 ? kv.x : 0.0f;
+                kv.y = in1 ? kv.y : 0.0f;
+              }
+              acc[u] = __ffma2_rn(w2, kv, acc[u]);
             }
           }
         }
-      };
-      run(std::integral_constant<int, 2>{});     // 16-column chunks: three sets of row sums stay in registers
-      if (!all) {                                // the accumulator is free again
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.tempty[buf]);
-      }
-      float fa[4], fb[4], fe[4];
+        float v = 0.0f;
+        if (hi > lo) {
+          float f4[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        fa[u] = quad_sum(aA[u].x + aA[u].y);
-        fb[u] = quad_sum(aB[u].x + aB[u].y);
-        fe[u] = quad_sum(aE[u].x + aE[u].y);
-      }
-      // this lane's row rq = g4 + 8 us: its row term and row weight, summed over
-      // the warp (a new block's item needs only the sum over B)
-      const float fac = (KIND == K_GAUSS && fast) ? ex2_approx(pick4(rc, us)) : 1.0f;
-      const float wr = pick4(wp, us);
-      tE = WS::rows(wr, fac, pick4(fe, us));
-      if (kind == 0) {
-        tA = WS::rows(wr, fac, pick4(fa, us));
-        tB = WS::rows(wr, fac, pick4(fb, us));
+          for (int u = 0; u < 4; ++u) f4[u] = quad_sum(acc[u].x + acc[u].y);
+          v = pick4(f4, us);
+        }
+        if (!lead) sh.ex[all ? qlo - 1 : slot * 2 + t][cls][q * 32 + rq] = v;
+        else add_class(cls, v);
       }
     }
-    // The item's four sums (A, Bdd, E for kind 0; M for kind 1) over its 128
-    // rows: the quadrant warps' sums meet in shared memory and one warp
-    // adds them in quadrant order (group by group in the all-groups mode).
-    double* out = s.wpart + ((int64_t)item * GPT + ph) * 4;
-    const bool first = ((warp - 2) & 3) == 0;   // the group's first warp
-    const int src = lane == 3 ? 2 : lane;       // M is the E sum of a kind-1 item
-    const bool keep = (lane < 3) == (kind == 0);
-    if (!all) {
-      Sum (*wq)[4] = reinterpret_cast<Sum (*)[4]>(sh.x.wq[g][gi & 1u]);
-      if (lane == 0) {
-        wq[q][0] = tA;
-        wq[q][1] = tB;
-        wq[q][2] = tE;
-      }
-      __syncwarp();
-      if (lane == 0 && !dead) mbar_arrive(&sh.mempty[ms]);
-      asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory");   // every warp of the group, dead or not
-      if (first && !dead && lane < 4) {
-        const Sum v = WS::add(WS::add(WS::add(wq[0][src], wq[1][src]), wq[2][src]), wq[3][src]);
-        out[lane] = keep ? WS::value(v) : 0.0;
-      }
-      ++gi;
-    } else {
-      Sum (*wr)[4][4] = reinterpret_cast<Sum (*)[4][4]>(sh.x.wred[local & 1u]);
-      if (lane == 0) {
-        wr[g][q][0] = tA;
-        wr[g][q][1] = tB;
-        wr[g][q][2] = tE;
-      }
+    if (!all) {                                  // the accumulator and the slot are free again
       tc_fence_before();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory");
-      if (lead) {
-        if (first && !dead && lane < 4) {
-          Sum v = WS::zero();
-          for (int o = 0; o < QPP; ++o)
-            v = WS::add(v, WS::add(WS::add(WS::add(wr[g + o][0][src], wr[g + o][1][src]), wr[g + o][2][src]),
-                                   wr[g + o][3][src]));
-          out[lane] = keep ? WS::value(v) : 0.0;
-        }
-        __syncwarp();
-        if (lane == 0 && !dead) {
-          mbar_arrive(&sh.tempty[buf]);
-          mbar_arrive(&sh.mempty[ms]);
-        }
+      pl.arrive(&sh.tempty[buf]);
+      pl.arrive(&sh.mempty[ms]);
+    }
+  }
+  if (all) {
+    tc_fence_before();
+    pl.sync_all();
+    if (pl.frees() && !dead) {
+      pl.arrive(&sh.tempty[buf]);
+      pl.arrive(&sh.mempty[ms]);
+    }
+  } else {
+    pl.sync_team();
+  }
+  if (lead && rows_here)
+    for (int o = nq; o < NGRP; ++o) {
+      const float (*ex)[TM] = sh.ex[all ? o - 1 : slot * 2 + o - nq];
+      for (int cls = 0; cls < 3; ++cls) add_class(cls, ex[cls][q * 32 + rq]);
+    }
+  if (all) pl.sync_all();                        // the exchange buffer may be written again
+  else pl.sync_team();
+  if (!lead) return;
+  if (rows_here) {
+    rE = WS::rows(rE, wrow);
+    if (kind == 0) {
+      rA = WS::rows(rA, wrow);
+      rB = WS::rows(rB, wrow);
+    }
+  }
+  // the four quadrants' sums (A, Bdd, E for kind 0; M for kind 1) in quadrant order
+  Sum (*wq)[4] = reinterpret_cast<Sum (*)[4]>(sh.wq[slot][turn & 1u]);
+  if (lane == 0) {
+    wq[q][0] = rA;
+    wq[q][1] = rB;
+    wq[q][2] = rE;
+  }
+  pl.sync_group();                               // every warp of the group, dead or not
+  if (q == 2) {                                  // the group's first warp
+    if (!dead && lane < 4) {
+      const int src = lane == 3 ? 2 : lane;      // M is the E sum of a kind-1 item
+      const bool keep = (lane < 3) == (kind == 0);
+      const Sum v = WS::add(WS::add(WS::add(wq[0][src], wq[1][src]), wq[2][src]), wq[3][src]);
+      s.wpart[(int64_t)item * 4 + lane] = keep ? WS::value(v) : 0.0;
+    }
+    if (norms) {                                 // hand the item to the norm warp
+      __syncwarp();
+      if (lane == 0) {
+        const uint32_t ns = local % NSLOT;
+        const bool ok = mbar_wait(&sh.nempty[ns], ((local / NSLOT) & 1u) ^ 1u);
+        sh.nj[ns] = ok && !dead ? center : -1;
+        mbar_arrive(&sh.nfull[ns]);
       }
+    }
+  }
+}
+
+// The epilogue warps (2-17): window items [rw.lo, rw.hi) first (MODE 1, 2),
+// then distance items [rd.lo, rd.hi) (MODE 0, 2).
+template <int KIND, int MODE, int TNV>
+__device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rw, Range rd, int T,
+                                         int rows, int warp, int lane, bool all, bool norms) {
+  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
+  const Place<TNV> pl(warp, lane, all);
+  // part[] must hold GPT partials per tile and wpart[] one slot of four sums
+  // per window item, as the host sized them (Dev::ppt, Dev::wslots)
+  bool dead = (MODE != 1 && s.ppt != Geo<TNV>::GPT) || (MODE != 0 && s.wslots != 1);
+  if (dead && lane == 0 && warp == 2) atomicOr(s.status, ST_CAPACITY);
+  const int nw = MODE == 0 ? 0 : rw.hi - rw.lo;
+  const int n = nw + (MODE == 1 ? 0 : rd.hi - rd.lo);
+  auto wait = [&](uint32_t local) {
+    const uint32_t buf = local % NACC, ms = local % MS;
+    const bool ok = dead || (mbar_wait(&sh.mfull[ms], (local / MS) & 1u) &&
+                             mbar_wait(&sh.tfull[buf], (local / NACC) & 1u));
+    if (__any_sync(0xffffffffu, !ok)) {
+      if (lane == 0 && !dead) atomicOr(s.status, ST_TIMEOUT);
+      dead = true;
+    }
+    if (!dead) tc_fence_after();
+  };
+  uint32_t local = 0;
+  if constexpr (MODE != 0) {
+    uint32_t turn = 0;                           // window items this team has taken
+    for (; (int)local < nw; ++local) {
+      if (!pl.mine(local)) continue;
+      wait(local);
+      window_item<KIND, TNV>(s, sh, tmem, pl, local, turn++, rw.lo + (int)local, norms, dead);
+    }
+  }
+  if constexpr (MODE != 1) {
+    for (; (int)local < n; ++local) {
+      if (!pl.mine(local)) continue;
+      wait(local);
+      const int item = rd.lo + (int)local - nw;
+      dist_item<KIND, TNV>(s, sh, tmem, pl, local, item % T, (item / T) * TM, rows, dead);
+    }
+  }
+}
+
+// The norm warp (a launch with norms): counts every finished window item of
+// this CTA at its center; whoever finishes a center's last item carries its
+// norm (norm_update). The item's sums were written by the epilogue before its
+// arrival on nfull; the fences order them before the count and the counts of
+// all items before the norm's reads.
+template <int TNV>
+__device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int nw, int lane) {
+  for (uint32_t i = 0; (int)i < nw; ++i) {
+    const uint32_t ns = i % NSLOT;
+    const bool ok = mbar_wait(&sh.nfull[ns], (i / NSLOT) & 1u);
+    if (__any_sync(0xffffffffu, !ok)) {
+      if (lane == 0) atomicOr(s.status, ST_TIMEOUT);
+      return;
+    }
+    const int j = sh.nj[ns];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.nempty[ns]);
+    if (j < 0) continue;
+    int last = 0;
+    if (lane == 0) {
+      __threadfence();
+      last = atomicAdd(&s.wdone[j], 1) + 1 == s.wpair_cnt[j];
+    }
+    if (__shfl_sync(0xffffffffu, last, 0)) {
+      __threadfence();
+      norm_update(s, j);
     }
   }
 }
@@ -870,7 +941,6 @@ __device__ __forceinline__ void pair_epilogue(const Dev& s, Shared<TNV>& sh, uin
 // (global support rows, both 4-aligned) and its ranges. Row and column tiles
 // start at the range starts rounded down to a multiple of 4 rows; rows and
 // columns outside the ranges are masked by position.
-template <int TNV>
 __device__ __forceinline__ void pair_item(const Dev& s, int w, int& ya, int& yb, ItemDesc& d) {
   const WPair pr = s.wpairs[w];
   const Plan P = s.plan[pr.j];
@@ -878,7 +948,7 @@ __device__ __forceinline__ void pair_item(const Dev& s, int w, int& ya, int& yb,
   if (pr.kind == 0) { r0 = P.head_c; r1 = P.head_c + P.ndrop; c0 = P.head_c; }
   else { r0 = P.tail_c; r1 = P.tail_new; c0 = P.tail_c; }
   const int ra = (r0 & ~3) + pr.rt * TM;
-  const int ca = (c0 & ~3) + pr.ct * TNV;
+  const int ca = (c0 & ~3) + pr.ct * WPASS_TNV;
   const int base = pr.j * s.cap;
   ya = base + ra;
   yb = base + ca;
@@ -888,7 +958,8 @@ __device__ __forceinline__ void pair_item(const Dev& s, int w, int& ya, int& yb,
   d.dnew = P.head_new - ca;
   d.told = P.tail_c - ca;
   d.tnew = P.tail_new - ca;
-  d.pad0 = d.pad1 = 0;
+  d.j = pr.j;
+  d.pad0 = 0;
 }
 
 // This CTA's items: a contiguous range of the launch's items, in row-tile-
@@ -903,33 +974,49 @@ __device__ __forceinline__ Range my_range(int total, int cta, int ncta) {
 }
 
 // MODE 0: distance pass (A = batch tile, B = support tile, one FP32 partial per row).
-// MODE 1: window pass (A and B = support rows of one center, four FP64 sums per
-//         TMEM lane quadrant).
-// Both passes only sum over columns, so a tile can be split along its
-// columns with no merge.
+// MODE 1: window pass (A and B = support rows of one center, four FP64 sums per item).
+// MODE 2: both, the window items of the previous step's update first: they are
+//         a few dozen rows each and by themselves leave the chip waiting on
+//         their latency, while as a few more items per CTA they cost their work.
+//         With the window pass and the weight update as launches of their own
+//         16 iterations and a scoring call took 1307 us on the 1e6 x 128 workload
+//         (k = 100, b = 4096) and 468 us at 2000 x 16 (b = 256), now 1266 and 407.
+// norms (MODE 1, 2): the norm warp carries ||C_j||^2 once a center's items are done.
+//
+// Both passes only sum over columns, so a tile can be split along its columns
+// with no merge. Columns past a tile's width are neither multiplied (the MMA's
+// N is the width rounded up to 16) nor read back.
 //
 // Metadata: distance-pass tiles start on a multiple of 4 support rows and
 // support weights are 0 outside the windows, so an item's column metadata
 // (||y||^2, w, data index) and row metadata (||x||^2, data index) are plain
 // contiguous, 16-byte aligned ranges; window-pass tiles start 4-aligned by
-// construction. The producer copies them with bulk async copies into a ring
-// of slots next to the operands, so nothing on the epilogue's path waits on a
-// global load. Tile descriptors are fetched 32 items at a time, one per
-// producer lane.
+// construction. The metadata warp copies them into a ring of slots next to
+// the operands, so nothing on the epilogue's path waits on a global load.
+// Item descriptors are fetched 32 at a time, one per lane.
 template <int KIND, int MODE, int OP, int TNV>
-__device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUtensorMap* tmA,
-                                             const CUtensorMap* tmB, int cta, int ncta,
+__device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUtensorMap* tmA, const CUtensorMap* tmB,
+                                             const CUtensorMap* tmW, const CUtensorMap* tmN, int cta, int ncta,
+                                             bool norms = false,
                                              Range ovr = Range{-1, -1}, int flags = TC_ALLOC | TC_FREE) {
   constexpr bool X3 = OP == OP_X3;
   constexpr int KSE = OP == OP_TF32 ? 32 : KS;   // operand elements per slice row
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
-  constexpr int BT = TNV * KS * 2;               // one B slice (TNV rows x 128 bytes)
+  // one B slice: the rows its live columns need (a box of 64, 128 or TNV rows) x 128 bytes
+  auto slice_bytes = [](uint32_t ncol) {
+    return (TNV > 64 && ncol > 64u ? (TNV > 128 && ncol > 128u ? TNV : 128) : 64) * KS * 2;
+  };
+  // the MMA's N: an item's live columns, whole 16s
+  auto live_cols = [](bool win, int wd) {
+    const int most = win ? WPASS_TNV : TNV;
+    return (uint32_t)(wd <= 0 ? 16 : wd >= most ? most : (wd + 15) & ~15);
+  };
   constexpr int AH = X3 ? 2 : 1;                 // hi (and lo) tiles per operand
+  static_assert(MODE == 0 || TNV >= WPASS_TNV, "a stage holds a window item's B tile");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   Shared<TNV>& sh = *reinterpret_cast<Shared<TNV>*>(smem + RING_BYTES);
   constexpr uint32_t TMEM_COLS = Geo<TNV>::TMEM_COLS;
-  constexpr uint32_t IDESC = idesc<TNV, OP>();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nks = s.dp / KSE;
   const Layout L = layout<X3, TNV>(nks);
@@ -954,6 +1041,10 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
         mbar_inval(&sh.mfull[i]);
         mbar_inval(&sh.mempty[i]);
       }
+      for (int i = 0; i < NSLOT; ++i) {
+        mbar_inval(&sh.nfull[i]);
+        mbar_inval(&sh.nempty[i]);
+      }
       mbar_inval(&sh.mma_done);
     }
     // every stage's pair, not only the layout's L.nst: a later segment may use more
@@ -971,6 +1062,10 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
       mbar_init(&sh.mfull[i], META_ARRIVALS);
       mbar_init(&sh.mempty[i], 4 * Geo<TNV>::GPT);
     }
+    for (int i = 0; i < NSLOT; ++i) {
+      mbar_init(&sh.nfull[i], 1);
+      mbar_init(&sh.nempty[i], 1);
+    }
     mbar_init(&sh.mma_done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -986,303 +1081,258 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   const uint32_t tmem = sh.tmem_base;
   const int R = (rows + TM - 1) / TM;
 
-  // Streaming stage for slice sl: lanes issue A_hi, A_lo (split form), B_hi,
-  // B_lo in one instruction; with b_only, only the B tiles.
-  auto stream_issue = [&](uint8_t* st, uint64_t* bar, int sl, int ya, int yb, bool b_only) {
-    const int nl = 2 * AH;
-    if (lane < nl) {
-      const bool isb = lane >= AH;
-      const int hl = X3 ? (lane & 1) : 0;
-      if (isb || !b_only) {
-        const int x = hl ? s.dp + sl * KSE : sl * KSE;
-        uint8_t* dst = st + (isb ? AH * A_BYTES + hl * BT : hl * A_BYTES);
-        tma_load_2d(dst, isb ? tmB : tmA, bar, x, isb ? yb : ya);
-      }
-    }
+  // Streaming stage for slice sl: A_hi, A_lo (split form), B_hi, B_lo.
+  auto stream_issue = [&](bool lead, uint8_t* st, uint64_t* bar, int sl, const CUtensorMap* ta, int ya,
+                          const CUtensorMap* tb, int yb, int bt) {
+    const int x = sl * KSE;
+    tma_load_2d(lead, st, ta, bar, x, ya);
+    if (X3) tma_load_2d(lead, st + A_BYTES, ta, bar, s.dp + x, ya);
+    tma_load_2d(lead, st + AH * A_BYTES, tb, bar, x, yb);
+    if (X3) tma_load_2d(lead, st + AH * A_BYTES + bt, tb, bar, s.dp + x, yb);
   };
 
-  // Metadata of one item as 16-byte chunks: the column arrays (TNV floats
-  // each: ||y||^2, w, data index) then the row arrays (128 each: distance
-  // pass ||x||^2, data index; window pass ||y||^2, data index, w).
-  constexpr int NCC = TNV / 4, NRA = MODE == 0 ? 2 : 3;
-  constexpr int NCHUNK = 3 * NCC + 32 * NRA;
-  constexpr uint32_t META_ALL = (1u << (3 + NRA)) - 1u;
-  constexpr uint32_t META_PRE = (1u << 0) | (1u << 2);   // column norms and data indices: earlier steps' data
-  // arrays: bit a of `which` selects array a (0-2 columns, 3.. rows)
-  auto meta_copy = [&](MetaSlot<TNV>& m, int ya, int yb, uint32_t which) {
-    for (int c = lane; c < NCHUNK; c += 32) {
-      const int a = c < 3 * NCC ? c / NCC : 3 + (c - 3 * NCC) / 32;
-      const int o = 4 * (c < 3 * NCC ? c % NCC : (c - 3 * NCC) % 32);
-      if (!((which >> a) & 1u)) continue;
-      float* dst = a < 3 ? m.col[a] : m.row[a - 3];
-      const float* src;
-      if (a == 0) src = s.yn + yb;
-      else if (a == 1) src = s.w32 + yb;
-      else if (a == 2) src = (const float*)s.yi + yb;
-      else if (MODE == 0) src = a == 3 ? s.xbn + ya : (const float*)s.xbi + ya;
-      else src = a == 3 ? s.yn + ya : (a == 4 ? (const float*)s.yi + ya : s.w32 + ya);
-      cp16(dst + o, src + o);
+  // Metadata of one item, 16 bytes per lane and copy: the column arrays
+  // (||y||^2, w, data index of the B rows; the second 128 of them only where
+  // the item has that many) and the row arrays (distance item ||x||^2, data
+  // index; window item ||y||^2, data index, w). Window items read the weights
+  // before the update (wwin). Straight-line on purpose: as a loop that worked out
+  // each chunk's array by division this took one warp about as long as an
+  // item's arithmetic takes the epilogue.
+  auto meta_copy = [&](MetaSlot<TNV>& m, int ya, int yb, int ncol, bool win) {
+    const float *c0 = s.yn + yb, *c1 = (win ? s.wwin : s.w32) + yb, *c2 = (const float*)s.yi + yb;
+    const float *r0 = (win ? s.yn : s.xbn) + ya, *r1 = (const float*)(win ? s.yi : s.xbi) + ya;
+    const int o = 4 * lane;
+    if (TNV >= 128 || lane < TNV / 4) {
+      cp16(m.col[0] + o, c0 + o);
+      cp16(m.col[1] + o, c1 + o);
+      cp16(m.col[2] + o, c2 + o);
+    }
+    if (TNV > 128 && ncol > 128) {
+      cp16(m.col[0] + (TNV - 128) + o, c0 + 128 + o);
+      cp16(m.col[1] + (TNV - 128) + o, c1 + 128 + o);
+      cp16(m.col[2] + (TNV - 128) + o, c2 + 128 + o);
+    }
+    cp16(m.row[0] + o, r0 + o);
+    cp16(m.row[1] + o, r1 + o);
+    if (MODE != 0 && win) cp16(m.row[2] + o, s.wwin + ya + o);
+  };
+  static_assert(TNV == 64 || TNV == 128 || TNV == 256, "meta_copy covers these tiles");
+
+  // The CTA's items: window items, then distance items. With s.pre_b (set per
+  // launch when the kernel just ahead writes neither the tile and pair lists
+  // nor the plans: the batch gather, the row moves or this pass itself) the
+  // lists are read, and the descriptors of the first 32 items fetched, one per
+  // lane, before the grid-dependency wait.
+  int T = 1, total = 0;
+  Range rw{0, 0}, rd{0, 0};
+  auto ranges = [&]() {
+    int np = 0;
+    if constexpr (MODE != 0) np = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
+    if constexpr (MODE != 1) T = *s.ntiles;
+    total = MODE == 1 ? np : R * T;
+    if (ovr.lo >= 0) {
+      (MODE == 1 ? rw : rd) = ovr;
+    } else if (MODE == 2 && np > 0 && ncta == s.nsplit) {
+      const int2 lo = s.split[cta], hi = s.split[cta + 1];   // by work (the sort/plan)
+      rw = Range{lo.x, hi.x};
+      rd = Range{lo.y, hi.y};
+    } else {
+      rw = my_range(np, cta, ncta);
+      rd = my_range(R * T, cta, ncta);
     }
   };
-
-  // Distance pass with s.pre_b (set per launch when the kernel just ahead, the
-  // batch gather or this pass itself, writes none of it): before the
-  // grid-dependency wait the producer fetches the descriptors of its first 32
-  // items (one per lane) and stages the B tile of its first item, and the
-  // metadata warp stages that item's column norms and indices. They come from
-  // the sort, plan and row moves of earlier steps. The column weights (written
-  // by the previous step's weight update, which may still be running beside
-  // the gather), the batch rows and their metadata follow after the wait.
-  int npre = 0;                                  // first-item stages already on their way
-  bool meta_pre = false;                         // first item's column norms and indices on their way
-  int pya_pre = 0, pyb_pre = 0;                  // this lane's first-round item: its A and B rows
-  ItemDesc pd_pre{};
-  bool desc_pre = false;
-  if constexpr (MODE == 0) {
-    if ((warp == 0 || warp == MWARP) && s.pre_b) {
-      const int T0 = *s.ntiles;
-      const Range r0 = my_range(R * T0, cta, ncta);
-      const int mine0 = r0.lo + lane;
-      if (mine0 < r0.hi) {
-        pya_pre = (mine0 / T0) * TM;
-        pyb_pre = s.tiles[mine0 % T0].row0;
-      }
-      desc_pre = true;
-      const int yb0 = __shfl_sync(0xffffffffu, pyb_pre, 0);
-      if (r0.lo < r0.hi) {
-        if (warp == MWARP) {
-          meta_copy(sh.ring[0], 0, yb0, META_PRE);   // column norms and indices
-          meta_pre = true;
-        } else if (L.res) {
-          if (lane == 0) {
-            sh.anew[0] = 1u;                          // the first item brings the first A tile
-            mbar_expect_tx(&sh.full[0], L.sb);
-          }
-          __syncwarp();
-          tile_issue(lane, L.nsl, nks, s.dp, KSE, ring, BT, tmB, &sh.full[0], yb0);
-          npre = 1;
-        } else {
-          npre = nks < L.nst ? nks : L.nst;
-          for (int sl = 0; sl < npre; ++sl) {
-            if (lane == 0) mbar_expect_tx(&sh.full[sl], L.sb);   // covers the A slice issued after the wait
-            __syncwarp();
-            stream_issue(ring + sl * L.sb, &sh.full[sl], sl, 0, yb0, true);
-          }
-        }
-      }
+  int pya = 0, pyb = 0;                          // this lane's prefetched item: A and B rows
+  ItemDesc pd{};
+  // descriptors of items local .. local + 31, one per lane; a distance item's
+  // width goes in tnew
+  auto fetch_desc = [&](int local) {
+    const int nw = rw.hi - rw.lo, mine = local + lane;
+    if (MODE != 0 && mine < nw) {
+      pair_item(s, rw.lo + mine, pya, pyb, pd);
+    } else if (MODE != 1 && rd.lo + mine - nw < rd.hi) {
+      const int item = rd.lo + mine - nw;
+      const Tile t = s.tiles[item % T];
+      pya = (item / T) * TM;
+      pyb = t.row0;
+      pd.tnew = t.ncols;
     }
-  } else {
-    // window pass: its pair list and plans come from the sort/plan kernel two
-    // launches back (the row moves just ahead write neither), so the producer
-    // and the metadata warp fetch their first 32 pair descriptors before the wait
-    if (warp == 0 || warp == MWARP) {
-      const Range r0 = ovr.lo >= 0 ? ovr : my_range(*s.nwpairs, cta, ncta);
-      const int mine0 = r0.lo + lane;
-      if (mine0 < r0.hi) pair_item<TNV>(s, mine0, pya_pre, pyb_pre, pd_pre);
-      desc_pre = true;
-    }
+  };
+  const bool desc_pre = s.pre_b != 0;
+  if (desc_pre) {
+    ranges();
+    if (warp <= 1 || warp == MWARP) fetch_desc(0);
+    if (warp == 0 && lane < 4)   // the first copy does not wait for its descriptor
+      asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)(lane == 0 ? tmA : lane == 1 ? tmB : lane == 2 ? tmW : tmN))
+                   : "memory");
   }
-  KKM_GRID_DEP_WAIT();   // everything above reads only data of earlier steps
+  KKM_GRID_DEP_WAIT();       // everything above reads only data of earlier steps
   KKM_LAUNCH_DEPENDENTS();   // the next kernel may set itself up; it waits before reading our output
-
-  const int T = MODE == 0 ? *s.ntiles : 1;
-  const int total = (MODE == 0) ? R * T : *s.nwpairs;
-  const Range rg = ovr.lo >= 0 ? ovr : my_range(total, cta, ncta);
+  if (!desc_pre) ranges();
+  const int nw = rw.hi - rw.lo, n = nw + rd.hi - rd.lo;
   // All epilogue groups on each item (instead of a team per item) when the
   // run has fewer than NTEAM items per SM. The choice depends on the run
   // alone, never on how a launch splits its items, so an item's sums come out
   // the same in a run's own launch and in a run group's.
   const bool all_groups = total < Geo<TNV>::NTEAM * s.num_sms;
 
-  // descriptors of the next 32 items, one per lane (producer and metadata warp)
-  auto fetch_desc = [&](int item, uint32_t local, int& pya, int& pyb, ItemDesc& pd) {
-    const int mine = item + lane;
-    if (mine >= rg.hi) return;
-    if (local == 0 && desc_pre) {
-      pya = pya_pre;
-      pyb = pyb_pre;
-      pd = pd_pre;
-    } else if constexpr (MODE == 0) {
-      pya = (mine / T) * TM;
-      pyb = s.tiles[mine % T].row0;
-    } else {
-      pair_item<TNV>(s, mine, pya, pyb, pd);
-    }
-  };
-
   if (warp == 0) {
     // ------------------------------------------------- operand producer (one warp)
-    // Lane 0 waits on the barriers and posts the expected bytes; the slices of
-    // a tile are issued by several lanes at once.
+    const bool lead = lane == 0;
     bool ok = true;
-    uint32_t it = 0, local = 0, na = 0;          // stage fills, items visited, A tiles
-    int cur_ya = -1;                             // the resident A tile's first row
-    int pya = 0, pyb = 0;                        // this lane's prefetched item: A and B row
-    ItemDesc pd{};
-    for (int item = rg.lo; item < rg.hi; ++item, ++local) {
-      if ((local & 31u) == 0) fetch_desc(item, local, pya, pyb, pd);
-      const int src = (int)(local & 31u);
+    uint32_t it = 0, na = 0;                     // stage fills, A tiles
+    int cur_ya = -1;                             // the resident A tile's first row (window items: support rows)
+    bool cur_win = false;
+    for (int local = 0; local < n && ok; ++local) {
+      if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
+      const int src = local & 31;
       const int ya = __shfl_sync(0xffffffffu, pya, src);
       const int yb = __shfl_sync(0xffffffffu, pyb, src);
-      const bool new_a = L.res && ya != cur_ya;
+      const int wd = __shfl_sync(0xffffffffu, pd.tnew, src);
+      const bool win = MODE != 0 && local < nw;
+      const uint32_t ncol = live_cols(win, wd);
+      const CUtensorMap* ta = win ? tmW : tmA;
+      const CUtensorMap* tb = TNV == 64 || ncol <= 64u ? tmN : TNV > 128 && ncol > 128u ? tmB : tmW;
+      const int bt = slice_bytes(ncol);
+      const bool new_a = L.res && (ya != cur_ya || win != cur_win);
       if (L.res) {
         // one stage: the item's whole B tile
         const int st = it % L.nst;
-        const uint32_t ph = (it / L.nst) & 1u;
-        const bool pre = MODE == 0 && local == 0 && npre > 0;
-        if (!pre) {
-          if (lane == 0) {
-            if (!mbar_wait(&sh.empty[st], ph ^ 1u)) ok = false;
-            sh.anew[st] = new_a ? 1u : 0u;             // published by the arrive below
-            if (ok) mbar_expect_tx(&sh.full[st], L.sb);
-          }
-          if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
-          tile_issue(lane, L.nsl, nks, s.dp, KSE, ring + st * L.sb, BT, tmB, &sh.full[st], yb);
-        }
+        ok = warp_wait(&sh.empty[st], ((it / L.nst) & 1u) ^ 1u);
+        if (!ok) break;
+        if (lead) sh.mark[st] = new_a ? 1u : 0u;   // published by the arrive below
+        mbar_expect_tx(lead, &sh.full[st], (uint32_t)(L.nsl * bt));
+        tile_issue(lead, L.nsl, nks, s.dp, KSE, ring + st * L.sb, bt, tb, &sh.full[st], yb);
         ++it;
         if (new_a) {
           // the item's B tile is queued (the MMA warp sees the new-A mark on it
           // and releases the old A tile); then the new A tile
-          if (lane == 0) {
-            if (na > 0 && !mbar_wait(&sh.afree, (na - 1) & 1u)) ok = false;
-            if (ok) mbar_expect_tx(&sh.afull, (uint32_t)L.a_bytes);
-          }
-          if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
-          tile_issue(lane, L.nsl, nks, s.dp, KSE, smem, A_BYTES, tmA, &sh.afull, ya);
+          ok = na == 0 || warp_wait(&sh.afree, (na - 1) & 1u);
+          if (!ok) break;
+          mbar_expect_tx(lead, &sh.afull, (uint32_t)L.a_bytes);
+          tile_issue(lead, L.nsl, nks, s.dp, KSE, smem, A_BYTES, ta, &sh.afull, ya);
           ++na;
           cur_ya = ya;
+          cur_win = win;
         }
       } else {
         for (int sl = 0; sl < nks; ++sl, ++it) {
           const int st = it % L.nst;
-          const uint32_t ph = (it / L.nst) & 1u;
-          const bool pre = MODE == 0 && local == 0 && sl < npre;   // B slices and expected bytes sent before the wait
-          if (lane == 0) {
-            if (!mbar_wait(&sh.empty[st], ph ^ 1u)) ok = false;
-            if (ok && !pre) mbar_expect_tx(&sh.full[st], L.sb);
-          }
-          if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
-          if (pre) {   // the A slice only
-            if (lane < AH) {
-              const int x = lane ? s.dp + sl * KSE : sl * KSE;
-              tma_load_2d(ring + st * L.sb + lane * A_BYTES, tmA, &sh.full[st], x, ya);
-            }
-          } else {
-            stream_issue(ring + st * L.sb, &sh.full[st], sl, ya, yb, false);
-          }
+          ok = warp_wait(&sh.empty[st], ((it / L.nst) & 1u) ^ 1u);
+          if (!ok) break;
+          mbar_expect_tx(lead, &sh.full[st], (uint32_t)(AH * (A_BYTES + bt)));
+          stream_issue(lead, ring + st * L.sb, &sh.full[st], sl, ta, ya, tb, yb, bt);
         }
-        if (!ok) break;
       }
     }
-    if (lane == 0) {
-      // the copies in flight must land before the CTA may exit: the last fill
-      // of every stage and the last A tile
-      for (uint32_t q = (it > (uint32_t)L.nst ? it - L.nst : 0u); q < it; ++q)
-        if (!mbar_wait(&sh.full[q % L.nst], (q / L.nst) & 1u)) ok = false;
-      if (na > 0 && !mbar_wait(&sh.afull, (na - 1) & 1u)) ok = false;
-      if (!ok) atomicOr(s.status, ST_TIMEOUT);
-    }
+    // the copies in flight must land before the CTA may exit: the last fill
+    // of every stage and the last A tile
+    for (uint32_t q = (it > (uint32_t)L.nst ? it - L.nst : 0u); q < it; ++q)
+      if (!warp_wait(&sh.full[q % L.nst], (q / L.nst) & 1u)) ok = false;
+    if (na > 0 && !warp_wait(&sh.afull, (na - 1) & 1u)) ok = false;
+    if (lead && !ok) atomicOr(s.status, ST_TIMEOUT);
   } else if (warp == MWARP) {
     // ------------------------------------------------------ metadata (one warp)
     // Every lane copies its share of an item's metadata and arrives on the
     // slot's barrier once its copies have landed; lane 0 also arrives after
-    // writing the window-pass ranges, which publishes them.
+    // writing the item's ranges, which publishes them.
     bool ok = true;
-    uint32_t local = 0;
-    int pya = 0, pyb = 0;
-    ItemDesc pd{};
-    for (int item = rg.lo; item < rg.hi; ++item, ++local) {
-      if ((local & 31u) == 0) fetch_desc(item, local, pya, pyb, pd);
-      const int src = (int)(local & 31u);
+    for (int local = 0; local < n; ++local) {
+      if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
+      const int src = local & 31;
       const int ya = __shfl_sync(0xffffffffu, pya, src);
       const int yb = __shfl_sync(0xffffffffu, pyb, src);
+      const bool win = MODE != 0 && local < nw;
       const int ms = local % MS;
-      if (lane == 0 && !mbar_wait(&sh.mempty[ms], ((local / MS) & 1u) ^ 1u)) ok = false;
+      if (lane == 0 && !mbar_wait(&sh.mempty[ms], (((uint32_t)local / MS) & 1u) ^ 1u)) ok = false;
       if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
       MetaSlot<TNV>& m = sh.ring[ms];
-      if constexpr (MODE == 1) {
-        ItemDesc d;
+      ItemDesc d{};
+      d.tnew = __shfl_sync(0xffffffffu, pd.tnew, src);
+      if constexpr (MODE != 0) {
         d.kind = __shfl_sync(0xffffffffu, pd.kind, src);
         d.rlo = __shfl_sync(0xffffffffu, pd.rlo, src);
         d.rhi = __shfl_sync(0xffffffffu, pd.rhi, src);
         d.dnew = __shfl_sync(0xffffffffu, pd.dnew, src);
         d.told = __shfl_sync(0xffffffffu, pd.told, src);
-        d.tnew = __shfl_sync(0xffffffffu, pd.tnew, src);
-        d.pad0 = d.pad1 = 0;
-        if (lane == 0) m.desc = d;
+        d.j = __shfl_sync(0xffffffffu, pd.j, src);
       }
-      meta_copy(m, ya, yb, (local == 0 && meta_pre) ? META_ALL & ~META_PRE : META_ALL);
+      if (lane == 0) m.desc = d;
+      meta_copy(m, ya, yb, d.tnew, win);
       cp_arrive_noinc(&sh.mfull[ms]);
       if (lane == 0) mbar_arrive(&sh.mfull[ms]);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");   // nothing in flight when the CTA exits
     if (lane == 0 && !ok) atomicOr(s.status, ST_TIMEOUT);
   } else if (warp == 1) {
-    // -------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      uint32_t it = 0, local = 0, na = 0;
-      const uint32_t abase = smem_u32(smem), rbase = smem_u32(ring);
-      // descriptors of a slice's tiles; a 32-byte K step adds 2 to the address field
-      auto mma_slice = [&](uint32_t d, uint32_t ahi, uint32_t alo, uint32_t bhi, uint32_t blo, bool first) {
-        const uint64_t dah = sw128_desc(ahi), dbh = sw128_desc(bhi);
+    // ---------------------------------------------------- MMA issuer (one warp)
+    const bool lead = lane == 0;
+    bool ok = true;
+    uint32_t it = 0, na = 0;
+    const uint32_t abase = smem_u32(smem), rbase = smem_u32(ring);
+    // the four K steps of a slice
+    auto mma_slice = [&](uint32_t d, uint32_t id, uint32_t ahi, uint32_t alo, uint32_t bhi, uint32_t blo,
+                         bool first) {
+      const uint32_t ah = desc_lo(ahi), bh = desc_lo(bhi), al = desc_lo(alo), bl = desc_lo(blo);
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        mma_op<OP>(lead, d, ah + 2u * k, bh + 2u * k, id, (first && k == 0) ? 0u : 1u);
         if constexpr (X3) {
-          const uint64_t dal = sw128_desc(alo), dbl = sw128_desc(blo);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            mma_op<OP>(d, dah + 2u * k, dbh + 2u * k, IDESC, (first && k == 0) ? 0u : 1u);
-            mma_op<OP>(d, dah + 2u * k, dbl + 2u * k, IDESC, 1u);
-            mma_op<OP>(d, dal + 2u * k, dbh + 2u * k, IDESC, 1u);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)   // four 32-byte K steps per 128-byte slice row
-            mma_op<OP>(d, dah + 2u * k, dbh + 2u * k, IDESC, (first && k == 0) ? 0u : 1u);
+          mma_op<OP>(lead, d, ah + 2u * k, bl + 2u * k, id, 1u);
+          mma_op<OP>(lead, d, al + 2u * k, bh + 2u * k, id, 1u);
         }
-      };
-      for (int item = rg.lo; ok && item < rg.hi; ++item, ++local) {
-        const uint32_t buf = local % NACC, bph = (local / NACC) & 1u;
-        if (!mbar_wait(&sh.tempty[buf], bph ^ 1u)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d = tmem + buf * TNV;
-        if (L.res) {
-          const int st = it % L.nst;
-          if (!mbar_wait(&sh.full[st], (it / L.nst) & 1u)) { ok = false; break; }
-          tc_fence_after();
-          if (sh.anew[st]) {
-            // a new resident A tile: release the old one once its MMAs are done, wait for the new one
-            if (na > 0) mma_commit(&sh.afree);
-            if (!mbar_wait(&sh.afull, na & 1u)) { ok = false; break; }
-            tc_fence_after();
-            ++na;
-          }
-          const uint32_t b0 = rbase + (uint32_t)(st * L.sb);
-          for (int sl = 0; sl < nks; ++sl)
-            mma_slice(d, abase + sl * A_BYTES, abase + (nks + sl) * A_BYTES, b0 + sl * BT, b0 + (nks + sl) * BT,
-                      sl == 0);
-          mma_commit(&sh.empty[st]);
-          ++it;
-        } else {
-          for (int sl = 0; sl < nks; ++sl, ++it) {
-            const int st = it % L.nst;
-            if (!mbar_wait(&sh.full[st], (it / L.nst) & 1u)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t a0 = rbase + (uint32_t)(st * L.sb), b0 = a0 + AH * A_BYTES;
-            mma_slice(d, a0, a0 + A_BYTES, b0, b0 + BT, sl == 0);
-            mma_commit(&sh.empty[st]);
-          }
-          if (!ok) break;
-        }
-        mma_commit(&sh.tfull[buf]);
       }
-      mma_commit(&sh.mma_done);
-      if (!mbar_wait(&sh.mma_done, 0)) ok = false;
-      if (!ok) atomicOr(s.status, ST_TIMEOUT);
+    };
+    for (int local = 0; local < n && ok; ++local) {
+      if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
+      const int wd = __shfl_sync(0xffffffffu, pd.tnew, local & 31);
+      const uint32_t ncol = live_cols(MODE != 0 && local < nw, wd);
+      const uint32_t id = idesc<OP>(ncol);
+      const int bt = slice_bytes(ncol);
+      const uint32_t buf = local % NACC, bph = ((uint32_t)local / NACC) & 1u;
+      ok = warp_wait(&sh.tempty[buf], bph ^ 1u);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d = tmem + buf * TNV;
+      if (L.res) {
+        const int st = it % L.nst;
+        ok = warp_wait(&sh.full[st], (it / L.nst) & 1u);
+        if (!ok) break;
+        tc_fence_after();
+        if (__any_sync(0xffffffffu, sh.mark[st])) {
+          // a new resident A tile: release the old one once its MMAs are done, wait for the new one
+          if (na > 0) mma_commit(lead, &sh.afree);
+          ok = warp_wait(&sh.afull, na & 1u);
+          if (!ok) break;
+          tc_fence_after();
+          ++na;
+        }
+        const uint32_t b0 = rbase + (uint32_t)(st * L.sb);
+        for (int sl = 0; sl < nks; ++sl)
+          mma_slice(d, id, abase + sl * A_BYTES, abase + (nks + sl) * A_BYTES, b0 + sl * bt, b0 + (nks + sl) * bt,
+                    sl == 0);
+        mma_commit(lead, &sh.empty[st]);
+        ++it;
+      } else {
+        for (int sl = 0; sl < nks; ++sl, ++it) {
+          const int st = it % L.nst;
+          ok = warp_wait(&sh.full[st], (it / L.nst) & 1u);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t a0 = rbase + (uint32_t)(st * L.sb), b0 = a0 + AH * A_BYTES;
+          mma_slice(d, id, a0, a0 + A_BYTES, b0, b0 + bt, sl == 0);
+          mma_commit(lead, &sh.empty[st]);
+        }
+        if (!ok) break;
+      }
+      mma_commit(lead, &sh.tfull[buf]);
     }
-  } else if constexpr (MODE == 0) {
-    dist_epilogue<KIND, TNV>(s, sh, tmem, rg, T, rows, warp, lane, all_groups);
-  } else {
-    pair_epilogue<KIND, TNV>(s, sh, tmem, rg, warp, lane, all_groups);
+    mma_commit(lead, &sh.mma_done);
+    if (!warp_wait(&sh.mma_done, 0)) ok = false;
+    if (lead && !ok) atomicOr(s.status, ST_TIMEOUT);
+  } else if (warp < MWARP) {
+    epilogue<KIND, MODE, TNV>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_groups, norms);
+  } else if constexpr (MODE != 0) {
+    if (norms) norm_warp<TNV>(s, sh, nw, lane);
   }
   tc_fence_before();
   __syncthreads();
@@ -1294,10 +1344,48 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
 }
 
 template <int KIND, int MODE, int OP, int TNV>
-__global__ void __launch_bounds__(NTHREADS, 1)
-    k_dist_tc(Dev s, int rows, const __grid_constant__ CUtensorMap tmA,
-              const __grid_constant__ CUtensorMap tmB) {
-  dist_tc_body<KIND, MODE, OP, TNV>(s, rows, &tmA, &tmB, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(nthreads<MODE>(), 1)
+    k_dist_tc(Dev s, int rows, int norms, const __grid_constant__ CUtensorMap tmA,
+              const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmW,
+              const __grid_constant__ CUtensorMap tmN) {
+  dist_tc_body<KIND, MODE, OP, TNV>(s, rows, &tmA, &tmB, &tmW, &tmN, blockIdx.x, gridDim.x, norms != 0);
+}
+
+template <int KIND, int MODE, int OP, int TNV>
+cudaError_t launch_form(const Dev& s, const CUtensorMap* m, int rows, bool norms, cudaStream_t st) {
+  static std::atomic<uint64_t> attr{0};
+  {
+    const cudaError_t e = smem_limit_once(k_dist_tc<KIND, MODE, OP, TNV>, smem_bytes<TNV>(), attr);
+    if (e != cudaSuccess) return e;
+  }
+  // one CTA per SM, but never more CTAs than the most items this launch can
+  // have: small runs then leave SMs free for the kernels of other runs
+  const int64_t most = (MODE != 1 ? (int64_t)((rows + TM - 1) / TM) * s.max_tiles : 0) +
+                       (MODE != 0 ? (int64_t)s.max_pairs : 0);
+  const int grid = MODE == 2 ? s.nsplit : (int)(most < s.num_sms ? (most > 0 ? most : 1) : s.num_sms);
+  // maps: [0] batch rows, 128-row boxes; support rows with [1] 128-row, [2] 64-row, [3] 256-row boxes
+  return launch_pdl(k_dist_tc<KIND, MODE, OP, TNV>, dim3(grid), dim3(nthreads<MODE>()), smem_bytes<TNV>(), st, s,
+                    rows, norms ? 1 : 0, m[0], m[3], m[1], m[2]);
+}
+
+template <int MODE, int OP, int TNV>
+cudaError_t launch_kind(const Dev& s, const CUtensorMap* m, int rows, bool norms, cudaStream_t st) {
+  switch (s.kind) {
+    case K_GAUSS: return launch_form<K_GAUSS, MODE, OP, TNV>(s, m, rows, norms, st);
+    case K_LAPLACE: return launch_form<K_LAPLACE, MODE, OP, TNV>(s, m, rows, norms, st);
+    case K_LINEAR: return launch_form<K_LINEAR, MODE, OP, TNV>(s, m, rows, norms, st);
+    default: return launch_form<K_POLY, MODE, OP, TNV>(s, m, rows, norms, st);
+  }
+}
+
+template <int MODE, int TNV>
+cudaError_t launch_mode(const Dev& s, const void* maps, int rows, bool norms, cudaStream_t st) {
+  const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
+  switch (s.form) {
+    case FORM_BF16X3: return launch_kind<MODE, OP_X3, TNV>(s, m, rows, norms, st);
+    case FORM_TF32: return launch_kind<MODE, OP_TF32, TNV>(s, m, rows, norms, st);
+    default: return launch_kind<MODE, OP_BF16, TNV>(s, m, rows, norms, st);
+  }
 }
 
 // Run groups. A launch covers the runs of one class (same form, kernel kind
@@ -1374,7 +1462,7 @@ __device__ __forceinline__ int group_find(const GroupPhase& g, long long A, long
 }
 
 template <int KIND, int MODE, int OP, int TNV>
-__global__ void __launch_bounds__(NTHREADS, 1) k_group_tc(GroupPhase g) {
+__global__ void __launch_bounds__(nthreads<MODE>(), 1) k_group_tc(GroupPhase g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   Shared<TNV>& sh = *reinterpret_cast<Shared<TNV>*>(smem + RING_BYTES);
@@ -1413,19 +1501,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_group_tc(GroupPhase g) {
       static_assert(sizeof(Dev) % 16 == 0, "Dev copied in 16-byte words");
       const int4* src = reinterpret_cast<const int4*>(&gr.s);
       int4* dst = reinterpret_cast<int4*>(&sh.gdev);
-      for (int i = threadIdx.x; i < (int)(sizeof(Dev) / 16); i += NTHREADS) dst[i] = src[i];
+      for (int i = threadIdx.x; i < (int)(sizeof(Dev) / 16); i += nthreads<MODE>()) dst[i] = src[i];
     }
     __syncthreads();
     const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(gr.maps);
-    const CUtensorMap* a = MODE == 0 ? &m[0] : &m[1];
-    const CUtensorMap* b = TNV == 256 ? &m[3] : (TNV == 128 ? &m[1] : &m[2]);
     if (warp == 0) {
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)a) : "memory");
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)b) : "memory");
+      for (int i = 0; i < 4; ++i)
+        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)&m[i]) : "memory");
     }
     // the body starts and ends on CTA barriers, so gseg is read by every
     // thread before warp 0 writes the next segment
-    dist_tc_body<KIND, MODE, OP, TNV>(sh.gdev, sh.gdev.b, a, b, 0, 1, seg, flags);
+    dist_tc_body<KIND, MODE, OP, TNV>(sh.gdev, sh.gdev.b, &m[0], &m[3], &m[1], &m[2], 0, 1, false, seg, flags);
     flags = TC_REINIT;
     rnext = r + 1;
   }

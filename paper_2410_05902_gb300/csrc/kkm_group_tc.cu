@@ -14,7 +14,7 @@ cudaError_t launch_group_form(const GroupPhase& g, int ctas, cudaStream_t st) {
     const cudaError_t e = smem_limit_once(k_group_tc<KIND, MODE, OP, TNV>, smem_bytes<TNV>(), attr);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(k_group_tc<KIND, MODE, OP, TNV>, dim3(ctas), dim3(NTHREADS), smem_bytes<TNV>(), st, g);
+  return launch_pdl(k_group_tc<KIND, MODE, OP, TNV>, dim3(ctas), dim3(nthreads<MODE>()), smem_bytes<TNV>(), st, g);
 }
 
 template <int MODE, int OP, int TNV>

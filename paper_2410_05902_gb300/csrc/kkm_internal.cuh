@@ -80,7 +80,7 @@ struct Plan {
   int32_t c1_new;    // C_1 kept after this update
 };
 
-struct Dev {
+struct alignas(16) Dev {
   // problem
   int64_t n;
   int32_t d, k, b, tau, cap, nbcap;
@@ -95,8 +95,8 @@ struct Dev {
   uint64_t seed;
   int32_t tn;        // support rows per distance tile
   int32_t ppt;       // partials per distance tile in part[] (2 for 256-row tcgen05 tiles: one per column half)
-  int32_t pre_b;     // distance pass: stage the support operand, its metadata and the tile list before
-                     // the grid-dependency wait (launch_dist_tc sets it per launch, only after the gather)
+  int32_t pre_b;     // tcgen05 passes: read the tile and pair lists before the grid-dependency wait
+                     // (set per launch, where the kernel just ahead writes neither)
   int32_t pair_rows, pair_cols; // window-pass tile: row and column counts (64x64 SIMT, 128x128 tcgen05)
   int32_t walign;    // window-pass tiles start at range starts rounded down to this many rows (1 SIMT, 4 tcgen05)
   int32_t bpad;      // rows of the batch buffers (>= b, multiple of 128)
@@ -115,6 +115,10 @@ struct Dev {
   int32_t* yi;
   double* w64;
   float* w32;
+  float* wo32;       // FP32 weights before the pending update (k_update), for its window pass
+  double* wo64;      // the same in FP64 (FP32 form only, whose window pass reads FP64 weights)
+  const float* wwin; // the weights the window pass reads: wo32, or w32 where the pass runs before the update
+  const double* wwin64;   // FP32 form: wo64 or w64
   // per center
   int32_t* head;
   int32_t* tail;
@@ -141,6 +145,10 @@ struct Dev {
   int32_t* comp_total; // [1] rows copied by this step's compactions
   Tile* tiles;       // [max_tiles]
   int32_t* ntiles;   // [1]
+  int2* split;       // [nsplit + 1] first window item and first distance item of each CTA of a step's launch
+  int32_t nsplit;    // its CTAs
+  int32_t tile_floor;  // least work of a tile: its operand copies (see tile_work)
+  int32_t win_work;    // work of a window-pass item, on the same scale
   int32_t* tile_first; // [k]
   int32_t* tile_cnt;   // [k]
   float* part;       // [max_tiles * ppt * bpad] per-tile weighted kernel sums (ppt partials per tile)
@@ -151,10 +159,12 @@ struct Dev {
   double* ncum;      // [k] points assigned to each center so far (N^j of the sklearn rate)
   const double* rtab; // [2 (b + 1)]: 1/n at [n] and sqrt(n / b) at [b + 1 + n], n = 0..b (host-computed)
   double* wpart;     // [max_pairs][wslots][4 sums]: A, Bdd, E, M partials per tile
-  int32_t wslots;    // partial slots per window-pass tile (SIMT: 4, slot 0 used; tcgen05: one per team group)
+  int32_t wslots;    // partial slots per window-pass tile (SIMT: 4, slot 0 used; tcgen05: 1)
   int64_t* iter;     // [1] next iteration number
   int32_t* status;   // [1] sticky device status bits
-  int32_t* fin_pending;   // [1] 1 while a step's weight update (k_finalize) is still to run
+  int32_t* wdone;    // [k] finished window items of the pending update (k_sort_plan clears them)
+  int64_t* gnext;    // [1] the iteration whose batch has been scored (its successor's batch may be gathered)
+  int32_t* fin_pending;   // [1] 1 while a step's window pass and center norms are still to run
   int64_t* stats;    // [3] steps, support rows, tiles
   double* obj;       // [1] last batch objective
   float* cmpart;     // [k][32] FP32 lane partials of sum_{x in B_j} <phi(x), C_j>
@@ -209,6 +219,71 @@ inline cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, si
 }
 
 // ---------------------------------------------------------------- helpers
+// Work of a distance tile in units of one 16-column chunk of an epilogue group
+// (about 470 cycles): five for what an item costs whatever its width, one per
+// chunk of its wider column half, and at least what its operand copies take.
+// With the items split by count the CTAs of the 1e6 x 128 workload's launch
+// ended 44.9 to 56.8 us after its start, split by work 41 to 49.
+__host__ __device__ inline int tile_work(int ncols, int tn, int floor_) {
+  const int half = tn == 256 ? 128 : tn;
+  const int w = 5 + ((ncols < half ? ncols : half) + 15) / 16;
+  return w > floor_ ? w : floor_;
+}
+
+__device__ __forceinline__ double warp_sum_f64(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// alpha_i^j for b_j = n > 0 points, N points in all (this batch included), beta = sqrt(b_j / b).
+__device__ __forceinline__ double learning_rate(const Dev& s, double n, double N, double beta) {
+  if (s.lr == 0) return beta;
+  return s.lr == 2 ? n / N : s.eta;    // sklearn: the running-mean rate
+}
+
+// Sec. 4: ||C'||^2 = (1-a)^2 ||R||^2 + 2a(1-a) <R, m> + a^2 ||m||^2 with m =
+// cm(B_j) and R = C - D, the part of the old center Eq. (1) keeps. cmc =
+// <C, m>, inv_n = 1 / b_j. One function for every caller, so that a run's
+// norms come out the same to the bit however its launches are grouped.
+static __device__ __noinline__ double norm_recurrence(double a, double cmc, double inv_n, double cn_old, double A,
+                                                      double Bdd, double E, double M) {
+  const double keep = 1.0 - a;
+  const double m2 = M * inv_n * inv_n;
+  const double R2 = cn_old - 2.0 * A + Bdd;
+  const double Rm = cmc - E * inv_n;
+  return keep * keep * R2 + 2.0 * a * keep * Rm + a * a * m2;
+}
+
+// ||C_j||^2 after the update, by one warp, once all of center j's window items
+// are in wpart: the sums in k_finalize's order (element e of a center's partials
+// is sum e & 3; eight strided runs, then run by run), the recurrence on lane 0.
+__device__ __forceinline__ void norm_update(const Dev& s, int j) {
+  const int lane = threadIdx.x & 31;
+  const int n = s.plan[j].cnt, per = s.wslots * 4;
+  const int cnt = s.wpair_cnt[j] * per;
+  const double* wp = s.wpart + (int64_t)s.wpair_first[j] * per;
+  const double part = (double)s.cmpart[(int64_t)j * 32 + lane];
+  const double inv_n = s.rtab[n], a = s.alpha[j], cn_old = s.cnorm[j];
+  double qt = 0.0;
+  for (int w = 0; w < 8 && w * 32 < cnt; ++w) {
+    double acc = 0.0;
+    for (int e = w * 32 + lane; e < cnt; e += 256) acc += __ldcg(wp + e);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    qt += acc;
+  }
+  const double A = __shfl_sync(0xffffffffu, qt, 0), Bdd = __shfl_sync(0xffffffffu, qt, 1);
+  const double E = __shfl_sync(0xffffffffu, qt, 2), M = __shfl_sync(0xffffffffu, qt, 3);
+  const double cmc = warp_sum_f64(part) * inv_n;
+  if (lane == 0) {
+    const double cn = norm_recurrence(a, cmc, inv_n, cn_old, A, Bdd, E, M);
+    s.cmc[j] = cmc;
+    s.cnorm[j] = cn;
+    s.cnorm32[j] = (float)cn;
+  }
+}
+
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t m) { return (a + m - 1) / m * m; }
 
 // SplitMix64 (Steele, Lea, Flood 2014): output `counter` of the sequential
@@ -267,20 +342,21 @@ struct TabBuf {
 // ------------------------------------------------------------ launchers
 // All return cudaGetLastError() of their launches.
 cudaError_t launch_sample(const Dev& s, cudaStream_t st);
-// rotated: the gather follows the previous step's k_finalize, does its work
-// and releases the distance pass before its grid-dependency wait (neither
-// touches before its wait what finalize writes), then clears fin_pending
-cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st, bool rotated = false);
+cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st);
 cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, cudaStream_t st);
 cudaError_t launch_dist_simt(const Dev& s, int rows, cudaStream_t st);
 cudaError_t launch_argmin(const Dev& s, int rows, const int32_t* forced, int32_t* assign_out,
                           float* mind_out, float* dist_out, bool update, cudaStream_t st);
-// set_pending: the step's k_finalize runs at the start of the next step (or a flush)
+// set_pending: the step's window pass and norms run in the next step's distance pass (or a flush)
 cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st, bool set_pending = false);
 cudaError_t launch_move(const Dev& s, cudaStream_t st);
-cudaError_t launch_wgram(const Dev& s, cudaStream_t st);
-// if_pending: a no-op unless fin_pending is set
-cudaError_t launch_finalize(const Dev& s, cudaStream_t st, bool if_pending = false);
+// The row moves and the weight update in one launch; with next, the gather of
+// the following batch beside them, into next's batch buffers (next_idx: its
+// indices, or NULL for the built-in sampler).
+cudaError_t launch_update(const Dev& s, const Dev* next, const int32_t* next_idx, cudaStream_t st);
+// norms: a no-op unless fin_pending is set, and every center's norm follows its last item
+cudaError_t launch_wgram(const Dev& s, cudaStream_t st, bool norms = false);
+cudaError_t launch_finalize(const Dev& s, cudaStream_t st);
 // batch objective at fixed assignments and its adjoint (kkm_grad.cu): two
 // launches. ws holds grad_workspace_doubles(s, m) doubles, zeroed when it is
 // allocated (its first int is the row kernel's finished-block counter, which
@@ -376,14 +452,19 @@ cudaError_t launch_lloyd_dist(const Dev& g, const LloydBuf& L, float* out, cudaS
 cudaError_t tc_prepare(Dev& s, void* maps);
 // one bounded mbarrier wait (the passes' own), limited to limit_ns; out[0] = 1 when it ran out
 cudaError_t launch_wait_probe(uint64_t limit_ns, int arrive, int* out, cudaStream_t st);
+// bytes the tcgen05 passes copy per item against a B tile of `cols` rows; with_a: its A tile too
+int64_t tc_item_bytes(const Dev& s, int cols, bool with_a);
 // partials the distance pass writes per tile of tn support rows (Dev::ppt)
 int tc_parts_per_tile(int tn);
 // stage_early: the kernel just ahead on `st` (the batch gather, or this pass
-// itself) writes none of the support tiles, their metadata or the tile list,
-// so the pass may stage them before its grid-dependency wait.
+// itself) writes neither the tile list nor the pair list and plans, so the
+// pass may read them before its grid-dependency wait.
 cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_t st, bool stage_early = false);
 // The window pass reads its pair list and plans before its grid-dependency
-// wait: launch it only right after k_move (which writes neither).
-cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st);
+// wait: launch it only right after k_move, k_update or a kernel that writes neither.
+cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st, bool norms = false);
+// A step's distance pass with the window items of the pending update ahead of
+// it (none unless fin_pending is set) and their center norms; s.tn 128 or 256.
+cudaError_t launch_step_tc(const Dev& s, const void* maps, cudaStream_t st);
 
 }  // namespace kkm

@@ -11,11 +11,7 @@ namespace kkm {
 
 namespace {
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+__device__ __forceinline__ double warp_sum(double v) { return warp_sum_f64(v); }
 
 // Exclusive scan of one int per thread over a block of exactly 1024 threads.
 // Returns the exclusive prefix; *total receives the block sum.
@@ -46,39 +42,42 @@ __device__ int block_exclusive_scan_1024(int v, int* total) {
   return excl;
 }
 
-// Exclusive scans of three ints per thread over a block of exactly 1024
-// threads, in one pass (two barriers plus one that frees the scratch).
-__device__ void block_exclusive_scan3_1024(const int (&v)[3], int (&excl)[3], int (&total)[3]) {
-  __shared__ int wsum3[32][3];
+// Exclusive scans of N ints per thread over a block of exactly 1024 threads,
+// in one pass (two barriers plus one that frees the scratch).
+template <int N>
+__device__ void block_exclusive_scans_1024(const int (&v)[N], int (&excl)[N], int (&total)[N]) {
+  __shared__ int wsums[32][N];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x[3] = {v[0], v[1], v[2]};
+  int x[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) x[q] = v[q];
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < N; ++q) {
       const int y = __shfl_up_sync(0xffffffffu, x[q], o);
       if (lane >= o) x[q] += y;
     }
   if (lane == 31)
-    for (int q = 0; q < 3; ++q) wsum3[warp][q] = x[q];
+    for (int q = 0; q < N; ++q) wsums[warp][q] = x[q];
   __syncthreads();
   if (warp == 0) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      int t = wsum3[lane][q];
+    for (int q = 0; q < N; ++q) {
+      int t = wsums[lane][q];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, t, o);
         if (lane >= o) t += y;
       }
-      wsum3[lane][q] = t;   // inclusive warp-total prefix
+      wsums[lane][q] = t;   // inclusive warp-total prefix
     }
   }
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    excl[q] = x[q] - v[q] + (warp > 0 ? wsum3[warp - 1][q] : 0);
-    total[q] = wsum3[31][q];
+  for (int q = 0; q < N; ++q) {
+    excl[q] = x[q] - v[q] + (warp > 0 ? wsums[warp - 1][q] : 0);
+    total[q] = wsums[31][q];
   }
   __syncthreads();
 }
@@ -203,13 +202,14 @@ __global__ void k_sample(Dev s) {
 }
 
 // One warp per batch slot: X[idx] -> batch row, norm, data index. With idx
-// NULL the slot's index is drawn here: SplitMix64 output (i-1)*b + slot.
-__device__ __forceinline__ void gather_one(const Dev& s, const int32_t* __restrict__ idx, int warp) {
+// NULL the slot's index is drawn here: SplitMix64 output (it-1)*b + slot.
+__device__ __forceinline__ void gather_one(const Dev& s, const int32_t* __restrict__ idx, int warp,
+                                           const int64_t* it) {
   int64_t i;
   if (idx) {
     i = idx[warp];
   } else {
-    const uint64_t c = (uint64_t)(*s.iter - 1) * (uint64_t)s.b + (uint64_t)warp;
+    const uint64_t c = (uint64_t)(*it - 1) * (uint64_t)s.b + (uint64_t)warp;
     i = index_below(splitmix64(s.seed, c), (uint64_t)s.n);
     if ((threadIdx.x & 31) == 0) s.bidx[warp] = (int32_t)i;
   }
@@ -224,32 +224,16 @@ __device__ __forceinline__ void gather_one(const Dev& s, const int32_t* __restri
   }
 }
 
-// Not rotated: waits first, then lets the distance pass stage what it reads
-// from earlier steps (the support tiles, their norms and indices, the tile
-// list; this kernel writes none of it). Rotated (launched right after the
-// previous step's k_finalize): the rows are gathered first, while finalize
-// runs (finalize touches none of the batch buffers, the indices or the
-// iteration counter), and the distance pass is released at once: its early
-// staging reads nothing finalize writes (it loads the weights after its own
-// wait, which returns once this kernel, and so finalize, has completed).
-// Then the wait and the clear of fin_pending.
-__device__ __forceinline__ void gather_body(const Dev& s, const int32_t* __restrict__ idx, int rotated, int bid) {
-  if (!rotated) {
-    KKM_GRID_DEP_WAIT();
-    KKM_LAUNCH_DEPENDENTS();
-  }
+// Waits first, then lets the distance pass read the tile and pair lists,
+// which this kernel does not write.
+__device__ __forceinline__ void gather_body(const Dev& s, const int32_t* __restrict__ idx, int bid) {
+  KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();
   const int warp = (bid * blockDim.x + threadIdx.x) >> 5;
-  if (warp < s.b) gather_one(s, idx, warp);
-  if (rotated) {
-    KKM_LAUNCH_DEPENDENTS();
-    KKM_GRID_DEP_WAIT();
-    if (bid == 0 && threadIdx.x == 0) *s.fin_pending = 0;
-  }
+  if (warp < s.b) gather_one(s, idx, warp, s.iter);
 }
 
-__global__ void k_gather_batch(Dev s, const int32_t* __restrict__ idx, int rotated) {
-  gather_body(s, idx, rotated, blockIdx.x);
-}
+__global__ void k_gather_batch(Dev s, const int32_t* __restrict__ idx) { gather_body(s, idx, blockIdx.x); }
 
 __global__ void k_gather_query(Dev s, const float* __restrict__ Q, int64_t ldq, int rows) {
   KKM_GRID_DEP_WAIT();
@@ -275,18 +259,17 @@ constexpr int AM_WARPS = 16;
 __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_t* __restrict__ forced,
                                             int32_t* __restrict__ assign_out, float* __restrict__ mind_out,
                                             float* __restrict__ dist_out, int update, int bid) {
-  // Before the wait: the tile tables, the center norms, the batch rows' norms
-  // and the forced assignments. They come from kernels that completed before
-  // this one was launched (it is launched once the distance pass has passed
-  // its own wait): the sort/plan, the weight update and the gather.
+  // Before the wait: the tile tables, the batch rows' norms and the forced
+  // assignments. They come from kernels that completed before this one was
+  // launched (it is launched once the distance pass has passed its own wait):
+  // the sort/plan and the gather. The center norms come after it: the
+  // distance pass carries those of the previous step's update.
   __shared__ float r_best[AM_WARPS][32], r_inner[AM_WARPS][32], r_f[AM_WARPS][32];
   __shared__ int r_j[AM_WARPS][32];
   __shared__ int c_first[1024], c_cnt[1024];
-  __shared__ float c_norm[1024];
   for (int j = threadIdx.x; j < s.k; j += 32 * AM_WARPS) {   // a tile holds ppt consecutive partials
     c_first[j] = s.tile_first[j] * s.ppt;
     c_cnt[j] = s.tile_cnt[j] * s.ppt;
-    c_norm[j] = s.cnorm32[j];
   }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int x = bid * 32 + lane;
@@ -296,19 +279,21 @@ __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_
   const int fa = forced ? forced[xr] : -1;
   KKM_GRID_DEP_WAIT();       // the distance pass's partial sums
   KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top
+  if (update && bid == 0 && threadIdx.x == 0) *s.gnext = *s.iter + 1;   // the sort/plan advances iter
   __syncthreads();
   float best = 3.0e38f, best_inner = 0.0f, f_inner = 0.0f;
   int bj = 0x7fffffff;
   const float* part = s.part + xr;
   const int64_t ld = s.bpad;
   for (int j0 = w; j0 < s.k; j0 += 4 * AM_WARPS) {
-    float v[4][4];
+    float v[4][4], cn[4];
     int t0[4], nt[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int j = j0 + u * AM_WARPS;
       t0[u] = j < s.k ? c_first[j] : 0;
       nt[u] = j < s.k ? c_cnt[j] : 0;
+      cn[u] = j < s.k ? s.cnorm32[j] : 0.0f;
 #pragma unroll
       for (int t = 0; t < 4; ++t) v[u][t] = t < nt[u] ? part[(int64_t)(t0[u] + t) * ld] : 0.0f;
     }
@@ -324,7 +309,7 @@ __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_
         if (t + 3 < nt[u]) i3 += part[(int64_t)(t0[u] + t + 3) * ld];
       }
       const float inner = (i0 + i1) + (i2 + i3);
-      const float dist = fmaf(-2.0f, inner, kxx + c_norm[j]);
+      const float dist = fmaf(-2.0f, inner, kxx + cn[u]);
       if (dist_out && live) dist_out[(int64_t)x * s.k + j] = dist;
       if (dist < best) { best = dist; bj = j; best_inner = inner; }   // j increases: ties keep the lowest
       if (j == fa) f_inner = inner;
@@ -368,8 +353,8 @@ __global__ void __launch_bounds__(32 * AM_WARPS) k_argmin(Dev s, int rows, const
   argmin_body(s, rows, forced, assign_out, mind_out, dist_out, update, blockIdx.x);
 }
 
-__device__ int tile_count(const Dev& s, int& head, int& size);
-__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total);
+__device__ int tile_count(const Dev& s, int& head, int& size, int& work);
+__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total, int before, int work, int nwin);
 
 // Single CTA of 1024 threads. Stable counting sort of the batch by center,
 // alpha_i^j, <C_j, cm(B_j)>, and the per-center window plan: compaction,
@@ -578,14 +563,16 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, in
   // one scan for the compaction offsets, the window-pass tiles and the next
   // step's distance tiles (the distance pass and argmin of this step have
   // already consumed the current tile list)
-  const int nt = tile_count(s, thead, tsize);
-  int v3[3] = {ncomp, npairs, nt}, ex3[3], tot3[3];
-  block_exclusive_scan3_1024(v3, ex3, tot3);
+  int twork = 0;
+  const int nt = tile_count(s, thead, tsize, twork);
+  int v3[4] = {ncomp, npairs, nt, twork}, ex3[4], tot3[4];
+  block_exclusive_scans_1024(v3, ex3, tot3);
   const int ptotal = tot3[1];
   if (tid < k) {
     s.comp_off[tid] = ex3[0];
     s.wpair_first[tid] = ex3[1];
     s.wpair_cnt[tid] = npairs;
+    s.wdone[tid] = 0;
     base[tid] = ex3[1];
     tot[tid] = npairs;
   }
@@ -599,7 +586,8 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, in
     *s.iter += 1;
     if (set_pending) *s.fin_pending = 1;
   }
-  tiles_write(s, ex3[2], nt, thead, tsize, tot3[2]);   // its barrier also publishes base/tot
+  tiles_write(s, ex3[2], nt, thead, tsize, tot3[2], ex3[3], tot3[3],
+              min(ptotal, s.max_pairs));   // its barrier also publishes base/tot
   // where k_move puts each sorted batch row: after the window's tail (after
   // the compaction, when there is one), in sorted order
   for (int r = tid; r < b; r += 1024) {
@@ -629,13 +617,11 @@ __global__ void __launch_bounds__(1024) k_sort_plan(Dev s, double* obj_out, int 
 }
 
 // The append of the new blocks and the compaction of the windows that need
-// it, one warp per row: work items 0..b-1 append batch row perm[w] at the end
+// it (with their weights, unless the weight update moves those), one warp per row: work items 0..b-1 append batch row perm[w] at the end
 // of its center's window; items b.. copy the compacting windows' rows down to
 // row 0, all compactions laid end to end (comp_off). Sources and destinations
 // never overlap (see the capacity argument in kkm_internal.cuh).
-__device__ __forceinline__ void move_body(const Dev& s, int bid, int nblk) {
-  KKM_GRID_DEP_WAIT();
-  KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top (or only stages earlier steps' data)
+__device__ __forceinline__ void move_body(const Dev& s, bool weights, int bid, int nblk) {
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   const int nwarps = nblk * wpb;
@@ -665,14 +651,106 @@ __device__ __forceinline__ void move_body(const Dev& s, int bid, int nblk) {
       if (lane == 0) {
         s.yn[dst] = s.yn[src];
         s.yi[dst] = s.yi[src];
-        s.w64[dst] = s.w64[src];
-        s.w32[dst] = s.w32[src];
+        if (weights) {
+          s.w64[dst] = s.w64[src];
+          s.w32[dst] = s.w32[src];
+        }
       }
     }
   }
 }
 
-__global__ void k_move(Dev s) { move_body(s, blockIdx.x, gridDim.x); }
+__global__ void k_move(Dev s) {
+  KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top (or only reads the sort/plan's lists)
+  move_body(s, true, blockIdx.x, gridDim.x);
+}
+
+// The weight update of center j (a block of 256): alpha_j, N^j, the window
+// bounds and the weights. Rows [head_new, tail_c) decay by (1 - alpha), rows
+// [tail_c, tail_new) get alpha / b_j, rows that left the window get 0, and a
+// compacted window's weights move with its rows. wo32 (and wo64) keep the old
+// window's weights for the window pass, which runs after this update.
+__device__ __forceinline__ void weights_body(const Dev& s, int j) {
+  const int tid = threadIdx.x;
+  const Plan P = s.plan[j];
+  const int n = P.cnt;
+  if (n == 0) return;
+  __shared__ double keep_s, wnew_s;
+  const int64_t base = (int64_t)j * s.cap;
+  const int size = min(P.tail_c, s.cap) - P.head_c;             // the old window
+  const int src = P.src_head >= 0 ? P.src_head : P.head_c;
+  if (tid == 0) {
+    const double dn = (double)n, inv_n = s.rtab[n], N = s.ncum[j] + dn;
+    const double a = learning_rate(s, dn, N, s.rtab[s.b + 1 + n]);
+    s.ncum[j] = N;
+    s.alpha[j] = a;
+    s.head[j] = P.head_new;
+    s.tail[j] = P.tail_new;
+    s.c1[j] = P.c1_new;
+    keep_s = 1.0 - a;
+    wnew_s = a * inv_n;
+  }
+  double w[4];                                   // the first 1024 rows' old weights, loaded ahead of the rate
+  float o[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = tid + 256 * u;
+    w[u] = r < size ? s.w64[base + src + r] : 0.0;
+    o[u] = r < size ? s.w32[base + src + r] : 0.0f;
+  }
+  __syncthreads();
+  const double keep = keep_s, wnew = wnew_s;
+  const float wnew32 = (float)wnew;
+  for (int r0 = 0; r0 < size; r0 += 1024) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + tid + 256 * u;
+      if (r >= size) continue;
+      if (r0 > 0) {
+        w[u] = s.w64[base + src + r];
+        o[u] = s.w32[base + src + r];
+      }
+      const int64_t dst = base + P.head_c + r;
+      const double v = P.head_c + r < P.head_new ? 0.0 : w[u] * keep;
+      s.wo32[dst] = o[u];
+      if (s.wo64) s.wo64[dst] = w[u];
+      s.w64[dst] = v;
+      s.w32[dst] = (float)v;
+      if (P.src_head >= 0) {                     // never overlaps the compacted window
+        s.w64[base + src + r] = 0.0;
+        s.w32[base + src + r] = 0.0f;
+      }
+    }
+  }
+  // window-pass tiles start at the window's start rounded down to 4 rows, and
+  // the rows that adds carry weight 0
+  if (tid < (P.head_c & 3)) s.wo32[base + P.head_c - 1 - tid] = 0.0f;
+  for (int r = P.tail_c + tid; r < min(P.tail_new, s.cap); r += 256) {
+    s.w64[base + r] = wnew;
+    s.w32[base + r] = wnew32;
+  }
+}
+
+// The row moves and the weight update in one launch, and beside them the
+// gather of the next batch when the caller knows it (gblocks > 0): blocks
+// [0, gblocks) gather into g's batch buffers before the grid-dependency wait,
+// while the sort/plan's one block runs (they read the data, the batch counter
+// that the argmin left and the caller's indices), the next k blocks each
+// update a center's weights, the rest move rows.
+__global__ void __launch_bounds__(256) k_update(Dev s, Dev g, const int32_t* __restrict__ idx, int gblocks) {
+  const int bid = blockIdx.x;
+  if (bid < gblocks) {
+    const int warp = (bid * 256 + (int)threadIdx.x) >> 5;
+    if (warp < g.b) gather_one(g, idx, warp, g.gnext);
+  }
+  KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();   // the next kernel reads only the sort/plan's lists before its own wait
+  if (bid < gblocks) return;
+  const int c = bid - gblocks;
+  if (c < s.k) weights_body(s, c);
+  else move_body(s, false, c - s.k, (int)gridDim.x - gblocks - s.k);
+}
 
 // Tile list of the distance pass (block of 1024, k <= 1024). Thread j < k
 // passes the window [head, head + size) of center j. Tiles start at head
@@ -681,19 +759,28 @@ __global__ void k_move(Dev s) { move_body(s, blockIdx.x, gridDim.x); }
 // Tile counts of one center's window (thread j < k): the window [head,
 // head + size) is widened down to a multiple of 4 rows, so every tile starts
 // 4-aligned and its metadata copies are 16-byte aligned.
-__device__ int tile_count(const Dev& s, int& head, int& size) {
+// Also the work of the window's tiles: all but the last are full.
+__device__ int tile_count(const Dev& s, int& head, int& size, int& work) {
   if (size > 0) {
     size += head & 3;
     head &= ~3;
   }
-  return (int)threadIdx.x < s.k ? (size + s.tn - 1) / s.tn : 0;
+  const int nt = (int)threadIdx.x < s.k ? (size + s.tn - 1) / s.tn : 0;
+  work = nt > 0 ? (nt - 1) * tile_work(s.tn, s.tn, s.tile_floor) +
+                      tile_work(size - (nt - 1) * s.tn, s.tn, s.tile_floor)
+                : 0;
+  return nt;
 }
 
 // Writes the tile list given each center's first tile and count (exclusive
-// scan over centers, total): tile_first/tile_cnt, ntiles, and one Tile per
-// thread, its center found by a binary search over the first tiles.
-__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total) {
-  __shared__ int t_first[1024], t_nt[1024], t_head[1024], t_size[1024];
+// scan over centers, total) and the work before it: tile_first/tile_cnt,
+// ntiles, and one Tile per thread, its center found by a binary search over
+// the first tiles. Then the split of the next step's launch: nwin window items
+// of win_work each and the R x total distance items on one line of work, of
+// which every CTA takes an equal stretch (the items that start in it).
+__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total, int before, int work,
+                            int nwin) {
+  __shared__ int t_first[1024], t_nt[1024], t_head[1024], t_size[1024], t_before[1024];
   const int tid = threadIdx.x;
   if (tid == 0) {
     *s.ntiles = total <= s.max_tiles ? total : s.max_tiles;
@@ -707,8 +794,10 @@ __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size,
     t_nt[tid] = fits ? nt : 0;
     t_head[tid] = head;
     t_size[tid] = size;
+    t_before[tid] = before;
   }
   __syncthreads();
+  const int full = tile_work(s.tn, s.tn, s.tile_floor);
   const int lim = total <= s.max_tiles ? total : s.max_tiles;
   for (int t = tid; t < lim; t += 1024) {
     const int j = last_le(t_first, s.k, t);
@@ -718,13 +807,31 @@ __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size,
       s.tiles[t] = Tile{j, (int32_t)((int64_t)j * s.cap + t_head[j] + c), min(s.tn, t_size[j] - c), 0};
     }
   }
+  if (tid <= s.nsplit) {                         // nsplit <= 1023
+    const int64_t R = (s.b + 127) / 128, ww = (int64_t)nwin * s.win_work;
+    const int64_t p = (ww + R * work) * tid / s.nsplit, d = p > ww ? p - ww : 0;
+    const int64_t r = work > 0 ? d / work : R;
+    int64_t item = R * lim;
+    if (r < R) {
+      const int rem = (int)(d - r * work);       // the first tile with at least this much work before it
+      int t = 0;
+      if (rem > 0) {
+        const int j = last_le(t_before, s.k, rem - 1);
+        t = t_first[j] + min(t_nt[j], (rem - t_before[j] + full - 1) / full);
+      }
+      item = r * lim + min(t, lim);
+    }
+    s.split[tid] = make_int2(p >= ww ? nwin : (int)((p + s.win_work - 1) / s.win_work), (int)item);
+  }
 }
 
 __device__ void build_tiles_block(const Dev& s, int head, int size) {
-  const int nt = tile_count(s, head, size);
-  int total = 0;
-  const int first = block_exclusive_scan_1024(nt, &total);
-  tiles_write(s, first, nt, head, size, total);
+  int work = 0;
+  const int nt = tile_count(s, head, size, work);
+  const int v[2] = {nt, work};
+  int ex[2], tot[2];
+  block_exclusive_scans_1024(v, ex, tot);
+  tiles_write(s, ex[0], nt, head, size, tot[0], ex[1], tot[1], 0);
 }
 
 __device__ void build_tiles_block(const Dev& s) {
@@ -741,8 +848,9 @@ __global__ void __launch_bounds__(1024) k_build_tiles(Dev s) {
   build_tiles_block(s);
 }
 
-// One block of 256 threads per center j that received points, FP64 where the
-// values accumulate over iterations:
+// Run groups: one block of 256 threads per center j that received points (a
+// run's own steps split this between k_update and the distance pass's norm
+// warps, with the same values), FP64 where the values accumulate over iterations:
 //   alpha_j = sqrt(b_j / b) (or eta), <C_j, cm(B_j)> = (1/b_j) sum_x <phi(x), C_j>
 //   (from k_sort_plan's 32 FP32 lane partials), the window-pass sums, the
 //   Sec. 4 recurrence for ||C_j||^2 corrected for the rows Eq. (1) drops, and
@@ -753,19 +861,18 @@ __global__ void __launch_bounds__(1024) k_build_tiles(Dev s) {
 // The scalar chain has no FP64 division or square root: 1/b_j and the beta
 // rate sqrt(b_j / b) come from a table the host fills at kkm_init, and the
 // thread's operands are loaded before the window sums so their latency overlaps.
-__device__ __forceinline__ void finalize_body(const Dev& s, int if_pending, int bid) {
-  // Before the wait: the pending flag, the plan, the running count, the old
-  // norm, the rate table, the pair range and the sort/plan's partials of
-  // <phi(x), C_j>. Their writers (the sort/plan, the gather, earlier weight
-  // updates) completed before this kernel was launched: it is launched once
-  // the kernel ahead (the window pass, or a full dependency) has passed its
-  // own wait. Only the window-pass sums need the wait, and no block returns
-  // before it, so this kernel never completes ahead of the one it follows.
+__device__ __forceinline__ void finalize_body(const Dev& s, int bid) {
+  // Before the wait: the plan, the running count, the old norm, the rate
+  // table, the pair range and the sort/plan's partials of <phi(x), C_j>. Their
+  // writers (the sort/plan, earlier weight updates) completed before this
+  // kernel was launched: it is launched once the kernel ahead (the window
+  // pass, or a full dependency) has passed its own wait. Only the window-pass
+  // sums need the wait, and no block returns before it, so this kernel never
+  // completes ahead of the one it follows.
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = bid;
-  const bool skip = if_pending && *s.fin_pending == 0;   // nothing to apply (the first step, or after a flush)
   const Plan P = s.plan[j];
   double ncum_j = 0.0, cn_old = 0.0, inv_n = 0.0, beta = 0.0;
-  if (tid == 0 && !skip && P.cnt > 0) {
+  if (tid == 0 && P.cnt > 0) {
     ncum_j = s.ncum[j];
     cn_old = s.cnorm[j];
     inv_n = s.rtab[P.cnt];
@@ -777,13 +884,13 @@ __device__ __forceinline__ void finalize_body(const Dev& s, int if_pending, int 
   const int per = s.wslots * 4;
   const int p0 = s.wpair_first[j];
   const int np = (p0 + s.wpair_cnt[j] <= s.max_pairs) ? s.wpair_cnt[j] : 0;
-  if (warp == 0 && !skip && P.cnt > 0) {
+  if (warp == 0 && P.cnt > 0) {
     const double v = warp_sum((double)s.cmpart[(int64_t)j * 32 + lane]);
     if (lane == 0) cm_s = v;
   }
   KKM_GRID_DEP_WAIT();
-  KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top (or, the rotated gather, touches none of this)
-  if (skip || P.cnt == 0) return;
+  KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top
+  if (P.cnt == 0) return;
   // window-pass sums: element e of a tile's partials is sum e & 3 (A, Bdd, E, M);
   // with a stride of 256 every thread stays on sum tid & 3
   const double* wp = s.wpart + (int64_t)p0 * per;
@@ -806,20 +913,12 @@ __device__ __forceinline__ void finalize_body(const Dev& s, int if_pending, int 
       const double dn = (double)n;
       const double N = ncum_j + dn;      // points assigned to j so far, this batch included
       s.ncum[j] = N;
-      double a;
-      if (s.lr == 0) a = beta;               // sqrt(b_j / b)
-      else if (s.lr == 2) a = dn / N;        // sklearn: the running-mean rate
-      else a = s.eta;
+      const double a = learning_rate(s, dn, N, beta);
       const double keep = 1.0 - a;
       s.alpha[j] = a;
       const double cmc = cm_s * inv_n;
       s.cmc[j] = cmc;
-      // Sec. 4: ||C'||^2 = (1-a)^2 ||R||^2 + 2a(1-a) <R, m> + a^2 ||m||^2 with
-      // m = cm(B_j) and R = C - D, the part of the old center Eq. (1) keeps
-      const double m2 = M * inv_n * inv_n;
-      const double R2 = cn_old - 2.0 * A + Bdd;
-      const double Rm = cmc - E * inv_n;
-      const double cn = keep * keep * R2 + 2.0 * a * keep * Rm + a * a * m2;
+      const double cn = norm_recurrence(a, cmc, inv_n, cn_old, A, Bdd, E, M);
       s.cnorm[j] = cn;
       s.cnorm32[j] = (float)cn;
       s.head[j] = P.head_new;
@@ -856,7 +955,7 @@ __device__ __forceinline__ void finalize_body(const Dev& s, int if_pending, int 
   }
 }
 
-__global__ void __launch_bounds__(256) k_finalize(Dev s, int if_pending) { finalize_body(s, if_pending, blockIdx.x); }
+__global__ void __launch_bounds__(256) k_finalize(Dev s) { finalize_body(s, blockIdx.x); }
 
 // Seeds every window with C_1^j = phi(x_{init_idx[j]}), weight 1, ||C||^2 = K(x,x).
 __global__ void k_init_centers(Dev s, const int32_t* __restrict__ init_idx) {
@@ -1223,7 +1322,7 @@ __device__ __forceinline__ int group_run(const GroupPhase& g, int& local, int& n
 __global__ void k_group_gather(GroupPhase g) {
   int local, nblk;
   const int r = group_run(g, local, nblk);
-  gather_body(g.runs[r].s, nullptr, 0, local);
+  gather_body(g.runs[r].s, nullptr, local);
 }
 
 __global__ void __launch_bounds__(32 * AM_WARPS) k_group_argmin(GroupPhase g) {
@@ -1242,13 +1341,15 @@ __global__ void __launch_bounds__(1024) k_group_sort_plan(GroupPhase g) {
 __global__ void k_group_move(GroupPhase g) {
   int local, nblk;
   const int r = group_run(g, local, nblk);
-  move_body(g.runs[r].s, local, nblk);
+  KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();
+  move_body(g.runs[r].s, true, local, nblk);
 }
 
 __global__ void __launch_bounds__(256) k_group_finalize(GroupPhase g) {
   int local, nblk;
   const int r = group_run(g, local, nblk);
-  finalize_body(g.runs[r].s, 0, local);
+  finalize_body(g.runs[r].s, local);
 }
 
 // ------------------------------------------------------------------------
@@ -1469,8 +1570,8 @@ cudaError_t launch_sample(const Dev& s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st, bool rotated) {
-  cudaError_t e = launch_pdl(k_gather_batch, dim3((s.b * 32 + 255) / 256), dim3(256), 0, st, s, idx, rotated ? 1 : 0);
+cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st) {
+  cudaError_t e = launch_pdl(k_gather_batch, dim3((s.b * 32 + 255) / 256), dim3(256), 0, st, s, idx);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -1511,8 +1612,16 @@ cudaError_t launch_move(const Dev& s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const Dev& s, cudaStream_t st, bool if_pending) {
-  cudaError_t e = launch_pdl(k_finalize, dim3(s.k), dim3(256), 0, st, s, if_pending ? 1 : 0);
+cudaError_t launch_update(const Dev& s, const Dev* next, const int32_t* next_idx, cudaStream_t st) {
+  const int gblocks = next ? (s.b * 32 + 255) / 256 : 0;
+  const int blocks = gblocks + s.k + std::max((s.b + 7) / 8, s.num_sms * 2);
+  cudaError_t e = launch_pdl(k_update, dim3(blocks), dim3(256), 0, st, s, next ? *next : s, next_idx, gblocks);
+  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finalize(const Dev& s, cudaStream_t st) {
+  cudaError_t e = launch_pdl(k_finalize, dim3(s.k), dim3(256), 0, st, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
