@@ -343,10 +343,15 @@ struct TabBuf {
 // All return cudaGetLastError() of their launches.
 cudaError_t launch_sample(const Dev& s, cudaStream_t st);
 cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st);
-cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, cudaStream_t st);
+// id0 >= 0: the rows are the data points id0 ..; ahead: see k_gather_query
+cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, int64_t id0, bool ahead,
+                                cudaStream_t st);
 cudaError_t launch_dist_simt(const Dev& s, int rows, cudaStream_t st);
+// obj_acc: each block's FP64 sum of its rows' minima goes to obj_acc[block], or (obj_first false) is added to it
 cudaError_t launch_argmin(const Dev& s, int rows, const int32_t* forced, int32_t* assign_out,
-                          float* mind_out, float* dist_out, bool update, cudaStream_t st);
+                          float* mind_out, float* dist_out, bool update, cudaStream_t st, double* obj_acc = nullptr,
+                          bool obj_first = false);
+cudaError_t launch_sum(const double* a, int n, double* out, cudaStream_t st);   // sum of n doubles
 // set_pending: the step's window pass and norms run in the next step's distance pass (or a flush)
 cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st, bool set_pending = false);
 cudaError_t launch_move(const Dev& s, cudaStream_t st);

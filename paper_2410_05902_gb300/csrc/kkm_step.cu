@@ -235,15 +235,23 @@ __device__ __forceinline__ void gather_body(const Dev& s, const int32_t* __restr
 
 __global__ void k_gather_batch(Dev s, const int32_t* __restrict__ idx) { gather_body(s, idx, blockIdx.x); }
 
-__global__ void k_gather_query(Dev s, const float* __restrict__ Q, int64_t ldq, int rows) {
-  KKM_GRID_DEP_WAIT();
+// A warp per query row. id0 >= 0: the rows are the data points id0, id0 + 1, ..
+// and keep their index, so that one meeting its own support copy gets ||x - y||
+// = 0 exactly. ahead: the launch ahead is the distance pass of the chunk before
+// (which reads the other batch buffers), so the rows are gathered beside it,
+// before the grid-dependency wait.
+__global__ void k_gather_query(Dev s, const float* __restrict__ Q, int64_t ldq, int rows, int64_t id0, int ahead) {
+  if (!ahead) KKM_GRID_DEP_WAIT();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (warp >= rows) return;
-  double nrm = warp_store_row(s, Q + (int64_t)warp * ldq, warp, false);
-  if ((threadIdx.x & 31) == 0) {
-    s.xbn[warp] = (float)nrm;
-    s.xbi[warp] = -1;
+  if (warp < rows) {
+    double nrm = warp_store_row(s, Q + (int64_t)warp * ldq, warp, false);
+    if ((threadIdx.x & 31) == 0) {
+      s.xbn[warp] = (float)nrm;
+      s.xbi[warp] = id0 >= 0 ? (int32_t)(id0 + warp) : -1;
+    }
   }
+  if (ahead) KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();   // the next kernel reads only the tile tables before its own wait
 }
 
 // Block of 16 warps per 32 batch rows: lane = row, warp w handles centers
@@ -258,7 +266,8 @@ constexpr int AM_WARPS = 16;
 
 __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_t* __restrict__ forced,
                                             int32_t* __restrict__ assign_out, float* __restrict__ mind_out,
-                                            float* __restrict__ dist_out, int update, int bid) {
+                                            float* __restrict__ dist_out, double* __restrict__ obj_acc,
+                                            int obj_first, int update, int bid) {
   // Before the wait: the tile tables, the batch rows' norms and the forced
   // assignments. They come from kernels that completed before this one was
   // launched (it is launched once the distance pass has passed its own wait):
@@ -320,13 +329,18 @@ __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_
   r_inner[w][lane] = best_inner;
   r_f[w][lane] = f_inner;
   __syncthreads();
-  if (w != 0 || !live) return;
+  if (w != 0) return;
   for (int o = 1; o < AM_WARPS; ++o) {
     const float ob = r_best[o][lane];
     const int oj = r_j[o][lane];
     if (ob < best || (ob == best && oj < bj)) { best = ob; bj = oj; best_inner = r_inner[o][lane]; }
     f_inner += r_f[o][lane];   // only the warp owning fa is non-zero
   }
+  if (obj_acc) {               // this block's rows of every chunk, in chunk order
+    const double t = warp_sum(live ? (double)best : 0.0);
+    if (lane == 0) obj_acc[bid] = obj_first ? t : obj_acc[bid] + t;
+  }
+  if (!live) return;
   int a = bj;
   float a_inner = best_inner;
   if (forced) {
@@ -349,8 +363,9 @@ __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_
 __global__ void __launch_bounds__(32 * AM_WARPS) k_argmin(Dev s, int rows, const int32_t* __restrict__ forced,
                                                           int32_t* __restrict__ assign_out,
                                                           float* __restrict__ mind_out,
-                                                          float* __restrict__ dist_out, int update) {
-  argmin_body(s, rows, forced, assign_out, mind_out, dist_out, update, blockIdx.x);
+                                                          float* __restrict__ dist_out,
+                                                          double* __restrict__ obj_acc, int obj_first, int update) {
+  argmin_body(s, rows, forced, assign_out, mind_out, dist_out, obj_acc, obj_first, update, blockIdx.x);
 }
 
 __device__ int tile_count(const Dev& s, int& head, int& size, int& work);
@@ -1006,6 +1021,15 @@ __global__ void k_load_rows(Dev s) {
   }
 }
 
+// The sum of n doubles into *out (single warp, fixed order).
+__global__ void __launch_bounds__(32) k_sum(const double* __restrict__ a, int n, double* out) {
+  KKM_GRID_DEP_WAIT();
+  double t = 0.0;
+  for (int i = threadIdx.x; i < n; i += 32) t += a[i];
+  t = warp_sum(t);
+  if (threadIdx.x == 0) *out = t;
+}
+
 // scale * (FP64 sum of mind[0..rows)) into *out (single CTA, fixed order).
 __global__ void __launch_bounds__(1024) k_mind_sum(Dev s, int rows, double scale, double* out) {
   KKM_GRID_DEP_WAIT();
@@ -1329,7 +1353,7 @@ __global__ void __launch_bounds__(32 * AM_WARPS) k_group_argmin(GroupPhase g) {
   int local, nblk;
   const int r = group_run(g, local, nblk);
   const Dev& s = g.runs[r].s;
-  argmin_body(s, s.b, nullptr, nullptr, nullptr, nullptr, 1, local);
+  argmin_body(s, s.b, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1, local);
 }
 
 __global__ void __launch_bounds__(1024) k_group_sort_plan(GroupPhase g) {
@@ -1576,18 +1600,27 @@ cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, cudaStream_t st) {
+cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, int64_t id0, bool ahead,
+                                cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  cudaError_t e = launch_pdl(k_gather_query, dim3((rows * 32 + 255) / 256), dim3(256), 0, st, s, Q, ldq, rows);
+  cudaError_t e = launch_pdl(k_gather_query, dim3((rows * 32 + 255) / 256), dim3(256), 0, st, s, Q, ldq, rows, id0,
+                             ahead ? 1 : 0);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
 cudaError_t launch_argmin(const Dev& s, int rows, const int32_t* forced, int32_t* assign_out,
-                          float* mind_out, float* dist_out, bool update, cudaStream_t st) {
+                          float* mind_out, float* dist_out, bool update, cudaStream_t st, double* obj_acc,
+                          bool obj_first) {
   if (rows <= 0) return cudaSuccess;
   cudaError_t e = launch_pdl(k_argmin, dim3((rows + 31) / 32), dim3(32 * AM_WARPS), 0, st, s, rows, forced,
-                             assign_out, mind_out, dist_out, update ? 1 : 0);
+                             assign_out, mind_out, dist_out, obj_acc, obj_first ? 1 : 0, update ? 1 : 0);
+  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sum(const double* a, int n, double* out, cudaStream_t st) {
+  cudaError_t e = launch_pdl(k_sum, dim3(1), dim3(32), 0, st, a, n, out);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
