@@ -15,6 +15,8 @@
 // where W is the old window, D its dropped prefix (old weights) and B the new
 // block. Each tile writes its four FP64 partial sums; k_finalize adds them in
 // tile order.
+#include <algorithm>
+
 #include "kkm_internal.cuh"
 
 namespace kkm {
@@ -44,38 +46,68 @@ __device__ __forceinline__ float4 load4(const void* rowp, int k, int dp) {
   }
 }
 
-// acc[i][j] = sum_k A[ty*4+i][k] * B[tx*4+j][k] for a 64x64 tile. A and B point
-// at the tiles' first rows (element type by form); rows are `ld` elements apart
-// and the product runs over kend columns (zero padded, a multiple of BK).
-// DIFF: acc[i][j] = sum_k (A[ty*4+i][k] - B[tx*4+j][k])^2 instead.
-template <int F, bool DIFF = false>
+// Operand chunks of BK columns, two buffers: columns of 16 MR rows of A and 64 of B.
+template <int MR> struct GramSmem {
+  float A[2][BK][16 * MR + 4];
+  float B[2][BK][BN + 4];
+};
+
+// acc[i][j] = sum_k A[ty*MR+i][k] * B[tx*4+j][k] for a 16 MR x 64 tile. A and B
+// point at the tiles' first rows (element type by form); rows are `ld` elements
+// apart and the product runs over kend columns (zero padded, a multiple of BK).
+// DIFF: acc[i][j] = sum_k (A[ty*MR+i][k] - B[tx*4+j][k])^2 instead. The next BK
+// columns are loaded into registers while the current ones are multiplied out of
+// shared memory, with one barrier per BK columns. Each sum is one chain over k
+// whatever MR is.
+template <int F, int MR, bool DIFF>
 __device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void* __restrict__ B,
-                                          int ld, int kend, int dp, float (&acc)[4][4],
-                                          float (*As)[BM + 4], float (*Bs)[BN + 4]) {
+                                          int ld, int kend, int dp, float (&acc)[MR][4], GramSmem<MR>& sm) {
+  constexpr int NA = MR / 4;                     // 64-row slices of A a loader thread fills
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int lr = tid >> 2, lk = (tid & 3) * 4;   // loader: row, k offset
   const int esz = (F == FORM_FP32) ? 4 : 2;
   const char* arow = (const char*)A + (int64_t)lr * ld * esz;
   const char* brow = (const char*)B + (int64_t)lr * ld * esz;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MR; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-  for (int k0 = 0; k0 < kend; k0 += BK) {
-    const float4 a = load4<F>(arow, k0 + lk, dp);
-    const float4 b = load4<F>(brow, k0 + lk, dp);
-    __syncthreads();
-    As[lk + 0][lr] = a.x; As[lk + 1][lr] = a.y; As[lk + 2][lr] = a.z; As[lk + 3][lr] = a.w;
-    Bs[lk + 0][lr] = b.x; Bs[lk + 1][lr] = b.y; Bs[lk + 2][lr] = b.z; Bs[lk + 3][lr] = b.w;
-    __syncthreads();
+  float4 a[NA], b;
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) a[q] = load4<F>(arow + (int64_t)q * 64 * ld * esz, k0 + lk, dp);
+    b = load4<F>(brow, k0 + lk, dp);
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int r = q * 64 + lr;
+      sm.A[buf][lk + 0][r] = a[q].x; sm.A[buf][lk + 1][r] = a[q].y;
+      sm.A[buf][lk + 2][r] = a[q].z; sm.A[buf][lk + 3][r] = a[q].w;
+    }
+    sm.B[buf][lk + 0][lr] = b.x; sm.B[buf][lk + 1][lr] = b.y;
+    sm.B[buf][lk + 2][lr] = b.z; sm.B[buf][lk + 3][lr] = b.w;
+  };
+  load(0);
+  __syncthreads();                               // the previous tile's readers are done
+  store(0);
+  int buf = 0;
+  for (int k0 = 0; k0 < kend; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < kend;
+    if (more) load(k0 + BK);
+    __syncthreads();                             // this buffer is filled, the other one read
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float ar[4] = {av.x, av.y, av.z, av.w};
+      float ar[MR];
+#pragma unroll
+      for (int i = 0; i < MR; i += 4) {
+        const float4 av = *reinterpret_cast<const float4*>(&sm.A[buf][kk][ty * MR + i]);
+        ar[i] = av.x; ar[i + 1] = av.y; ar[i + 2] = av.z; ar[i + 3] = av.w;
+      }
+      const float4 bv = *reinterpret_cast<const float4*>(&sm.B[buf][kk][tx * 4]);
       const float br[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < MR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if constexpr (DIFF) {
@@ -86,6 +118,7 @@ __device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void
           }
         }
     }
+    if (more) store(buf ^ 1);
   }
 }
 
@@ -95,83 +128,113 @@ __device__ __forceinline__ const void* rows_ptr(const Dev& s, bool support, int6
   else return (support ? s.ybh : s.xbh) + row * s.ld;
 }
 
-__device__ __forceinline__ float sum16(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 8);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  return v;
-}
-
-// Item w of a run's distance pass (row tile w % R of support tile w / R).
-template <int F>
-__device__ __forceinline__ void dist_simt_item(const Dev& s, int rows, int R, int w, float (*As)[BM + 4],
-                                               float (*Bs)[BN + 4]) {
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const bool lap = s.kind == K_LAPLACE;
-  {
-    const int t = w / R, rt = w % R;
-    const Tile T = s.tiles[t];
-    float acc[4][4];
-    // Laplacian kernel: ||x - y||^2 from the differences. Through ||x||^2 +
-    // ||y||^2 - 2 <x, y> a query row equal to a support row (no data index to
-    // recognise it by) keeps d2 ~ eps ||x||^2, which the square root magnifies.
-    if (lap)
-      gram_tile<F, true>(rows_ptr<F>(s, false, (int64_t)rt * BM), rows_ptr<F>(s, true, T.row0), s.ld,
-                         F == FORM_FP32 ? s.ld : s.dp, s.dp, acc, As, Bs);
-    else
-      gram_tile<F>(rows_ptr<F>(s, false, (int64_t)rt * BM), rows_ptr<F>(s, true, T.row0), s.ld,
-                   F == FORM_FP32 ? s.ld : s.dp, s.dp, acc, As, Bs);
-    float yn[4], wy[4];
-    int yi[4];
+// One level of the row sums' tree: N rows' values, half of them handed to the
+// lane across `o`, which keeps the other half. The lane whose bit o is set keeps the upper half.
+template <int N>
+__device__ __forceinline__ void fold_rows(float (&v)[N], int o) {
+  const bool up = (threadIdx.x & o) != 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = tx * 4 + j;
-      const bool ok = c < T.ncols;
-      const int64_t g = (int64_t)T.row0 + (ok ? c : 0);
-      yn[j] = s.yn[g];
-      yi[j] = s.yi[g];
-      wy[j] = ok ? s.w32[g] : 0.0f;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = rt * BM + ty * 4 + i;
-      const int rr = r < rows ? r : 0;
-      const float xn = s.xbn[rr];
-      const int xi = s.xbi[rr];
-      float sum = 0.0f;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool same = xi >= 0 && xi == yi[j];
-        const float kv = lap ? exp2f(sqrtf(same ? 0.0f : acc[i][j]) * s.negc)
-                             : kernel_from_gram(s.kind, acc[i][j], xn, yn[j], same, s.negc, (float)s.coef0,
-                                                s.degree);
-        sum += (tx * 4 + j < T.ncols) ? wy[j] * kv : 0.0f;
-      }
-      sum = sum16(sum);
-      if (tx == 0 && r < rows) s.part[(int64_t)t * s.bpad + r] = sum;
-    }
+  for (int i = 0; i < N / 2; ++i) {
+    const float keep = up ? v[i + N / 2] : v[i], give = up ? v[i] : v[i + N / 2];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
   }
 }
 
-template <int F>
-__device__ __forceinline__ void dist_simt_body(const Dev& s, int rows, int bid, int nblk) {
-  KKM_GRID_DEP_WAIT();
-  KKM_LAUNCH_DEPENDENTS();
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN + 4];
-  const int R = (rows + BM - 1) / BM;
-  const int total = R * (*s.ntiles);
-  for (int w = bid; w < total; w += nblk) dist_simt_item<F>(s, rows, R, w, As, Bs);
+// The weighted kernel sums of a tile's rows (16 MR rows, 64 columns): per thread
+// four columns in order, then the 16 threads of a row in a tree over lane bits
+// 3, 2, 1, 0. The tree works on all of a thread's rows at once, each level
+// halving the rows a lane holds: MR + 16 / MR - 1 shuffles or so instead of 4 MR.
+template <int KIND, int MR>
+__device__ __forceinline__ void dist_simt_sums(const Dev& s, int rows, int t, int row0, const Tile& T,
+                                               const float (&acc)[MR][4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float yn[4], wy[4];
+  int yi[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = tx * 4 + j;
+    const bool ok = c < T.ncols;
+    const int64_t g = (int64_t)T.row0 + (ok ? c : 0);
+    yn[j] = s.yn[g];
+    yi[j] = s.yi[g];
+    wy[j] = ok ? s.w32[g] : 0.0f;
+  }
+  float v[MR];
+#pragma unroll
+  for (int i = 0; i < MR; ++i) {
+    const int r = row0 + ty * MR + i;
+    const int rr = r < rows ? r : 0;
+    const float xn = s.xbn[rr];
+    const int xi = s.xbi[rr];
+    float sum = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool same = xi >= 0 && xi == yi[j];
+      const float kv = KIND == K_LAPLACE ? exp2f(sqrtf(same ? 0.0f : acc[i][j]) * s.negc)
+                                         : kernel_from_gram(KIND, acc[i][j], xn, yn[j], same, s.negc, (float)s.coef0,
+                                                            s.degree);
+      sum += (tx * 4 + j < T.ncols) ? wy[j] * kv : 0.0f;
+    }
+    v[i] = sum;
+  }
+  int row = 0, o = 8;                            // the row this lane ends up with; lanes left to add over
+  if constexpr (MR == 8) {
+    float (&v8)[8] = v;
+    fold_rows(v8, 8);
+    row = (tx & 8) >> 1;
+    o = 4;
+  }
+  float v4[4] = {v[0], v[1], v[2], v[3]};
+  fold_rows(v4, o);
+  row += (tx & o) ? 2 : 0;
+  o >>= 1;
+  float v2[2] = {v4[0], v4[1]};
+  fold_rows(v2, o);
+  row += (tx & o) ? 1 : 0;
+  o >>= 1;
+  float sum = v2[0];
+  const int mask = 2 * o - 1;                    // lanes that end up with the same row
+  for (; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  const int r = row0 + ty * MR + row;
+  if ((tx & mask) == 0 && r < rows) s.part[(int64_t)t * s.bpad + r] = sum;
 }
 
-template <int F>
-__global__ void __launch_bounds__(NT) k_dist_simt(Dev s, int rows) { dist_simt_body<F>(s, rows, blockIdx.x, gridDim.x); }
+// Item w of a run's distance pass (row tile w % R of support tile w / R; 16 MR rows a tile).
+template <int F, int MR>
+__device__ __forceinline__ void dist_simt_item(const Dev& s, int rows, int R, int w, GramSmem<MR>& sm) {
+  const int t = w / R, row0 = (w % R) * 16 * MR;
+  const Tile T = s.tiles[t];
+  const void *A = rows_ptr<F>(s, false, row0), *B = rows_ptr<F>(s, true, T.row0);
+  const int kend = F == FORM_FP32 ? s.ld : s.dp;
+  float acc[MR][4];
+  // Laplacian kernel: ||x - y||^2 from the differences. Through ||x||^2 +
+  // ||y||^2 - 2 <x, y> a query row equal to a support row (no data index to
+  // recognise it by) keeps d2 ~ eps ||x||^2, which the square root magnifies.
+  if (s.kind == K_LAPLACE) {
+    gram_tile<F, MR, true>(A, B, s.ld, kend, s.dp, acc, sm);
+    dist_simt_sums<K_LAPLACE, MR>(s, rows, t, row0, T, acc);
+    return;
+  }
+  gram_tile<F, MR, false>(A, B, s.ld, kend, s.dp, acc, sm);
+  if (s.kind == K_GAUSS) dist_simt_sums<K_GAUSS, MR>(s, rows, t, row0, T, acc);
+  else if (s.kind == K_LINEAR) dist_simt_sums<K_LINEAR, MR>(s, rows, t, row0, T, acc);
+  else dist_simt_sums<K_POLY, MR>(s, rows, t, row0, T, acc);
+}
+
+template <int F, int MR>
+__global__ void __launch_bounds__(NT) k_dist_simt(Dev s, int rows) {
+  KKM_GRID_DEP_WAIT();
+  KKM_LAUNCH_DEPENDENTS();
+  __shared__ __align__(16) GramSmem<MR> sm;
+  const int R = (rows + 16 * MR - 1) / (16 * MR);
+  const int total = R * (*s.ntiles);
+  for (int w = blockIdx.x; w < total; w += gridDim.x) dist_simt_item<F, MR>(s, rows, R, w, sm);
+}
 
 // Pair w of a run's window pass; its four sums go to wpart[w] (slot 0).
 template <int F>
-__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms, float (*As)[BM + 4],
-                                                float (*Bs)[BN + 4], double (*red)[NT / 32]) {
+__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms, GramSmem<4>& sm,
+                                                double (*red)[NT / 32]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
   {
     const WPair pr = s.wpairs[w];
@@ -183,8 +246,23 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms,
     else { r0 = P.tail_c; rn = P.cnt; c0 = P.tail_c; cn = P.cnt; }
     const int rs = r0 + pr.rt * BM, cs = c0 + pr.ct * BN;
     float acc[4][4];
-    gram_tile<F>(rows_ptr<F>(s, true, base + rs), rows_ptr<F>(s, true, base + cs), s.ld,
-                 F == FORM_FP32 ? s.ld : s.dp, s.dp, acc, As, Bs);
+    gram_tile<F, 4, false>(rows_ptr<F>(s, true, base + rs), rows_ptr<F>(s, true, base + cs), s.ld,
+                           F == FORM_FP32 ? s.ld : s.dp, s.dp, acc, sm);
+    // FP64 issues at 1/64 of the FP32 rate on this chip, so the row weight is
+    // taken out of the column sums: a conversion and one to two FP64 operations
+    // per element where the product of both weights took four to five
+    double yw[4];
+    float yn[4];
+    int yi[4], qp[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int qc = pr.ct * BN + tx * 4 + j;
+      qp[j] = qc < cn ? cs + tx * 4 + j : -1;            // position in the region
+      const int64_t q = base + (qp[j] >= 0 ? qp[j] : cs);
+      yn[j] = s.yn[q];
+      yi[j] = s.yi[q];
+      yw[j] = pr.kind == 0 && qp[j] >= 0 && qp[j] < P.tail_c ? s.wwin64[q] : 0.0;
+    }
     double sA = 0.0, sB = 0.0, sE = 0.0, sM = 0.0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -193,37 +271,38 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms,
       const int64_t p = base + rs + ty * 4 + i;
       const float xn = s.yn[p];
       const int xi = s.yi[p];
-      const double wp = s.wwin64[p];
+      double ra = 0.0, rb = 0.0, re = 0.0;             // this row's W (not D), D and B columns
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int qc = pr.ct * BN + tx * 4 + j;
-        if (qc >= cn) continue;
-        const int qpos = cs + tx * 4 + j;                 // position in the region
-        const int64_t q = base + qpos;
-        const double kv = (double)kernel_from_gram(s.kind, acc[i][j], xn, s.yn[q], xi == s.yi[q],
-                                                   s.negc, (float)s.coef0, s.degree);
-        if (pr.kind == 0) {
-          if (qpos < P.tail_c) {
-            const double ww = wp * s.wwin64[q] * kv;
-            sA += ww;
-            if (qpos < P.head_new) sB += ww;
-          } else {
-            sE += wp * kv;
-          }
-        } else {
-          sM += kv;
-        }
+        if (qp[j] < 0) continue;
+        const double kv = (double)kernel_from_gram(s.kind, acc[i][j], xn, yn[j], xi == yi[j], s.negc,
+                                                   (float)s.coef0, s.degree);
+        if (pr.kind != 0) sM += kv;
+        else if (qp[j] >= P.tail_c) re += kv;
+        else if (qp[j] < P.head_new) rb += yw[j] * kv;
+        else ra += yw[j] * kv;
+      }
+      if (pr.kind == 0) {
+        const double wp = s.wwin64[p];
+        sA += wp * (ra + rb);
+        sB += wp * rb;
+        sE += wp * re;
       }
     }
-    // fixed-order block reduction of the four sums
+    // fixed-order block reduction of the four sums: two levels hand half of them
+    // to the other lane, so that lanes 0, 8, 16, 24 end with sA, sE, sB, sM
+    {
+      const bool hi = lane & 16, up = lane & 8;
+      double k0 = hi ? sB : sA, k1 = hi ? sM : sE;
+      k0 += __shfl_xor_sync(0xffffffffu, hi ? sA : sB, 16);
+      k1 += __shfl_xor_sync(0xffffffffu, hi ? sE : sM, 16);
+      double v = up ? k1 : k0;
+      v += __shfl_xor_sync(0xffffffffu, up ? k0 : k1, 8);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sA += __shfl_xor_sync(0xffffffffu, sA, o);
-      sB += __shfl_xor_sync(0xffffffffu, sB, o);
-      sE += __shfl_xor_sync(0xffffffffu, sE, o);
-      sM += __shfl_xor_sync(0xffffffffu, sM, o);
+      for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      // red[0..3]: sA, sB, sE, sM
+      if ((lane & 7) == 0) red[(hi ? 1 : 0) + (up ? 2 : 0)][warp] = v;
     }
-    if (lane == 0) { red[0][warp] = sA; red[1][warp] = sB; red[2][warp] = sE; red[3][warp] = sM; }
     __syncthreads();
     if (tid < 16) {   // slot 0 holds the tile's sums, slots 1-3 are zero
       double v = 0.0;
@@ -250,11 +329,10 @@ template <int F>
 __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bid, int nblk) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN + 4];
+  __shared__ __align__(16) GramSmem<4> sm;
   __shared__ double red[4][NT / 32];
   const int total = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
-  for (int w = bid; w < total; w += nblk) wgram_simt_item<F>(s, w, norms, As, Bs, red);
+  for (int w = bid; w < total; w += nblk) wgram_simt_item<F>(s, w, norms, sm, red);
 }
 
 template <int F>
@@ -273,8 +351,7 @@ template <int F, int MODE>
 __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN + 4];
+  __shared__ __align__(16) GramSmem<4> sm;
   __shared__ double red[4][NT / 32];
   __shared__ int off[GROUP_MAX_RUNS + 1];
   const int nr = g.nruns < GROUP_MAX_RUNS ? g.nruns : GROUP_MAX_RUNS;
@@ -297,22 +374,35 @@ __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
       else hi = mid;
     }
     const Dev& s = g.runs[lo].s;
-    if constexpr (MODE == 0) dist_simt_item<F>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], As, Bs);
-    else wgram_simt_item<F>(s, w - off[lo], false, As, Bs, red);
+    if constexpr (MODE == 0) dist_simt_item<F, 4>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], sm);
+    else wgram_simt_item<F>(s, w - off[lo], false, sm, red);
   }
 }
 
 }  // namespace
 
+// 2048 x 64 batch rows against about 11000 support rows (k = 50): the whole
+// iteration took 188 us, 131 of it this pass, with 64-row tiles, one buffer and
+// a runtime kernel kind; now 150 us with the window pass's fewer FP64 operations.
+// 128-row tiles where the pass still has two items for every SM: a thread's 8 x
+// 4 products take three shared-memory reads per 32 FMAs, the 64-row tile's 4 x 4
+// two per 16. The number of support tiles is known on the device only; a full
+// window has at least tau / 64 of them, a center without one at most none.
+template <int F>
+static cudaError_t launch_dist_form(const Dev& s, int rows, cudaStream_t st) {
+  const int64_t tiles = (int64_t)s.k * std::max(1, s.tau / BN);
+  if (rows > BM && (rows + 127) / 128 * tiles >= 2 * s.num_sms)
+    return launch_pdl(k_dist_simt<F, 8>, dim3(s.num_sms * 3), dim3(NT), 0, st, s, rows);
+  return launch_pdl(k_dist_simt<F, 4>, dim3(s.num_sms * 4), dim3(NT), 0, st, s, rows);
+}
+
 cudaError_t launch_dist_simt(const Dev& s, int rows, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  const int blocks = s.num_sms * 4;
   switch (s.form) {
-    case FORM_FP32: return launch_pdl(k_dist_simt<FORM_FP32>, dim3(blocks), dim3(NT), 0, st, s, rows);
-    case FORM_BF16: return launch_pdl(k_dist_simt<FORM_BF16>, dim3(blocks), dim3(NT), 0, st, s, rows);
-    default: return launch_pdl(k_dist_simt<FORM_BF16X3>, dim3(blocks), dim3(NT), 0, st, s, rows);
+    case FORM_FP32: return launch_dist_form<FORM_FP32>(s, rows, st);
+    case FORM_BF16: return launch_dist_form<FORM_BF16>(s, rows, st);
+    default: return launch_dist_form<FORM_BF16X3>(s, rows, st);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_wgram(const Dev& s, cudaStream_t st, bool norms) {
