@@ -62,11 +62,16 @@ cudaError_t tc_prepare(Dev& s, void* maps_out) {
   return cudaSuccess;
 }
 
+// Whether a launch's batch tile stays in shared memory between items (layout()).
+static bool tc_resident(const Dev& s, int cols) {
+  const int64_t nsl = s.dp / (s.form == FORM_TF32 ? 32 : KS) * (s.form == FORM_BF16X3 ? 2 : 1);
+  return nsl * A_BYTES <= A_RES_MAX && (RING_BYTES - nsl * A_BYTES) / (nsl * cols * KS * 2) >= 2;
+}
+
 int64_t tc_item_bytes(const Dev& s, int cols, bool with_a) {
   const int nsl = s.dp / (s.form == FORM_TF32 ? 32 : KS) * (s.form == FORM_BF16X3 ? 2 : 1);
   const int64_t b = (int64_t)nsl * cols * KS * 2, a = (int64_t)nsl * A_BYTES;
-  const bool resident = a <= A_RES_MAX && (RING_BYTES - a) / b >= 2;   // layout()
-  return b + (with_a || !resident ? a : 0);
+  return b + (with_a || !tc_resident(s, cols) ? a : 0);
 }
 
 int tc_parts_per_tile(int tn) {
@@ -79,6 +84,11 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
   // ahead writes none of what it stages (the gather, or this pass itself)
   Dev d = s;
   d.pre_b = (stage_early && s.pre_b) ? 1 : 0;
+  // CTA pairs where the operands stream and the row tiles pair up with little left over: an odd last
+  // row tile costs the pair a whole one
+  const int R = (rows + TM - 1) / TM;
+  if (d.tn == 256 && !tc_resident(d, 256) && R >= 2 && (R % 2 == 0 || R >= 5))
+    return launch_dist_pair(d, maps, rows, st);
   if (d.tn == 64) return launch_mode<0, 64>(d, maps, rows, false, st);
   if (d.tn == 256) return launch_mode<0, 256>(d, maps, rows, false, st);
   return launch_mode<0, 128>(d, maps, rows, false, st);

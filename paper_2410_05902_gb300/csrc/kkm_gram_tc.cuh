@@ -43,6 +43,18 @@
 // sums meet in shared memory (chosen per run, so that a run's results do not
 // depend on how a launch splits its items).
 //
+// CTA pairs (PAIR, distance pass with 256-column tiles whose operands stream):
+// two CTAs of a cluster take two row tiles against the same support tile, and
+// the tcgen05 pair form multiplies both at once: each CTA stages its own A rows
+// and half of the B rows, so a 128-byte slice costs 32 KB of operand traffic per
+// CTA where a CTA alone takes 48 KB. Alone, operands arrived at about 42 bytes per
+// clock and SM while the MMAs could use 96, which is what bounded rows of
+// more than 128 BF16 columns.
+// The even CTA's MMA warp issues for both; its full barriers count both CTAs' copies,
+// its commits arrive on both CTAs' stage and accumulator barriers, and both
+// epilogues release an accumulator at the even CTA. Row tiles, partials and their
+// sums are those of the single-CTA form, bit for bit.
+//
 // Gaussian kernel values without a per-element row term: with rc = -log2(e)
 // ||x||^2 / kappa and t = (2 log2(e) / kappa) g - log2(e) ||y||^2 / kappa,
 //   K(x, y) = 2^(rc + t) = 2^rc 2^t,
@@ -54,6 +66,7 @@
 // makes the role stop. On the way out the producer waits for its last copies
 // to land and the MMA warp waits for its last MMAs, so TMEM is freed only once
 // nothing is in flight.
+#include <algorithm>
 #include <cstddef>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -133,6 +146,19 @@ __device__ __forceinline__ Layout layout(int nks) {
   return L;
 }
 
+// CTA pairs always stream: a stage holds one slice of A and of this CTA's half of B.
+template <bool X3>
+__device__ __forceinline__ Layout pair_layout(int nks) {
+  Layout L;
+  L.nsl = nks * (X3 ? 2 : 1);
+  L.res = false;
+  L.a_bytes = 0;
+  L.sb = (X3 ? 2 : 1) * 2 * A_BYTES;
+  const int n = RING_BYTES / L.sb;
+  L.nst = n < STAGES ? n : STAGES;
+  return L;
+}
+
 // The slices of a whole tile (hi slices, then lo slices at column dp) into dst + t * tb.
 __device__ __forceinline__ void tile_issue(bool lead, int n, int nks, int dp, int kse, uint8_t* dst, int tb,
                                            const CUtensorMap* tm, uint64_t* bar, int y) {
@@ -145,9 +171,9 @@ __device__ __forceinline__ void tile_issue(bool lead, int n, int nks, int dp, in
 // 10-12, both K-major (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in
 // bits 24-28.
 template <int OP>
-__device__ __forceinline__ uint32_t idesc(uint32_t n) {
+__device__ __forceinline__ uint32_t idesc(uint32_t n, uint32_t m = TM) {
   constexpr uint32_t t = OP == OP_TF32 ? 2u : 1u;
-  return (1u << 4) | (t << 7) | (t << 10) | ((n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+  return (1u << 4) | (t << 7) | (t << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
 // An item's ranges. Distance item: only tnew, the tile's columns. Window item:
@@ -296,27 +322,68 @@ constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // One MMA on a 32-byte K step of the 128-byte swizzled rows: K = 16 BF16
 // values (kind::f16) or K = 8 TF32 values (kind::tf32).
-template <int OP>
+// PAIR: M = 256, rows 0-127 in this CTA and 128-255 in its peer (the addresses
+// hold in both).
+template <int OP, bool PAIR = false>
 __device__ __forceinline__ void mma_op(bool lead, uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
                                        uint32_t accum) {
-#define KKM_MMA(kind)                                                                            \
+#define KKM_MMA(group, kind)                                                                     \
   asm volatile(                                                                                  \
       "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t" \
       "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"                                       \
-      "@q tcgen05.mma.cta_group::1." kind " [%0], da, db, %3, p;\n\t}"                           \
+      "@q tcgen05.mma.cta_group::" group "." kind " [%0], da, db, %3, p;\n\t}"                   \
       ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(idesc), "r"(accum), "r"(DESC_HI), "r"((uint32_t)lead) \
       : "memory")
-  if constexpr (OP == OP_TF32) KKM_MMA("kind::tf32");
-  else KKM_MMA("kind::f16");
+  if constexpr (OP == OP_TF32 && PAIR) KKM_MMA("2", "kind::tf32");
+  else if constexpr (OP == OP_TF32) KKM_MMA("1", "kind::tf32");
+  else if constexpr (PAIR) KKM_MMA("2", "kind::f16");
+  else KKM_MMA("1", "kind::f16");
 #undef KKM_MMA
 }
 
+template <bool PAIR = false>
 __device__ __forceinline__ void mma_commit(bool lead, uint64_t* bar) {
+#define KKM_COMMIT(group)                                                                          \
+  asm volatile(                                                                                    \
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"                                            \
+      "@q tcgen05.commit.cta_group::" group ".mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" \
+      ::"r"(smem_u32(bar)), "r"((uint32_t)lead)                                                    \
+      : "memory")
+  if constexpr (PAIR) KKM_COMMIT("2");
+  else KKM_COMMIT("1");
+#undef KKM_COMMIT
+}
+
+// CTA pairs. The address of a shared variable in the pair's even CTA:
+__device__ __forceinline__ uint32_t lead_addr(const void* p) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
+  return a;
+}
+// both CTAs' threads meet here
+__device__ __forceinline__ void pair_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// a copy into this CTA's shared memory that counts at a barrier of the even CTA
+__device__ __forceinline__ void tma_load_2d_pair(bool lead, void* dst, const CUtensorMap* map, uint32_t bar, int x,
+                                                 int y) {
   asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(bar), "r"(x), "r"(y), "r"((uint32_t)lead)
+      : "memory");
+}
+// arrives on the barrier at bar's address in both CTAs once the pair's MMAs so far are done
+__device__ __forceinline__ void mma_commit_pair(bool lead, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t.reg .b16 both;\n\tsetp.ne.b32 q, %1, 0;\n\tmov.b16 both, 3;\n\t"
+      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], both;\n\t}"
       ::"r"(smem_u32(bar)), "r"((uint32_t)lead)
       : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
 // A whole warp's wait, the same answer on every lane.
@@ -567,6 +634,15 @@ template <int TNV> struct Place {
     __syncwarp();
     if (lane == 0) mbar_arrive(b);
   }
+  // the accumulator's barrier: the even CTA's, where the pair's MMAs are issued
+  template <bool PAIR> __device__ void arrive_acc(uint64_t* b) const {
+    if constexpr (PAIR) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(lead_addr(b));
+    } else {
+      arrive(b);
+    }
+  }
   __device__ void sync_all() const { asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory"); }
   __device__ void sync_group() const { asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory"); }
   __device__ void sync_team() const {
@@ -581,7 +657,7 @@ template <int TNV> struct Place {
 // chunks past it are skipped, and the last partial may be plain 0. A warp
 // covers its quadrant's 32 rows; it releases the accumulator once its last
 // chunk is in registers and the metadata slot once its arithmetic is done.
-template <int KIND, int TNV>
+template <int KIND, int TNV, bool PAIR>
 __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem, const Place<TNV>& pl,
                                           uint32_t local, int tile, int row0, int rows, bool dead) {
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT, QPP = Place<TNV>::QPP;
@@ -623,7 +699,7 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
     auto release = [&]() {                      // the accumulator is free again
       if (!all) {
         tc_fence_before();
-        pl.arrive(&sh.tempty[buf]);
+        pl.template arrive_acc<PAIR>(&sh.tempty[buf]);
       }
     };
     constexpr int NB = DIST_NB, CW = 8 * NB;
@@ -683,7 +759,7 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
         *out = v;
       }
       if (!dead) {
-        pl.arrive(&sh.tempty[buf]);
+        pl.template arrive_acc<PAIR>(&sh.tempty[buf]);
         pl.arrive(&sh.mempty[ms]);
       }
     }
@@ -867,9 +943,9 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
 
 // The epilogue warps (2-17): window items [rw.lo, rw.hi) first (MODE 1, 2),
 // then distance items [rd.lo, rd.hi) (MODE 0, 2).
-template <int KIND, int MODE, int TNV>
+template <int KIND, int MODE, int TNV, bool PAIR>
 __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rw, Range rd, int T,
-                                         int rows, int warp, int lane, bool all, bool norms) {
+                                         int rows, int warp, int lane, bool all, bool norms, int rank) {
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
   const Place<TNV> pl(warp, lane, all);
   // part[] must hold GPT partials per tile and wpart[] one slot of four sums
@@ -902,7 +978,8 @@ __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t
       if (!pl.mine(local)) continue;
       wait(local);
       const int item = rd.lo + (int)local - nw;
-      dist_item<KIND, TNV>(s, sh, tmem, pl, local, item % T, (item / T) * TM, rows, dead);
+      dist_item<KIND, TNV, PAIR>(s, sh, tmem, pl, local, item % T, (PAIR ? 2 * (item / T) + rank : item / T) * TM,
+                                 rows, dead);
     }
   }
 }
@@ -994,14 +1071,16 @@ __device__ __forceinline__ Range my_range(int total, int cta, int ncta) {
 // construction. The metadata warp copies them into a ring of slots next to
 // the operands, so nothing on the epilogue's path waits on a global load.
 // Item descriptors are fetched 32 at a time, one per lane.
-template <int KIND, int MODE, int OP, int TNV>
+template <int KIND, int MODE, int OP, int TNV, bool PAIR = false>
 __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUtensorMap* tmA, const CUtensorMap* tmB,
                                              const CUtensorMap* tmW, const CUtensorMap* tmN, int cta, int ncta,
                                              bool norms = false,
                                              Range ovr = Range{-1, -1}, int flags = TC_ALLOC | TC_FREE) {
+  static_assert(!PAIR || (MODE == 0 && TNV == 256), "CTA pairs take 256-column distance items");
   constexpr bool X3 = OP == OP_X3;
   constexpr int KSE = OP == OP_TF32 ? 32 : KS;   // operand elements per slice row
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
+  const int rank = PAIR ? cta & 1 : 0;           // the CTA's place in its pair
   // one B slice: the rows its live columns need (a box of 64, 128 or TNV rows) x 128 bytes
   auto slice_bytes = [](uint32_t ncol) {
     return (TNV > 64 && ncol > 64u ? (TNV > 128 && ncol > 128u ? TNV : 128) : 64) * KS * 2;
@@ -1011,6 +1090,8 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     const int most = win ? WPASS_TNV : TNV;
     return (uint32_t)(wd <= 0 ? 16 : wd >= most ? most : (wd + 15) & ~15);
   };
+  // a pair's N: whole 32s, half of the columns from each CTA's B rows
+  auto pair_cols = [](int wd) { return (uint32_t)(wd <= 0 ? 32 : wd >= TNV ? TNV : (wd + 31) & ~31); };
   constexpr int AH = X3 ? 2 : 1;                 // hi (and lo) tiles per operand
   static_assert(MODE == 0 || TNV >= WPASS_TNV, "a stage holds a window item's B tile");
   extern __shared__ uint8_t smem_raw[];
@@ -1019,7 +1100,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   constexpr uint32_t TMEM_COLS = Geo<TNV>::TMEM_COLS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nks = s.dp / KSE;
-  const Layout L = layout<X3, TNV>(nks);
+  const Layout L = PAIR ? pair_layout<X3>(nks) : layout<X3, TNV>(nks);
   uint8_t* const ring = smem + L.a_bytes;        // stages (resident A sits below them)
 
   if (threadIdx.x == 0) {
@@ -1056,7 +1137,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     mbar_init(&sh.afree, 1);
     for (int i = 0; i < NACC; ++i) {
       mbar_init(&sh.tfull[i], 1);
-      mbar_init(&sh.tempty[i], 4 * Geo<TNV>::GPT);   // the warps of one team
+      mbar_init(&sh.tempty[i], (PAIR ? 2 : 1) * 4 * Geo<TNV>::GPT);   // the warps of one team (of both CTAs)
     }
     for (int i = 0; i < MS; ++i) {
       mbar_init(&sh.mfull[i], META_ARRIVALS);
@@ -1070,13 +1151,25 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1 && (flags & TC_ALLOC)) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(&sh.tmem_base)), "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                   ::"r"(smem_u32(&sh.tmem_base)), "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                   ::"r"(smem_u32(&sh.tmem_base)), "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) {
+    __syncwarp();
+    pair_sync();                                 // the peer's barriers are initialised too
+  } else {
+    __syncthreads();
+  }
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
   const int R = (rows + TM - 1) / TM;
@@ -1136,6 +1229,8 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
       const int2 lo = s.split[cta], hi = s.split[cta + 1];   // by work (the sort/plan)
       rw = Range{lo.x, hi.x};
       rd = Range{lo.y, hi.y};
+    } else if (PAIR) {                           // pairs of row tiles; both CTAs walk the same items
+      rd = my_range((R + 1) / 2 * T, cta >> 1, ncta >> 1);
     } else {
       rw = my_range(np, cta, ncta);
       rd = my_range(R * T, cta, ncta);
@@ -1152,7 +1247,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     } else if (MODE != 1 && rd.lo + mine - nw < rd.hi) {
       const int item = rd.lo + mine - nw;
       const Tile t = s.tiles[item % T];
-      pya = (item / T) * TM;
+      pya = (PAIR ? 2 * (item / T) + rank : item / T) * TM;
       pyb = t.row0;
       pd.tnew = t.ncols;
     }
@@ -1214,6 +1309,24 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
           cur_ya = ya;
           cur_win = win;
         }
+      } else if constexpr (PAIR) {
+        // this CTA's A rows (past the last row tile: zeros) and its half of the
+        // MMA's B rows; the even CTA's barrier counts the bytes of both CTAs
+        const int half = (int)pair_cols(wd) / 2;
+        const CUtensorMap* th = half <= 64 ? tmN : tmW;
+        const int hb = (half <= 64 ? 64 : 128) * KS * 2, yh = yb + rank * half;
+        for (int sl = 0; sl < nks; ++sl, ++it) {
+          const int st = it % L.nst, x = sl * KSE;
+          ok = warp_wait(&sh.empty[st], ((it / L.nst) & 1u) ^ 1u);
+          if (!ok) break;
+          if (rank == 0) mbar_expect_tx(lead, &sh.full[st], (uint32_t)(2 * AH * (A_BYTES + hb)));
+          const uint32_t bar = lead_addr(&sh.full[st]);
+          uint8_t* sp = ring + st * L.sb;
+          tma_load_2d_pair(lead, sp, ta, bar, x, ya);
+          if (X3) tma_load_2d_pair(lead, sp + A_BYTES, ta, bar, s.dp + x, ya);
+          tma_load_2d_pair(lead, sp + AH * A_BYTES, th, bar, x, yh);
+          if (X3) tma_load_2d_pair(lead, sp + (AH + 1) * A_BYTES, th, bar, s.dp + x, yh);
+        }
       } else {
         for (int sl = 0; sl < nks; ++sl, ++it) {
           const int st = it % L.nst;
@@ -1225,9 +1338,11 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
       }
     }
     // the copies in flight must land before the CTA may exit: the last fill
-    // of every stage and the last A tile
-    for (uint32_t q = (it > (uint32_t)L.nst ? it - L.nst : 0u); q < it; ++q)
-      if (!warp_wait(&sh.full[q % L.nst], (q / L.nst) & 1u)) ok = false;
+    // of every stage and the last A tile. A pair's copies count at the even CTA,
+    // and both CTAs meet before they exit; the odd one waits for the last
+    // arrivals that the even CTA's commits send it.
+    for (uint32_t q = (it > (uint32_t)L.nst ? it - L.nst : 0u); q < it && (ok || !PAIR); ++q)
+      if (!warp_wait(rank == 0 ? &sh.full[q % L.nst] : &sh.empty[q % L.nst], (q / L.nst) & 1u)) ok = false;
     if (na > 0 && !warp_wait(&sh.afull, (na - 1) & 1u)) ok = false;
     if (lead && !ok) atomicOr(s.status, ST_TIMEOUT);
   } else if (warp == MWARP) {
@@ -1257,7 +1372,8 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
         d.j = __shfl_sync(0xffffffffu, pd.j, src);
       }
       if (lane == 0) m.desc = d;
-      meta_copy(m, ya, yb, d.tnew, win);
+      // the last pair's second row tile may lie past the batch: nothing of it is written
+      meta_copy(m, PAIR ? min(ya, (R - 1) * TM) : ya, yb, d.tnew, win);
       cp_arrive_noinc(&sh.mfull[ms]);
       if (lane == 0) mbar_arrive(&sh.mfull[ms]);
     }
@@ -1275,14 +1391,36 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
       const uint32_t ah = desc_lo(ahi), bh = desc_lo(bhi), al = desc_lo(alo), bl = desc_lo(blo);
 #pragma unroll
       for (uint32_t k = 0; k < 4; ++k) {
-        mma_op<OP>(lead, d, ah + 2u * k, bh + 2u * k, id, (first && k == 0) ? 0u : 1u);
+        mma_op<OP, PAIR>(lead, d, ah + 2u * k, bh + 2u * k, id, (first && k == 0) ? 0u : 1u);
         if constexpr (X3) {
-          mma_op<OP>(lead, d, ah + 2u * k, bl + 2u * k, id, 1u);
-          mma_op<OP>(lead, d, al + 2u * k, bh + 2u * k, id, 1u);
+          mma_op<OP, PAIR>(lead, d, ah + 2u * k, bl + 2u * k, id, 1u);
+          mma_op<OP, PAIR>(lead, d, al + 2u * k, bh + 2u * k, id, 1u);
         }
       }
     };
-    for (int local = 0; local < n && ok; ++local) {
+    if constexpr (PAIR) {
+      for (int local = 0; local < n && ok && rank == 0; ++local) {
+        if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
+        const uint32_t id = idesc<OP>(pair_cols(__shfl_sync(0xffffffffu, pd.tnew, local & 31)), 2 * TM);
+        const uint32_t buf = local % NACC, bph = ((uint32_t)local / NACC) & 1u;
+        ok = warp_wait(&sh.tempty[buf], bph ^ 1u);
+        if (!ok) break;
+        asm volatile("fence.acq_rel.cluster;" ::: "memory");   // the peer's releases
+        tc_fence_after();
+        for (int sl = 0; sl < nks; ++sl, ++it) {
+          const int st = it % L.nst;
+          ok = warp_wait(&sh.full[st], (it / L.nst) & 1u);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t a0 = rbase + (uint32_t)(st * L.sb), b0 = a0 + AH * A_BYTES;
+          mma_slice(tmem + buf * TNV, id, a0, a0 + A_BYTES, b0, b0 + A_BYTES, sl == 0);
+          mma_commit_pair(lead, &sh.empty[st]);
+        }
+        if (!ok) break;
+        mma_commit_pair(lead, &sh.tfull[buf]);
+      }
+    }
+    for (int local = 0; local < n && ok && !PAIR; ++local) {
       if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
       const int wd = __shfl_sync(0xffffffffu, pd.tnew, local & 31);
       const uint32_t ncol = live_cols(MODE != 0 && local < nw, wd);
@@ -1326,15 +1464,26 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
       }
       mma_commit(lead, &sh.tfull[buf]);
     }
-    mma_commit(lead, &sh.mma_done);
-    if (!warp_wait(&sh.mma_done, 0)) ok = false;
+    if (rank == 0) {                             // a pair's MMAs are all the even CTA's
+      mma_commit<PAIR>(lead, &sh.mma_done);
+      if (!warp_wait(&sh.mma_done, 0)) ok = false;
+    }
     if (lead && !ok) atomicOr(s.status, ST_TIMEOUT);
   } else if (warp < MWARP) {
-    epilogue<KIND, MODE, TNV>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_groups, norms);
+    epilogue<KIND, MODE, TNV, PAIR>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_groups, norms, rank);
   } else if constexpr (MODE != 0) {
     if (norms) norm_warp<TNV>(s, sh, nw, lane);
   }
   tc_fence_before();
+  if constexpr (PAIR) {
+    __syncwarp();
+    pair_sync();                                 // every copy, MMA, arrival and read of both CTAs is done
+    if (warp == 1) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+    return;
+  }
   __syncthreads();
   if (warp == 1 && (flags & TC_FREE)) {
     tc_fence_after();
@@ -1366,6 +1515,35 @@ cudaError_t launch_form(const Dev& s, const CUtensorMap* m, int rows, bool norms
   // maps: [0] batch rows, 128-row boxes; support rows with [1] 128-row, [2] 64-row, [3] 256-row boxes
   return launch_pdl(k_dist_tc<KIND, MODE, OP, TNV>, dim3(grid), dim3(nthreads<MODE>()), smem_bytes<TNV>(), st, s,
                     rows, norms ? 1 : 0, m[0], m[3], m[1], m[2]);
+}
+
+// The distance pass on CTA pairs.
+template <int KIND, int OP>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(nthreads<0>(), 1)
+    k_dist_pair(Dev s, int rows, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmN) {
+  dist_tc_body<KIND, 0, OP, 256, true>(s, rows, &tmA, &tmB, &tmW, &tmN, blockIdx.x, gridDim.x);
+}
+
+template <int KIND, int OP>
+cudaError_t launch_pair_form(const Dev& s, const CUtensorMap* m, int rows, cudaStream_t st) {
+  static std::atomic<uint64_t> attr{0};
+  const cudaError_t e = smem_limit_once(k_dist_pair<KIND, OP>, smem_bytes<256>(), attr);
+  if (e != cudaSuccess) return e;
+  const int64_t most = (int64_t)((rows + 2 * TM - 1) / (2 * TM)) * s.max_tiles;
+  const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(most, s.num_sms / 2));
+  return launch_pdl(k_dist_pair<KIND, OP>, dim3(2 * pairs), dim3(nthreads<0>()), smem_bytes<256>(), st, s, rows,
+                    m[0], m[3], m[1], m[2]);
+}
+
+template <int OP>
+cudaError_t launch_pair_kind(const Dev& s, const CUtensorMap* m, int rows, cudaStream_t st) {
+  switch (s.kind) {
+    case K_GAUSS: return launch_pair_form<K_GAUSS, OP>(s, m, rows, st);
+    case K_LAPLACE: return launch_pair_form<K_LAPLACE, OP>(s, m, rows, st);
+    case K_LINEAR: return launch_pair_form<K_LINEAR, OP>(s, m, rows, st);
+    default: return launch_pair_form<K_POLY, OP>(s, m, rows, st);
+  }
 }
 
 template <int MODE, int OP, int TNV>
