@@ -378,12 +378,11 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
     }
     c->use_tc = true;
   }
-  s.tn = c->use_tc ? (cfg->dist_tile == 0 ? 256 : cfg->dist_tile) : 64;
   // The table form's blocks are a few dozen rows a center: 64-row tiles while the
-  // row tile of X stays in shared memory between them, 256 once it streams with
-  // every tile (its bytes are then most of a tile's).
-  if (tab && c->use_tc && cfg->dist_tile == 0 && kkm::tc_item_bytes(s, 64, false) != kkm::tc_item_bytes(s, 64, true))
-    s.tn = 64;
+  // row tile of X stays in shared memory between them. Once it streams with every
+  // tile, its bytes are most of a tile's: 128-row tiles, two to a pass over it.
+  const auto table_tile = [&] { return kkm::tc_item_bytes(s, 64, false) == kkm::tc_item_bytes(s, 64, true) ? 128 : 64; };
+  s.tn = !c->use_tc ? 64 : cfg->dist_tile != 0 ? cfg->dist_tile : tab ? table_tile() : 256;
   s.ppt = c->use_tc ? kkm::tc_parts_per_tile(s.tn) : 1;
   s.pair_rows = c->use_tc ? 128 : 64;
   s.pair_cols = c->use_tc ? kkm::WPASS_TNV : 64;

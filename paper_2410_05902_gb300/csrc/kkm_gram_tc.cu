@@ -87,7 +87,7 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
   // CTA pairs where the operands stream and the row tiles pair up with little left over: an odd last
   // row tile costs the pair a whole one
   const int R = (rows + TM - 1) / TM;
-  if (d.tn == 256 && !tc_resident(d, 256) && R >= 2 && (R % 2 == 0 || R >= 5))
+  if (d.tn >= 128 && !tc_resident(d, d.tn) && R >= 2 && (R % 2 == 0 || R >= 5))
     return launch_dist_pair(d, maps, rows, st);
   if (d.tn == 64) return launch_mode<0, 64>(d, maps, rows, false, st);
   if (d.tn == 256) return launch_mode<0, 256>(d, maps, rows, false, st);

@@ -43,7 +43,7 @@
 // sums meet in shared memory (chosen per run, so that a run's results do not
 // depend on how a launch splits its items).
 //
-// CTA pairs (PAIR, distance pass with 256-column tiles whose operands stream):
+// CTA pairs (PAIR, distance pass of 128- or 256-column tiles whose operands stream):
 // two CTAs of a cluster take two row tiles against the same support tile, and
 // the tcgen05 pair form multiplies both at once: each CTA stages its own A rows
 // and half of the B rows, so a 128-byte slice costs 32 KB of operand traffic per
@@ -52,8 +52,9 @@
 // more than 128 BF16 columns.
 // The even CTA's MMA warp issues for both; its full barriers count both CTAs' copies,
 // its commits arrive on both CTAs' stage and accumulator barriers, and both
-// epilogues release an accumulator at the even CTA. Row tiles, partials and their
-// sums are those of the single-CTA form, bit for bit.
+// epilogues release an accumulator at the even CTA. With 128-column tiles two
+// items of a row tile share one pass over its slices. Row tiles, partials and
+// their sums are those of the single-CTA form, bit for bit.
 //
 // Gaussian kernel values without a per-element row term: with rc = -log2(e)
 // ||x||^2 / kappa and t = (2 log2(e) / kappa) g - log2(e) ||y||^2 / kappa,
@@ -146,7 +147,8 @@ __device__ __forceinline__ Layout layout(int nks) {
   return L;
 }
 
-// CTA pairs always stream: a stage holds one slice of A and of this CTA's half of B.
+// CTA pairs always stream: a stage holds one slice of A and of this CTA's half of
+// B: 128 rows of one 256-column tile, or 64 of each of two 128-column tiles.
 template <bool X3>
 __device__ __forceinline__ Layout pair_layout(int nks) {
   Layout L;
@@ -1076,7 +1078,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
                                              const CUtensorMap* tmW, const CUtensorMap* tmN, int cta, int ncta,
                                              bool norms = false,
                                              Range ovr = Range{-1, -1}, int flags = TC_ALLOC | TC_FREE) {
-  static_assert(!PAIR || (MODE == 0 && TNV == 256), "CTA pairs take 256-column distance items");
+  static_assert(!PAIR || (MODE == 0 && TNV >= 128), "CTA pairs take distance items of 128 or 256 columns");
   constexpr bool X3 = OP == OP_X3;
   constexpr int KSE = OP == OP_TF32 ? 32 : KS;   // operand elements per slice row
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
@@ -1091,6 +1093,8 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     return (uint32_t)(wd <= 0 ? 16 : wd >= most ? most : (wd + 15) & ~15);
   };
   // a pair's N: whole 32s, half of the columns from each CTA's B rows
+  constexpr int GRP = PAIR && TNV == 128 ? 2 : 1;   // items that share a pass over their row tile
+  constexpr int HB = TNV / 2 * KS * 2;              // bytes of half a tile's B slice
   auto pair_cols = [](int wd) { return (uint32_t)(wd <= 0 ? 32 : wd >= TNV ? TNV : (wd + 31) & ~31); };
   constexpr int AH = X3 ? 2 : 1;                 // hi (and lo) tiles per operand
   static_assert(MODE == 0 || TNV >= WPASS_TNV, "a stage holds a window item's B tile");
@@ -1311,22 +1315,32 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
         }
       } else if constexpr (PAIR) {
         // this CTA's A rows (past the last row tile: zeros) and its half of the
-        // MMA's B rows; the even CTA's barrier counts the bytes of both CTAs
+        // MMA's B rows, for one or two items; the even CTA's barrier counts the
+        // bytes of both CTAs
+        const bool two = GRP == 2 && local + 1 < n && src < 31 && __shfl_sync(0xffffffffu, pya, (src + 1) & 31) == ya;
         const int half = (int)pair_cols(wd) / 2;
         const CUtensorMap* th = half <= 64 ? tmN : tmW;
         const int hb = (half <= 64 ? 64 : 128) * KS * 2, yh = yb + rank * half;
+        const int yh2 = __shfl_sync(0xffffffffu, pyb, (src + 1) & 31) +
+                        rank * ((int)pair_cols(__shfl_sync(0xffffffffu, pd.tnew, (src + 1) & 31)) / 2);
         for (int sl = 0; sl < nks; ++sl, ++it) {
           const int st = it % L.nst, x = sl * KSE;
           ok = warp_wait(&sh.empty[st], ((it / L.nst) & 1u) ^ 1u);
           if (!ok) break;
-          if (rank == 0) mbar_expect_tx(lead, &sh.full[st], (uint32_t)(2 * AH * (A_BYTES + hb)));
+          if (rank == 0)
+            mbar_expect_tx(lead, &sh.full[st], (uint32_t)(2 * AH * (A_BYTES + (two ? 2 * hb : hb))));
           const uint32_t bar = lead_addr(&sh.full[st]);
-          uint8_t* sp = ring + st * L.sb;
+          uint8_t *sp = ring + st * L.sb, *sb = sp + AH * A_BYTES;
           tma_load_2d_pair(lead, sp, ta, bar, x, ya);
           if (X3) tma_load_2d_pair(lead, sp + A_BYTES, ta, bar, s.dp + x, ya);
-          tma_load_2d_pair(lead, sp + AH * A_BYTES, th, bar, x, yh);
-          if (X3) tma_load_2d_pair(lead, sp + (AH + 1) * A_BYTES, th, bar, s.dp + x, yh);
+          tma_load_2d_pair(lead, sb, th, bar, x, yh);
+          if (X3) tma_load_2d_pair(lead, sb + HB, th, bar, s.dp + x, yh);
+          if (two) {
+            tma_load_2d_pair(lead, sb + AH * HB, th, bar, x, yh2);
+            if (X3) tma_load_2d_pair(lead, sb + (AH + 1) * HB, th, bar, s.dp + x, yh2);
+          }
         }
+        if (two) ++local;
       } else {
         for (int sl = 0; sl < nks; ++sl, ++it) {
           const int st = it % L.nst;
@@ -1401,9 +1415,14 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     if constexpr (PAIR) {
       for (int local = 0; local < n && ok && rank == 0; ++local) {
         if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
-        const uint32_t id = idesc<OP>(pair_cols(__shfl_sync(0xffffffffu, pd.tnew, local & 31)), 2 * TM);
-        const uint32_t buf = local % NACC, bph = ((uint32_t)local / NACC) & 1u;
-        ok = warp_wait(&sh.tempty[buf], bph ^ 1u);
+        const int src = local & 31, nx = (src + 1) & 31;
+        const bool two = GRP == 2 && local + 1 < n && src < 31 &&
+                         __shfl_sync(0xffffffffu, pya, nx) == __shfl_sync(0xffffffffu, pya, src);
+        const uint32_t id = idesc<OP>(pair_cols(__shfl_sync(0xffffffffu, pd.tnew, src)), 2 * TM);
+        const uint32_t id2 = idesc<OP>(pair_cols(__shfl_sync(0xffffffffu, pd.tnew, nx)), 2 * TM);
+        const uint32_t buf = local % NACC, buf2 = (local + 1) % NACC;
+        ok = warp_wait(&sh.tempty[buf], (((uint32_t)local / NACC) & 1u) ^ 1u) &&
+             (!two || warp_wait(&sh.tempty[buf2], (((uint32_t)(local + 1) / NACC) & 1u) ^ 1u));
         if (!ok) break;
         asm volatile("fence.acq_rel.cluster;" ::: "memory");   // the peer's releases
         tc_fence_after();
@@ -1413,11 +1432,16 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
           if (!ok) break;
           tc_fence_after();
           const uint32_t a0 = rbase + (uint32_t)(st * L.sb), b0 = a0 + AH * A_BYTES;
-          mma_slice(tmem + buf * TNV, id, a0, a0 + A_BYTES, b0, b0 + A_BYTES, sl == 0);
+          mma_slice(tmem + buf * TNV, id, a0, a0 + A_BYTES, b0, b0 + HB, sl == 0);
+          if (two) mma_slice(tmem + buf2 * TNV, id2, a0, a0 + A_BYTES, b0 + AH * HB, b0 + (AH + 1) * HB, sl == 0);
           mma_commit_pair(lead, &sh.empty[st]);
         }
         if (!ok) break;
         mma_commit_pair(lead, &sh.tfull[buf]);
+        if (two) {
+          mma_commit_pair(lead, &sh.tfull[buf2]);
+          ++local;
+        }
       }
     }
     for (int local = 0; local < n && ok && !PAIR; ++local) {
@@ -1518,31 +1542,31 @@ cudaError_t launch_form(const Dev& s, const CUtensorMap* m, int rows, bool norms
 }
 
 // The distance pass on CTA pairs.
-template <int KIND, int OP>
+template <int KIND, int OP, int TNV>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(nthreads<0>(), 1)
     k_dist_pair(Dev s, int rows, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmN) {
-  dist_tc_body<KIND, 0, OP, 256, true>(s, rows, &tmA, &tmB, &tmW, &tmN, blockIdx.x, gridDim.x);
+  dist_tc_body<KIND, 0, OP, TNV, true>(s, rows, &tmA, &tmB, &tmW, &tmN, blockIdx.x, gridDim.x);
 }
 
-template <int KIND, int OP>
+template <int KIND, int OP, int TNV>
 cudaError_t launch_pair_form(const Dev& s, const CUtensorMap* m, int rows, cudaStream_t st) {
   static std::atomic<uint64_t> attr{0};
-  const cudaError_t e = smem_limit_once(k_dist_pair<KIND, OP>, smem_bytes<256>(), attr);
+  const cudaError_t e = smem_limit_once(k_dist_pair<KIND, OP, TNV>, smem_bytes<TNV>(), attr);
   if (e != cudaSuccess) return e;
   const int64_t most = (int64_t)((rows + 2 * TM - 1) / (2 * TM)) * s.max_tiles;
   const int pairs = (int)std::max<int64_t>(1, std::min<int64_t>(most, s.num_sms / 2));
-  return launch_pdl(k_dist_pair<KIND, OP>, dim3(2 * pairs), dim3(nthreads<0>()), smem_bytes<256>(), st, s, rows,
+  return launch_pdl(k_dist_pair<KIND, OP, TNV>, dim3(2 * pairs), dim3(nthreads<0>()), smem_bytes<TNV>(), st, s, rows,
                     m[0], m[3], m[1], m[2]);
 }
 
-template <int OP>
+template <int OP, int TNV>
 cudaError_t launch_pair_kind(const Dev& s, const CUtensorMap* m, int rows, cudaStream_t st) {
   switch (s.kind) {
-    case K_GAUSS: return launch_pair_form<K_GAUSS, OP>(s, m, rows, st);
-    case K_LAPLACE: return launch_pair_form<K_LAPLACE, OP>(s, m, rows, st);
-    case K_LINEAR: return launch_pair_form<K_LINEAR, OP>(s, m, rows, st);
-    default: return launch_pair_form<K_POLY, OP>(s, m, rows, st);
+    case K_GAUSS: return launch_pair_form<K_GAUSS, OP, TNV>(s, m, rows, st);
+    case K_LAPLACE: return launch_pair_form<K_LAPLACE, OP, TNV>(s, m, rows, st);
+    case K_LINEAR: return launch_pair_form<K_LINEAR, OP, TNV>(s, m, rows, st);
+    default: return launch_pair_form<K_POLY, OP, TNV>(s, m, rows, st);
   }
 }
 

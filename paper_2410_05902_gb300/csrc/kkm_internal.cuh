@@ -468,7 +468,7 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
 // The window pass reads its pair list and plans before its grid-dependency
 // wait: launch it only right after k_move, k_update or a kernel that writes neither.
 cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st, bool norms = false);
-// The distance pass on CTA pairs (256-column tiles, streamed operands).
+// The distance pass on CTA pairs (streamed operands, s.tn 128 or 256).
 cudaError_t launch_dist_pair(const Dev& s, const void* maps, int rows, cudaStream_t st);
 // A step's distance pass with the window items of the pending update ahead of
 // it (none unless fin_pending is set) and their center norms; s.tn 128 or 256.
