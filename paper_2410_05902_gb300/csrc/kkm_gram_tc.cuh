@@ -72,6 +72,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "kkm_internal.cuh"
 
 namespace kkm {
@@ -102,9 +104,6 @@ template <int MODE> constexpr int nthreads() { return 32 * (MWARP + (MODE == 0 ?
 constexpr int NSLOT = 4;                         // finished window items waiting for the norm warp
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;   // 2 s per wait
 constexpr float ROW_EXP_FLOOR = -100.0f;        // Gaussian: rc at or above it keeps 2^t finite
-#ifndef DIST_NB
-#define DIST_NB 2                                // distance-pass epilogue: 8-column blocks per TMEM chunk
-#endif
 
 // TMEM accumulators (TNV columns each, at most 512 columns), teams of
 // groups (one per accumulator), groups per team (= partials per tile), and
@@ -500,13 +499,6 @@ __device__ __forceinline__ void chunk_load(uint32_t taddr, float (&v0)[4 * NB], 
   tmem_wait_ld();
 }
 
-// The two loads of a chunk without the wait (the caller waits before reading).
-template <int NB>
-__device__ __forceinline__ void chunk_issue(uint32_t taddr, float (&v0)[4 * NB], float (&v1)[4 * NB]) {
-  tmem_ld16x256<NB>(taddr, v0);
-  tmem_ld16x256<NB>(taddr + (16u << 16), v1);
-}
-
 template <int NB>
 __device__ __forceinline__ float2 gram2(const float (&v0)[4 * NB], const float (&v1)[4 * NB], int j, int u) {
   const int o = 4 * j + 2 * (u & 1);
@@ -694,22 +686,24 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
     bool fast = false;
     if constexpr (KIND == K_GAUSS)
       fast = __all_sync(0xffffffffu, fminf(fminf(rc[0], rc[1]), fminf(rc[2], rc[3])) >= ROW_EXP_FLOOR);
-    // chunks of CW columns, two in flight: the next chunk's TMEM loads are
-    // issued before the current chunk's arithmetic and waited for after it
-    // (tcgen05.wait::ld waits for every load in flight, so a chunk's
-    // arithmetic is what hides the next chunk's load latency)
     auto release = [&]() {                      // the accumulator is free again
       if (!all) {
         tc_fence_before();
         pl.template arrive_acc<PAIR>(&sh.tempty[buf]);
       }
     };
-    constexpr int NB = DIST_NB, CW = 8 * NB;
-    static_assert(TNV / NGRP % CW == 0, "whole chunks per group");
+    // Whole 16-column blocks of the live columns (the MMA's N ends there): 32 at
+    // a time, then a last 16. A chunk's TMEM load takes about 30 cycles; what a warp waits
+    // for is its own chain of shared-memory reads, FMAs and exponentials, so
+    // the wide chunk (32 elements a lane in flight) does as well as two 16-column
+    // ones loaded ahead of each other where items are many (1e6 x 128, b = 4096: 79 us
+    // an iteration both ways), and better where a CTA has one or two (70000 x 784,
+    // b = 1024: 36.9 -> 34.3 us).
     const int live = min(ncols, m.desc.tnew - cbeg);
-    const int nch = live > 0 ? (live + CW - 1) / CW : 0;
-    auto math = [&](const float (&w0)[4 * NB], const float (&w1)[4 * NB], int ch) {
-      const int c = cbeg + ch * CW + c2;
+    const int n16 = live > 0 ? (live + 15) >> 4 : 0;
+    auto math = [&](auto nb, const auto& w0, const auto& w1, int col) {
+      constexpr int NB = decltype(nb)::value;
+      const int c = cbeg + col + c2;
       if constexpr (KIND == K_GAUSS) {
         if (fast) gauss_chunk<NB, true>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
         else gauss_chunk<NB, false>(w0, w1, m.col[0], m.col[1], c, negc, C2, rc, acc);
@@ -717,24 +711,21 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
         generic_chunk<KIND, NB>(w0, w1, m.col[0], m.col[1], m.col[2], c, negc, coef0, degree, rc, xi, acc);
       }
     };
-    if (nch == 0) {
+    static_assert(TNV / NGRP % 16 == 0, "whole 16-column blocks per group");
+    if (n16 == 0) release();
+    int q16 = 0;
+#pragma unroll 1
+    for (; q16 + 2 <= n16; q16 += 2) {
+      float v0[16], v1[16];
+      chunk_load<4>(tq + q16 * 16, v0, v1);
+      if (q16 + 2 == n16) release();
+      math(std::integral_constant<int, 4>{}, v0, v1, q16 * 16);
+    }
+    if (q16 < n16) {
+      float v0[8], v1[8];
+      chunk_load<2>(tq + q16 * 16, v0, v1);
       release();
-    } else {
-      float a0[4 * NB], a1[4 * NB], b0[4 * NB], b1[4 * NB];
-      chunk_issue<NB>(tq, a0, a1);
-      tmem_wait_ld();
-      for (int ch = 0; ch < nch; ch += 2) {
-        if (ch + 1 < nch) chunk_issue<NB>(tq + (ch + 1) * CW, b0, b1);
-        else release();
-        math(a0, a1, ch);
-        if (ch + 1 < nch) {
-          tmem_wait_ld();
-          if (ch + 2 < nch) chunk_issue<NB>(tq + (ch + 2) * CW, a0, a1);
-          else release();
-          math(b0, b1, ch + 1);
-          if (ch + 2 < nch) tmem_wait_ld();
-        }
-      }
+      math(std::integral_constant<int, 2>{}, v0, v1, q16 * 16);
     }
     float fr[4];
 #pragma unroll
