@@ -216,7 +216,7 @@ template <int TNV> struct Shared {
   uint32_t tmem_base;
   uint32_t pad;
   long long gtot;                // run groups: the class's weighted item total
-  int gseg[4];                   // run groups: the next segment (run, first item, end item)
+  int gseg[4];                   // run groups: the next segment (run, first item, end item), whole CTAs per run
   alignas(16) Dev gdev;          // run groups: the segment's run (a shared copy: no reloads after global stores)
   alignas(16) MetaSlot<TNV> ring[Geo<TNV>::MS];   // 16-byte asynchronous copies land here
   float red[2][NGRP][4][32];     // distance items, all-groups mode: row sums (item parity, group, quadrant, row)
@@ -1586,8 +1586,9 @@ cudaError_t launch_mode(const Dev& s, const void* maps, int rows, bool norms, cu
 // row tiles x support tiles; window pass: its pair list) are laid end to end
 // in one weighted item space, an item of run r weighing
 // max(5, 2 nks_r m_r) (m = 3 for the split form: the MMA share next to the
-// epilogue's fixed share), and CTA c takes the items whose start falls in
-// [c W / G, (c + 1) W / G). It walks its range run by run: each stretch of
+// epilogue's fixed share). Where the shares allow it each CTA belongs to one run
+// (group_whole_ctas); otherwise CTA c takes the items whose start falls in
+// [c W / G, (c + 1) W / G) and walks its range run by run: each stretch of
 // one run's items is a segment, run with that run's Dev and TMA descriptors
 // (read from device memory; the host wrote them before the group's first
 // launch, and the acquire fence orders that write before the tensor-map
@@ -1654,6 +1655,50 @@ __device__ __forceinline__ int group_find(const GroupPhase& g, long long A, long
   return -1;
 }
 
+// Whole CTAs per run (up to 32 runs, a lane each, warp-wide): the runs'
+// boundaries in the weighted item space rounded to CTA boundaries, a run's
+// items dealt evenly to its CTAs. A CTA then has one segment: filling and draining
+// the pass's pipeline a second time costs as much as several items. Four steps of
+// eight runs (k 5-100, d 16-256, b 256-2048): 740 -> 693 us.
+// False, for the split by exact weight, where a run would get no CTA or
+// the rounding would give some CTA over an eighth more than its share. r = -1: no items.
+template <int MODE>
+__device__ __forceinline__ bool group_whole_ctas(const GroupPhase& g, int cta, int ncta, int& r, int& lo, int& hi) {
+  if (g.nruns > 32) return false;
+  const int lane = threadIdx.x & 31;
+  int n = 0, om = 1;
+  if (lane < g.nruns) {
+    const Dev& s = g.runs[lane].s;
+    n = group_items<MODE>(s);
+    om = group_weight(s);
+  }
+  const long long w = (long long)n * om;
+  long long incl = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const long long W = __shfl_sync(0xffffffffu, incl, 31);
+  r = -1;
+  lo = hi = 0;
+  if (W == 0) return true;
+  const int c0 = (int)((2 * (incl - w) * ncta + W) / (2 * W)), c1 = (int)((2 * incl * ncta + W) / (2 * W));
+  // w / (c1 - c0) <= (9 / 8) W / ncta
+  const bool fits = n == 0 || (c1 > c0 && 8 * w * ncta <= 9 * W * (c1 - c0));
+  if (!__all_sync(0xffffffffu, fits)) return false;
+  const unsigned own = __ballot_sync(0xffffffffu, n > 0 && cta >= c0 && cta < c1);
+  if (own) {
+    r = __ffs(own) - 1;
+    const int nr = __shfl_sync(0xffffffffu, n, r), a = __shfl_sync(0xffffffffu, c0, r),
+              b = __shfl_sync(0xffffffffu, c1, r);
+    lo = (int)((long long)nr * (cta - a) / (b - a));
+    hi = (int)((long long)nr * (cta - a + 1) / (b - a));
+    if (lo == hi) r = -1;
+  }
+  return true;
+}
+
 template <int KIND, int MODE, int OP, int TNV>
 __global__ void __launch_bounds__(nthreads<MODE>(), 1) k_group_tc(GroupPhase g) {
   extern __shared__ uint8_t smem_raw[];
@@ -1663,17 +1708,25 @@ __global__ void __launch_bounds__(nthreads<MODE>(), 1) k_group_tc(GroupPhase g) 
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
   if (warp == 0) {
-    int lo = 0, hi = 0;
+    int r = -1, lo = 0, hi = 0;
     long long total = 0;
-    group_find<MODE>(g, -1, -1, 0, lo, hi, total);
+    const bool whole = group_whole_ctas<MODE>(g, blockIdx.x, gridDim.x, r, lo, hi);
+    if (lane == 0) {
+      sh.gseg[0] = r;
+      sh.gseg[1] = lo;
+      sh.gseg[2] = hi;
+      sh.gseg[3] = whole;
+    }
+    if (!whole) group_find<MODE>(g, -1, -1, 0, lo, hi, total);
     if (lane == 0) sh.gtot = total;
   }
   __syncthreads();
   const long long W = sh.gtot;
+  const bool whole = sh.gseg[3] != 0;
   const long long A = W * (long long)blockIdx.x / gridDim.x, B = W * (long long)(blockIdx.x + 1) / gridDim.x;
   int flags = TC_ALLOC, rnext = 0;
   for (;;) {
-    if (warp == 0) {
+    if (warp == 0 && !whole) {
       int lo = 0, hi = 0;
       long long total = 0;
       const int r = A < B ? group_find<MODE>(g, A, B, rnext, lo, hi, total) : -1;
@@ -1706,6 +1759,7 @@ __global__ void __launch_bounds__(nthreads<MODE>(), 1) k_group_tc(GroupPhase g) 
     // thread before warp 0 writes the next segment
     dist_tc_body<KIND, MODE, OP, TNV>(sh.gdev, sh.gdev.b, &m[0], &m[3], &m[1], &m[2], 0, 1, false, seg, flags);
     flags = TC_REINIT;
+    if (whole) break;
     rnext = r + 1;
   }
   if (flags == TC_REINIT && warp == 1) {   // TMEM was allocated by the first segment
