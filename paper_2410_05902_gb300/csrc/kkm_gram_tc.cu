@@ -84,10 +84,18 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
   // ahead writes none of what it stages (the gather, or this pass itself)
   Dev d = s;
   d.pre_b = (stage_early && s.pre_b) ? 1 : 0;
-  // CTA pairs where the operands stream and the row tiles pair up with little left over: an odd last
-  // row tile costs the pair a whole one
+  // CTA pairs where the operands stream, an item's MMAs are long (16 or more
+  // times a BF16 slice's four) or two items share a row tile's slices
+  // (128-column tiles), and the row tiles pair up with little left over: an odd
+  // last one costs the pair a whole one. Shorter items are bound by the
+  // epilogue, and a pair waits for the slower of its two. Scoring 20000 rows
+  // against 64 centers of about 216 rows, pairs and single CTAs: BF16 d = 256 (4
+  // slices) 543 and 494 us, d = 784 (13) 914 and 922; split BF16 d = 128 (6 slices'
+  // MMAs) 582 and 521, d = 256 (12) 797 and 735, d = 784 (39) 1773 and 1932; TF32
+  // d = 128 (4) 538 and 485, d = 784 (25) 1381 and 1463.
   const int R = (rows + TM - 1) / TM;
-  if (d.tn >= 128 && !tc_resident(d, d.tn) && R >= 2 && (R % 2 == 0 || R >= 5))
+  const int mmas = d.dp / (d.form == FORM_TF32 ? 32 : KS) * (d.form == FORM_BF16X3 ? 3 : 1);
+  if (d.tn >= 128 && !tc_resident(d, d.tn) && (d.tn == 128 || mmas >= 16) && R >= 2 && (R % 2 == 0 || R >= 5))
     return launch_dist_pair(d, maps, rows, st);
   if (d.tn == 64) return launch_mode<0, 64>(d, maps, rows, false, st);
   if (d.tn == 256) return launch_mode<0, 256>(d, maps, rows, false, st);

@@ -18,9 +18,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("kernel", ["gaussian", "laplacian", "linear"])
-@pytest.mark.parametrize("precision,d", [("bf16", 129), ("bf16", 784), ("bf16x3", 65), ("bf16x3", 257),
-                                         ("tf32", 65), ("tf32", 230)])
-def test_paired_row_tiles_match_oracle(kernel, precision, d):
+@pytest.mark.parametrize("precision,d,tile", [
+    ("bf16", 300, 128), ("bf16", 784, 128), ("bf16x3", 129, 128), ("bf16x3", 257, 128), ("tf32", 129, 128),
+    ("tf32", 230, 128), ("bf16", 1030, 256), ("bf16x3", 321, 256), ("tf32", 490, 256)])
+def test_paired_row_tiles_match_oracle(kernel, precision, d, tile):
     torch = torch_cuda()
     from paper_2410_05902_gb300.kkm import KKM
     n, k, b, tau = 3000, 5, 900, 260
@@ -28,7 +29,7 @@ def test_paired_row_tiles_match_oracle(kernel, precision, d):
     sigma = inputs.median_sigma(X, seed=1)
     param = {"gaussian": 2 * sigma * sigma, "laplacian": sigma, "linear": 1.0}[kernel]
     run = KKM(torch.from_numpy(X).cuda(), k, b, kernel=kernel, param=param, tau=tau, precision=precision,
-              init_idx=inputs.init_indices(n, k, seed=3))
+              dist_tile=tile, init_idx=inputs.init_indices(n, k, seed=3))
     for batch in inputs.batch_stream(n, b, 3, seed=4):
         run.step(torch.from_numpy(batch.astype(np.int32)).cuda())
     st = run.get_state()
