@@ -65,3 +65,22 @@ def test_table_blocks_of_wide_rows_match_oracle(counts):
         dist, _, _ = p.gpu_step(B, forced=rec.assign)
         assert dist_rel_err(dist, rec.dist) <= DIST_TOL["bf16"]
     p.close()
+
+
+def test_paired_table_steps_replayed_from_a_graph():
+    torch = torch_cuda()
+    from paper_2410_05902_gb300.kkm import KKM
+    X, _ = inputs.isotropic_mixture(1500, 450, 4, seed=13)
+    sigma = inputs.median_sigma(X, seed=1)
+    out = []
+    for graph in (False, True):
+        run = KKM(torch.from_numpy(X).cuda(), 4, 300, kernel="gaussian", param=2 * sigma * sigma, tau=0, algo="table",
+                  precision="bf16", seed=3, init_idx=inputs.init_indices(len(X), 4, seed=3))
+        run.graph(graph)
+        run.steps(40)            # eager steps and two replays of sixteen, or forty eager ones
+        dist = torch.empty((300, 4), dtype=torch.float32, device="cuda")
+        run.step(torch.arange(300, dtype=torch.int32, device="cuda"), None, None, dist, None)
+        out.append((dist.cpu().numpy(), run.objective()))
+        run.close()
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1]
