@@ -698,7 +698,7 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
     // the wide chunk (32 elements a lane in flight) does as well as two 16-column
     // ones loaded ahead of each other where items are many (1e6 x 128, b = 4096: 79 us
     // an iteration both ways), and better where a CTA has one or two (70000 x 784,
-    // b = 1024: 36.9 -> 34.3 us).
+    // b = 1024: 36.9 -> 34.3 to 35.7 us).
     const int live = min(ncols, m.desc.tnew - cbeg);
     const int n16 = live > 0 ? (live + 15) >> 4 : 0;
     auto math = [&](auto nb, const auto& w0, const auto& w1, int col) {
