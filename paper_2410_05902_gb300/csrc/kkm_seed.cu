@@ -188,15 +188,17 @@ __device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int t) {
 }
 
 // D^2(x) = min(D^2(x), Delta(x, c)) for c = chosen[t] (first draw: = Delta),
-// then (last block) draw t + 1. DOT (linear and polynomial kernels): <x, c>
-// and ||x||^2 in FP64. Otherwise ||x - c||^2 in FP32 triples; a warp with a sum
-// that left the range where every product is exact (below 2^-60 but not 0,
-// above 2^120, or not finite) sums that tile again in FP64.
+// then (last block) draw t + 1. DOT (linear and polynomial kernels): <x, c>,
+// ||x||^2 and ||c||^2 in FP64, all three in the same order, so that Delta of a
+// row that equals the center's is exactly 0 (||c||^2 is the block's first
+// warp's). Otherwise ||x - c||^2 in FP32 triples; a warp with a sum that left
+// the range where every product is exact (below 2^-60 but not 0, above 2^120,
+// or not finite) sums that tile again in FP64.
 template <bool DOT>
 __global__ void __launch_bounds__(PP_ROWS) k_pp_draw(PPArgs a, int t) {
   extern __shared__ __align__(16) float crow[];       // [round_up(d, 32)] the center's row
   __shared__ __align__(16) float tiles[PP_ROWS / 32][32][PP_PITCH];
-  __shared__ double red[PP_ROWS / 32];
+  __shared__ double red[PP_ROWS / 32], cself;
   __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * PP_ROWS + 32 * w, x = row0 + lane;
@@ -216,16 +218,16 @@ __global__ void __launch_bounds__(PP_ROWS) k_pp_draw(PPArgs a, int t) {
         __syncwarp();
         stage_tile(a, row0, f0, tile);
       }
-      const double cl = crow[f0 + lane];
-      scc = fma(cl, cl, scc);                         // a lane per feature
       for (int f = 0; f < PP_F; ++f) {
         const double xv = tile[lane][f], cv = crow[f0 + f];
         sxy = fma(xv, cv, sxy);
         sxx = fma(xv, xv, sxx);
+        if (w == 0) scc = fma(cv, cv, scc);
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) scc += __shfl_xor_sync(0xffffffffu, scc, o);
+    if (threadIdx.x == 0) cself = scc;
+    __syncthreads();
+    scc = cself;
     delta = kernel_fp64(a.kind, 0.0, sxx, a.param, a.coef0, a.degree) -
             2.0 * kernel_fp64(a.kind, 0.0, sxy, a.param, a.coef0, a.degree) +
             kernel_fp64(a.kind, 0.0, scc, a.param, a.coef0, a.degree);
