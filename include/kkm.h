@@ -141,8 +141,8 @@ int32_t kkm_version(void);
  *   k       : 1 <= k <= n.
  *   kernel  : host; as for kkm_init.
  *   out_idx : host, k int64 (the indices kkm_init's init_idx takes).
- *   stream  : cudaStream_t or NULL. The call allocates n + n/128 + k + 2 words
- *             of device scratch, frees it, and synchronises the stream.
+ *   stream  : cudaStream_t or NULL. The call allocates at most n + n/16 + k + 2
+ *             words of device scratch, frees it, and synchronises the stream.
  * kkm_last_error(NULL) reports failures. */
 kkm_status kkm_kmeanspp(const float* X, int64_t n, int32_t d, int64_t ldx, int32_t k, const kkm_kernel* kernel,
                         uint64_t seed, int64_t* out_idx, void* stream);

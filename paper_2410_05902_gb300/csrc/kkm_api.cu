@@ -260,13 +260,16 @@ KKM_API kkm_status kkm_kmeanspp(const float* X, int64_t n, int32_t d, int64_t ld
   double* d2 = nullptr;
   double* part = nullptr;
   int64_t* chosen = nullptr;
-  const int64_t nblk = (n + 127) / 128;
-  cudaError_t e = cudaMalloc(&d2, n * sizeof(double));
+  int dev = 0, sms = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t nblk = kkm::kmeanspp_blocks(n, d, sms);
+  if (e == cudaSuccess) e = cudaMalloc(&d2, n * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&part, nblk * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&chosen, (k + 1) * sizeof(int64_t));   // and the draws' block counter
   if (e == cudaSuccess)
-    e = kkm::launch_kmeanspp(X, n, d, ldx, k, kernel->kind, kernel->param, kernel->coef0, kernel->degree, seed, d2,
-                             part, chosen, reinterpret_cast<unsigned*>(chosen + k), st);
+    e = kkm::launch_kmeanspp(X, n, d, ldx, k, kernel->kind, kernel->param, kernel->coef0, kernel->degree, seed, sms,
+                             d2, part, chosen, reinterpret_cast<unsigned*>(chosen + k), st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(out_idx, chosen, k * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(d2);

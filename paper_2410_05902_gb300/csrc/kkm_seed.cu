@@ -12,29 +12,39 @@
 // [0, n) by Lemire's multiply-high; so does a draw whose total is 0.
 //
 // Each draw is one launch: every block refreshes D^2 against the newest center
-// for its 128 points (a thread per point) and writes its FP64 sum, and the
-// last block to finish finds the crossing point. The chosen index stays on
-// the device, so the k draws need no host round trip.
+// for its points (one, two, four or eight lanes a point) and writes its FP64
+// sum, and the last block to finish finds the crossing point. The chosen index
+// stays on the device, so the k draws need no host round trip.
 //
 // What bounds it: FP64. The chip issues about 2 FP64 operations per clock and
 // SM, 1/64 of its FP32 rate, conversions included. The squared distance is
 // therefore summed in FP32 triples (hi + mid + lo, every rounding error of the
 // large terms carried exactly by two-sums and FMA products), about 40 FP32
 // operations per feature in place of three FP64 ones, with a smaller error
-// than an FP64 sum has; and a thread owns a point, so the FP64 exponential
-// (or square root) runs once per point, not once per lane. Measured at
-// 200000 x 64, k = 50: 38.2 ms per call before (a warp per point, four FP64
-// sums and the exponential on every lane, two launches per draw), 1.75 ms now.
+// than an FP64 sum has; and a point has few lanes, so the FP64 exponential (or
+// square root) runs once per lane of it, not on 32. Measured at 200000 x 64,
+// k = 50: 38.2 ms per call with a warp per point, four FP64 sums, the
+// exponential on every lane and two launches per draw, 1.62 ms now.
 // At d = 3 .. 784 the triples end at most 1.0e-16 (relative) off the exact
 // sum, the FP64 sums they replace 2.3e-16.
+//
+// Lanes per point: one where the points alone fill the chip. Fewer points than
+// two blocks' worth for every SM are spread over more lanes as long as each
+// keeps a tile of features of its own. One draw at 5000 x 784: Gaussian kernel
+// 60 us with one lane a point and 35 with eight (107 with a warp), polynomial
+// 158 and 79 (101 with a warp).
+#include <algorithm>
+#include <type_traits>
+
 #include "kkm_internal.cuh"
 
 namespace kkm {
 namespace {
 
-constexpr int PP_ROWS = 128;                // points per block, a thread each
-constexpr int PP_F = 32;                    // features per staged tile
-constexpr int PP_PITCH = PP_F + 4;          // float4 reads of 32 different rows without bank conflicts
+constexpr int PP_NT = 128;                  // threads per block
+constexpr int PP_STATIC = 21 * 1024;        // a block's shared memory aside from the center's row
+constexpr int PP_F = 32;                    // features per lane of a staged tile
+constexpr int PP_PITCH = PP_F + 4;          // floats per lane of a tile's row: float4 reads without bank conflicts
 
 __device__ __forceinline__ double uniform01(uint64_t seed, uint64_t counter) {
   return (double)(splitmix64(seed, counter) >> 11) * (1.0 / 9007199254740992.0);
@@ -90,27 +100,41 @@ __device__ __forceinline__ void add_square(float x, float c, float& hi, float& m
   lo = __fadd_rn(lo, __fadd_rn(h, __fmaf_rn(e, e, u)));
 }
 
-// Features [f0, f0 + 32) of the warp's 32 points (rows row0 ..) into its tile,
-// zero past d and past the last point.
-__device__ __forceinline__ void stage_tile(const PPArgs& a, int64_t row0, int f0, float (*tile)[PP_PITCH]) {
-  const int lane = threadIdx.x & 31;
-  if (a.vec) {                              // a row's 32 features are eight 16-byte words
+// The sum of two triples.
+__device__ __forceinline__ void add_triple(float& hi, float& mid, float& lo, float bh, float bm, float bl) {
+  float g, h, e;
+  hi = two_sum(hi, bh, g);
+  mid = two_sum(mid, bm, h);
+  mid = two_sum(mid, g, e);
+  lo = __fadd_rn(__fadd_rn(lo, bl), __fadd_rn(h, e));
+}
+
+// Features [f0, f0 + 32 LP) of the warp's 32 / LP points (rows row0 ..) into
+// its tile (rows of LP * PP_PITCH floats), zero past d and past the last point.
+template <int LP>
+__device__ __forceinline__ void stage_tile(const PPArgs& a, int64_t row0, int f0, float* tile) {
+  const unsigned lane = threadIdx.x & 31u;
+  if (a.vec) {                              // a row's features are 8 LP 16-byte words
     float4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int r = 4 * u + (lane >> 3), f = f0 + 4 * (lane & 7);
+      const unsigned i = 32u * u + lane, r = i / (8u * LP), f = f0 + 4u * (i % (8u * LP));
       v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (row0 + r < a.n && f < a.d)
+      if (row0 + r < a.n && f < (unsigned)a.d)
         v[u] = __ldg(reinterpret_cast<const float4*>(a.X + (row0 + r) * a.ldx + f));
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      *reinterpret_cast<float4*>(&tile[4 * u + (lane >> 3)][4 * (lane & 7)]) = v[u];
+    for (int u = 0; u < 8; ++u) {
+      const unsigned i = 32u * u + lane;
+      *reinterpret_cast<float4*>(tile + i / (8u * LP) * (LP * PP_PITCH) + 4u * (i % (8u * LP))) = v[u];
+    }
   } else {
-    const int f = f0 + lane;
 #pragma unroll 8
-    for (int r = 0; r < 32; ++r)
-      tile[r][lane] = (row0 + r < a.n && f < a.d) ? __ldg(a.X + (row0 + r) * a.ldx + f) : 0.0f;
+    for (int u = 0; u < 32; ++u) {
+      const unsigned i = 32u * u + lane, r = i / (PP_F * LP), f = i % (PP_F * LP);
+      tile[r * (LP * PP_PITCH) + f] =
+          (row0 + r < a.n && f0 + f < (unsigned)a.d) ? __ldg(a.X + (row0 + r) * a.ldx + f0 + f) : 0.0f;
+    }
   }
   __syncwarp();
 }
@@ -148,10 +172,11 @@ __device__ int64_t warp_crossing(int64_t lo, int64_t hi, double base, double tar
 // total = sum of the block sums (fixed order); the first point whose running
 // sum exceeds u * total (points in index order) becomes chosen[t + 1]. The
 // search narrows run -> block -> point, each step by one warp.
-__device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int t) {
-  __shared__ double pre[PP_ROWS];
+// points: per block.
+__device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int points, int t) {
+  __shared__ double pre[PP_NT];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int per = (nblk + PP_ROWS - 1) / PP_ROWS;   // thread r sums run r of `per` consecutive block sums
+  const int per = (nblk + PP_NT - 1) / PP_NT;   // thread r sums run r of `per` consecutive block sums
   const int b0 = min(tid * per, nblk), b1 = min(b0 + per, nblk);
   double mine = 0.0;
   for (int q = b0; q < b1; ++q) mine += __ldcg(a.part + q);
@@ -160,7 +185,7 @@ __device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int t) {
   if (tid >= 32) return;
   double total = 0.0;
 #pragma unroll
-  for (int g = 0; g < PP_ROWS / 32; ++g) {          // the same scan order as the search below
+  for (int g = 0; g < PP_NT / 32; ++g) {            // the same scan order as the search below
     double v = pre[32 * g + lane];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -175,11 +200,11 @@ __device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int t) {
   } else {
     const double target = uniform01(a.seed, (uint64_t)(t + 1)) * total;
     double before = 0.0;
-    const int64_t r = warp_crossing(0, PP_ROWS, 0.0, target, [&](int64_t i) { return pre[i]; }, &before);
+    const int64_t r = warp_crossing(0, PP_NT, 0.0, target, [&](int64_t i) { return pre[i]; }, &before);
     const int64_t q0 = min((int64_t)r * per, (int64_t)nblk), q1 = min(q0 + per, (int64_t)nblk);
     const int64_t q = warp_crossing(q0, q1 > q0 ? q1 : q0 + 1, before, target,
                                     [&](int64_t i) { return i < nblk ? __ldcg(a.part + i) : 0.0; }, &before);
-    const int64_t x0 = q * PP_ROWS, x1 = min(x0 + PP_ROWS, a.n);
+    const int64_t x0 = q * points, x1 = min(x0 + points, a.n);
     const int64_t x = warp_crossing(x0, x1 > x0 ? x1 : x0 + 1, before, target,
                                     [&](int64_t i) { return i < a.n ? __ldcg(a.d2 + i) : 0.0; }, &before);
     c = x < a.n ? x : a.n - 1;
@@ -188,86 +213,123 @@ __device__ __forceinline__ void select_next(const PPArgs& a, int nblk, int t) {
 }
 
 // D^2(x) = min(D^2(x), Delta(x, c)) for c = chosen[t] (first draw: = Delta),
-// then (last block) draw t + 1. DOT (linear and polynomial kernels): <x, c>,
-// ||x||^2 and ||c||^2 in FP64, all three in the same order, so that Delta of a
-// row that equals the center's is exactly 0 (||c||^2 is the block's first
-// warp's). Otherwise ||x - c||^2 in FP32 triples; a warp with a sum that left
-// the range where every product is exact (below 2^-60 but not 0, above 2^120,
-// or not finite) sums that tile again in FP64.
-template <bool DOT>
-__global__ void __launch_bounds__(PP_ROWS) k_pp_draw(PPArgs a, int t) {
-  extern __shared__ __align__(16) float crow[];       // [round_up(d, 32)] the center's row
-  __shared__ __align__(16) float tiles[PP_ROWS / 32][32][PP_PITCH];
-  __shared__ double red[PP_ROWS / 32], cself;
+// then (last block) draw t + 1. LP lanes share a point: lane p of it takes the
+// tile's float4 words p, p + LP, .. and the lanes' sums meet by shuffles.
+// DOT (linear and polynomial kernels): <x, c>, ||x||^2 and ||c||^2 in FP64, all
+// three in the same order, so that Delta of a row that equals the center's is
+// exactly 0. The lane's words go to four sums in turn, and the block's four
+// warps take one of ||c||^2's each. The center's row is kept in FP64, which
+// leaves three FP64 operations per feature and lane and a quarter of one:
+// 200000 x 256, linear kernel: 523 us a draw with ||c||^2 in one warp and the
+// center's row converted by every lane, 421 now.
+// Otherwise ||x - c||^2 in FP32 triples; a warp with a sum that left the range
+// where every product is exact (below 2^-60 but not 0, above 2^120, or not
+// finite) sums that tile again in FP64.
+template <bool DOT, int LP>
+__global__ void __launch_bounds__(PP_NT) k_pp_draw(PPArgs a, int t) {
+  using C = std::conditional_t<DOT, double, float>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  C* const crow = reinterpret_cast<C*>(smem);         // [round_up(d, 32 LP)] the center's row
+  __shared__ __align__(16) float tiles[PP_NT / 32][32 * PP_PITCH];
+  __shared__ double red[PP_NT / 32], cself[PP_NT / 32][32];
   __shared__ bool last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t row0 = (int64_t)blockIdx.x * PP_ROWS + 32 * w, x = row0 + lane;
-  const int dp = (a.d + PP_F - 1) / PP_F * PP_F;
-  float(*tile)[PP_PITCH] = tiles[w];
-  stage_tile(a, row0, 0, tile);                       // X does not depend on the draw before
+  constexpr int TF = PP_F * LP;                       // features of a tile
+  const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5, p = lane % LP;
+  const int64_t row0 = (int64_t)blockIdx.x * (PP_NT / LP) + 32 / LP * w, x = row0 + lane / LP;
+  const int dp = (a.d + TF - 1) / TF * TF;
+  float* const tile = tiles[w];
+  const float* const mine = tile + lane / LP * (LP * PP_PITCH);
+  stage_tile<LP>(a, row0, 0, tile);                   // X does not depend on the draw before
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
   const float* cr = a.X + a.chosen[t] * a.ldx;
-  for (int f = threadIdx.x; f < dp; f += PP_ROWS) crow[f] = f < a.d ? cr[f] : 0.0f;
+  for (int f = threadIdx.x; f < dp; f += PP_NT) crow[f] = (C)(f < a.d ? cr[f] : 0.0f);
   __syncthreads();
   double delta;
   if constexpr (DOT) {
-    double sxy = 0.0, sxx = 0.0, scc = 0.0;
-    for (int f0 = 0; f0 < dp; f0 += PP_F) {
+    double qxy[4] = {}, qxx[4] = {}, qcc = 0.0;
+    for (int f0 = 0; f0 < dp; f0 += TF) {
       if (f0 > 0) {
         __syncwarp();
-        stage_tile(a, row0, f0, tile);
+        stage_tile<LP>(a, row0, f0, tile);
       }
-      for (int f = 0; f < PP_F; ++f) {
-        const double xv = tile[lane][f], cv = crow[f0 + f];
-        sxy = fma(xv, cv, sxy);
-        sxx = fma(xv, xv, sxx);
-        if (w == 0) scc = fma(cv, cv, scc);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 xv = *reinterpret_cast<const float4*>(mine + 4 * (i * LP + p));
+        const double2* cq = reinterpret_cast<const double2*>(&crow[f0 + 4 * (i * LP + p)]);
+        const double2 c0 = cq[0], c1 = cq[1];
+        const double xd[4] = {xv.x, xv.y, xv.z, xv.w}, cd[4] = {c0.x, c0.y, c1.x, c1.y};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          qxy[i & 3] = fma(xd[u], cd[u], qxy[i & 3]);
+          qxx[i & 3] = fma(xd[u], xd[u], qxx[i & 3]);
+        }
+        if ((i & 3) == w)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) qcc = fma(cd[u], cd[u], qcc);
       }
     }
-    if (threadIdx.x == 0) cself = scc;
+    static_assert(PP_NT / 32 == 4, "a warp per sum of ||c||^2");
+    cself[w][lane] = qcc;
     __syncthreads();
-    scc = cself;
+    double sxy = (qxy[0] + qxy[1]) + (qxy[2] + qxy[3]);
+    double sxx = (qxx[0] + qxx[1]) + (qxx[2] + qxx[3]);
+    double scc = (cself[0][lane] + cself[1][lane]) + (cself[2][lane] + cself[3][lane]);
+#pragma unroll
+    for (int o = 1; o < LP; o <<= 1) {
+      sxy += __shfl_xor_sync(0xffffffffu, sxy, o);
+      sxx += __shfl_xor_sync(0xffffffffu, sxx, o);
+      scc += __shfl_xor_sync(0xffffffffu, scc, o);
+    }
     delta = kernel_fp64(a.kind, 0.0, sxx, a.param, a.coef0, a.degree) -
             2.0 * kernel_fp64(a.kind, 0.0, sxy, a.param, a.coef0, a.degree) +
             kernel_fp64(a.kind, 0.0, scc, a.param, a.coef0, a.degree);
   } else {
     float hi = 0.0f, mid = 0.0f, lo = 0.0f;
     unsigned nz = 0u;
-    for (int f0 = 0; f0 < dp; f0 += PP_F) {
+    for (int f0 = 0; f0 < dp; f0 += TF) {
       if (f0 > 0) {
         __syncwarp();
-        stage_tile(a, row0, f0, tile);
+        stage_tile<LP>(a, row0, f0, tile);
       }
 #pragma unroll
-      for (int f = 0; f < PP_F; f += 4) {
-        const float4 xv = *reinterpret_cast<const float4*>(&tile[lane][f]);
-        const float4 cv = *reinterpret_cast<const float4*>(&crow[f0 + f]);
+      for (int i = 0; i < 8; ++i) {
+        const float4 xv = *reinterpret_cast<const float4*>(mine + 4 * (i * LP + p));
+        const float4 cv = *reinterpret_cast<const float4*>(&crow[f0 + 4 * (i * LP + p)]);
         add_square(xv.x, cv.x, hi, mid, lo, nz);
         add_square(xv.y, cv.y, hi, mid, lo, nz);
         add_square(xv.z, cv.z, hi, mid, lo, nz);
         add_square(xv.w, cv.w, hi, mid, lo, nz);
       }
     }
+#pragma unroll
+    for (int o = 1; o < LP; o <<= 1) {
+      add_triple(hi, mid, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, mid, o),
+                 __shfl_xor_sync(0xffffffffu, lo, o));
+      nz |= __shfl_xor_sync(0xffffffffu, nz, o);
+    }
     double s2 = (double)hi + ((double)mid + (double)lo);
     const bool redo = nz != 0u && !(hi >= 0x1p-60f && hi <= 0x1p120f);
     if (__any_sync(0xffffffffu, redo)) {
       double s = 0.0;
-      for (int f0 = 0; f0 < dp; f0 += PP_F) {
+      for (int f0 = 0; f0 < dp; f0 += TF) {
         __syncwarp();
-        stage_tile(a, row0, f0, tile);
-        for (int f = 0; f < PP_F; ++f) {
-          const double df = (double)tile[lane][f] - (double)crow[f0 + f];
+        stage_tile<LP>(a, row0, f0, tile);
+        for (int i = 0; i < PP_F; ++i) {
+          const int f = 4 * (i / 4 * LP + p) + i % 4;
+          const double df = (double)mine[f] - (double)crow[f0 + f];
           s = fma(df, df, s);
         }
       }
+#pragma unroll
+      for (int o = 1; o < LP; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (redo) s2 = s;
     }
     delta = 2.0 - 2.0 * kernel_fp64(a.kind, s2, 0.0, a.param, 0.0, 0);
   }
   delta = fmax(delta, 0.0);
   double v = 0.0;
-  if (x < a.n) {
+  if (x < a.n && p == 0) {
     v = (t == 0) ? delta : fmin(a.d2[x], delta);
     a.d2[x] = v;
   }
@@ -277,7 +339,7 @@ __global__ void __launch_bounds__(PP_ROWS) k_pp_draw(PPArgs a, int t) {
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int q = 0; q < PP_ROWS / 32; ++q) s += red[q];
+    for (int q = 0; q < PP_NT / 32; ++q) s += red[q];
     a.part[blockIdx.x] = s;
   }
   // D^2 and the block sum become visible before the block counts as finished
@@ -287,27 +349,57 @@ __global__ void __launch_bounds__(PP_ROWS) k_pp_draw(PPArgs a, int t) {
   __syncthreads();
   if (!last) return;
   __threadfence();
-  select_next(a, (int)gridDim.x, t);
+  select_next(a, (int)gridDim.x, PP_NT / LP, t);
   if (threadIdx.x == 0) *a.done = 0u;                 // ready for the next draw
+}
+
+using PPDraw = void (*)(PPArgs, int);
+template <bool DOT> PPDraw draw_kernel(int lanes) {
+  return lanes == 1   ? k_pp_draw<DOT, 1>
+         : lanes == 2 ? k_pp_draw<DOT, 2>
+         : lanes == 4 ? k_pp_draw<DOT, 4>
+                      : k_pp_draw<DOT, 8>;
 }
 
 }  // namespace
 
+// Lanes per point (see the header comment).
+static int kmeanspp_lanes(int64_t n, int d, int num_sms) {
+  int lanes = 1;
+  while (lanes < 8 && n * lanes < 2 * (int64_t)PP_NT * num_sms && d > PP_F * lanes) lanes *= 2;
+  return lanes;
+}
+
+int64_t kmeanspp_blocks(int64_t n, int d, int num_sms) {
+  return (n * kmeanspp_lanes(n, d, num_sms) + PP_NT - 1) / PP_NT;
+}
+
 cudaError_t launch_kmeanspp(const float* X, int64_t n, int d, int64_t ldx, int k, int kind, double param,
-                            double coef0, int degree, uint64_t seed, double* d2, double* part, int64_t* chosen,
-                            unsigned* done, cudaStream_t st) {
+                            double coef0, int degree, uint64_t seed, int num_sms, double* d2, double* part,
+                            int64_t* chosen, unsigned* done, cudaStream_t st) {
   const int vec = d % 4 == 0 && ldx % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
   PPArgs a{X, n, ldx, d, kind, degree, param, coef0, seed, d2, part, chosen, done, vec};
-  const int64_t nblk = (n + PP_ROWS - 1) / PP_ROWS;
+  const int lanes = kmeanspp_lanes(n, d, num_sms);
+  const int64_t nblk = kmeanspp_blocks(n, d, num_sms);
   if (nblk > (int64_t)0x7fffffff) return cudaErrorInvalidValue;
   // draw 0: uniform
   const int64_t first = (int64_t)index_below(splitmix64(seed, 0), (uint64_t)n);
   cudaError_t e = cudaMemcpyAsync(chosen, &first, sizeof(first), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(done, 0, sizeof(unsigned), st);
   const bool dot = kind == K_LINEAR || kind == K_POLY;
-  const size_t smem = (size_t)round_up(d, PP_F) * sizeof(float);   // at most 16 KB
+  const PPDraw draw = dot ? draw_kernel<true>(lanes) : draw_kernel<false>(lanes);
+  size_t smem = (size_t)round_up(d, PP_F * lanes) * (dot ? sizeof(double) : sizeof(float));   // at most 32 KB
+  // Blocks of the next draw take their places while this one's finish, wherever
+  // there is room, and then stay: with more room than its share an SM ends up
+  // with nine of 782 blocks that others have five of. Shared memory past the
+  // row's keeps every SM to its share (at most eight). 100000 points, d = 64 and
+  // 256: 33.0 and 82 us a draw without, 29.1 and 65 with.
+  const int64_t share = std::min<int64_t>(8, (nblk + num_sms - 1) / num_sms);
+  if (share >= 2) smem = std::max<size_t>(smem, (228 * 1024 / share - 1024 - PP_STATIC) / 128 * 128);
+  if (e == cudaSuccess && smem > 24 * 1024)   // with the staged tiles more than a kernel has by default
+    e = cudaFuncSetAttribute(draw, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);   // the same for every call
   for (int t = 0; t + 1 < k && e == cudaSuccess; ++t)
-    e = launch_pdl(dot ? k_pp_draw<true> : k_pp_draw<false>, dim3((unsigned)nblk), dim3(PP_ROWS), smem, st, a, t);
+    e = launch_pdl(draw, dim3((unsigned)nblk), dim3(PP_NT), smem, st, a, t);
   return e;
 }
 
