@@ -458,9 +458,14 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   if (!tab) ALLOC(s.split, s.nsplit + 1); ALLOC(s.tile_cnt, k);
   ALLOC(s.part, (size_t)s.max_tiles * s.ppt * s.bpad);
   ALLOC(s.wpairs, s.max_pairs); ALLOC(s.nwpairs, 1); ALLOC(s.wpair_first, k); ALLOC(s.wpair_cnt, k);
-  s.wslots = c->use_tc ? 1 : 4;   // window-pass partial slots (of four sums) per item
-  ALLOC(s.wpart, (size_t)s.max_pairs * s.wslots * 4);
-  ALLOC(s.iter, 1); ALLOC(s.gnext, 1); ALLOC(s.wdone, k); ALLOC(s.fin_pending, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
+  ALLOC(s.wpart, (size_t)s.max_pairs * 4);
+  {
+    const size_t slots = (size_t)kkm::win_segment_slots(s.max_pairs, k);
+    ALLOC(s.wseg, slots * 4);
+    ALLOC(s.wdone, slots);
+    ALLOC(s.cdone, k);
+  }
+  ALLOC(s.iter, 1); ALLOC(s.gnext, 1); ALLOC(s.fin_pending, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
   {
     // the finalise step's rate sqrt(n/b) and 1/n, by the host's correctly rounded
     // FP64 operations (the same values the device would compute)

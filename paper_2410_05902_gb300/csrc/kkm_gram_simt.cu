@@ -231,10 +231,9 @@ __global__ void __launch_bounds__(NT) k_dist_simt(Dev s, int rows) {
   for (int w = blockIdx.x; w < total; w += gridDim.x) dist_simt_item<F, MR>(s, rows, R, w, sm);
 }
 
-// Pair w of a run's window pass; its four sums go to wpart[w] (slot 0).
+// Pair w of a run's window pass; its four sums go to wpart[w].
 template <int F>
-__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms, GramSmem<4>& sm,
-                                                double (*red)[NT / 32]) {
+__device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, GramSmem<4>& sm, double (*red)[NT / 32]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
   {
     const WPair pr = s.wpairs[w];
@@ -304,24 +303,13 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, bool norms,
       if ((lane & 7) == 0) red[(hi ? 1 : 0) + (up ? 2 : 0)][warp] = v;
     }
     __syncthreads();
-    if (tid < 16) {   // slot 0 holds the tile's sums, slots 1-3 are zero
+    if (tid < 4) {
       double v = 0.0;
       if (tid < 4)
         for (int q = 0; q < NT / 32; ++q) v += red[tid][q];
-      s.wpart[(int64_t)w * 16 + tid] = v;
+      s.wpart[(int64_t)w * 4 + tid] = v;
     }
     __syncthreads();
-    if (norms && warp == 0) {   // whoever finishes a center's last pair carries its norm
-      int last = 0;
-      if (lane == 0) {
-        __threadfence();
-        last = atomicAdd(&s.wdone[pr.j], 1) + 1 == s.wpair_cnt[pr.j];
-      }
-      if (__shfl_sync(0xffffffffu, last, 0)) {
-        __threadfence();
-        norm_update(s, pr.j);
-      }
-    }
   }
 }
 
@@ -332,7 +320,26 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   __shared__ __align__(16) GramSmem<4> sm;
   __shared__ double red[4][NT / 32];
   const int total = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
-  for (int w = bid; w < total; w += nblk) wgram_simt_item<F>(s, w, norms, sm, red);
+  // Norms are reported by the first warp, whose first four lanes wrote the sums.
+  // Many items a block: a contiguous range each, so that its reports are few;
+  // few: strided, so that a center's items spread over the chip. FP32, d = 64,
+  // 90 % of the batch in one of 10 centers, us a step strided and contiguous:
+  // b = 1024 (1.5 items a block) 85 and 92, b = 2048 (6) 221 and 208, b = 8192
+  // (75) 2649 and 2459.
+  if (total < 4 * nblk) {
+    for (int w = bid; w < total; w += nblk) {
+      wgram_simt_item<F>(s, w, sm, red);
+      const int j = s.wpairs[w].j;
+      if (norms && threadIdx.x < 32) norm_report(s, j, (w - s.wpair_first[j]) / WSEG, 1);
+    }
+    return;
+  }
+  const int lo = (int)((int64_t)bid * total / nblk), hi = (int)((int64_t)(bid + 1) * total / nblk);
+  NormReports reports(hi);
+  for (int w = lo; w < hi; ++w) {
+    wgram_simt_item<F>(s, w, sm, red);
+    if (norms && threadIdx.x < 32) reports.done(s, w, s.wpairs[w].j);
+  }
 }
 
 template <int F>
@@ -375,7 +382,7 @@ __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
     }
     const Dev& s = g.runs[lo].s;
     if constexpr (MODE == 0) dist_simt_item<F, 4>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], sm);
-    else wgram_simt_item<F>(s, w - off[lo], false, sm, red);
+    else wgram_simt_item<F>(s, w - off[lo], sm, red);
   }
 }
 

@@ -941,9 +941,8 @@ __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t
                                          int rows, int warp, int lane, bool all, bool norms, int rank) {
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
   const Place<TNV> pl(warp, lane, all);
-  // part[] must hold GPT partials per tile and wpart[] one slot of four sums
-  // per window item, as the host sized them (Dev::ppt, Dev::wslots)
-  bool dead = (MODE != 1 && s.ppt != Geo<TNV>::GPT) || (MODE != 0 && s.wslots != 1);
+  // part[] must hold GPT partials per tile, as the host sized it (Dev::ppt)
+  bool dead = MODE != 1 && s.ppt != Geo<TNV>::GPT;
   if (dead && lane == 0 && warp == 2) atomicOr(s.status, ST_CAPACITY);
   const int nw = MODE == 0 ? 0 : rw.hi - rw.lo;
   const int n = nw + (MODE == 1 ? 0 : rd.hi - rd.lo);
@@ -977,13 +976,12 @@ __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t
   }
 }
 
-// The norm warp (a launch with norms): counts every finished window item of
-// this CTA at its center; whoever finishes a center's last item carries its
-// norm (norm_update). The item's sums were written by the epilogue before its
-// arrival on nfull; the fences order them before the count and the counts of
-// all items before the norm's reads.
+// The norm warp (a launch with norms): reports every finished window item of
+// this CTA (items lo, lo + 1, ..). The item's sums were written by the epilogue
+// before its arrival on nfull.
 template <int TNV>
-__device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int nw, int lane) {
+__device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int lo, int nw, int lane) {
+  NormReports reports(lo + nw);
   for (uint32_t i = 0; (int)i < nw; ++i) {
     const uint32_t ns = i % NSLOT;
     const bool ok = mbar_wait(&sh.nfull[ns], (i / NSLOT) & 1u);
@@ -994,16 +992,7 @@ __device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int nw,
     const int j = sh.nj[ns];
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.nempty[ns]);
-    if (j < 0) continue;
-    int last = 0;
-    if (lane == 0) {
-      __threadfence();
-      last = atomicAdd(&s.wdone[j], 1) + 1 == s.wpair_cnt[j];
-    }
-    if (__shfl_sync(0xffffffffu, last, 0)) {
-      __threadfence();
-      norm_update(s, j);
-    }
+    reports.done(s, lo + (int)i, j);
   }
 }
 
@@ -1487,7 +1476,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   } else if (warp < MWARP) {
     epilogue<KIND, MODE, TNV, PAIR>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_groups, norms, rank);
   } else if constexpr (MODE != 0) {
-    if (norms) norm_warp<TNV>(s, sh, nw, lane);
+    if (norms) norm_warp<TNV>(s, sh, rw.lo, nw, lane);
   }
   tc_fence_before();
   if constexpr (PAIR) {

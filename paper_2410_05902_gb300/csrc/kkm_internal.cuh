@@ -158,11 +158,12 @@ struct alignas(16) Dev {
   int32_t* wpair_cnt;   // [k]
   double* ncum;      // [k] points assigned to each center so far (N^j of the sklearn rate)
   const double* rtab; // [2 (b + 1)]: 1/n at [n] and sqrt(n / b) at [b + 1 + n], n = 0..b (host-computed)
-  double* wpart;     // [max_pairs][wslots][4 sums]: A, Bdd, E, M partials per tile
-  int32_t wslots;    // partial slots per window-pass tile (SIMT: 4, slot 0 used; tcgen05: 1)
+  double* wpart;     // [max_pairs][4 sums]: A, Bdd, E, M partials per window item
+  double* wseg;      // [win_segment_slots][4 sums]: the same per segment of a center's items
   int64_t* iter;     // [1] next iteration number
   int32_t* status;   // [1] sticky device status bits
-  int32_t* wdone;    // [k] finished window items of the pending update (k_sort_plan clears them)
+  int32_t* wdone;    // [win_segment_slots] finished items of each segment (k_sort_plan clears them)
+  int32_t* cdone;    // [k] finished segments (k_sort_plan clears them)
   int64_t* gnext;    // [1] the iteration whose batch has been scored (its successor's batch may be gathered)
   int32_t* fin_pending;   // [1] 1 while a step's window pass and center norms are still to run
   int64_t* stats;    // [3] steps, support rows, tiles
@@ -255,23 +256,74 @@ static __device__ __noinline__ double norm_recurrence(double a, double cmc, doub
   return keep * keep * R2 + 2.0 * a * keep * Rm + a * a * m2;
 }
 
-// ||C_j||^2 after the update, by one warp, once all of center j's window items
-// are in wpart: the sums in k_finalize's order (element e of a center's partials
-// is sum e & 3; eight strided runs, then run by run), the recurrence on lane 0.
-__device__ __forceinline__ void norm_update(const Dev& s, int j) {
+// The window items of a center are added up in segments of WSEG items, then the
+// segments' sums: a center's items grow with the square of its rows (two at 40
+// rows, 768 at 1900), and as one list read by the warp that finishes the last
+// of them the sum was tens of microseconds that the argmin waits for. A segment
+// is summed by the warp that finishes the last item in it, wherever that runs,
+// with all its loads in flight at once. 90 % of the batch in one of 10 centers,
+// d = 64, us a step with one list and with segments: BF16 b = 4096 120 and 88,
+// b = 8192 392 and 276; FP32 b = 2048 346 and 208, b = 8192 4683 and 2459.
+constexpr int WSEG = 64;
+__host__ __device__ inline int win_segments(int items) { return (items + WSEG - 1) / WSEG; }
+// Place of the first segment of center j, whose items start at `first`: no two
+// centers' segments meet, and all lie below win_segment_slots.
+__host__ __device__ inline int win_segment_slot(int first, int j) { return first / WSEG + j; }
+__host__ __device__ inline int win_segment_slots(int items, int k) { return items / WSEG + k + 1; }
+
+// Sums of n / 4 partials of four values each by a warp (element e belongs to
+// value e & 3): lane l ends with value l & 3. One order for every caller.
+__device__ __forceinline__ double sum_partials(const double* p, int n) {
   const int lane = threadIdx.x & 31;
-  const int n = s.plan[j].cnt, per = s.wslots * 4;
-  const int cnt = s.wpair_cnt[j] * per;
-  const double* wp = s.wpart + (int64_t)s.wpair_first[j] * per;
+  double acc = 0.0;
+  for (int e0 = 0; e0 < n; e0 += 256) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + 32 * u + lane;
+      v[u] = e < n ? __ldcg(p + e) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + 32 * u < n) acc += v[u];
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+
+// Whether this warp's `m` arrivals are the last of `of` on the counter; what
+// the earlier ones wrote before theirs is then visible.
+__device__ __forceinline__ bool last_arrival(int32_t* counter, int m, int of) {
+  int last = 0;
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    last = atomicAdd(counter, m) + m == of;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return false;
+  __threadfence();
+  return true;
+}
+
+// A warp's report of m finished window items of segment q of center j (their
+// sums are in wpart): the last of a segment adds it up, the last of a center's
+// segments adds those and carries ||C_j||^2 through the update. A fence and an
+// atomic take longer than an item's arithmetic, so consecutive items of a
+// segment are reported together (NormReports).
+__device__ __forceinline__ void norm_report(const Dev& s, int j, int q, int m) {
+  const int lane = threadIdx.x & 31;
+  const int first = s.wpair_first[j], cnt = s.wpair_cnt[j];
+  const int nseg = win_segments(cnt), slot = win_segment_slot(first, j), here = min(WSEG, cnt - q * WSEG);
+  if (!last_arrival(s.wdone + slot + q, m, here)) return;
+  const int n = s.plan[j].cnt;
   const double part = (double)s.cmpart[(int64_t)j * 32 + lane];
   const double inv_n = s.rtab[n], a = s.alpha[j], cn_old = s.cnorm[j];
-  double qt = 0.0;
-  for (int w = 0; w < 8 && w * 32 < cnt; ++w) {
-    double acc = 0.0;
-    for (int e = w * 32 + lane; e < cnt; e += 256) acc += __ldcg(wp + e);
-#pragma unroll
-    for (int o = 4; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    qt += acc;
+  double qt = sum_partials(s.wpart + (int64_t)(first + q * WSEG) * 4, here * 4);
+  if (nseg > 1) {
+    if (lane < 4) __stcg(s.wseg + (int64_t)(slot + q) * 4 + lane, qt);
+    __syncwarp();
+    if (!last_arrival(s.cdone + j, 1, nseg)) return;
+    qt = sum_partials(s.wseg + (int64_t)slot * 4, nseg * 4);
   }
   const double A = __shfl_sync(0xffffffffu, qt, 0), Bdd = __shfl_sync(0xffffffffu, qt, 1);
   const double E = __shfl_sync(0xffffffffu, qt, 2), M = __shfl_sync(0xffffffffu, qt, 3);
@@ -283,6 +335,22 @@ __device__ __forceinline__ void norm_update(const Dev& s, int j) {
     s.cnorm32[j] = (float)cn;
   }
 }
+
+// Gathers the reports of a warp that finishes the items lo, .. , hi - 1 in
+// order: one per segment. done(item, j): item of center j is finished (j < 0: it
+// was skipped, and its center keeps its norm).
+struct NormReports {
+  int hi, m = 0;
+  __device__ explicit NormReports(int hi_) : hi(hi_) {}
+  __device__ __forceinline__ void done(const Dev& s, int item, int j) {
+    const int jn = item + 1 < hi ? s.wpairs[item + 1].j : -1;
+    const int jc = s.wpairs[item].j, at = item - s.wpair_first[jc];
+    m += j >= 0 ? 1 : 0;
+    if (jn == jc && (at + 1) % WSEG != 0) return;
+    if (m > 0) norm_report(s, jc, at / WSEG, m);
+    m = 0;
+  }
+};
 
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t m) { return (a + m - 1) / m * m; }
 

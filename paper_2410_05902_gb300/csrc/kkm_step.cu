@@ -587,10 +587,11 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, in
     s.comp_off[tid] = ex3[0];
     s.wpair_first[tid] = ex3[1];
     s.wpair_cnt[tid] = npairs;
-    s.wdone[tid] = 0;
+    s.cdone[tid] = 0;
     base[tid] = ex3[1];
     tot[tid] = npairs;
   }
+  for (int e = tid; e < win_segment_slots(min(ptotal, s.max_pairs), k); e += 1024) s.wdone[e] = 0;
   if (tid == 0) {
     *s.comp_total = tot3[0];
     *s.nwpairs = ptotal <= s.max_pairs ? ptotal : s.max_pairs;
@@ -893,10 +894,8 @@ __device__ __forceinline__ void finalize_body(const Dev& s, int bid) {
     inv_n = s.rtab[P.cnt];
     beta = s.rtab[s.b + 1 + P.cnt];
   }
-  __shared__ double red[8][4];
   __shared__ double cm_s;
   __shared__ double keep_s, wnew_s;
-  const int per = s.wslots * 4;
   const int p0 = s.wpair_first[j];
   const int np = (p0 + s.wpair_cnt[j] <= s.max_pairs) ? s.wpair_cnt[j] : 0;
   if (warp == 0 && P.cnt > 0) {
@@ -906,22 +905,17 @@ __device__ __forceinline__ void finalize_body(const Dev& s, int bid) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top
   if (P.cnt == 0) return;
-  // window-pass sums: element e of a tile's partials is sum e & 3 (A, Bdd, E, M);
-  // with a stride of 256 every thread stays on sum tid & 3
-  const double* wp = s.wpart + (int64_t)p0 * per;
-  double acc = 0.0;
-#pragma unroll 8
-  for (int e = tid; e < np * per; e += 256) acc += wp[e];
-#pragma unroll
-  for (int o = 4; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane < 4) red[warp][lane] = acc;
+  // window-pass sums (A, Bdd, E, M), segment by segment as norm_item adds them
+  const int nseg = win_segments(np);
+  double* const wseg = s.wseg + (int64_t)win_segment_slot(p0, j) * 4;
+  for (int q = warp; q < nseg; q += 8) {
+    const double v = sum_partials(s.wpart + (int64_t)(p0 + q * WSEG) * 4, min(WSEG, np - q * WSEG) * 4);
+    if (lane < 4) __stcg(wseg + q * 4 + lane, v);
+  }
   __syncthreads();
   const int n = P.cnt;
   if (warp == 0) {
-    // lane t < 4 adds sum t over the eight warps, in warp order
-    double qt = 0.0;
-    if (lane < 4)
-      for (int w = 0; w < 8; ++w) qt += red[w][lane];
+    const double qt = sum_partials(wseg, nseg * 4);
     const double A = __shfl_sync(0xffffffffu, qt, 0), Bdd = __shfl_sync(0xffffffffu, qt, 1);
     const double E = __shfl_sync(0xffffffffu, qt, 2), M = __shfl_sync(0xffffffffu, qt, 3);
     if (lane == 0) {
