@@ -390,7 +390,6 @@ def time_form(form, args, X, Xd, kappa, init, rank, world, dev, barrier):
     # replay, and the single-step one for a remainder) are captured here
     for _ in range(max(2, -(-args.warmup // K))):
         run.steps(K)
-    run.flush()
     run.sync()
     run.stats(reset=True)
     run.launches(reset=True)
@@ -401,7 +400,6 @@ def time_form(form, args, X, Xd, kappa, init, rank, world, dev, barrier):
         barrier()
         ev0.record(stream)
         run.steps(K)                          # the fixed-iteration loop with the built-in sampler
-        run.flush()                           # the last step's weight update (each step queues the previous one's)
         ev1.record(stream)
         barrier()
         return ev0.elapsed_time(ev1)
@@ -630,7 +628,7 @@ def run_ours(args):
             "timing": {"support_rows_S": r["S"], "state_prep_iters": PREP_ITERS,
                        "blocks": r["blocks"], "block_ms_median": r["ms"], "block_ms_p10": r["block_ms_p10"],
                        "block_ms_p90": r["block_ms_p90"], "block_ms_first": r["block_ms_first"],
-                       "region": f"{r['blocks']} blocks of exactly {args.steps} steps (kkm_steps + flush), "
+                       "region": f"{r['blocks']} blocks of exactly {args.steps} steps (kkm_steps), "
                                  "each bracketed by barrier + synchronize and CUDA events; ms_per_step from "
                                  "the median block; graphs captured during the warm-up",
                        "step_launch": "eager kernel launches" if args.no_graph else

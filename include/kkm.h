@@ -201,25 +201,25 @@ kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d, int64_t
  *   batch_obj_out : device, one double, or NULL. Receives
  *                   f_{B_i}(C_i) = (1/b) sum_x min_j Delta(x, C_i^j) (Sec. 3).
  * An index out of range is found on the device, and it poisons the context.
- * The last kernel of the weight update (k_finalize) is queued at the start of
- * the next kkm_step, where it runs beside the next batch's gather, or by the
- * next call that reads or replaces the centers (every call below but
- * kkm_stats and the timing and launch counters), or by kkm_flush. The
- * outputs above do not depend on it. */
+ * All of the step's kernels are queued when the call returns. */
 kkm_status kkm_step(kkm_ctx* ctx, const int32_t* batch_idx, const int32_t* forced_assign,
                     int32_t* assign_out, float* dist_out, double* batch_obj_out);
 
-/* kkm_flush -- queues the weight update the last kkm_step left pending, if
- * any, on the context's stream (asynchronous; nothing to do otherwise). */
+/* kkm_flush -- every call queues all of its own work, so there is nothing to do
+ * unless a call of several steps failed on the way: then the center norms of
+ * its last step are queued here, or by the next call that needs them.
+ * Asynchronous. */
 kkm_status kkm_flush(kkm_ctx* ctx);
 
 /* kkm_steps -- n iterations of kkm_step with the built-in sampler and no
- * outputs: the fixed-iteration loop of the experiments (Sec. 6). With graphs
- * enabled (kkm_graph_enable) it replays a captured graph of 16 iterations,
- * inside which consecutive iterations meet through programmatic dependent
- * launch, and runs the remainder one step at a time. The result is the same,
- * bit for bit, as n calls of kkm_step(ctx, NULL, NULL, NULL, NULL, NULL).
- * Asynchronous; n >= 0. */
+ * outputs: the fixed-iteration loop of the experiments (Sec. 6). An
+ * iteration's window pass (the center norms) runs in the distance launch of the
+ * next one, the last one's in a launch of its own. With graphs enabled
+ * (kkm_graph_enable) it replays captured graphs of up to 16 iterations, inside
+ * which consecutive iterations meet through programmatic dependent launch (a
+ * graph is captured when its length and place in the call first occur). The
+ * result is the same, bit for bit, as n calls of
+ * kkm_step(ctx, NULL, NULL, NULL, NULL, NULL). Asynchronous; n >= 0. */
 kkm_status kkm_steps(kkm_ctx* ctx, int64_t n);
 
 /* kkm_step_eval -- kkm_step (device sampler when batch_idx is NULL) that

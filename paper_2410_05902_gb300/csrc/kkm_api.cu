@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <tuple>
 #include <unordered_set>
@@ -58,8 +59,9 @@ struct kkm_ctx {
   char* d_qslot[2] = {nullptr, nullptr};
   size_t q_nb4 = 0;
   cudaEvent_t qdone[2] = {nullptr, nullptr};
-  cudaGraphExec_t gexec_q[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [slot][host indices]
-  bool fin_pending = false;          // the last step's window pass and norms are still to run (see flush)
+  cudaGraphExec_t gexec_q[2][8] = {};   // [slot][host indices + 2 * (first of its call) + 4 * (last of its call)]
+  bool fin_pending = false;          // a call in progress: the last queued step's window pass and norms are still to queue
+  bool own_work = false;             // steps queued on `stream` since it was last synchronised
   // the second set of batch buffers and its descriptors: within a captured run
   // of steps the batches alternate, so that one can be gathered while the
   // rows of the other still move (the first set is s's own)
@@ -85,7 +87,8 @@ struct kkm_ctx {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   const void* gkey[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  cudaGraphExec_t gexec_multi = nullptr;     // kkm_steps: STEPS_PER_GRAPH sampler steps per replay
+  // kkm_steps: the graphs of its chains, by 4 * steps + 2 * (first of its call) + (last of its call)
+  std::map<int, cudaGraphExec_t> gexec_run;
   // table form of Algorithm 1 (kkm_config.algo = KKM_ALGO_TABLE)
   bool tab = false;
   kkm::TabBuf tb{};
@@ -127,17 +130,18 @@ void free_all(kkm_ctx* c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   c->gexec = nullptr;
   for (int q = 0; q < 2; ++q) {
-    for (int h = 0; h < 2; ++h) {
-      if (c->gexec_q[q][h]) cudaGraphExecDestroy(c->gexec_q[q][h]);
-      c->gexec_q[q][h] = nullptr;
+    for (cudaGraphExec_t& ge : c->gexec_q[q]) {
+      if (ge) cudaGraphExecDestroy(ge);
+      ge = nullptr;
     }
     if (c->qdone[q]) cudaEventDestroy(c->qdone[q]);
     c->qdone[q] = nullptr;
   }
   if (c->h_qstage) cudaFreeHost(c->h_qstage);
   c->h_qstage = nullptr;
-  if (c->gexec_multi) cudaGraphExecDestroy(c->gexec_multi);
-  c->gexec_multi = nullptr;
+  for (auto& g : c->gexec_run)
+    if (g.second) cudaGraphExecDestroy(g.second);
+  c->gexec_run.clear();
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   c->cap_stream = nullptr;
   for (void* p : c->allocs) cudaFree(p);
@@ -160,22 +164,22 @@ kkm_status check_usable(kkm_ctx* c) {
   return KKM_OK;
 }
 
-// A step (windows form, kkm_step) ends with its row moves and weights and
-// leaves its window pass, and the center norms that follow from it, to the
-// next step's distance pass. Every call that reads or replaces the centers
-// first runs it here (on the context's stream).
+// Within a call of several steps (windows form) a step's window pass, and the
+// center norms that follow from it, run in the next step's distance launch; the
+// last step's has a launch of its own before the call returns. Only a call that
+// failed in between leaves it pending, and then the next call that reads or
+// replaces the centers runs it here first (on the context's stream).
 kkm_status flush(kkm_ctx* c) {
   if (!c->fin_pending) return KKM_OK;
-  cudaError_t e = c->use_tc ? kkm::launch_wgram_tc(c->s, c->tmaps, c->stream, true)
-                            : kkm::launch_wgram(c->s, c->stream, true);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->s.fin_pending, 0, sizeof(int32_t), c->stream);
+  const cudaError_t e = c->use_tc ? kkm::launch_wgram_tc(c->s, c->tmaps, c->stream, true)
+                                  : kkm::launch_wgram(c->s, c->stream, true);
   if (e != cudaSuccess) return cuda_fail(c, e, "pending center norms");
   c->fin_pending = false;
   c->launches += 1;
   return KKM_OK;
 }
 
-// check_usable, then the pending weight update.
+// check_usable, then what a failed call left pending.
 kkm_status check_ready(kkm_ctx* c) {
   const kkm_status st = check_usable(c);
   return st != KKM_OK ? st : flush(c);
@@ -189,6 +193,7 @@ kkm_status sync_and_check(kkm_ctx* c) {
   if (e != cudaSuccess) return cuda_fail(c, e, "status read");
   e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
+  c->own_work = false;
   const int32_t st = *c->h_status;
   if (st != 0) {
     c->poisoned = true;
@@ -220,12 +225,15 @@ Dev batch_view(const kkm_ctx* c, int buf) {
   return v;
 }
 
-// A run whose window pass has a launch of its own ahead of the distance pass:
-// the FP32 form, and 64-row distance tiles (narrower than a window item's).
+// A run whose window pass always has a launch of its own: the FP32 form, and
+// 64-row distance tiles (narrower than a window item's).
 bool split_window(const kkm_ctx* c) { return !c->use_tc || c->s.tn < kkm::WPASS_TNV; }
 
-// Kernels of one step of a run's own sequence, its gather aside.
-int step_kernels(const kkm_ctx* c) { return c->tab ? 6 : split_window(c) ? 5 : 4; }
+// Kernels of a chain of m steps (enqueue_steps; last: it ends its call).
+int chain_kernels(const kkm_ctx* c, int m, bool last) {
+  if (c->tab) return 7 * m;
+  return 1 + 4 * m + (split_window(c) ? m : last ? 1 : 0);   // the gathers but the first are in the step before
+}
 
 }  // namespace
 
@@ -465,7 +473,7 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
     ALLOC(s.wdone, slots);
     ALLOC(s.cdone, k);
   }
-  ALLOC(s.iter, 1); ALLOC(s.gnext, 1); ALLOC(s.fin_pending, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
+  ALLOC(s.iter, 1); ALLOC(s.gnext, 1); ALLOC(s.status, 1); ALLOC(s.stats, 3); ALLOC(s.obj, 1);
   {
     // the finalise step's rate sqrt(n/b) and 1/n, by the host's correctly rounded
     // FP64 operations (the same values the device would compute)
@@ -605,16 +613,18 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
 // Place of a step in a run of steps queued together.
 struct StepPlace {
   int buf = 0;                       // batch buffer set
+  bool window = false;               // the window pass of the step before runs in this distance launch
+  bool close = true;                 // this step's own window pass is queued at its end
   bool gathered = false;             // the step before gathered this batch
   bool next = false;                 // gather the next step's batch beside this step's row moves
   const int32_t* next_idx = nullptr; // its indices (NULL: built-in sampler)
 };
 
 // The kernel sequence of one step, queued on `st`.
-// rotated (a run's own steps, windows form): the window pass and the center
-// norms of the step before run in this step's distance pass (nothing unless
-// they are pending), and this step leaves its own pending. Otherwise (run
-// groups) the window pass and k_finalize end the step.
+// rotated (a run's own steps, windows form): the weight update runs beside the
+// row moves, and the window pass with the center norms follows it (at.close) or
+// goes into the next step's distance launch. Otherwise (run groups) the window
+// pass and k_finalize end the step.
 static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch_idx,
                                const int32_t* forced_assign, int32_t* assign_out, float* dist_out,
                                double* batch_obj_out, bool timed, bool rotated, const StepPlace& at = StepPlace{}) {
@@ -647,14 +657,10 @@ static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch
     v.wwin = s.w32;
     v.wwin64 = s.w64;
   }
-  if (rotated && (timed || split_window(c))) {
-    KKM_CU(c->use_tc ? kkm::launch_wgram_tc(v, maps, st, true) : kkm::launch_wgram(v, st, true), "window Gram");
-    if (timed) KKM_CU(cudaMemsetAsync(s.fin_pending, 0, sizeof(int32_t), st), "pending flag");
-  }
   if (!at.gathered) KKM_CU(kkm::launch_gather_batch(v, batch_idx, st), "batch gather");
   if (timed) KKM_CU(cudaEventRecord(c->ev[2 * c->ev_used], st), "timing event");
   for (int r = 0; r < (timed ? c->timing_reps : 1); ++r) {   // the distance pass alone is idempotent
-    if (rotated && !timed && !split_window(c)) KKM_CU(kkm::launch_step_tc(v, maps, st), "step kernel (tcgen05)");
+    if (at.window) KKM_CU(kkm::launch_step_tc(v, maps, st), "step kernel (tcgen05)");
     else if (c->use_tc) KKM_CU(kkm::launch_dist_tc(v, maps, s.b, st, true), "distance kernel (tcgen05)");
     else KKM_CU(kkm::launch_dist_simt(v, s.b, st), "distance kernel");
   }
@@ -663,10 +669,12 @@ static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch
     c->ev_reps[c->ev_used++] = c->timing_reps;
   }
   KKM_CU(kkm::launch_argmin(v, s.b, forced_assign, assign_out, nullptr, dist_out, true, st), "argmin");
-  KKM_CU(kkm::launch_sort_plan(v, batch_obj_out, st, rotated), "sort/plan");
+  KKM_CU(kkm::launch_sort_plan(v, batch_obj_out, st), "sort/plan");
   if (rotated) {
     const Dev nx = batch_view(c, at.buf ^ 1);
     KKM_CU(kkm::launch_update(v, at.next ? &nx : nullptr, at.next_idx, st), "row moves and weights");
+    if (at.close)
+      KKM_CU(c->use_tc ? kkm::launch_wgram_tc(v, maps, st, true) : kkm::launch_wgram(v, st, true), "window Gram");
     return KKM_OK;
   }
   KKM_CU(kkm::launch_move(v, st), "row moves");
@@ -676,16 +684,21 @@ static kkm_status enqueue_step(kkm_ctx* c, cudaStream_t st, const int32_t* batch
   return KKM_OK;
 }
 
-// `m` steps queued together on `st`: in the windows form the batches alternate
-// between the two buffer sets, each gathered beside the row moves of the step
-// before. idx, asg and obj give step i's pointers.
+// A chain of `m` steps queued together on `st`: in the windows form the batches
+// alternate between the two buffer sets, each gathered beside the row moves of
+// the step before, and a step's window pass runs in the next one's distance
+// launch (first: the chain starts its call, nothing is pending; last: it ends
+// its call and leaves nothing pending). idx, asg and obj give step i's pointers.
 template <class Idx, class Asg, class Obj>
-static kkm_status enqueue_steps(kkm_ctx* c, cudaStream_t st, int m, Idx idx, Asg asg, Obj obj) {
+static kkm_status enqueue_steps(kkm_ctx* c, cudaStream_t st, int m, bool first, bool last, Idx idx, Asg asg,
+                                Obj obj) {
   kkm_status r = KKM_OK;
   for (int i = 0; i < m && r == KKM_OK; ++i) {
     StepPlace at;
     if (!c->tab) {
       at.buf = i & 1;
+      at.window = !split_window(c) && !(first && i == 0);
+      at.close = split_window(c) || (last && i + 1 == m);
       at.gathered = i > 0;
       at.next = i + 1 < m;
       at.next_idx = at.next ? idx(i + 1) : nullptr;
@@ -697,7 +710,7 @@ static kkm_status enqueue_steps(kkm_ctx* c, cudaStream_t st, int m, Idx idx, Asg
 
 KKM_API kkm_status kkm_step(kkm_ctx* c, const int32_t* batch_idx, const int32_t* forced_assign,
                             int32_t* assign_out, float* dist_out, double* batch_obj_out) {
-  kkm_status st = check_usable(c);
+  kkm_status st = check_ready(c);
   if (st != KKM_OK) return st;
   if (c->s.tau == 0 && !c->tab && c->iteration > c->max_iters)
     return fail(c, KKM_ESTATE, "untruncated run: max_iters iterations already done");
@@ -730,60 +743,69 @@ KKM_API kkm_status kkm_step(kkm_ctx* c, const int32_t* batch_idx, const int32_t*
     if (st != KKM_OK) return st;
     ++c->eager_steps;
   }
-  c->launches += 1 + step_kernels(c) + (timed ? c->timing_reps - (split_window(c) || c->tab ? 1 : 0) : 0);
-  c->fin_pending = !c->tab;
+  c->launches += chain_kernels(c, 1, true) + (timed ? c->timing_reps - 1 : 0);
+  c->own_work = true;
   ++c->iteration;
   return KKM_OK;
 }
 
 KKM_API kkm_status kkm_flush(kkm_ctx* c) { return check_ready(c); }
 
-// Iterations the kkm_steps graph holds. Within it consecutive steps meet
+// Most iterations a kkm_steps graph holds. Within it consecutive steps meet
 // through programmatic dependent launch, as the kernels of one step do;
 // between two graph launches they do not.
 constexpr int STEPS_PER_GRAPH = 16;
 
 KKM_API kkm_status kkm_steps(kkm_ctx* c, int64_t n) {
-  kkm_status st = check_usable(c);
+  kkm_status st = check_ready(c);
   if (st != KKM_OK) return st;
   if (n < 0) return fail(c, KKM_EINVAL, "n must be >= 0");
   if (c->s.tau == 0 && !c->tab && c->iteration - 1 + n > c->max_iters)
     return fail(c, KKM_ESTATE, "untruncated run: n steps would pass max_iters");
   const bool timed = c->timing && c->ev_used < (int64_t)c->ev.size() / 2;
   int64_t left = n;
-  if (c->graph_on && !timed) {
-    if (c->eager_steps == 0 && left > 0) {   // the first step runs eagerly, as kkm_step's does
-      st = kkm_step(c, nullptr, nullptr, nullptr, nullptr, nullptr);
+  if (c->graph_on && !timed && c->eager_steps == 0 && left > 0) {   // the first step runs eagerly, as kkm_step's does
+    st = kkm_step(c, nullptr, nullptr, nullptr, nullptr, nullptr);
+    if (st != KKM_OK) return st;
+    --left;
+  }
+  const auto none = [](int) -> int32_t* { return nullptr; };
+  const auto no_obj = [](int) -> double* { return nullptr; };
+  for (bool first = true; left > 0 && !timed; first = false) {
+    const int m = (int)std::min<int64_t>(STEPS_PER_GRAPH, left);
+    const bool last = left == m;
+    if (c->graph_on) {
+      cudaGraphExec_t& ge = c->gexec_run[4 * m + (first ? 2 : 0) + (last ? 1 : 0)];
+      if (!ge) {
+        if (!c->cap_stream)
+          KKM_CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
+        KKM_CU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
+        st = enqueue_steps(c, c->cap_stream, m, first, last, none, none, no_obj);
+        cudaGraph_t g = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
+        if (st != KKM_OK) {
+          if (g) cudaGraphDestroy(g);
+          return st;
+        }
+        if (e != cudaSuccess) return cuda_fail(c, e, "end capture");
+        const cudaError_t ei = cudaGraphInstantiate(&ge, g, 0);
+        cudaGraphDestroy(g);
+        if (ei != cudaSuccess) {
+          ge = nullptr;
+          return cuda_fail(c, ei, "graph instantiate");
+        }
+      }
+      KKM_CU(cudaGraphLaunch(ge, c->stream), "graph launch");
+    } else {
+      st = enqueue_steps(c, c->stream, m, first, last, none, none, no_obj);
       if (st != KKM_OK) return st;
-      --left;
+      c->eager_steps += m;
     }
-    if (left >= STEPS_PER_GRAPH && !c->gexec_multi) {
-      if (!c->cap_stream)
-        KKM_CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
-      KKM_CU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-      st = enqueue_steps(
-          c, c->cap_stream, STEPS_PER_GRAPH, [](int) -> const int32_t* { return nullptr; },
-          [](int) -> int32_t* { return nullptr; }, [](int) -> double* { return nullptr; });
-      cudaGraph_t g = nullptr;
-      const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
-      if (st != KKM_OK) {
-        if (g) cudaGraphDestroy(g);
-        return st;
-      }
-      if (e != cudaSuccess) return cuda_fail(c, e, "end capture");
-      const cudaError_t ei = cudaGraphInstantiate(&c->gexec_multi, g, 0);
-      cudaGraphDestroy(g);
-      if (ei != cudaSuccess) {
-        c->gexec_multi = nullptr;
-        return cuda_fail(c, ei, "graph instantiate");
-      }
-    }
-    for (; left >= STEPS_PER_GRAPH; left -= STEPS_PER_GRAPH) {
-      KKM_CU(cudaGraphLaunch(c->gexec_multi, c->stream), "graph launch");
-      c->launches += STEPS_PER_GRAPH * step_kernels(c) + (c->tab ? STEPS_PER_GRAPH : 1);
-      c->iteration += STEPS_PER_GRAPH;
-      c->fin_pending = !c->tab;
-    }
+    c->launches += chain_kernels(c, m, last);
+    c->iteration += m;
+    c->fin_pending = !c->tab && !split_window(c) && !last;
+    c->own_work = true;
+    left -= m;
   }
   for (; left > 0; --left) {
     st = kkm_step(c, nullptr, nullptr, nullptr, nullptr, nullptr);
@@ -801,7 +823,7 @@ KKM_API kkm_status kkm_graph_enable(kkm_ctx* c, int32_t enable) {
 
 KKM_API kkm_status kkm_step_host(kkm_ctx* c, const int32_t* batch_idx, int32_t* assign_out,
                                  double* batch_obj_out) {
-  kkm_status st = check_usable(c);
+  kkm_status st = check_ready(c);
   if (st != KKM_OK) return st;
   const int b = c->s.b;
   if (c->host_pending) {            // an earlier call did not get to wait: its kernels may still read the area
@@ -838,20 +860,21 @@ double* q_obj(char* slot, size_t nb4, int i) {
 }
 
 // Queues m steps reading slot q (indices from it when host_idx, else the
-// built-in sampler) and writing their results there.
-kkm_status q_enqueue(kkm_ctx* c, int q, int m, bool host_idx) {
+// built-in sampler) and writing their results there. first, last: the chunk's
+// place in its call.
+kkm_status q_enqueue(kkm_ctx* c, int q, int m, bool host_idx, bool first, bool last) {
   const size_t nb4 = c->q_nb4;
   char* d = c->d_qslot[q];
   auto idx = [=](int i) -> const int32_t* { return host_idx ? q_idx(d, nb4, i) : nullptr; };
   auto asg = [=](int i) { return q_asg(d, nb4, i); };
   auto obj = [=](int i) { return q_obj(d, nb4, i); };
   if (c->graph_on && m == HOST_CHUNK) {
-    cudaGraphExec_t& ge = c->gexec_q[q][host_idx ? 1 : 0];
+    cudaGraphExec_t& ge = c->gexec_q[q][(host_idx ? 1 : 0) + (first ? 2 : 0) + (last ? 4 : 0)];
     if (!ge) {
       if (!c->cap_stream)
         KKM_CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
       KKM_CU(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-      const kkm_status st = enqueue_steps(c, c->cap_stream, HOST_CHUNK, idx, asg, obj);
+      const kkm_status st = enqueue_steps(c, c->cap_stream, HOST_CHUNK, first, last, idx, asg, obj);
       cudaGraph_t g = nullptr;
       const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
       if (st != KKM_OK) {
@@ -868,20 +891,21 @@ kkm_status q_enqueue(kkm_ctx* c, int q, int m, bool host_idx) {
     }
     KKM_CU(cudaGraphLaunch(ge, c->stream), "graph launch");
   } else {
-    const kkm_status st = enqueue_steps(c, c->stream, m, idx, asg, obj);
+    const kkm_status st = enqueue_steps(c, c->stream, m, first, last, idx, asg, obj);
     if (st != KKM_OK) return st;
     c->eager_steps += m;
   }
-  c->launches += m * step_kernels(c) + (c->tab ? m : 1);
+  c->launches += chain_kernels(c, m, last);
   c->iteration += m;
-  c->fin_pending = !c->tab;
+  c->fin_pending = !c->tab && !split_window(c) && !last;
+  c->own_work = true;
   return KKM_OK;
 }
 }  // namespace
 
 KKM_API kkm_status kkm_steps_host(kkm_ctx* c, int64_t n, const int32_t* batch_idx, int32_t* assign_out,
                                   double* batch_obj_out) {
-  kkm_status st = check_usable(c);
+  kkm_status st = check_ready(c);
   if (st != KKM_OK) return st;
   if (n < 0) return fail(c, KKM_EINVAL, "n must be >= 0");
   if (c->s.tau == 0 && !c->tab && c->iteration - 1 + n > c->max_iters)
@@ -922,13 +946,14 @@ KKM_API kkm_status kkm_steps_host(kkm_ctx* c, int64_t n, const int32_t* batch_id
     return s;
   };
   int q = 0;
+  const int64_t j0 = j;
   while (j < n) {
     const int m = (int)std::min<int64_t>(HOST_CHUNK, n - j);
     st = drain(q);
     if (st != KKM_OK) return abort_with(st);
     if (batch_idx)
       for (int i = 0; i < m; ++i) std::memcpy(q_idx(c->h_qslot[q], c->q_nb4, i), batch_idx + (j + i) * b, row);
-    st = q_enqueue(c, q, m, batch_idx != nullptr);
+    st = q_enqueue(c, q, m, batch_idx != nullptr, j == j0, j + m == n);
     if (st != KKM_OK) return abort_with(st);
     const cudaError_t e = cudaEventRecord(c->qdone[q], c->stream);
     if (e != cudaSuccess) return abort_with(cuda_fail(c, e, "chunk event"));
@@ -1081,8 +1106,6 @@ KKM_API kkm_status kkm_step_eval(kkm_ctx* c, const int32_t* batch_idx, double* o
   if (st != KKM_OK) return st;
   if (!obj_before_dev || !obj_after_dev) return fail(c, KKM_EINVAL, "obj_before_dev and obj_after_dev are required");
   st = kkm_step(c, batch_idx, nullptr, nullptr, nullptr, obj_before_dev);
-  if (st != KKM_OK) return st;
-  st = flush(c);                     // the step's weight update
   if (st != KKM_OK) return st;
   // f_{B_i}(C_{i+1}): the distance pass and argmin again on the same batch
   // rows, against the windows, weights and norms the step just wrote
@@ -1734,9 +1757,10 @@ KKM_API kkm_status kkm_group_step(kkm_group* g) {
     if (c->poisoned) return gfail(g, KKM_ESTATE, "a run is poisoned");
     if (c->s.tau == 0 && !c->tab && c->iteration > c->max_iters)
       return gfail(g, KKM_ESTATE, "an untruncated run has done max_iters iterations");
-    if (c->fin_pending) {               // a kkm_step on the run since the last group step
+    if (c->own_work) {                  // the run stepped on its own stream since the last group step
       if (flush(c) != KKM_OK || cudaStreamSynchronize(c->stream) != cudaSuccess)
-        return gfail(g, KKM_ECUDA, "pending weight update of a run");
+        return gfail(g, KKM_ECUDA, "a run's own steps");
+      c->own_work = false;
     }
   }
   if (g->steps == 0) {

@@ -319,7 +319,7 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   KKM_LAUNCH_DEPENDENTS();
   __shared__ __align__(16) GramSmem<4> sm;
   __shared__ double red[4][NT / 32];
-  const int total = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
+  const int total = *s.nwpairs;
   // Norms are reported by the first warp, whose first four lanes wrote the sums.
   // Many items a block: a contiguous range each, so that its reports are few;
   // few: strided, so that a center's items spread over the chip. FP32, d = 64,

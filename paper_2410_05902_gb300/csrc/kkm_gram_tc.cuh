@@ -1204,7 +1204,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   Range rw{0, 0}, rd{0, 0};
   auto ranges = [&]() {
     int np = 0;
-    if constexpr (MODE != 0) np = norms && *s.fin_pending == 0 ? 0 : *s.nwpairs;
+    if constexpr (MODE != 0) np = *s.nwpairs;
     if constexpr (MODE != 1) T = *s.ntiles;
     total = MODE == 1 ? np : R * T;
     if (ovr.lo >= 0) {

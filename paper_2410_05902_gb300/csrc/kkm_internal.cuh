@@ -115,7 +115,7 @@ struct alignas(16) Dev {
   int32_t* yi;
   double* w64;
   float* w32;
-  float* wo32;       // FP32 weights before the pending update (k_update), for its window pass
+  float* wo32;       // FP32 weights before the last update (k_update), for its window pass
   double* wo64;      // the same in FP64 (FP32 form only, whose window pass reads FP64 weights)
   const float* wwin; // the weights the window pass reads: wo32, or w32 where the pass runs before the update
   const double* wwin64;   // FP32 form: wo64 or w64
@@ -165,7 +165,6 @@ struct alignas(16) Dev {
   int32_t* wdone;    // [win_segment_slots] finished items of each segment (k_sort_plan clears them)
   int32_t* cdone;    // [k] finished segments (k_sort_plan clears them)
   int64_t* gnext;    // [1] the iteration whose batch has been scored (its successor's batch may be gathered)
-  int32_t* fin_pending;   // [1] 1 while a step's window pass and center norms are still to run
   int64_t* stats;    // [3] steps, support rows, tiles
   double* obj;       // [1] last batch objective
   float* cmpart;     // [k][32] FP32 lane partials of sum_{x in B_j} <phi(x), C_j>
@@ -420,14 +419,13 @@ cudaError_t launch_argmin(const Dev& s, int rows, const int32_t* forced, int32_t
                           float* mind_out, float* dist_out, bool update, cudaStream_t st, double* obj_acc = nullptr,
                           bool obj_first = false);
 cudaError_t launch_sum(const double* a, int n, double* out, cudaStream_t st);   // sum of n doubles
-// set_pending: the step's window pass and norms run in the next step's distance pass (or a flush)
-cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st, bool set_pending = false);
+cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st);
 cudaError_t launch_move(const Dev& s, cudaStream_t st);
 // The row moves and the weight update in one launch; with next, the gather of
 // the following batch beside them, into next's batch buffers (next_idx: its
 // indices, or NULL for the built-in sampler).
 cudaError_t launch_update(const Dev& s, const Dev* next, const int32_t* next_idx, cudaStream_t st);
-// norms: a no-op unless fin_pending is set, and every center's norm follows its last item
+// norms: every center's norm follows its last item (after k_update)
 cudaError_t launch_wgram(const Dev& s, cudaStream_t st, bool norms = false);
 cudaError_t launch_finalize(const Dev& s, cudaStream_t st);
 // batch objective at fixed assignments and its adjoint (kkm_grad.cu): two
@@ -539,8 +537,8 @@ cudaError_t launch_dist_tc(const Dev& s, const void* maps, int rows, cudaStream_
 cudaError_t launch_wgram_tc(const Dev& s, const void* maps, cudaStream_t st, bool norms = false);
 // The distance pass on CTA pairs (streamed operands, s.tn 128 or 256).
 cudaError_t launch_dist_pair(const Dev& s, const void* maps, int rows, cudaStream_t st);
-// A step's distance pass with the window items of the pending update ahead of
-// it (none unless fin_pending is set) and their center norms; s.tn 128 or 256.
+// A step's distance pass with the window items of the update before it ahead
+// of it and their center norms; s.tn 128 or 256.
 cudaError_t launch_step_tc(const Dev& s, const void* maps, cudaStream_t st);
 
 }  // namespace kkm

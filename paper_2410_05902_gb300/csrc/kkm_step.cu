@@ -375,7 +375,7 @@ __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size,
 // alpha_i^j, <C_j, cm(B_j)>, and the per-center window plan: compaction,
 // block push, the drops of Eq. (1), C_1 retirement, and the tile pairs of the
 // norm-recurrence Gram pass.
-__device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, int set_pending) {
+__device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();   // the next kernel waits at its top (or only stages earlier steps' data)
   extern __shared__ __align__(16) unsigned char smem[];
@@ -600,7 +600,6 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, in
     s.stats[1] += s_rows;
     s.stats[2] += tiles_used;
     *s.iter += 1;
-    if (set_pending) *s.fin_pending = 1;
   }
   tiles_write(s, ex3[2], nt, thead, tsize, tot3[2], ex3[3], tot3[3],
               min(ptotal, s.max_pairs));   // its barrier also publishes base/tot
@@ -628,8 +627,8 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out, in
   }
 }
 
-__global__ void __launch_bounds__(1024) k_sort_plan(Dev s, double* obj_out, int set_pending) {
-  sort_plan_body(s, obj_out, set_pending);
+__global__ void __launch_bounds__(1024) k_sort_plan(Dev s, double* obj_out) {
+  sort_plan_body(s, obj_out);
 }
 
 // The append of the new blocks and the compaction of the windows that need
@@ -1353,7 +1352,7 @@ __global__ void __launch_bounds__(32 * AM_WARPS) k_group_argmin(GroupPhase g) {
 __global__ void __launch_bounds__(1024) k_group_sort_plan(GroupPhase g) {
   int local, nblk;
   const int r = group_run(g, local, nblk);
-  sort_plan_body(g.runs[r].s, nullptr, 0);
+  sort_plan_body(g.runs[r].s, nullptr);
 }
 
 __global__ void k_group_move(GroupPhase g) {
@@ -1621,12 +1620,12 @@ cudaError_t launch_sum(const double* a, int n, double* out, cudaStream_t st) {
 
 int sort_plan_smem(int k, int b) { return k * (int)sizeof(Plan) + 4 * k * 4 + b * (4 + 2 + 2 + 2) + 32 * k * 2; }
 
-cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st, bool set_pending) {
+cudaError_t launch_sort_plan(const Dev& s, double* obj_out, cudaStream_t st) {
   const int smem = sort_plan_smem(s.k, s.b);
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = smem_limit_once(k_sort_plan, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(k_sort_plan, dim3(1), dim3(1024), smem, st, s, obj_out, set_pending ? 1 : 0);
+  e = launch_pdl(k_sort_plan, dim3(1), dim3(1024), smem, st, s, obj_out);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

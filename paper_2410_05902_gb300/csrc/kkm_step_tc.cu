@@ -1,4 +1,4 @@
-// A step's tcgen05 launch: the window items of the pending update and the
+// A step's tcgen05 launch: the window items of the update before and the
 // distance items of the batch (mode 2 of kkm_gram_tc.cuh), in a translation
 // unit of its own so that the two sets of kernels compile in parallel.
 #include "kkm_gram_tc.cuh"

@@ -499,7 +499,7 @@ class KKM:
         kkm_sync(self.ctx)
 
     def flush(self):
-        """Queue the weight update the last step left pending (asynchronous)."""
+        """Queue what a failed call of several steps left pending (nothing otherwise; asynchronous)."""
         kkm_flush(self.ctx)
 
     def get_state(self) -> dict:
