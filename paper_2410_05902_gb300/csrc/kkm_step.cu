@@ -311,11 +311,17 @@ __device__ __forceinline__ void argmin_body(const Dev& s, int rows, const int32_
       const int j = j0 + u * AM_WARPS;
       if (j >= s.k) break;
       float i0 = v[u][0], i1 = v[u][1], i2 = v[u][2], i3 = v[u][3];
-      for (int t = 4; t < nt[u]; t += 4) {
-        i0 += part[(int64_t)(t0[u] + t) * ld];
-        if (t + 1 < nt[u]) i1 += part[(int64_t)(t0[u] + t + 1) * ld];
-        if (t + 2 < nt[u]) i2 += part[(int64_t)(t0[u] + t + 2) * ld];
-        if (t + 3 < nt[u]) i3 += part[(int64_t)(t0[u] + t + 3) * ld];
+      for (int t = 4; t < nt[u]; t += 16) {     // 16 loads in flight: a center may have dozens of tiles
+        float p[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) p[q] = t + q < nt[u] ? part[(int64_t)(t0[u] + t + q) * ld] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 16; q += 4) {
+          i0 += p[q];
+          i1 += p[q + 1];
+          i2 += p[q + 2];
+          i3 += p[q + 3];
+        }
       }
       const float inner = (i0 + i1) + (i2 + i3);
       const float dist = fmaf(-2.0f, inner, kxx + cn[u]);
