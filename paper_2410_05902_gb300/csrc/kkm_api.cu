@@ -402,7 +402,7 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
     const int64_t tile_bytes = kkm::tc_item_bytes(s, s.tn, false);
     // operand copies in units of about 470 cycles, at 64 bytes per clock and SM
     s.tile_floor = (int32_t)std::min<int64_t>(tile_bytes / (64 * 470), 4096);
-    s.win_work = (int32_t)std::max<int64_t>(22, std::min<int64_t>(kkm::tc_item_bytes(s, kkm::WPASS_TNV, true) / (64 * 470), 4096));
+    s.win_floor = (int32_t)std::min<int64_t>(kkm::tc_item_bytes(s, kkm::WPASS_TNV, true) / (64 * 470), 4096);
   }
   const int64_t TR = s.pair_rows, TC = s.pair_cols;   // window-pass tile
   s.max_tiles = tab ? (int32_t)(k + (b + s.tn - 1) / s.tn + 1)
@@ -422,7 +422,6 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
   // CTAs of a step's tcgen05 launch: one per SM, but never more than its items
   s.nsplit = (int32_t)std::min<int64_t>(std::min(s.num_sms, 1023),
                                         (int64_t)((b + 127) / 128) * s.max_tiles + s.max_pairs);
-  if (!c->use_tc) s.win_work = 1;
 
   const int esz = kkm::f32_rows(s.form) ? 4 : 2;
   cudaError_t e = cudaSuccess;

@@ -34,11 +34,11 @@
 // few of them as possible: its B tile, and its A tile only when the row tile
 // changes (the batch tile stays resident while consecutive items share it).
 //
-// Teams: with four accumulators (64- and 128-column tiles) each group is a
-// team and takes every fourth item whole; with two (256-column tiles) two
-// groups form a team, take every other item and split its columns, each
-// writing its own partial. Either way every waiter on a barrier sees each of
-// its phases in order. A run with fewer than NTEAM items per SM runs every
+// Teams: with four accumulators (64- and 128-column tiles, window items) each
+// group is a team and takes every fourth item whole; with two (256-column
+// tiles) two groups form a team, take every other item and split its columns,
+// each writing its own partial. Either way every waiter on a barrier sees each
+// of its phases in order. A run with fewer than NTEAM items per SM runs every
 // item on all four groups, each on a quarter of the columns, and the groups'
 // sums meet in shared memory (chosen per run, so that a run's results do not
 // depend on how a launch splits its items).
@@ -112,9 +112,10 @@ template <int TNV> struct Geo {
   static constexpr int NACC = 512 / TNV < 4 ? 512 / TNV : 4;
   static constexpr int NTEAM = NACC < NGRP ? NACC : NGRP;
   static constexpr int GPT = NGRP / NTEAM;
-  static constexpr int MS = TNV == 256 ? 4 : TNV == 128 ? 6 : 8;
+  static constexpr int MS = TNV == 256 ? 5 : TNV == 128 ? 6 : 8;
   static constexpr uint32_t TMEM_COLS = (uint32_t)(NACC * TNV);
 };
+using WG = Geo<WPASS_TNV>;                       // window items' accumulators and teams, whatever the distance tile
 constexpr uint32_t META_ARRIVALS = 33;           // 32 lanes' asynchronous arrivals + lane 0's release
 
 __device__ __forceinline__ void tma_load_2d(bool lead, void* dst, const CUtensorMap* map, uint64_t* bar, int x,
@@ -207,6 +208,8 @@ template <int TNV> struct Shared {
   uint32_t mark[STAGES];         // 1: the stage's item brings a new resident A tile
   uint64_t tfull[4];
   uint64_t tempty[4];
+  uint64_t wfull[4];             // the same for window items
+  uint64_t wempty[4];
   uint64_t mfull[8];
   uint64_t mempty[8];
   uint64_t mma_done;
@@ -220,7 +223,7 @@ template <int TNV> struct Shared {
   alignas(16) Dev gdev;          // run groups: the segment's run (a shared copy: no reloads after global stores)
   alignas(16) MetaSlot<TNV> ring[Geo<TNV>::MS];   // 16-byte asynchronous copies land here
   float red[2][NGRP][4][32];     // distance items, all-groups mode: row sums (item parity, group, quadrant, row)
-  float ex[4][3][TM];            // window items: the other groups' quarter sums (quarter, sum, row)
+  float ex[3][3][TM];            // window items: the other groups' quarter sums (quarter, sum, row)
   double wq[NGRP][2][4][4];      // window items: quadrant sums (team, parity, quadrant, sum)
 };
 
@@ -263,8 +266,8 @@ __device__ __forceinline__ void mbar_expect_tx(bool lead, uint64_t* b, uint32_t 
       : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+__device__ __forceinline__ void mbar_arrive(uint64_t* b, uint32_t count = 1) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* b, uint32_t parity) {
@@ -622,11 +625,9 @@ template <int TNV> struct Place {
   __device__ Place(int warp, int lane_, bool all_)
       : g((warp - 2) >> 2), q(warp & 3), team(g / GPT), h(g % GPT), lane(lane_), all(all_) {}
   __device__ bool mine(uint32_t local) const { return all || (int)(local % Geo<TNV>::NTEAM) == team; }
-  // all-groups mode: the groups that free the accumulator and the slot (4 GPT arrivals on each)
-  __device__ bool frees() const { return !all || g % QPP == 0; }
-  __device__ void arrive(uint64_t* b) const {
+  __device__ void arrive(uint64_t* b, uint32_t count = 1) const {
     __syncwarp();
-    if (lane == 0) mbar_arrive(b);
+    if (lane == 0) mbar_arrive(b, count);
   }
   // the accumulator's barrier: the even CTA's, where the pair's MMAs are issued
   template <bool PAIR> __device__ void arrive_acc(uint64_t* b) const {
@@ -639,9 +640,6 @@ template <int TNV> struct Place {
   }
   __device__ void sync_all() const { asm volatile("bar.sync 1, %0;" ::"n"(32 * NEPI) : "memory"); }
   __device__ void sync_group() const { asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory"); }
-  __device__ void sync_team() const {
-    if constexpr (GPT == 2) asm volatile("bar.sync %0, 256;" ::"r"(6 + team) : "memory");
-  }
 };
 
 // One distance-pass item: group h of the team takes the columns [h TNV / GPT,
@@ -653,8 +651,8 @@ template <int TNV> struct Place {
 // chunk is in registers and the metadata slot once its arithmetic is done.
 template <int KIND, int TNV, bool PAIR>
 __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem, const Place<TNV>& pl,
-                                          uint32_t local, int tile, int row0, int rows, bool dead) {
-  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT, QPP = Place<TNV>::QPP;
+                                          uint32_t local, uint32_t buf, int tile, int row0, int rows, bool dead) {
+  constexpr int MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT, QPP = Place<TNV>::QPP;
   const int g = pl.g, q = pl.q, lane = pl.lane;
   const bool all = pl.all;
   const int g4 = lane >> 2, us = lane & 3, c2 = 2 * us;
@@ -667,7 +665,7 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
   const int cbeg = all ? g * ncols : pl.h * ncols;
   const int ph = all ? g / QPP : pl.h;          // this group's partial
   const bool lead = !all || g % QPP == 0;       // writes the partial
-  const uint32_t buf = local % NACC, ms = local % MS;
+  const uint32_t ms = local % MS;
   const MetaSlot<TNV>& m = sh.ring[ms];
   float f = 0.0f;
   if (!dead) {
@@ -767,14 +765,19 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
 // The sums of an item do not depend on how its 128 columns are dealt to the
 // groups: the columns are four quarters of 32, a row's FP32 sum of each quarter
 // is taken by one thread quad, and the quarters are added in order, as pairs.
-// A team of two groups takes two quarters each, a team of one takes all four,
-// and in the all-groups mode each group takes one; the lead group gets the
-// others' quarter sums through shared memory. `turn` counts the team's items
-// (buffer parity).
+// A group alone takes all four; in the all-groups mode each group takes one, and
+// the first gets the others' quarter sums through shared memory. `turn` counts
+// the group's items (buffer parity).
+// Window items have four accumulators and four teams whatever the launch's
+// distance tile, as in a launch of their own; beside 256-column tiles two teams
+// of two groups met twice an item to exchange their column sums.
 template <int KIND, int TNV>
-__device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem, const Place<TNV>& pl,
-                                            uint32_t local, uint32_t turn, int item, bool norms, bool dead) {
-  constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS, GPT = Geo<TNV>::GPT;
+__device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem,
+                                            const Place<WPASS_TNV>& pl, uint32_t local, uint32_t turn, int item,
+                                            bool norms, bool dead) {
+  constexpr int MS = Geo<TNV>::MS;
+  constexpr uint32_t SLOT_ARRIVALS = Geo<TNV>::GPT;   // a warp's share of a metadata slot's release
+  static_assert(WG::NACC == 4 && WG::GPT == 1 && WPASS_TNV == 128, "four quarters, a group each or one group's");
   using WS = WindowSum<KIND>;
   using Sum = typename WS::T;
   static_assert(sizeof(Sum) == sizeof(double), "a shared-memory slot holds one sum");
@@ -785,9 +788,9 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
   const float2 C2 = make_float2(-2.0f * negc, -2.0f * negc);
   const float coef0 = (float)s.coef0;
   const int degree = s.degree;
-  const uint32_t buf = local % NACC, ms = local % MS;
+  const uint32_t buf = local % WG::NACC, ms = local % MS;
   const MetaSlot<TNV>& m = sh.ring[ms];
-  const int nq = all ? 1 : NGRP / GPT, qlo = all ? pl.g : pl.h * nq;   // this group's quarters
+  const int nq = all ? 1 : NGRP, qlo = all ? pl.g : 0;     // this group's quarters
   const bool lead = qlo == 0;
   const int slot = all ? 0 : pl.team;
   Sum rA = WS::zero(), rB = WS::zero(), rE = WS::zero();   // this lane's row rq: W, D and B columns
@@ -816,7 +819,7 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
       const int r = q * 32 + rq;
       wrow = r >= dsc.rlo && r < dsc.rhi ? (kind == 0 ? m.row[2][r] : 1.0f) : 0.0f;
     }
-    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * TNV;
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * WPASS_TNV;
     constexpr int NB = 2, CW = 8 * NB;
     for (int t = 0; t < nq; ++t) {
       const int cb = (qlo + t) * 32;
@@ -872,33 +875,28 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
           for (int u = 0; u < 4; ++u) f4[u] = quad_sum(acc[u].x + acc[u].y);
           v = pick4(f4, us);
         }
-        if (!lead) sh.ex[all ? qlo - 1 : slot * 2 + t][cls][q * 32 + rq] = v;
+        if (!lead) sh.ex[qlo - 1][cls][q * 32 + rq] = v;
         else add_class(cls, v);
       }
     }
     if (!all) {                                  // the accumulator and the slot are free again
       tc_fence_before();
-      pl.arrive(&sh.tempty[buf]);
-      pl.arrive(&sh.mempty[ms]);
+      pl.arrive(&sh.wempty[buf]);
+      pl.arrive(&sh.mempty[ms], SLOT_ARRIVALS);
     }
   }
   if (all) {
     tc_fence_before();
     pl.sync_all();
-    if (pl.frees() && !dead) {
-      pl.arrive(&sh.tempty[buf]);
-      pl.arrive(&sh.mempty[ms]);
+    if (lead && !dead) {
+      pl.arrive(&sh.wempty[buf]);
+      pl.arrive(&sh.mempty[ms], SLOT_ARRIVALS);
     }
-  } else {
-    pl.sync_team();
+    if (lead && rows_here)
+      for (int o = 1; o < NGRP; ++o)
+        for (int cls = 0; cls < 3; ++cls) add_class(cls, sh.ex[o - 1][cls][q * 32 + rq]);
+    pl.sync_all();                               // the exchange buffer may be written again
   }
-  if (lead && rows_here)
-    for (int o = nq; o < NGRP; ++o) {
-      const float (*ex)[TM] = sh.ex[all ? o - 1 : slot * 2 + o - nq];
-      for (int cls = 0; cls < 3; ++cls) add_class(cls, ex[cls][q * 32 + rq]);
-    }
-  if (all) pl.sync_all();                        // the exchange buffer may be written again
-  else pl.sync_team();
   if (!lead) return;
   if (rows_here) {
     rE = WS::rows(rE, wrow);
@@ -938,18 +936,18 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
 // then distance items [rd.lo, rd.hi) (MODE 0, 2).
 template <int KIND, int MODE, int TNV, bool PAIR>
 __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t tmem, Range rw, Range rd, int T,
-                                         int rows, int warp, int lane, bool all, bool norms, int rank) {
+                                         int rows, int warp, int lane, bool all_w, bool all_d, bool norms,
+                                         int rank) {
   constexpr int NACC = Geo<TNV>::NACC, MS = Geo<TNV>::MS;
-  const Place<TNV> pl(warp, lane, all);
   // part[] must hold GPT partials per tile, as the host sized it (Dev::ppt)
   bool dead = MODE != 1 && s.ppt != Geo<TNV>::GPT;
   if (dead && lane == 0 && warp == 2) atomicOr(s.status, ST_CAPACITY);
   const int nw = MODE == 0 ? 0 : rw.hi - rw.lo;
   const int n = nw + (MODE == 1 ? 0 : rd.hi - rd.lo);
-  auto wait = [&](uint32_t local) {
-    const uint32_t buf = local % NACC, ms = local % MS;
-    const bool ok = dead || (mbar_wait(&sh.mfull[ms], (local / MS) & 1u) &&
-                             mbar_wait(&sh.tfull[buf], (local / NACC) & 1u));
+  // item `local`, whose accumulator's barrier is in its phase `turn`
+  auto wait = [&](uint32_t local, uint64_t* full, uint32_t turn) {
+    const uint32_t ms = local % MS;
+    const bool ok = dead || (mbar_wait(&sh.mfull[ms], (local / MS) & 1u) && mbar_wait(full, turn & 1u));
     if (__any_sync(0xffffffffu, !ok)) {
       if (lane == 0 && !dead) atomicOr(s.status, ST_TIMEOUT);
       dead = true;
@@ -958,20 +956,23 @@ __device__ __forceinline__ void epilogue(const Dev& s, Shared<TNV>& sh, uint32_t
   };
   uint32_t local = 0;
   if constexpr (MODE != 0) {
+    const Place<WPASS_TNV> pl(warp, lane, all_w);
     uint32_t turn = 0;                           // window items this team has taken
     for (; (int)local < nw; ++local) {
       if (!pl.mine(local)) continue;
-      wait(local);
+      wait(local, &sh.wfull[local % WG::NACC], local / WG::NACC);
       window_item<KIND, TNV>(s, sh, tmem, pl, local, turn++, rw.lo + (int)local, norms, dead);
     }
   }
   if constexpr (MODE != 1) {
+    const Place<TNV> pl(warp, lane, all_d);
     for (; (int)local < n; ++local) {
-      if (!pl.mine(local)) continue;
-      wait(local);
-      const int item = rd.lo + (int)local - nw;
-      dist_item<KIND, TNV, PAIR>(s, sh, tmem, pl, local, item % T, (PAIR ? 2 * (item / T) + rank : item / T) * TM,
-                                 rows, dead);
+      const uint32_t l = local - (uint32_t)nw, buf = l % NACC;
+      if (!pl.mine(l)) continue;
+      wait(local, &sh.tfull[buf], l / NACC);
+      const int item = rd.lo + (int)l;
+      dist_item<KIND, TNV, PAIR>(s, sh, tmem, pl, local, buf, item % T,
+                                 (PAIR ? 2 * (item / T) + rank : item / T) * TM, rows, dead);
     }
   }
 }
@@ -1034,12 +1035,13 @@ __device__ __forceinline__ Range my_range(int total, int cta, int ncta) {
 
 // MODE 0: distance pass (A = batch tile, B = support tile, one FP32 partial per row).
 // MODE 1: window pass (A and B = support rows of one center, four FP64 sums per item).
-// MODE 2: both, the window items of the previous step's update first: they are
-//         a few dozen rows each and by themselves leave the chip waiting on
-//         their latency, while as a few more items per CTA they cost their work.
-//         With the window pass and the weight update as launches of their own
-//         16 iterations and a scoring call took 1307 us on the 1e6 x 128 workload
-//         (k = 100, b = 4096) and 468 us at 2000 x 16 (b = 256), now 1266 and 407.
+// MODE 2: both, every CTA's share of the previous step's window items first. An
+//         evenly split batch has a few hundred of a few dozen rows each, which
+//         by themselves leave the chip waiting on their latency; as one or two
+//         more items per CTA they cost their work. With the window pass and the
+//         weight update as launches of their own 16 iterations and a scoring call
+//         took 1307 us on evenly split batches of 1e6 x 128 (k = 100, b = 4096)
+//         and 468 us at 2000 x 16 (b = 256), now 1266 and 407.
 // norms (MODE 1, 2): the norm warp carries ||C_j||^2 once a center's items are done.
 //
 // Both passes only sum over columns, so a tile can be split along its columns
@@ -1110,6 +1112,10 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
         mbar_inval(&sh.nfull[i]);
         mbar_inval(&sh.nempty[i]);
       }
+      for (int i = 0; i < WG::NACC && MODE != 0; ++i) {
+        mbar_inval(&sh.wfull[i]);
+        mbar_inval(&sh.wempty[i]);
+      }
       mbar_inval(&sh.mma_done);
     }
     // every stage's pair, not only the layout's L.nst: a later segment may use more
@@ -1122,6 +1128,10 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     for (int i = 0; i < NACC; ++i) {
       mbar_init(&sh.tfull[i], 1);
       mbar_init(&sh.tempty[i], (PAIR ? 2 : 1) * 4 * Geo<TNV>::GPT);   // the warps of one team (of both CTAs)
+    }
+    for (int i = 0; i < WG::NACC && MODE != 0; ++i) {
+      mbar_init(&sh.wfull[i], 1);
+      mbar_init(&sh.wempty[i], 4);               // the warps of one group
     }
     for (int i = 0; i < MS; ++i) {
       mbar_init(&sh.mfull[i], META_ARRIVALS);
@@ -1200,13 +1210,14 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   // nor the plans: the batch gather, the row moves or this pass itself) the
   // lists are read, and the descriptors of the first 32 items fetched, one per
   // lane, before the grid-dependency wait.
-  int T = 1, total = 0;
+  int T = 1, total = 0, np = 0;                  // support tiles, distance items, window items
   Range rw{0, 0}, rd{0, 0};
   auto ranges = [&]() {
-    int np = 0;
     if constexpr (MODE != 0) np = *s.nwpairs;
-    if constexpr (MODE != 1) T = *s.ntiles;
-    total = MODE == 1 ? np : R * T;
+    if constexpr (MODE != 1) {
+      T = *s.ntiles;
+      total = R * T;
+    }
     if (ovr.lo >= 0) {
       (MODE == 1 ? rw : rd) = ovr;
     } else if (MODE == 2 && np > 0 && ncta == s.nsplit) {
@@ -1248,11 +1259,12 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   KKM_LAUNCH_DEPENDENTS();   // the next kernel may set itself up; it waits before reading our output
   if (!desc_pre) ranges();
   const int nw = rw.hi - rw.lo, n = nw + rd.hi - rd.lo;
-  // All epilogue groups on each item (instead of a team per item) when the
-  // run has fewer than NTEAM items per SM. The choice depends on the run
+  // All epilogue groups on each item (instead of a team per item) when the run
+  // has fewer than NTEAM distance items per SM. The choice depends on the run
   // alone, never on how a launch splits its items, so an item's sums come out
-  // the same in a run's own launch and in a run group's.
-  const bool all_groups = total < Geo<TNV>::NTEAM * s.num_sms;
+  // the same in a run's own launch and in a run group's. (A window item's do
+  // either way.)
+  const bool all_d = total < Geo<TNV>::NTEAM * s.num_sms, all_w = np < WG::NTEAM * s.num_sms;
 
   if (warp == 0) {
     // ------------------------------------------------- operand producer (one warp)
@@ -1427,14 +1439,23 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     for (int local = 0; local < n && ok && !PAIR; ++local) {
       if ((local & 31) == 0 && !(local == 0 && desc_pre)) fetch_desc(local);
       const int wd = __shfl_sync(0xffffffffu, pd.tnew, local & 31);
-      const uint32_t ncol = live_cols(MODE != 0 && local < nw, wd);
+      const bool win = MODE != 0 && local < nw;
+      const uint32_t ncol = live_cols(win, wd);
       const uint32_t id = idesc<OP>(ncol);
       const int bt = slice_bytes(ncol);
-      const uint32_t buf = local % NACC, bph = ((uint32_t)local / NACC) & 1u;
-      ok = warp_wait(&sh.tempty[buf], bph ^ 1u);
+      const uint32_t l = win ? local : local - nw, nacc = win ? WG::NACC : NACC, buf = l % nacc;
+      uint64_t* const full = win ? &sh.wfull[buf] : &sh.tfull[buf];
+      const uint32_t d = tmem + buf * (win ? WPASS_TNV : TNV);
+      // the window items whose accumulators this one's first use covers
+      if (MODE == 2 && !win && l < (uint32_t)NACC)
+        for (int wb = (int)buf * (TNV / WPASS_TNV); wb < (int)(buf + 1) * (TNV / WPASS_TNV) && ok; ++wb) {
+          const int uses = nw > wb ? (nw - wb + WG::NACC - 1) / WG::NACC : 0;
+          if (uses > 0) ok = warp_wait(&sh.wempty[wb], (uint32_t)(uses - 1) & 1u);
+        }
+      if (!ok) break;
+      ok = warp_wait(win ? &sh.wempty[buf] : &sh.tempty[buf], ((l / nacc) & 1u) ^ 1u);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t d = tmem + buf * TNV;
       if (L.res) {
         const int st = it % L.nst;
         ok = warp_wait(&sh.full[st], (it / L.nst) & 1u);
@@ -1466,7 +1487,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
         }
         if (!ok) break;
       }
-      mma_commit(lead, &sh.tfull[buf]);
+      mma_commit(lead, full);
     }
     if (rank == 0) {                             // a pair's MMAs are all the even CTA's
       mma_commit<PAIR>(lead, &sh.mma_done);
@@ -1474,7 +1495,7 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
     }
     if (lead && !ok) atomicOr(s.status, ST_TIMEOUT);
   } else if (warp < MWARP) {
-    epilogue<KIND, MODE, TNV, PAIR>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_groups, norms, rank);
+    epilogue<KIND, MODE, TNV, PAIR>(s, sh, tmem, rw, rd, T, rows, warp, lane, all_w, all_d, norms, rank);
   } else if constexpr (MODE != 0) {
     if (norms) norm_warp<TNV>(s, sh, rw.lo, nw, lane);
   }

@@ -148,7 +148,7 @@ struct alignas(16) Dev {
   int2* split;       // [nsplit + 1] first window item and first distance item of each CTA of a step's launch
   int32_t nsplit;    // its CTAs
   int32_t tile_floor;  // least work of a tile: its operand copies (see tile_work)
-  int32_t win_work;    // work of a window-pass item, on the same scale
+  int32_t win_floor;   // least work of a window item (see window_work)
   int32_t* tile_first; // [k]
   int32_t* tile_cnt;   // [k]
   float* part;       // [max_tiles * ppt * bpad] per-tile weighted kernel sums (ppt partials per tile)
@@ -227,6 +227,17 @@ inline cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, si
 __host__ __device__ inline int tile_work(int ncols, int tn, int floor_) {
   const int half = tn == 256 ? 128 : tn;
   const int w = 5 + ((ncols < half ? ncols : half) + 15) / 16;
+  return w > floor_ ? w : floor_;
+}
+
+// Work of a window item beside tiles of tn rows, on the same scale: a 128 x 128
+// item takes a CTA about 4380 cycles where a full 256-row distance tile takes
+// 3690 (8192 x 64, BF16), narrow ones hardly less (weights by their columns made
+// the 1e6 x 128 workload 3 to 5 % slower), and all of them at least their
+// operand copies. few: the launch has so few items that all epilogue groups
+// work on each; then its reductions weigh most.
+__host__ __device__ inline int window_work(int tn, bool few, int floor_) {
+  const int w = few ? 22 : tn == 256 ? 15 : 30;
   return w > floor_ ? w : floor_;
 }
 

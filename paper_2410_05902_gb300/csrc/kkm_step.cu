@@ -375,7 +375,8 @@ __global__ void __launch_bounds__(32 * AM_WARPS) k_argmin(Dev s, int rows, const
 }
 
 __device__ int tile_count(const Dev& s, int& head, int& size, int& work);
-__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total, int before, int work, int nwin);
+__device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total, int before, int work,
+                            int nwin, int wwork);
 
 // Single CTA of 1024 threads. Stable counting sort of the batch by center,
 // alpha_i^j, <C_j, cm(B_j)>, and the per-center window plan: compaction,
@@ -581,6 +582,8 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out) {
     thead = P.head_new;
     tsize = P.tail_new - P.head_new;
   }
+  // few distance items (the next step's are about as many as this one's)
+  const bool few = (int64_t)((b + 127) / 128) * tiles_used < (s.tn == 256 ? 2 : 4) * s.num_sms;
   // one scan for the compaction offsets, the window-pass tiles and the next
   // step's distance tiles (the distance pass and argmin of this step have
   // already consumed the current tile list)
@@ -608,7 +611,7 @@ __device__ __forceinline__ void sort_plan_body(const Dev& s, double* obj_out) {
     *s.iter += 1;
   }
   tiles_write(s, ex3[2], nt, thead, tsize, tot3[2], ex3[3], tot3[3],
-              min(ptotal, s.max_pairs));   // its barrier also publishes base/tot
+              min(ptotal, s.max_pairs), window_work(s.tn, few, s.win_floor));   // its barrier also publishes base/tot
   // where k_move puts each sorted batch row: after the window's tail (after
   // the compaction, when there is one), in sorted order
   for (int r = tid; r < b; r += 1024) {
@@ -796,11 +799,18 @@ __device__ int tile_count(const Dev& s, int& head, int& size, int& work) {
 // Writes the tile list given each center's first tile and count (exclusive
 // scan over centers, total) and the work before it: tile_first/tile_cnt,
 // ntiles, and one Tile per thread, its center found by a binary search over
-// the first tiles. Then the split of the next step's launch: nwin window items
-// of win_work each and the R x total distance items on one line of work, of
-// which every CTA takes an equal stretch (the items that start in it).
+// the first tiles. Then the split of the next step's launch over its CTAs: each
+// takes its share of the nwin window items (wwork each) first and the rest of
+// its share of all work in distance items, so that window items end early in
+// every CTA and the norms that the argmin waits for are carried beside the
+// distance items. With all window items ahead of all distance items on one line
+// of work a third of the CTAs held nothing else and ended with the launch. A
+// step in BF16 then and now: 90 % of 8192 rows in one of 10 centers 261 and 213
+// us, half of 4096 in one of 100 92 and 80; the 1e6 x 128 workload 91.8 and 81.0.
+// Where the distance items are less than a window item per CTA that line of
+// work remains.
 __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size, int total, int before, int work,
-                            int nwin) {
+                            int nwin, int wwork) {
   __shared__ int t_first[1024], t_nt[1024], t_head[1024], t_size[1024], t_before[1024];
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -829,8 +839,11 @@ __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size,
     }
   }
   if (tid <= s.nsplit) {                         // nsplit <= 1023
-    const int64_t R = (s.b + 127) / 128, ww = (int64_t)nwin * s.win_work;
-    const int64_t p = (ww + R * work) * tid / s.nsplit, d = p > ww ? p - ww : 0;
+    const int64_t R = (s.b + 127) / 128, G = s.nsplit, ww = (int64_t)nwin * wwork;
+    const int64_t p = (ww + R * work) * tid / G;          // this CTA's start on the line of all work
+    const bool dealt = R * work >= G * (wwork + 2);       // no CTA has more in window items than its share of work
+    const int64_t witem = dealt ? (int64_t)nwin * tid / G : min((p + wwork - 1) / wwork, (int64_t)nwin);
+    const int64_t d = dealt ? p - witem * wwork : max(p - ww, (int64_t)0);
     const int64_t r = work > 0 ? d / work : R;
     int64_t item = R * lim;
     if (r < R) {
@@ -842,7 +855,7 @@ __device__ void tiles_write(const Dev& s, int first, int nt, int head, int size,
       }
       item = r * lim + min(t, lim);
     }
-    s.split[tid] = make_int2(p >= ww ? nwin : (int)((p + s.win_work - 1) / s.win_work), (int)item);
+    s.split[tid] = make_int2((int)witem, (int)item);
   }
 }
 
@@ -852,7 +865,7 @@ __device__ void build_tiles_block(const Dev& s, int head, int size) {
   const int v[2] = {nt, work};
   int ex[2], tot[2];
   block_exclusive_scans_1024(v, ex, tot);
-  tiles_write(s, ex[0], nt, head, size, tot[0], ex[1], tot[1], 0);
+  tiles_write(s, ex[0], nt, head, size, tot[0], ex[1], tot[1], 0, 1);
 }
 
 __device__ void build_tiles_block(const Dev& s) {
