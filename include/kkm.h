@@ -509,12 +509,14 @@ const char* kkm_noalloc_last_error(void);
 /* kkm_probe_bounded_wait -- the failure-detection path of the tcgen05 passes
  * on the current device. The paper has no counterpart. One thread waits on a
  * shared-memory mbarrier (the kind every role of the passes waits on) with the
- * passes' bounded wait, limited to limit_ns (1e3 .. 5e9). With arrive = 0
- * nothing arrives, so the wait runs out and the call returns KKM_ETIMEOUT, as
- * a step whose pass gave up reports through the context's status; with
- * arrive = 1 the thread arrives first and the call returns KKM_OK. Allocates
- * and frees one int of device memory and synchronises the stream. KKM_EINVAL
- * for arguments out of range (checked before any CUDA call). */
+ * passes' bounded wait, limited to limit_ns (1e3 .. 5e9), and then hands a value
+ * over through a slot as the passes' epilogue does. With arrive = 0 nothing
+ * arrives, so the wait runs out, the hand-over leaves the slot and its reader's
+ * barrier alone, and the call returns KKM_ETIMEOUT, as a step whose pass gave up
+ * reports through the context's status; with arrive = 1 the thread arrives first
+ * and the call returns KKM_OK. KKM_ESTATE if either did something else.
+ * Allocates and frees four ints of device memory and synchronises the stream.
+ * KKM_EINVAL for arguments out of range (checked before any CUDA call). */
 kkm_status kkm_probe_bounded_wait(int64_t limit_ns, int32_t arrive, void* stream);
 
 /* kkm_probe_unit_rate -- measured issue rate of one arithmetic unit on the

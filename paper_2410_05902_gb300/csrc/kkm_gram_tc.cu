@@ -6,17 +6,31 @@
 namespace kkm {
 namespace {
 
-// The passes' failure-detection path: thread 0 waits on an mbarrier of one
-// arrival with the passes' bounded wait. With arrive = 0 nothing arrives, so
-// the wait runs out after limit_ns; out[0] = 1 if it did.
+// The passes' failure-detection paths, by thread 0. First its bounded wait on an
+// mbarrier of one arrival; with arrive = 0 nothing arrives, so the wait runs out
+// after limit_ns and out[0] = 1. Then a hand-over through a slot that holds 7
+// and, with arrive = 0, is never freed: out[1] = 1 if it was refused, out[2] the
+// slot's value, out[3] = 1 if its reader was told.
 __global__ void k_wait_probe(uint64_t limit_ns, int arrive, int* out) {
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar, empty, full;
+  __shared__ int32_t slot;
   if (threadIdx.x != 0) return;
+  slot = 7;
   mbar_init(&bar, 1);
+  mbar_init(&empty, 1);
+  mbar_init(&full, 1);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  if (arrive) mbar_arrive(&bar);
+  if (arrive) {
+    mbar_arrive(&bar);
+    mbar_arrive(&empty);
+  }
   out[0] = mbar_wait(&bar, 0, limit_ns) ? 0 : 1;
+  out[1] = slot_put(&empty, 0, &slot, 3, &full, limit_ns) ? 0 : 1;
+  out[2] = slot;
+  out[3] = mbar_try_wait(&full, 0) ? 1 : 0;
   mbar_inval(&bar);
+  mbar_inval(&empty);
+  mbar_inval(&full);
 }
 
 }  // namespace

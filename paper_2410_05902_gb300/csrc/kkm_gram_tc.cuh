@@ -390,6 +390,18 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
+// One thread's hand-over of a value through a slot: waits for the slot to be
+// free (phase `parity` of empty), writes and arrives on full. On a wait that
+// runs out the slot and its barrier stay untouched, since the reader may not
+// have taken the value before; the caller gives up handing over.
+__device__ __forceinline__ bool slot_put(uint64_t* empty, uint32_t parity, int32_t* slot, int32_t v, uint64_t* full,
+                                         uint64_t limit_ns = WAIT_LIMIT_NS) {
+  if (!mbar_wait(empty, parity, limit_ns)) return false;
+  *slot = v;
+  mbar_arrive(full);
+  return true;
+}
+
 // A whole warp's wait, the same answer on every lane.
 __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(b, parity));
@@ -767,14 +779,15 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
 // is taken by one thread quad, and the quarters are added in order, as pairs.
 // A group alone takes all four; in the all-groups mode each group takes one, and
 // the first gets the others' quarter sums through shared memory. `turn` counts
-// the group's items (buffer parity).
+// the group's items (buffer parity). norms: finished items go to the norm warp
+// (cleared once a hand-over's wait has run out).
 // Window items have four accumulators and four teams whatever the launch's
 // distance tile, as in a launch of their own; beside 256-column tiles two teams
 // of two groups met twice an item to exchange their column sums.
 template <int KIND, int TNV>
 __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem,
                                             const Place<WPASS_TNV>& pl, uint32_t local, uint32_t turn, int item,
-                                            bool norms, bool dead) {
+                                            bool& norms, bool dead) {
   constexpr int MS = Geo<TNV>::MS;
   constexpr uint32_t SLOT_ARRIVALS = Geo<TNV>::GPT;   // a warp's share of a metadata slot's release
   static_assert(WG::NACC == 4 && WG::GPT == 1 && WPASS_TNV == 128, "four quarters, a group each or one group's");
@@ -922,11 +935,13 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
     }
     if (norms) {                                 // hand the item to the norm warp
       __syncwarp();
-      if (lane == 0) {
-        const uint32_t ns = local % NSLOT;
-        const bool ok = mbar_wait(&sh.nempty[ns], ((local / NSLOT) & 1u) ^ 1u);
-        sh.nj[ns] = ok && !dead ? center : -1;
-        mbar_arrive(&sh.nfull[ns]);
+      const uint32_t ns = local % NSLOT;
+      bool ok = true;
+      if (lane == 0)
+        ok = slot_put(&sh.nempty[ns], ((local / NSLOT) & 1u) ^ 1u, &sh.nj[ns], dead ? -1 : center, &sh.nfull[ns]);
+      if (!__shfl_sync(0xffffffffu, (int)ok, 0)) {   // the norm warp has given up: so does this one, at once
+        if (lane == 0) atomicOr(s.status, ST_TIMEOUT);
+        norms = false;
       }
     }
   }

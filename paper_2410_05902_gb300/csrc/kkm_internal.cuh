@@ -533,7 +533,7 @@ cudaError_t launch_lloyd_dist(const Dev& g, const LloydBuf& L, float* out, cudaS
 // tensor-core passes (BF16, split-BF16 and TF32 forms)
 // maps: 512 bytes, 64-byte aligned, holding the four CUtensorMap of the passes
 cudaError_t tc_prepare(Dev& s, void* maps);
-// one bounded mbarrier wait (the passes' own), limited to limit_ns; out[0] = 1 when it ran out
+// one bounded mbarrier wait and one hand-over (the passes' own), limited to limit_ns; out: four ints (k_wait_probe)
 cudaError_t launch_wait_probe(uint64_t limit_ns, int arrive, int* out, cudaStream_t st);
 // bytes the tcgen05 passes copy per item against a B tile of `cols` rows; with_a: its A tile too
 int64_t tc_item_bytes(const Dev& s, int cols, bool with_a);
