@@ -101,6 +101,7 @@ constexpr int NGRP = 4;                          // epilogue groups, one warp pe
 constexpr int MWARP = 2 + NEPI;                  // the metadata warp
 // TMA warp, MMA warp, epilogue, metadata warp and, where there are window items, the norm warp
 template <int MODE> constexpr int nthreads() { return 32 * (MWARP + (MODE == 0 ? 1 : 2)); }
+constexpr int WSUM_BYTES = 16;                   // a window sum in shared memory (FixedSum, or one FP64)
 constexpr int NSLOT = 4;                         // finished window items waiting for the norm warp
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;   // 2 s per wait
 constexpr float ROW_EXP_FLOOR = -100.0f;        // Gaussian: rc at or above it keeps 2^t finite
@@ -223,8 +224,7 @@ template <int TNV> struct Shared {
   alignas(16) Dev gdev;          // run groups: the segment's run (a shared copy: no reloads after global stores)
   alignas(16) MetaSlot<TNV> ring[Geo<TNV>::MS];   // 16-byte asynchronous copies land here
   float red[2][NGRP][4][32];     // distance items, all-groups mode: row sums (item parity, group, quadrant, row)
-  float ex[3][3][TM];            // window items: the other groups' quarter sums (quarter, sum, row)
-  double wq[NGRP][2][4][4];      // window items: quadrant sums (team, parity, quadrant, sum)
+  alignas(16) unsigned char wq[NGRP][2][3 * 4 * WSUM_BYTES];   // window items: sums (group, parity; class, quadrant)
 };
 
 template <int TNV> constexpr int smem_bytes() { return 1024 + RING_BYTES + (int)sizeof(Shared<TNV>); }
@@ -572,53 +572,81 @@ __device__ __forceinline__ float quad_sum(float v) {
   return v;
 }
 
-// A sum kept as h + l in two FP32 words (about 48 bits): the window pass adds
-// its row terms this way. FP64 issues at 1/64 of the FP32 rate on this chip (2
-// lane operations per clock and SM), and the 24 FP64 instructions that each of
-// the 16 epilogue warps took per item (conversions, products and three
-// 32-lane reductions) were about 6100 cycles of it, more than the rest of an
-// item. As pairs the same work is about 170 FP32 instructions per warp. The
-// terms are FP32 row sums, 2^-24 off by themselves. With the columns and row
-// quadrants outside an item's ranges skipped, the iteration went from 88.1 to
-// 79.2 us on the 1e6 x 128 workload (k = 100, b = 4096).
-struct Pair32 {
-  float h, l;
+// The window pass's sums where kernel values are at most 1 (Gaussian,
+// Laplacian). FP64 issues at 1/64 of the FP32 rate on this chip (2 lane
+// operations per clock and SM): the 24 FP64 instructions that each of the 16
+// epilogue warps took per item (conversions, products and three 32-lane
+// reductions) were about 6100 cycles of it, more than the rest of an item. Yet
+// the sums feed a recurrence and keep more than FP64's bits: a row's sum is
+// three FP32 words (Trip32: the errors of the first two words' sums are carried
+// exactly), and the 32 rows of a warp are added as fixed-point numbers of 66
+// bits below the largest row's exponent, three 22-bit limbs each, by integer
+// warp reductions (FixedSum), so that the sum is off by no more than 2^-60 of
+// itself. Only classes of columns that an item has are summed. 90 % of 8192 rows
+// in one of 10 centers, BF16: 213 us a step with sums of two FP32 words (48 bits)
+// for all three classes, 188 now; even batches of 4096 in 50 centers 53.4 and 54.9.
+struct Trip32 {
+  float h, m, l;
 };
-__device__ __forceinline__ Pair32 pair_scale(Pair32 x, float w) {
-  const float h = __fmul_rn(x.h, w);
-  return Pair32{h, __fmaf_rn(x.l, w, __fmaf_rn(x.h, w, -h))};
-}
-__device__ __forceinline__ Pair32 pair_add(Pair32 a, Pair32 b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float t = __fsub_rn(s, a.h);
-  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));   // a.h + b.h = s + e
-  return Pair32{s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
-}
-__device__ __forceinline__ Pair32 warp_pair_sum(Pair32 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    v = pair_add(v, Pair32{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
-  return v;
+// (l0 + 2^-22 l1 + 2^-44 l2) unit
+struct FixedSum {
+  int l0, l1, l2;
+  float unit;
+};
+// x, |x| < 2^22, as an integer, and what it leaves
+__device__ __forceinline__ int limb(float x, float& rest) {
+  constexpr float MAGIC = 12582912.0f;           // 1.5 * 2^23: the sum's last bit is 1
+  const float t = __fadd_rn(x, MAGIC);
+  rest = __fsub_rn(x, __fsub_rn(t, MAGIC));
+  return __float_as_int(t) - __float_as_int(MAGIC);
 }
 
-// The window pass's sums: pairs where kernel values are at most 1 (Gaussian,
-// Laplacian), FP64 where they have FP32's whole range. addf adds an FP32
-// quarter sum to a row's sum; rows gives the sum of w r over a warp's 32 rows.
+// zero; addf adds an FP32 quarter sum to a row's sum; rows gives the sum of w r
+// over a warp's 32 rows, value that sum in FP64.
 template <int KIND> struct WindowSum {
-  using T = Pair32;
-  static __device__ __forceinline__ T zero() { return T{0.0f, 0.0f}; }
-  static __device__ __forceinline__ T addf(T a, float b) { return pair_add(a, T{b, 0.0f}); }
-  static __device__ __forceinline__ T rows(T r, float w) { return warp_pair_sum(pair_scale(r, w)); }
-  static __device__ __forceinline__ T add(T a, T b) { return pair_add(a, b); }
-  static __device__ __forceinline__ double value(T a) { return (double)a.h + (double)a.l; }
+  using Row = Trip32;
+  using Sum = FixedSum;
+  static __device__ __forceinline__ Row zero() { return Row{0.0f, 0.0f, 0.0f}; }
+  static __device__ __forceinline__ Row addf(Row a, float b) {
+    float e, g;
+    const float h = two_sum(a.h, b, e), m = two_sum(a.m, e, g);
+    return Row{h, m, __fadd_rn(a.l, g)};
+  }
+  static __device__ __forceinline__ Sum rows(Row r, float w) {
+    // w r = h + m + l, m and l at most 2^-23 and 2^-46 or so of h
+    const float h = __fmul_rn(r.h, w), e = __fmaf_rn(r.h, w, -h);
+    const float q = __fmul_rn(r.m, w), f = __fmaf_rn(r.m, w, -q);
+    float g;
+    const float m = two_sum(q, e, g), l = __fadd_rn(__fmaf_rn(r.l, w, f), g);
+    const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(h) & 0x7fffffffu) >> 23;
+    if (top >= 255u) return Sum{0, 0, 0, __int_as_float(0x7fc00000)};   // a value that is not finite
+    // the unit is a power of two with every |h| below 2^21 units (nothing under 2^-100 needs its own)
+    const unsigned ex = top < 27u ? 27u : top;
+    const float inv = __uint_as_float((274u - ex) << 23), unit = __uint_as_float((ex - 20u) << 23);
+    float r1, r2, r3, r4, r5;
+    Sum s;
+    s.l0 = limb(__fmul_rn(h, inv), r1);
+    s.l1 = limb(__fmul_rn(r1, 0x1p22f), r2) + limb(__fmul_rn(__fmul_rn(m, inv), 0x1p22f), r3);
+    s.l2 = limb(__fmul_rn(__fadd_rn(r2, r3), 0x1p22f), r4) + limb(__fmul_rn(__fmul_rn(l, inv), 0x1p44f), r5);
+    s.l0 = __reduce_add_sync(0xffffffffu, s.l0);
+    s.l1 = __reduce_add_sync(0xffffffffu, s.l1);
+    s.l2 = __reduce_add_sync(0xffffffffu, s.l2);
+    s.unit = unit;
+    return s;
+  }
+  static __device__ __forceinline__ double value(Sum s) {
+    // l0 and l1 together are below 2^50
+    return fma((double)s.l2, 0x1p-22, (double)(((long long)s.l0 << 22) + s.l1)) * ((double)s.unit * 0x1p-22);
+  }
 };
+// FP64 where kernel values have FP32's whole range.
 struct WindowSum64 {
-  using T = double;
-  static __device__ __forceinline__ T zero() { return 0.0; }
-  static __device__ __forceinline__ T addf(T a, float b) { return a + (double)b; }
-  static __device__ __forceinline__ T rows(T r, float w) { return warp_sum_f64(r * (double)w); }
-  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
-  static __device__ __forceinline__ double value(T a) { return a; }
+  using Row = double;
+  using Sum = double;
+  static __device__ __forceinline__ Row zero() { return 0.0; }
+  static __device__ __forceinline__ Row addf(Row a, float b) { return a + (double)b; }
+  static __device__ __forceinline__ Sum rows(Row r, float w) { return warp_sum_f64(r * (double)w); }
+  static __device__ __forceinline__ double value(Sum a) { return a; }
 };
 template <> struct WindowSum<K_LINEAR> : WindowSum64 {};
 template <> struct WindowSum<K_POLY> : WindowSum64 {};
@@ -769,21 +797,27 @@ __device__ __forceinline__ void dist_item(const Dev& s, Shared<TNV>& sh, uint32_
   }
 }
 
-// One window-pass item: per element K(a, b) (its full exponent) into one of
-// three column sums per row (A: w_q on W, Bdd: w_q on D, E: 1 on B), then per
-// row the weight w_p (kind 0) or 1 (kind 1) and the sum over the 128 rows
-// (WindowSum). A row meeting its own copy (same data index) gets K = 1.
+// One window-pass item: per element K(a, b) (its full exponent) into the row's
+// sum over one of three classes of columns (w_q on D, w_q on the rest of W, 1 on
+// B), then per row the weight w_p (kind 0) or 1 (kind 1) and the sum over the 128
+// rows (WindowSum). A row meeting its own copy (same data index) gets K = 1.
 //
-// The sums of an item do not depend on how its 128 columns are dealt to the
-// groups: the columns are four quarters of 32, a row's FP32 sum of each quarter
-// is taken by one thread quad, and the quarters are added in order, as pairs.
-// A group alone takes all four; in the all-groups mode each group takes one, and
-// the first gets the others' quarter sums through shared memory. `turn` counts
-// the group's items (buffer parity). norms: finished items go to the norm warp
-// (cleared once a hand-over's wait has run out).
+// The columns are four quarters of 32; a row's FP32 sum of each quarter is taken
+// by one thread quad. A group alone takes all four and adds them in order before
+// the sum over the rows; in the all-groups mode each group takes one, with a sum
+// over the rows of its own, and the first group adds those. Which of the two
+// depends on the run's items alone (all_w), so that a run's norms come out the
+// same however its launches are grouped. `turn` counts the group's items (buffer
+// parity). norms: finished items go to the norm warp (cleared once a hand-over's
+// wait has run out).
 // Window items have four accumulators and four teams whatever the launch's
 // distance tile, as in a launch of their own; beside 256-column tiles two teams
 // of two groups met twice an item to exchange their column sums.
+// One copy of every part, in loops: as straight-line code for the three classes,
+// or with a second copy of the chunk's arithmetic that needs no masks, the
+// epilogue of a launch with both kinds of items outgrew the instruction cache.
+// 90 % of 8192 rows in one of 10 centers, split BF16: 295 and 249 us a step that
+// way, 231 in loops with the same sums.
 template <int KIND, int TNV>
 __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint32_t tmem,
                                             const Place<WPASS_TNV>& pl, uint32_t local, uint32_t turn, int item,
@@ -792,8 +826,9 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
   constexpr uint32_t SLOT_ARRIVALS = Geo<TNV>::GPT;   // a warp's share of a metadata slot's release
   static_assert(WG::NACC == 4 && WG::GPT == 1 && WPASS_TNV == 128, "four quarters, a group each or one group's");
   using WS = WindowSum<KIND>;
-  using Sum = typename WS::T;
-  static_assert(sizeof(Sum) == sizeof(double), "a shared-memory slot holds one sum");
+  using Row = typename WS::Row;
+  using Sum = typename WS::Sum;
+  static_assert(sizeof(Sum) <= WSUM_BYTES, "a shared-memory slot holds one sum");
   const int q = pl.q, lane = pl.lane;
   const int g4 = lane >> 2, us = lane & 3, c2 = 2 * us, rq = g4 + 8 * us;
   const bool all = pl.all;
@@ -805,133 +840,129 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
   const MetaSlot<TNV>& m = sh.ring[ms];
   const int nq = all ? 1 : NGRP, qlo = all ? pl.g : 0;     // this group's quarters
   const bool lead = qlo == 0;
-  const int slot = all ? 0 : pl.team;
-  Sum rA = WS::zero(), rB = WS::zero(), rE = WS::zero();   // this lane's row rq: W, D and B columns
-  auto add_class = [&](int cls, float v) {       // D is part of W
-    if (cls == 2) rE = WS::addf(rE, v);
-    else rA = WS::addf(rA, v);
-    if (cls == 0) rB = WS::addf(rB, v);
-  };
+  ItemDesc dsc{};                                // a dead warp's item has no columns
   float wrow = 0.0f;
-  int kind = 0, center = -1;
   bool rows_here = false;
+  float rc[4] = {};
+  int xi[4] = {};
   if (!dead) {
-    const ItemDesc dsc = m.desc;
-    kind = dsc.kind;
-    center = dsc.j;
+    dsc = m.desc;
     rows_here = dsc.rlo < q * 32 + 32 && dsc.rhi > q * 32;   // a quadrant may hold no row of the item
-    float rc[4];
-    int xi[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int r = q * 32 + g4 + 8 * u;
       rc[u] = (KIND == K_GAUSS) ? __fmul_rn(m.row[0][r], negc) : m.row[0][r];
       xi[u] = __float_as_int(m.row[1][r]);
     }
-    {
-      const int r = q * 32 + rq;
-      wrow = r >= dsc.rlo && r < dsc.rhi ? (kind == 0 ? m.row[2][r] : 1.0f) : 0.0f;
-    }
-    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * WPASS_TNV;
-    constexpr int NB = 2, CW = 8 * NB;
-    for (int t = 0; t < nq; ++t) {
-      const int cb = (qlo + t) * 32;
-      // the quarter's columns by class: 0 dropped rows D, 1 the rest of the old
-      // window W, 2 the new block B (columns from tnew on are in none); a chunk
-      // that straddles two classes goes through once for each
+    const int r = q * 32 + rq;
+    wrow = r >= dsc.rlo && r < dsc.rhi ? (dsc.kind == 0 ? m.row[2][r] : 1.0f) : 0.0f;
+  }
+  // Columns by class: 0 dropped rows D, 1 the rest of the old window W, 2 the new
+  // block B (columns from tnew on are in none; a new block's item needs only B).
+  // Most items have columns of one class alone, and the others cost nothing.
+  auto from = [&](int cls) { return cls == 0 ? 0 : max(cls == 1 ? dsc.dnew : dsc.told, 0); };
+  auto to = [&](int cls) { return min(cls == 0 ? dsc.dnew : cls == 1 ? dsc.told : dsc.tnew, WPASS_TNV); };
+  auto has = [&](int cls) { return (dsc.kind == 0 || cls == 2) && to(cls) > from(cls); };
+  auto release = [&]() {                         // the accumulator and the slot are free again
+    tc_fence_before();
+    pl.arrive(&sh.wempty[buf]);
+    pl.arrive(&sh.mempty[ms], SLOT_ARRIVALS);
+  };
+  const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + buf * WPASS_TNV;
+  auto sum_at = [&](int grp, int cls, int p) -> Sum& {
+    return *reinterpret_cast<Sum*>(sh.wq[grp][turn & 1u] + (cls * 4 + p) * WSUM_BYTES);
+  };
+  const int last = has(2) ? 2 : has(1) ? 1 : 0;
+  bool held = !all && !dead;
 #pragma unroll 1
-      for (int cls = 0; cls < 3; ++cls) {
-        const int lo = max(cb, cls == 0 ? 0 : cls == 1 ? dsc.dnew : dsc.told);
-        const bool need = rows_here && (kind == 0 || cls == 2);   // a new block's item needs only B
-        const int hi = need ? min(cb + 32, cls == 0 ? dsc.dnew : cls == 1 ? dsc.told : dsc.tnew) : 0;
-        float2 acc[4];
+  for (int cls = 0; cls < 3; ++cls) {
+    if (!has(cls)) continue;
+    Row r = WS::zero();
+#pragma unroll 1
+    for (int t = 0; t < nq; ++t) {
+      const int cb = (qlo + t) * 32, lo = max(cb, from(cls)), hi = rows_here ? min(cb + 32, to(cls)) : 0;
+      float2 acc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.0f, 0.0f);
-        for (int c0 = lo & ~(CW - 1); c0 < hi; c0 += CW) {
-          float v0[4 * NB], v1[4 * NB];
-          chunk_load<NB>(tq + c0, v0, v1);
+      for (int u = 0; u < 4; ++u) acc[u] = make_float2(0.0f, 0.0f);
+      constexpr int NB = 2, CW = 8 * NB;
+#pragma unroll 1
+      for (int c0 = lo & ~(CW - 1); c0 < hi; c0 += CW) {
+        float v0[4 * NB], v1[4 * NB];
+        chunk_load<NB>(tq + c0, v0, v1);
 #pragma unroll
-          for (int j = 0; j < NB; ++j) {
-            const int c = c0 + 8 * j + c2;
-            const float2 y2 = *reinterpret_cast<const float2*>(&m.col[0][c]);
-            float2 w2 = *reinterpret_cast<const float2*>(&m.col[1][c]);
-            const int2 i2 = *reinterpret_cast<const int2*>(&m.col[2][c]);
-            if (cls == 2) w2 = make_float2(1.0f, 1.0f);
-            const bool in0 = c >= lo && c < hi, in1 = c + 1 >= lo && c + 1 < hi;
-            w2 = make_float2(in0 ? w2.x : 0.0f, in1 ? w2.y : 0.0f);
+        for (int j = 0; j < NB; ++j) {
+          const int c = c0 + 8 * j + c2;
+          const float2 y2 = *reinterpret_cast<const float2*>(&m.col[0][c]);
+          float2 w2 = *reinterpret_cast<const float2*>(&m.col[1][c]);
+          const int2 i2 = *reinterpret_cast<const int2*>(&m.col[2][c]);
+          if (cls == 2) w2 = make_float2(1.0f, 1.0f);
+          const bool in0 = c >= lo && c < hi, in1 = c + 1 >= lo && c + 1 < hi;
+          w2 = make_float2(in0 ? w2.x : 0.0f, in1 ? w2.y : 0.0f);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const float2 gg = gram2<NB>(v0, v1, j, u);
-              float2 kv;
-              if constexpr (KIND == K_GAUSS) {
-                // every rounding spelled out: a run's norms must not depend on which
-                // kernel's compilation fuses a product into a sum
-                const float2 a = __ffma2_rn(gg, C2, __ffma2_rn(y2, make_float2(negc, negc),
-                                                               make_float2(rc[u], rc[u])));
-                kv.x = ex2_approx(xi[u] == i2.x ? 0.0f : a.x);
-                kv.y = ex2_approx(xi[u] == i2.y ? 0.0f : a.y);
-              } else {
-                kv = kernel_pair<KIND>(gg, rc[u], y2, xi[u], i2, negc, coef0, degree);
-              }
-              if constexpr (KIND == K_LINEAR || KIND == K_POLY) {   // unbounded outside the class
-                kv.x = in0 ? kv.x : 0.0f;
-                kv.y = in1 ? kv.y : 0.0f;
-              }
-              acc[u] = __ffma2_rn(w2, kv, acc[u]);
+          for (int u = 0; u < 4; ++u) {
+            const float2 gg = gram2<NB>(v0, v1, j, u);
+            float2 kv;
+            if constexpr (KIND == K_GAUSS) {
+              // every rounding spelled out: a run's norms must not depend on which
+              // kernel's compilation fuses a product into a sum
+              const float2 a = __ffma2_rn(gg, C2, __ffma2_rn(y2, make_float2(negc, negc),
+                                                             make_float2(rc[u], rc[u])));
+              kv.x = ex2_approx(xi[u] == i2.x ? 0.0f : a.x);
+              kv.y = ex2_approx(xi[u] == i2.y ? 0.0f : a.y);
+            } else {
+              kv = kernel_pair<KIND>(gg, rc[u], y2, xi[u], i2, negc, coef0, degree);
             }
+            if constexpr (KIND == K_LINEAR || KIND == K_POLY) {   // unbounded outside the class
+              kv.x = in0 ? kv.x : 0.0f;
+              kv.y = in1 ? kv.y : 0.0f;
+            }
+            acc[u] = __ffma2_rn(w2, kv, acc[u]);
           }
         }
-        float v = 0.0f;
-        if (hi > lo) {
-          float f4[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) f4[u] = quad_sum(acc[u].x + acc[u].y);
-          v = pick4(f4, us);
-        }
-        if (!lead) sh.ex[qlo - 1][cls][q * 32 + rq] = v;
-        else add_class(cls, v);
       }
+      float v = 0.0f;
+      if (hi > lo) {
+        float f4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) f4[u] = quad_sum(acc[u].x + acc[u].y);
+        v = pick4(f4, us);
+      }
+      r = WS::addf(r, v);
     }
-    if (!all) {                                  // the accumulator and the slot are free again
-      tc_fence_before();
-      pl.arrive(&sh.wempty[buf]);
-      pl.arrive(&sh.mempty[ms], SLOT_ARRIVALS);
+    if (held && cls == last) {
+      release();
+      held = false;
     }
+    const Sum t = WS::rows(r, wrow);
+    if (lane == 0) sum_at(pl.g, cls, q) = t;
   }
+  if (held) release();
+  const int kind = dsc.kind, center = dsc.j;
   if (all) {
     tc_fence_before();
-    pl.sync_all();
-    if (lead && !dead) {
-      pl.arrive(&sh.wempty[buf]);
-      pl.arrive(&sh.mempty[ms], SLOT_ARRIVALS);
-    }
-    if (lead && rows_here)
-      for (int o = 1; o < NGRP; ++o)
-        for (int cls = 0; cls < 3; ++cls) add_class(cls, sh.ex[o - 1][cls][q * 32 + rq]);
-    pl.sync_all();                               // the exchange buffer may be written again
+    pl.sync_all();                               // every warp, dead or not
+    if (!lead) return;                           // (their next sums go to the other parity)
+    if (!dead) release();
+  } else {
+    pl.sync_group();                             // every warp of the group, dead or not
   }
-  if (!lead) return;
-  if (rows_here) {
-    rE = WS::rows(rE, wrow);
-    if (kind == 0) {
-      rA = WS::rows(rA, wrow);
-      rB = WS::rows(rB, wrow);
-    }
-  }
-  // the four quadrants' sums (A, Bdd, E for kind 0; M for kind 1) in quadrant order
-  Sum (*wq)[4] = reinterpret_cast<Sum (*)[4]>(sh.wq[slot][turn & 1u]);
-  if (lane == 0) {
-    wq[q][0] = rA;
-    wq[q][1] = rB;
-    wq[q][2] = rE;
-  }
-  pl.sync_group();                               // every warp of the group, dead or not
   if (q == 2) {                                  // the group's first warp
-    if (!dead && lane < 4) {
-      const int src = lane == 3 ? 2 : lane;      // M is the E sum of a kind-1 item
-      const bool keep = (lane < 3) == (kind == 0);
-      const Sum v = WS::add(WS::add(WS::add(wq[0][src], wq[1][src]), wq[2][src]), wq[3][src]);
-      s.wpart[(int64_t)item * 4 + lane] = keep ? WS::value(v) : 0.0;
+    if (!dead) {                                 // lane 4 cls + p: quadrant p's sum of class cls
+      double v = 0.0;
+      if (lane < 12 && has(lane >> 2)) {
+        v = WS::value(sum_at(pl.g, lane >> 2, lane & 3));
+        if (all)
+          v = (v + WS::value(sum_at(1, lane >> 2, lane & 3))) +
+              (WS::value(sum_at(2, lane >> 2, lane & 3)) + WS::value(sum_at(3, lane >> 2, lane & 3)));
+      }
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      const double vd = __shfl_sync(0xffffffffu, v, 0), vw = __shfl_sync(0xffffffffu, v, 4),
+                   vb = __shfl_sync(0xffffffffu, v, 8);
+      // A over W (D and the rest), Bdd over D, E (kind 0) or M (kind 1) over B
+      if (lane < 4)
+        s.wpart[(int64_t)item * 4 + lane] =
+            lane == 0 ? vd + vw : lane == 1 ? vd : lane == (kind == 0 ? 2 : 3) ? vb : 0.0;
     }
     if (norms) {                                 // hand the item to the norm warp
       __syncwarp();

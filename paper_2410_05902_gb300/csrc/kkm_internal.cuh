@@ -417,6 +417,14 @@ struct TabBuf {
   int32_t bs_rows;     // rows of the support buffer (k * cap + 256)
 };
 
+// s + e = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+
 // ------------------------------------------------------------ launchers
 // All return cudaGetLastError() of their launches.
 cudaError_t launch_sample(const Dev& s, cudaStream_t st);

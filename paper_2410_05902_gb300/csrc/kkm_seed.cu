@@ -72,14 +72,6 @@ struct PPArgs {
   int vec;             // rows may be read 16 bytes at a time
 };
 
-// s + e = a + b exactly (Knuth's two-sum).
-__device__ __forceinline__ float two_sum(float a, float b, float& e) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return s;
-}
-
 // hi + mid + lo += (x - c)^2. x - c = s + e exactly; s^2 = p + q and 2 s e =
 // t + u exactly (FMA products); hi and mid collect their terms by two-sums, lo
 // the errors of mid's sums and the terms below 2^-46 s^2 in plain FP32. nz
