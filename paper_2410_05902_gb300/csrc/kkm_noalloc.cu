@@ -158,9 +158,11 @@ __device__ __forceinline__ void pair_square(float& h, float& l, float v) {
 // Y and of a pass's query rows Q, FP32-rounded, eight lanes a row. The squares
 // are summed as FP32 pairs (48 bits): FP64 issues at 1/64 of the FP32 rate on
 // this chip, and a warp per row with a 32-lane FP64 reduction took longer than
-// the Gram tiles of a small call. Sums near the ends of the FP32 range (where
-// a square's error term leaves it), zeros and non-finite ones are taken again
-// in FP64. VEC: rows on 16-byte boundaries (as NaGram's).
+// the Gram tiles of a small call. A pair only stands where every sum within
+// its error rounds to the same FP32 value, so that the norms are those of FP64
+// sums to the bit; the others (one row in thousands), sums near the ends of the
+// FP32 range (where a square's error term leaves it), zeros and non-finite ones
+// are taken again in FP64. VEC: rows on 16-byte boundaries (as NaGram's).
 template <bool VEC>
 __global__ void __launch_bounds__(NT) k_na_prepare(Scratch* sc, int tiles, const int32_t* __restrict__ seg_off,
                                                    int k, int S, const float* __restrict__ Y, int64_t ldy, int ny,
@@ -198,7 +200,10 @@ __global__ void __launch_bounds__(NT) k_na_prepare(Scratch* sc, int tiles, const
     pair_add(h, l, bh, bl);
   }
   float out = __fadd_rn(h, l);
-  const bool redo = live && !(h > 1e-25f && h < 1e37f);
+  // m additions into a pair: each rounds l, at most m 2^-24 h, by 2^-24 of it;
+  // twice that bounds their sum and the roundings of the bound itself
+  const float m = (float)(d / 8 + 8), err = __fmul_rn(h, m * m * 0x1p-47f);
+  const bool redo = live && (!(h > 1e-25f && h < 1e37f) || __fadd_rn(h, __fsub_rn(l, err)) != __fadd_rn(h, __fadd_rn(l, err)));
   if (__any_sync(0xffffffffu, redo)) {
     double acc = 0.0;
     for (int q = sub; q < dl; q += 8) acc += (double)p[q] * (double)p[q];
