@@ -329,8 +329,7 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   if (total < 4 * nblk) {
     for (int w = bid; w < total; w += nblk) {
       wgram_simt_item<F>(s, w, sm, red);
-      const int j = s.wpairs[w].j;
-      if (norms && threadIdx.x < 32) norm_report(s, j, (w - s.wpair_first[j]) / WSEG, 1);
+      if (norms && threadIdx.x < 32) norm_report(s, ItemPlace(s, w, s.wpairs[w].j), 1);
     }
     return;
   }
@@ -338,7 +337,10 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   NormReports reports(hi);
   for (int w = lo; w < hi; ++w) {
     wgram_simt_item<F>(s, w, sm, red);
-    if (norms && threadIdx.x < 32) reports.done(s, w, s.wpairs[w].j);
+    if (norms && threadIdx.x < 32) {
+      reports.next(s, w);
+      reports.done(s, true);
+    }
   }
 }
 

@@ -588,11 +588,11 @@ __device__ __forceinline__ float quad_sum(float v) {
 struct Trip32 {
   float h, m, l;
 };
-// (l0 + 2^-22 l1 + 2^-44 l2) unit
+// (l0 + 2^-22 l1 + 2^-44 l2) 2^e
 struct FixedSum {
-  int l0, l1, l2;
-  float unit;
+  int l0, l1, l2, e;
 };
+constexpr int NOT_FINITE = 1 << 20;              // e of a sum with a value that is not finite
 // x, |x| < 2^22, as an integer, and what it leaves
 __device__ __forceinline__ int limb(float x, float& rest) {
   constexpr float MAGIC = 12582912.0f;           // 1.5 * 2^23: the sum's last bit is 1
@@ -619,10 +619,10 @@ template <int KIND> struct WindowSum {
     float g;
     const float m = two_sum(q, e, g), l = __fadd_rn(__fmaf_rn(r.l, w, f), g);
     const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(h) & 0x7fffffffu) >> 23;
-    if (top >= 255u) return Sum{0, 0, 0, __int_as_float(0x7fc00000)};   // a value that is not finite
-    // the unit is a power of two with every |h| below 2^21 units (nothing under 2^-100 needs its own)
+    if (top >= 255u) return Sum{0, 0, 0, NOT_FINITE};
+    // every |h| is below 2^21 times 2^e (nothing under 2^-100 needs a unit of its own)
     const unsigned ex = top < 27u ? 27u : top;
-    const float inv = __uint_as_float((274u - ex) << 23), unit = __uint_as_float((ex - 20u) << 23);
+    const float inv = __uint_as_float((274u - ex) << 23);
     float r1, r2, r3, r4, r5;
     Sum s;
     s.l0 = limb(__fmul_rn(h, inv), r1);
@@ -631,12 +631,18 @@ template <int KIND> struct WindowSum {
     s.l0 = __reduce_add_sync(0xffffffffu, s.l0);
     s.l1 = __reduce_add_sync(0xffffffffu, s.l1);
     s.l2 = __reduce_add_sync(0xffffffffu, s.l2);
-    s.unit = unit;
+    s.e = (int)ex - 147;
     return s;
   }
   static __device__ __forceinline__ double value(Sum s) {
-    // l0 and l1 together are below 2^50
-    return fma((double)s.l2, 0x1p-22, (double)(((long long)s.l0 << 22) + s.l1)) * ((double)s.unit * 0x1p-22);
+    if (s.e == NOT_FINITE) return __longlong_as_double(0x7ff8000000000000ll);
+    // l0 and l1 (together below 2^50) and l2 as the last bits of doubles of known
+    // exponents: one FP64 subtraction each and one addition
+    const long long q = ((long long)s.l0 << 22) + s.l1 + (1ll << 51);
+    const int k = (s.e - 22) << 20, k2 = (s.e - 44) << 20;
+    const double a = __hiloint2double(0x43300000 + (int)(q >> 32) + k, (int)q);
+    const double b = __hiloint2double(0x43300000 + k2, s.l2 ^ (int)0x80000000);
+    return (a - __hiloint2double(0x43380000 + k, 0)) + (b - __hiloint2double(0x43300000 + k2, (int)0x80000000));
   }
 };
 // FP64 where kernel values have FP32's whole range.
@@ -1031,6 +1037,7 @@ __device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int lo,
   NormReports reports(lo + nw);
   for (uint32_t i = 0; (int)i < nw; ++i) {
     const uint32_t ns = i % NSLOT;
+    reports.next(s, lo + (int)i);                // its reads overlap the wait
     const bool ok = mbar_wait(&sh.nfull[ns], (i / NSLOT) & 1u);
     if (__any_sync(0xffffffffu, !ok)) {
       if (lane == 0) atomicOr(s.status, ST_TIMEOUT);
@@ -1039,7 +1046,7 @@ __device__ __forceinline__ void norm_warp(const Dev& s, Shared<TNV>& sh, int lo,
     const int j = sh.nj[ns];
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.nempty[ns]);
-    reports.done(s, lo + (int)i, j);
+    reports.done(s, j >= 0);
   }
 }
 

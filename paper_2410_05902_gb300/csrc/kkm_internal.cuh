@@ -315,15 +315,22 @@ __device__ __forceinline__ bool last_arrival(int32_t* counter, int m, int of) {
   return true;
 }
 
-// A warp's report of m finished window items of segment q of center j (their
-// sums are in wpart): the last of a segment adds it up, the last of a center's
-// segments adds those and carries ||C_j||^2 through the update. A fence and an
-// atomic take longer than an item's arithmetic, so consecutive items of a
-// segment are reported together (NormReports).
-__device__ __forceinline__ void norm_report(const Dev& s, int j, int q, int m) {
-  const int lane = threadIdx.x & 31;
-  const int first = s.wpair_first[j], cnt = s.wpair_cnt[j];
-  const int nseg = win_segments(cnt), slot = win_segment_slot(first, j), here = min(WSEG, cnt - q * WSEG);
+// Where a window item's sums go.
+struct ItemPlace {
+  int j, first, cnt, q;   // its center, that center's first item and their number, its segment
+  __device__ ItemPlace() {}
+  __device__ ItemPlace(const Dev& s, int item, int j_)
+      : j(j_), first(s.wpair_first[j_]), cnt(s.wpair_cnt[j_]), q((item - first) / WSEG) {}
+};
+
+// A warp's report of m finished window items of a segment (their sums are in
+// wpart): the last of a segment adds it up, the last of a center's segments adds
+// those and carries ||C_j||^2 through the update. A fence and an atomic take
+// longer than an item's arithmetic, so consecutive items of a segment are
+// reported together (NormReports).
+__device__ __forceinline__ void norm_report(const Dev& s, const ItemPlace& at, int m) {
+  const int lane = threadIdx.x & 31, j = at.j, q = at.q, first = at.first;
+  const int nseg = win_segments(at.cnt), slot = win_segment_slot(first, j), here = min(WSEG, at.cnt - q * WSEG);
   if (!last_arrival(s.wdone + slot + q, m, here)) return;
   const int n = s.plan[j].cnt;
   const double part = (double)s.cmpart[(int64_t)j * 32 + lane];
@@ -346,18 +353,23 @@ __device__ __forceinline__ void norm_report(const Dev& s, int j, int q, int m) {
   }
 }
 
-// Gathers the reports of a warp that finishes the items lo, .. , hi - 1 in
-// order: one per segment. done(item, j): item of center j is finished (j < 0: it
-// was skipped, and its center keeps its norm).
+// Gathers the reports of a warp that finishes items in order up to hi - 1: one
+// per segment. next: the item it waits for; done: that item is finished (ok) or
+// was skipped, and then its center keeps its norm.
 struct NormReports {
   int hi, m = 0;
+  ItemPlace at;
+  bool send = false;
   __device__ explicit NormReports(int hi_) : hi(hi_) {}
-  __device__ __forceinline__ void done(const Dev& s, int item, int j) {
-    const int jn = item + 1 < hi ? s.wpairs[item + 1].j : -1;
-    const int jc = s.wpairs[item].j, at = item - s.wpair_first[jc];
-    m += j >= 0 ? 1 : 0;
-    if (jn == jc && (at + 1) % WSEG != 0) return;
-    if (m > 0) norm_report(s, jc, at / WSEG, m);
+  __device__ __forceinline__ void next(const Dev& s, int item) {
+    const int j = s.wpairs[item].j, jn = item + 1 < hi ? s.wpairs[item + 1].j : -1;
+    at = ItemPlace(s, item, j);
+    send = jn != j || (item + 1 - at.first) % WSEG == 0;
+  }
+  __device__ __forceinline__ void done(const Dev& s, bool ok) {
+    m += ok ? 1 : 0;
+    if (!send) return;
+    if (m > 0) norm_report(s, at, m);
     m = 0;
   }
 };
