@@ -433,7 +433,6 @@ KKM_API kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d,
       return bail(KKM_ENOMEM);                                   \
     }                                                            \
   } while (0)
-  ALLOC(s.bidx, b);
   if (esz == 4) ALLOC(s.xb32, (size_t)s.bpad * s.ld);
   else ALLOC(s.xbh, (size_t)s.bpad * s.ld);
   ALLOC(s.xbn, s.bpad);
@@ -1484,7 +1483,7 @@ kkm_status chain_enqueue(kkm_group* g, const kkm_group::Chain& c, cudaStream_t s
   for (const auto& p : c.dist) {
     if (r != KKM_OK) return r;
     r = ok(p.tc ? kkm::launch_group_tc(p.ph.g, 0, p.form, p.kind, p.tn, p.ph.blocks, st)
-                : kkm::launch_group_simt(p.ph.g, 0, p.form, p.ph.blocks, st),
+                : kkm::launch_group_simt(p.ph.g, 0, p.ph.blocks, st),
            "group distance pass");
   }
   if (r == KKM_OK) r = ok(kkm::launch_group_argmin(c.argmin.g, c.argmin.blocks, st), "group argmin");
@@ -1493,7 +1492,7 @@ kkm_status chain_enqueue(kkm_group* g, const kkm_group::Chain& c, cudaStream_t s
   for (const auto& p : c.window) {
     if (r != KKM_OK) return r;
     r = ok(p.tc ? kkm::launch_group_tc(p.ph.g, 1, p.form, p.kind, p.tn, p.ph.blocks, st)
-                : kkm::launch_group_simt(p.ph.g, 1, p.form, p.ph.blocks, st),
+                : kkm::launch_group_simt(p.ph.g, 1, p.ph.blocks, st),
            "group window pass");
   }
   if (r == KKM_OK) r = ok(kkm::launch_group_finalize(c.finalize.g, c.finalize.blocks, st), "group finalize");

@@ -13,8 +13,8 @@
 //   E   = sum_{p in D, q in B} w_p K(p, q)       = b_j <D, cm(B_j)>
 //   M   = sum_{p in B, q in B} K(p, q)           = b_j^2 ||cm(B_j)||^2
 // where W is the old window, D its dropped prefix (old weights) and B the new
-// block. Each tile writes its four FP64 partial sums; k_finalize adds them in
-// tile order.
+// block. Each tile writes its four FP64 partial sums, which are added in tile
+// order (NormReports; run groups: k_finalize).
 #include <algorithm>
 
 #include "kkm_internal.cuh"
@@ -24,28 +24,6 @@ namespace {
 
 constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
 
-// Four consecutive row values starting at column k, as the Gram product uses them:
-// FP32 rows as stored; BF16 rows as hi, or hi + lo for the split form.
-template <int F>
-__device__ __forceinline__ float4 load4(const void* rowp, int k, int dp) {
-  if constexpr (F == FORM_FP32) {
-    return *reinterpret_cast<const float4*>((const float*)rowp + k);
-  } else {
-    const __nv_bfloat16* r = (const __nv_bfloat16*)rowp;
-    const uint2 h = *reinterpret_cast<const uint2*>(r + k);
-    const __nv_bfloat162 h0 = *reinterpret_cast<const __nv_bfloat162*>(&h.x);
-    const __nv_bfloat162 h1 = *reinterpret_cast<const __nv_bfloat162*>(&h.y);
-    float4 v = make_float4(__low2float(h0), __high2float(h0), __low2float(h1), __high2float(h1));
-    if constexpr (F == FORM_BF16X3) {
-      const uint2 l = *reinterpret_cast<const uint2*>(r + dp + k);
-      const __nv_bfloat162 l0 = *reinterpret_cast<const __nv_bfloat162*>(&l.x);
-      const __nv_bfloat162 l1 = *reinterpret_cast<const __nv_bfloat162*>(&l.y);
-      v.x += __low2float(l0); v.y += __high2float(l0); v.z += __low2float(l1); v.w += __high2float(l1);
-    }
-    return v;
-  }
-}
-
 // Operand chunks of BK columns, two buffers: columns of 16 MR rows of A and 64 of B.
 template <int MR> struct GramSmem {
   float A[2][BK][16 * MR + 4];
@@ -53,21 +31,20 @@ template <int MR> struct GramSmem {
 };
 
 // acc[i][j] = sum_k A[ty*MR+i][k] * B[tx*4+j][k] for a 16 MR x 64 tile. A and B
-// point at the tiles' first rows (element type by form); rows are `ld` elements
-// apart and the product runs over kend columns (zero padded, a multiple of BK).
+// point at the tiles' first rows; rows are `ld` elements apart and the product
+// runs over all of them (zero padded, a multiple of BK).
 // DIFF: acc[i][j] = sum_k (A[ty*MR+i][k] - B[tx*4+j][k])^2 instead. The next BK
 // columns are loaded into registers while the current ones are multiplied out of
 // shared memory, with one barrier per BK columns. Each sum is one chain over k
 // whatever MR is.
-template <int F, int MR, bool DIFF>
-__device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void* __restrict__ B,
-                                          int ld, int kend, int dp, float (&acc)[MR][4], GramSmem<MR>& sm) {
+template <int MR, bool DIFF>
+__device__ __forceinline__ void gram_tile(const float* __restrict__ A, const float* __restrict__ B, int ld,
+                                          float (&acc)[MR][4], GramSmem<MR>& sm) {
   constexpr int NA = MR / 4;                     // 64-row slices of A a loader thread fills
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int lr = tid >> 2, lk = (tid & 3) * 4;   // loader: row, k offset
-  const int esz = (F == FORM_FP32) ? 4 : 2;
-  const char* arow = (const char*)A + (int64_t)lr * ld * esz;
-  const char* brow = (const char*)B + (int64_t)lr * ld * esz;
+  const float* arow = A + (int64_t)lr * ld + lk;
+  const float* brow = B + (int64_t)lr * ld + lk;
 #pragma unroll
   for (int i = 0; i < MR; ++i)
 #pragma unroll
@@ -75,8 +52,8 @@ __device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void
   float4 a[NA], b;
   auto load = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < NA; ++q) a[q] = load4<F>(arow + (int64_t)q * 64 * ld * esz, k0 + lk, dp);
-    b = load4<F>(brow, k0 + lk, dp);
+    for (int q = 0; q < NA; ++q) a[q] = *reinterpret_cast<const float4*>(arow + (int64_t)q * 64 * ld + k0);
+    b = *reinterpret_cast<const float4*>(brow + k0);
   };
   auto store = [&](int buf) {
 #pragma unroll
@@ -92,8 +69,8 @@ __device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void
   __syncthreads();                               // the previous tile's readers are done
   store(0);
   int buf = 0;
-  for (int k0 = 0; k0 < kend; k0 += BK, buf ^= 1) {
-    const bool more = k0 + BK < kend;
+  for (int k0 = 0; k0 < ld; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < ld;
     if (more) load(k0 + BK);
     __syncthreads();                             // this buffer is filled, the other one read
 #pragma unroll
@@ -120,12 +97,6 @@ __device__ __forceinline__ void gram_tile(const void* __restrict__ A, const void
     }
     if (more) store(buf ^ 1);
   }
-}
-
-template <int F>
-__device__ __forceinline__ const void* rows_ptr(const Dev& s, bool support, int64_t row) {
-  if constexpr (F == FORM_FP32) return (support ? s.y32 : s.xb32) + row * s.ld;
-  else return (support ? s.ybh : s.xbh) + row * s.ld;
 }
 
 // One level of the row sums' tree: N rows' values, half of them handed to the
@@ -200,39 +171,37 @@ __device__ __forceinline__ void dist_simt_sums(const Dev& s, int rows, int t, in
 }
 
 // Item w of a run's distance pass (row tile w % R of support tile w / R; 16 MR rows a tile).
-template <int F, int MR>
+template <int MR>
 __device__ __forceinline__ void dist_simt_item(const Dev& s, int rows, int R, int w, GramSmem<MR>& sm) {
   const int t = w / R, row0 = (w % R) * 16 * MR;
   const Tile T = s.tiles[t];
-  const void *A = rows_ptr<F>(s, false, row0), *B = rows_ptr<F>(s, true, T.row0);
-  const int kend = F == FORM_FP32 ? s.ld : s.dp;
+  const float *A = s.xb32 + (int64_t)row0 * s.ld, *B = s.y32 + (int64_t)T.row0 * s.ld;
   float acc[MR][4];
   // Laplacian kernel: ||x - y||^2 from the differences. Through ||x||^2 +
   // ||y||^2 - 2 <x, y> a query row equal to a support row (no data index to
   // recognise it by) keeps d2 ~ eps ||x||^2, which the square root magnifies.
   if (s.kind == K_LAPLACE) {
-    gram_tile<F, MR, true>(A, B, s.ld, kend, s.dp, acc, sm);
+    gram_tile<MR, true>(A, B, s.ld, acc, sm);
     dist_simt_sums<K_LAPLACE, MR>(s, rows, t, row0, T, acc);
     return;
   }
-  gram_tile<F, MR, false>(A, B, s.ld, kend, s.dp, acc, sm);
+  gram_tile<MR, false>(A, B, s.ld, acc, sm);
   if (s.kind == K_GAUSS) dist_simt_sums<K_GAUSS, MR>(s, rows, t, row0, T, acc);
   else if (s.kind == K_LINEAR) dist_simt_sums<K_LINEAR, MR>(s, rows, t, row0, T, acc);
   else dist_simt_sums<K_POLY, MR>(s, rows, t, row0, T, acc);
 }
 
-template <int F, int MR>
+template <int MR>
 __global__ void __launch_bounds__(NT) k_dist_simt(Dev s, int rows) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
   __shared__ __align__(16) GramSmem<MR> sm;
   const int R = (rows + 16 * MR - 1) / (16 * MR);
   const int total = R * (*s.ntiles);
-  for (int w = blockIdx.x; w < total; w += gridDim.x) dist_simt_item<F, MR>(s, rows, R, w, sm);
+  for (int w = blockIdx.x; w < total; w += gridDim.x) dist_simt_item<MR>(s, rows, R, w, sm);
 }
 
 // Pair w of a run's window pass; its four sums go to wpart[w].
-template <int F>
 __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, GramSmem<4>& sm, double (*red)[NT / 32]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
   {
@@ -245,8 +214,7 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, GramSmem<4>
     else { r0 = P.tail_c; rn = P.cnt; c0 = P.tail_c; cn = P.cnt; }
     const int rs = r0 + pr.rt * BM, cs = c0 + pr.ct * BN;
     float acc[4][4];
-    gram_tile<F, 4, false>(rows_ptr<F>(s, true, base + rs), rows_ptr<F>(s, true, base + cs), s.ld,
-                           F == FORM_FP32 ? s.ld : s.dp, s.dp, acc, sm);
+    gram_tile<4, false>(s.y32 + (base + rs) * s.ld, s.y32 + (base + cs) * s.ld, s.ld, acc, sm);
     // FP64 issues at 1/64 of the FP32 rate on this chip, so the row weight is
     // taken out of the column sums: a conversion and one to two FP64 operations
     // per element where the product of both weights took four to five
@@ -313,7 +281,6 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, GramSmem<4>
   }
 }
 
-template <int F>
 __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bid, int nblk) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
@@ -328,7 +295,7 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   // (75) 2649 and 2459.
   if (total < 4 * nblk) {
     for (int w = bid; w < total; w += nblk) {
-      wgram_simt_item<F>(s, w, sm, red);
+      wgram_simt_item(s, w, sm, red);
       if (norms && threadIdx.x < 32) norm_report(s, ItemPlace(s, w, s.wpairs[w].j), 1);
     }
     return;
@@ -336,7 +303,7 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   const int lo = (int)((int64_t)bid * total / nblk), hi = (int)((int64_t)(bid + 1) * total / nblk);
   NormReports reports(hi);
   for (int w = lo; w < hi; ++w) {
-    wgram_simt_item<F>(s, w, sm, red);
+    wgram_simt_item(s, w, sm, red);
     if (norms && threadIdx.x < 32) {
       reports.next(s, w);
       reports.done(s, true);
@@ -344,9 +311,8 @@ __device__ __forceinline__ void wgram_simt_body(const Dev& s, bool norms, int bi
   }
 }
 
-template <int F>
 __global__ void __launch_bounds__(NT) k_wgram_simt(Dev s, int norms) {
-  wgram_simt_body<F>(s, norms != 0, blockIdx.x, gridDim.x);
+  wgram_simt_body(s, norms != 0, blockIdx.x, gridDim.x);
 }
 
 // Run groups: the items of all the launch's runs laid end to end (distance
@@ -356,7 +322,7 @@ __global__ void __launch_bounds__(NT) k_wgram_simt(Dev s, int norms) {
 // run computes what its own launch would.
 constexpr int GROUP_MAX_RUNS = 1024;
 
-template <int F, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
   KKM_GRID_DEP_WAIT();
   KKM_LAUNCH_DEPENDENTS();
@@ -383,8 +349,8 @@ __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
       else hi = mid;
     }
     const Dev& s = g.runs[lo].s;
-    if constexpr (MODE == 0) dist_simt_item<F, 4>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], sm);
-    else wgram_simt_item<F>(s, w - off[lo], sm, red);
+    if constexpr (MODE == 0) dist_simt_item<4>(s, s.b, (s.b + BM - 1) / BM, w - off[lo], sm);
+    else wgram_simt_item(s, w - off[lo], sm, red);
   }
 }
 
@@ -397,46 +363,21 @@ __global__ void __launch_bounds__(NT) k_group_simt(GroupPhase g) {
 // 4 products take three shared-memory reads per 32 FMAs, the 64-row tile's 4 x 4
 // two per 16. The number of support tiles is known on the device only; a full
 // window has at least tau / 64 of them, a center without one at most none.
-template <int F>
-static cudaError_t launch_dist_form(const Dev& s, int rows, cudaStream_t st) {
-  const int64_t tiles = (int64_t)s.k * std::max(1, s.tau / BN);
-  if (rows > BM && (rows + 127) / 128 * tiles >= 2 * s.num_sms)
-    return launch_pdl(k_dist_simt<F, 8>, dim3(s.num_sms * 3), dim3(NT), 0, st, s, rows);
-  return launch_pdl(k_dist_simt<F, 4>, dim3(s.num_sms * 4), dim3(NT), 0, st, s, rows);
-}
-
 cudaError_t launch_dist_simt(const Dev& s, int rows, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  switch (s.form) {
-    case FORM_FP32: return launch_dist_form<FORM_FP32>(s, rows, st);
-    case FORM_BF16: return launch_dist_form<FORM_BF16>(s, rows, st);
-    default: return launch_dist_form<FORM_BF16X3>(s, rows, st);
-  }
+  const int64_t tiles = (int64_t)s.k * std::max(1, s.tau / BN);
+  if (rows > BM && (rows + 127) / 128 * tiles >= 2 * s.num_sms)
+    return launch_pdl(k_dist_simt<8>, dim3(s.num_sms * 3), dim3(NT), 0, st, s, rows);
+  return launch_pdl(k_dist_simt<4>, dim3(s.num_sms * 4), dim3(NT), 0, st, s, rows);
 }
 
 cudaError_t launch_wgram(const Dev& s, cudaStream_t st, bool norms) {
-  const int blocks = s.num_sms * 4;
-  switch (s.form) {
-    case FORM_FP32: return launch_pdl(k_wgram_simt<FORM_FP32>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
-    case FORM_BF16: return launch_pdl(k_wgram_simt<FORM_BF16>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
-    default: return launch_pdl(k_wgram_simt<FORM_BF16X3>, dim3(blocks), dim3(NT), 0, st, s, norms ? 1 : 0);
-  }
+  return launch_pdl(k_wgram_simt, dim3(s.num_sms * 4), dim3(NT), 0, st, s, norms ? 1 : 0);
 }
 
-cudaError_t launch_group_simt(const GroupPhase& g, int mode, int form, int blocks, cudaStream_t st) {
+cudaError_t launch_group_simt(const GroupPhase& g, int mode, int blocks, cudaStream_t st) {
   const dim3 grid(blocks > 0 ? blocks : 1), block(NT);
-  if (mode == 0) {
-    switch (form) {
-      case FORM_FP32: return launch_pdl(k_group_simt<FORM_FP32, 0>, grid, block, 0, st, g);
-      case FORM_BF16: return launch_pdl(k_group_simt<FORM_BF16, 0>, grid, block, 0, st, g);
-      default: return launch_pdl(k_group_simt<FORM_BF16X3, 0>, grid, block, 0, st, g);
-    }
-  }
-  switch (form) {
-    case FORM_FP32: return launch_pdl(k_group_simt<FORM_FP32, 1>, grid, block, 0, st, g);
-    case FORM_BF16: return launch_pdl(k_group_simt<FORM_BF16, 1>, grid, block, 0, st, g);
-    default: return launch_pdl(k_group_simt<FORM_BF16X3, 1>, grid, block, 0, st, g);
-  }
+  return launch_pdl(mode == 0 ? k_group_simt<0> : k_group_simt<1>, grid, block, 0, st, g);
 }
 
 }  // namespace kkm

@@ -103,7 +103,6 @@ struct alignas(16) Dev {
   int32_t max_tiles, max_pairs;
   const float* X;
   // batch
-  int32_t* bidx;     // [b] indices of the batch being processed
   float* xb32;       // [bpad * ld]   FP32 form
   __nv_bfloat16* xbh;// [bpad * ld]   BF16 forms
   float* xbn;        // [bpad]
@@ -175,15 +174,24 @@ struct alignas(16) Dev {
 // anything the predecessor writes (a no-op when launched without the attribute).
 #define KKM_GRID_DEP_WAIT() asm volatile("griddepcontrol.wait;" ::: "memory")
 // Lets the next kernel in the stream start its pre-wait part. Issued only after
-// this kernel's own wait, so every kernel before it has completed by then,
-// with one exception: the rotated gather (which follows the previous step's
-// k_finalize) issues it before its wait. The distance pass it releases reads
-// before its own wait only what the previous step's sort, plan and row moves
-// wrote, and those completed before the gather was launched. The step kernels
-// all issue it; each of them waits at its first statement, except the
-// tcgen05 passes, whose pre-wait part sets up shared memory and TMEM and
-// (distance pass after the gather only) stages data of earlier steps, and
-// the rotated gather.
+// this kernel's own wait, so that every kernel before it has completed, and by
+// every block of it, so that the pre-wait part of the next kernel runs beside
+// this one and beside nothing earlier. It may therefore read what kernels before
+// this one wrote, and write what only they read. Before their wait work:
+//   the tcgen05 passes: set up shared memory and TMEM and read the tile and pair
+//     lists (where the kernel ahead writes none of them: Dev::pre_b)
+//   k_argmin: the tile tables, the batch rows' norms, forced assignments
+//   k_finalize (run groups): plans, counts, norms and partials of the sort/plan
+//   k_update, its gather of the next batch into the other buffer set: beside it
+//     runs the sort/plan, which reads no batch rows. The last readers of that set
+//     were the previous step's row moves, and the distance pass and the argmin of
+//     this step have completed since. It reads the data, the caller's indices and
+//     the counter that the argmin left (gnext)
+//   k_gather_query, ahead of a chunk, into the other buffer set: beside it runs a
+//     chunk's distance pass, which reads its own set; the last readers of the
+//     other one, the kernels of the chunk before, have completed
+//   k_pp_draw: stages rows of the data
+// All others wait at their first statement.
 #define KKM_LAUNCH_DEPENDENTS() asm volatile("griddepcontrol.launch_dependents;" ::: "memory")
 
 // Raises `kern`'s dynamic shared-memory limit to `bytes` on the current device,
@@ -439,7 +447,6 @@ __device__ __forceinline__ float two_sum(float a, float b, float& e) {
 
 // ------------------------------------------------------------ launchers
 // All return cudaGetLastError() of their launches.
-cudaError_t launch_sample(const Dev& s, cudaStream_t st);
 cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st);
 // id0 >= 0: the rows are the data points id0 ..; ahead: see k_gather_query
 cudaError_t launch_gather_query(const Dev& s, const float* Q, int64_t ldq, int rows, int64_t id0, bool ahead,
@@ -514,7 +521,7 @@ cudaError_t launch_group_finalize(const GroupPhase& g, int blocks, cudaStream_t 
 // kernel kind and distance tile: tcgen05 (ctas persistent CTAs) ...
 cudaError_t launch_group_tc(const GroupPhase& g, int mode, int form, int kind, int tn, int ctas, cudaStream_t st);
 // ... or the FP32 CUDA-core passes
-cudaError_t launch_group_simt(const GroupPhase& g, int mode, int form, int blocks, cudaStream_t st);
+cudaError_t launch_group_simt(const GroupPhase& g, int mode, int blocks, cudaStream_t st);
 int sort_plan_smem(int k, int b);
 
 // ------------------------------------------------ full-batch kernel Lloyd

@@ -193,14 +193,6 @@ __device__ void warp_copy_row(const Dev& s, bool src_support, int64_t src_row, i
 }
 
 // ------------------------------------------------------------------ kernels
-__global__ void k_sample(Dev s) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= s.b) return;
-  const int64_t it = *s.iter;
-  const uint64_t c = (uint64_t)(it - 1) * (uint64_t)s.b + (uint64_t)t;
-  s.bidx[t] = (int32_t)index_below(splitmix64(s.seed, c), (uint64_t)s.n);
-}
-
 // One warp per batch slot: X[idx] -> batch row, norm, data index. With idx
 // NULL the slot's index is drawn here: SplitMix64 output (it-1)*b + slot.
 __device__ __forceinline__ void gather_one(const Dev& s, const int32_t* __restrict__ idx, int warp,
@@ -211,7 +203,6 @@ __device__ __forceinline__ void gather_one(const Dev& s, const int32_t* __restri
   } else {
     const uint64_t c = (uint64_t)(*it - 1) * (uint64_t)s.b + (uint64_t)warp;
     i = index_below(splitmix64(s.seed, c), (uint64_t)s.n);
-    if ((threadIdx.x & 31) == 0) s.bidx[warp] = (int32_t)i;
   }
   if (i < 0 || i >= s.n) {
     if ((threadIdx.x & 31) == 0) atomicOr(s.status, ST_BAD_BATCH_INDEX);
@@ -1601,11 +1592,6 @@ __global__ void __launch_bounds__(256) k_lloyd_dist(Dev g, LloydBuf L, float* __
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-cudaError_t launch_sample(const Dev& s, cudaStream_t st) {
-  k_sample<<<(s.b + 255) / 256, 256, 0, st>>>(s);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_gather_batch(const Dev& s, const int32_t* idx, cudaStream_t st) {
   cudaError_t e = launch_pdl(k_gather_batch, dim3((s.b * 32 + 255) / 256), dim3(256), 0, st, s, idx);
   if (e != cudaSuccess) return e;
