@@ -215,47 +215,56 @@ __device__ __forceinline__ void wgram_simt_item(const Dev& s, int w, GramSmem<4>
     const int rs = r0 + pr.rt * BM, cs = c0 + pr.ct * BN;
     float acc[4][4];
     gram_tile<4, false>(s.y32 + (base + rs) * s.ld, s.y32 + (base + cs) * s.ld, s.ld, acc, sm);
-    // FP64 issues at 1/64 of the FP32 rate on this chip, so the row weight is
-    // taken out of the column sums: a conversion and one to two FP64 operations
-    // per element where the product of both weights took four to five
-    double yw[4];
-    float yn[4];
-    int yi[4], qp[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int qc = pr.ct * BN + tx * 4 + j;
-      qp[j] = qc < cn ? cs + tx * 4 + j : -1;            // position in the region
-      const int64_t q = base + (qp[j] >= 0 ? qp[j] : cs);
-      yn[j] = s.yn[q];
-      yi[j] = s.yi[q];
-      yw[j] = pr.kind == 0 && qp[j] >= 0 && qp[j] < P.tail_c ? s.wwin64[q] : 0.0;
-    }
-    double sA = 0.0, sB = 0.0, sE = 0.0, sM = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int pr_ = pr.rt * BM + ty * 4 + i;         // row offset inside its range
-      if (pr_ >= rn) continue;
-      const int64_t p = base + rs + ty * 4 + i;
-      const float xn = s.yn[p];
-      const int xi = s.yi[p];
-      double ra = 0.0, rb = 0.0, re = 0.0;             // this row's W (not D), D and B columns
+    // FP64 issues at 1/64 of the FP32 rate on this chip. The row weight is taken
+    // out of the column sums, and a thread's 16 kernel values go through FP64 once
+    // for every class of columns that the item has (0 dropped rows, 1 the rest of
+    // the old window, 2 the new block; most items have one): a conversion and one
+    // FMA a value. With every value's class decided in the FP64 code 90 % of 8192
+    // rows in one of two centers, d = 64, took 2460 us a step, 2000 now.
+    const int c1 = pr.kind == 0 ? P.head_new : c0, c2 = pr.kind == 0 ? P.tail_c : c0, cend = c0 + cn;
+    float kv[4][4];
+    {
+      float yn[4];
+      int yi[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (qp[j] < 0) continue;
-        const double kv = (double)kernel_from_gram(s.kind, acc[i][j], xn, yn[j], xi == yi[j], s.negc,
-                                                   (float)s.coef0, s.degree);
-        if (pr.kind != 0) sM += kv;
-        else if (qp[j] >= P.tail_c) re += kv;
-        else if (qp[j] < P.head_new) rb += yw[j] * kv;
-        else ra += yw[j] * kv;
+        const int64_t q = base + min(cs + tx * 4 + j, cend - 1);
+        yn[j] = s.yn[q];
+        yi[j] = s.yi[q];
       }
-      if (pr.kind == 0) {
-        const double wp = s.wwin64[p];
-        sA += wp * (ra + rb);
-        sB += wp * rb;
-        sE += wp * re;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t p = base + rs + ty * 4 + i;
+        const float xn = s.yn[p];
+        const int xi = s.yi[p];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          kv[i][j] = kernel_from_gram(s.kind, acc[i][j], xn, yn[j], xi == yi[j], s.negc, (float)s.coef0, s.degree);
       }
     }
+    double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int cls = 0; cls < 3; ++cls) {
+      const int lo = cls == 0 ? c0 : cls == 1 ? c1 : c2, hi = cls == 0 ? c1 : cls == 1 ? c2 : cend;
+      if (max(lo, cs) >= min(hi, cs + BN)) continue;   // the item has no such columns
+      double yw[4];
+      bool in[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = cs + tx * 4 + j;
+        in[j] = c >= lo && c < hi;
+        yw[j] = cls < 2 && in[j] ? s.wwin64[base + c] : 1.0;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (pr.rt * BM + ty * 4 + i >= rn) continue;
+        double r = 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r = fma(yw[j], (double)(in[j] ? kv[i][j] : 0.0f), r);
+        sum[cls] = pr.kind == 0 ? fma(s.wwin64[base + rs + ty * 4 + i], r, sum[cls]) : sum[cls] + r;
+      }
+    }
+    const double sA = sum[0] + sum[1], sB = sum[0], sE = pr.kind == 0 ? sum[2] : 0.0, sM = pr.kind == 0 ? 0.0 : sum[2];
     // fixed-order block reduction of the four sums: two levels hand half of them
     // to the other lane, so that lanes 0, 8, 16, 24 end with sA, sE, sB, sM
     {
