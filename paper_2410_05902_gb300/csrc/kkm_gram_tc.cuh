@@ -902,7 +902,8 @@ __device__ __forceinline__ void window_item(const Dev& s, Shared<TNV>& sh, uint3
           float2 w2 = *reinterpret_cast<const float2*>(&m.col[1][c]);
           const int2 i2 = *reinterpret_cast<const int2*>(&m.col[2][c]);
           if (cls == 2) w2 = make_float2(1.0f, 1.0f);
-          const bool in0 = c >= lo && c < hi, in1 = c + 1 >= lo && c + 1 < hi;
+          const unsigned o = (unsigned)(c - lo), span = (unsigned)(hi - lo);
+          const bool in0 = o < span, in1 = o + 1u < span;
           w2 = make_float2(in0 ? w2.x : 0.0f, in1 ? w2.y : 0.0f);
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -1313,11 +1314,13 @@ __device__ __forceinline__ void dist_tc_body(const Dev& s, int rows, const CUten
   if (!desc_pre) ranges();
   const int nw = rw.hi - rw.lo, n = nw + rd.hi - rd.lo;
   // All epilogue groups on each item (instead of a team per item) when the run
-  // has fewer than NTEAM distance items per SM. The choice depends on the run
-  // alone, never on how a launch splits its items, so an item's sums come out
-  // the same in a run's own launch and in a run group's. (A window item's do
-  // either way.)
-  const bool all_d = total < Geo<TNV>::NTEAM * s.num_sms, all_w = np < WG::NTEAM * s.num_sms;
+  // has fewer than NTEAM distance items, or fewer than one window item, per SM.
+  // The choice depends on the run alone, never on how a launch splits its items,
+  // so an item's sums come out the same in a run's own launch and in a run
+  // group's. (Window items on all groups up to NTEAM per SM: single steps with
+  // half of 1024 rows in one of 100 centers 53.7 and 51.5 us; never: 2000 x 16,
+  // b = 256, 34.0 and 34.9.)
+  const bool all_d = total < Geo<TNV>::NTEAM * s.num_sms, all_w = np < s.num_sms;
 
   if (warp == 0) {
     // ------------------------------------------------- operand producer (one warp)
