@@ -175,8 +175,10 @@ kkm_status kkm_form_supported(int32_t precision, int32_t cc_major, int32_t cc_mi
  * KKM_ENOTSUP when cfg->precision is not FP32 and the device is not compute
  * capability 10.3 (see kkm_form_supported).
  * Allocates all device state up front: the support store of k*(2*tau + 4*b + 8)
- * rows (k*(1 + b*max_iters) when untruncated) and the step workspaces. No
- * later call allocates. Sets ||C_1^j||^2 = K(x, x). */
+ * rows (k*(1 + b*max_iters) when untruncated), with 12 bytes of weights a row
+ * and another 4 (FP32 form: 12) for the weights before an update, two sets of
+ * batch buffers, and the step workspaces. No later call allocates. Sets
+ * ||C_1^j||^2 = K(x, x). */
 kkm_status kkm_init(kkm_ctx** out, const float* X, int64_t n, int32_t d, int64_t ldx, int32_t k,
                     const kkm_kernel* kernel, int32_t b, const kkm_config* cfg,
                     const int64_t* init_idx, void* stream);
@@ -374,8 +376,10 @@ kkm_status kkm_stats(kkm_ctx* ctx, int64_t* steps, int64_t* support_rows, int64_
  * > 1 the step launches the kernel R times back to back between the two
  * events (it is idempotent: it rewrites the same partial sums from the same
  * inputs) and the record is the average, which leaves out the launch gap
- * that a single launch between two events includes. enable must be in
- * [0, 1000] (KKM_EINVAL otherwise). kkm_timing_read synchronises and writes
+ * that a single launch between two events includes. The window pass of the
+ * step has a launch of its own outside the record; within kkm_steps and
+ * kkm_steps_host, untimed, its items share the next step's distance launch.
+ * enable must be in [0, 1000] (KKM_EINVAL otherwise). kkm_timing_read synchronises and writes
  * the launches recorded and the sum of their per-launch milliseconds (host).
  * reset != 0 clears the record. */
 kkm_status kkm_timing_enable(kkm_ctx* ctx, int32_t enable);
