@@ -311,16 +311,19 @@ __device__ __forceinline__ double sum_partials(const double* p, int n) {
 }
 
 // Whether this warp's `m` arrivals are the last of `of` on the counter; what
-// the earlier ones wrote before theirs is then visible.
+// the earlier ones wrote before theirs is then visible. (Release and acquire on
+// the atomic itself.)
 __device__ __forceinline__ bool last_arrival(int32_t* counter, int m, int of) {
   int last = 0;
+  __syncwarp();
   if ((threadIdx.x & 31) == 0) {
-    __threadfence();
-    last = atomicAdd(counter, m) + m == of;
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(before) : "l"(counter), "r"(m) : "memory");
+    last = before + m == of;
   }
-  if (!__shfl_sync(0xffffffffu, last, 0)) return false;
-  __threadfence();
-  return true;
+  last = __shfl_sync(0xffffffffu, last, 0);
+  __syncwarp();
+  return last != 0;
 }
 
 // Where a window item's sums go.
